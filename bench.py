@@ -401,6 +401,10 @@ def time_window(win, steps, barrier, reduce_max, sampler=None):
     return ms, committed, ctx_mid, int(launches)
 
 
+# the kernels that read the weight matrices: "layers" is the one launch that runs all layers of a pass of few rows
+MATRIX_KERNELS = ("layers", "gemm", "gemm_lm_head_argmax")
+
+
 def kernel_shares(win, steps=6):
     """Share of each kind of kernel in the step, from a separate pass with an event pair around every launch (the
     pairs serialise the launches, so only the shares are used, never the absolute times)."""
@@ -495,18 +499,19 @@ def main():
 
     roofline = roofline_of_step(shape, B, k, ctx_mid, ms_step, peaks)
     roofline["peak_source"] = peaks["source"]
-    roofline["what"] = "whole verify step (draft, embedding, %d layers x 5 kernels, LM head + argmax, accept), graph-replayed" % shape.n_layers
+    roofline["what"] = "whole verify step (draft, embedding, %d layers, LM head + argmax, accept), graph-replayed" % shape.n_layers
     shares = kernel_shares(win)
     M = B * (k + 1)
-    gemm_share = sum(shares[n]["share"] for n in ("gemm", "gemm_lm_head_argmax") if n in shares)
-    gemm_launches = sum(shares[n]["launches_per_step"] for n in ("gemm", "gemm_lm_head_argmax") if n in shares)
+    gemm_share = sum(shares[n]["share"] for n in MATRIX_KERNELS if n in shares)
+    gemm_launches = sum(shares[n]["launches_per_step"] for n in MATRIX_KERNELS if n in shares)
     gemm_bytes = gemm_bytes_per_step(shape, M)
     gemm_us = gemm_share * ms_step * 1e3
     traffic = NCU_TRAFFIC.get((cfg.index, B, k))
     roofline["traffic"] = traffic["bytes_per_launch"] if traffic and traffic["kernel_sha256_16"] == kernel_digest() else None
     roofline["kernel_shares"] = shares
     roofline["dominant_kernel"] = {
-        "name": "gemm_fused_kernel (tcgen05 + TMA, cluster split-K, fused epilogues; 4 launches per layer + LM head)",
+        "name": ("layers_kernel (all decoder layers, attention included, as one cooperative launch) + LM head" if "layers" in shares else
+                 "gemm_fused_kernel (tcgen05 + TMA, cluster split-K, fused epilogues; 4 launches per layer + LM head)"),
         "share_of_step": gemm_share, "launches_per_step": gemm_launches,
         "bytes_per_launch": gemm_bytes / max(gemm_launches, 1), "us_per_launch": gemm_us / max(gemm_launches, 1),
         "achieved_gbs": gemm_bytes / max(gemm_us, 1e-9) / 1e3, "frac": gemm_bytes / max(gemm_us, 1e-9) / 1e3 / peaks["hbm_gbs"],

@@ -18,6 +18,8 @@ struct StepPlans {
     uint64_t rows;
     CUtensorMap tm_h, tm_o, tm_act, tm_h_lm;
     tasc::FusedPlan p_qkv, p_o, p_gu, p_down, p_lm;
+    bool persist;                                   // the layers run as one kernel (forward_persist.cu)
+    tasc::PersistPlan pp;
 };
 
 struct tasc_model {
@@ -28,12 +30,14 @@ struct tasc_model {
     std::vector<const float*> attn_norm, mlp_norm;
     std::vector<const void*> wqkv, wo, w_gate_up, w_down;
     float2* rope;                                   // [max_positions][head_dim / 2] (cos, sin), library-owned
+    tasc::LayerWeights* d_layers;                   // bf16 models: device copy of the layers' weight pointers, behind the rope table
     // tensor maps of the weight matrices (bf16 models): box = 64 columns x 128 rows (gate/up: 64 rows, see EPI_SWIGLU)
     std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
     CUtensorMap tm_lm;
     int qkv_rows, q_dim, kv_dim;
     int few_tiles;                                  // token tiles for 49..128 rows (see gemm_token_tile), from the layer's weight bytes
     double layer_mb;                                // projection weights of one layer, MB
+    bool aligned32;                                 // every layer matrix starts on a 32-byte boundary (forward_persist.cu)
     mutable std::mutex plan_mu;
     mutable std::vector<StepPlans> plans;           // most recently used last; a handful of (B, k, workspace) combinations
 };
@@ -68,8 +72,13 @@ struct Workspace {
     float* att_scratch;
     float* ssq;                   // [M][ceil(d / 128)] partial sums of squares of the residual rows (bf16 models)
     int ssq_slots;
+    double* ssq64;                // bf16 models, passes whose layers run as one kernel: [2 n_layers + 1][rows]
+    float* att_part;              // ... and their parked key ranges
+    unsigned* counters;           // ... grid barrier, attention groups
     size_t bytes;
 };
+
+constexpr int COUNTER_BAR = 0, COUNTER_GROUPS = 64, COUNTER_WORDS = COUNTER_GROUPS + PERSIST_MAX_GROUPS;
 
 // Rows a pass may carry: TASC_MAX_ROWS per sequence for a verify step, and for bf16 models at least PREFILL_ROWS
 // in all, so that a prefill of few sequences still runs passes of hundreds of rows (weights are read once per pass).
@@ -125,6 +134,10 @@ Workspace layout_workspace(const tasc_model* m, int B, void* base_) {
     w.att_scratch = L.take<float>(base, att_bytes / sizeof(float));
     w.ssq_slots = (d.d_model + 127) / 128;
     w.ssq = L.take<float>(base, M * w.ssq_slots * 4);      // passes of more than 128 rows keep four slots per 128 features
+    const bool bf16 = d.dtype == TASC_BF16;
+    w.ssq64 = L.take<double>(base, bf16 ? (size_t)(2 * d.n_layers + 1) * PERSIST_MAX_ROWS : 1);
+    w.att_part = L.take<float>(base, bf16 ? (size_t)PERSIST_MAX_UNITS * 16 * (d.head_dim + 2) : 1);
+    w.counters = L.take<unsigned>(base, bf16 ? COUNTER_WORDS : 1);
     w.bytes = L.off;
     return w;
 }
@@ -206,8 +219,24 @@ tasc_status forward_f32(const tasc_model* m, const tasc_kv* kv, const Workspace&
     return TASC_OK;
 }
 
+// Whether the layers of a pass run as one persistent kernel (forward_persist.cu).  Its phases cost about 2.5 us less than
+// kernels of their own, but a CTA reads the activations of all its token rows itself, so what it loses grows with rows
+// times width.  A step in us, five kernels per layer against one kernel:
+//     rows            7 MB per layer (135M)      30 MB (0.5B)             94 MB (1.5B)
+//     up to 8         798 / 578 - 818 / 591      897 / 652 - 940 / 702    1350 / 1122 - 1419 / 1172
+//     9 - 16          830 / 620 - 811 / 628      919 / 829 - 910 / 826    1412 / 1658
+//     17 - 32         857 / 770 - 868 / 789      951 / 972                -
+//     33 - 64         1006 / 814 - 945 / 819     -                        -
+//     96, 380 keys    1033 / 1077                -                        -
+// Its attention has at most one unit per SM and 12 key ranges, so the keys of a unit are bounded too (94 MB per layer, one
+// sequence of 4,000 tokens: 1559 / 1427 at 341 keys per unit).
+bool persist_pays(const tasc_model* m, int M, int max_ctx, const PersistPlan& pp) {
+    if (max_ctx / pp.splits > 512) return false;
+    return M <= 8 || (M <= 16 && m->layer_mb <= 48.0) || (M <= 64 && m->layer_mb <= 12.0);
+}
+
 // bf16 models: five launches per layer (QKV+RoPE+KV append, attention, O+residual, gate/up+SiLU*mul, down+residual),
-// each with programmatic stream serialisation; see gemm_fused.cu and attention_mma.cu.
+// each with programmatic stream serialisation (gemm_fused.cu, attention_mma.cu), or one launch for all layers.
 tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace& w, const RowSource& src, int B, int R,
                          bool lm_head, float* logits, cudaStream_t s) {
     const tasc_model_desc& d = m->desc;
@@ -230,6 +259,10 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
             const double big_mb = 2.0 * 2.0 * (double)d.d_ff * d.d_model / 1e6;      // the largest matrix of a layer (gate/up)
             const bool wide_pass = M > 128 && big_mb >= WIDE_MATRIX_MB && (M >= WIDE_ROWS || m->layer_mb >= WIDE_LAYER_MB);
             const double wide_min_mb = wide_pass ? WIDE_MATRIX_MB : -1.0;
+            sp.persist = !wide_pass && m->aligned32 &&
+                         plan_persist(d.n_layers, M, B, R, d.d_model, m->q_dim, d.n_q_heads, d.n_kv_heads, d.head_dim, d.d_ff, max_ctx,
+                                      d.page_size, sp.pp) &&
+                         persist_pays(m, M, max_ctx, sp.pp);
             sp.TB = gemm_token_tile(M, true, m->few_tiles, wide_min_mb >= 0.0);
             sp.rows = (uint64_t)((M + sp.TB - 1) / sp.TB) * 2 * sp.TB;
             if ((st = encode_tmap_bf16(&sp.tm_h, w.h, sp.rows, d.d_model, 2 * sp.TB)) != TASC_OK) return st;
@@ -265,9 +298,26 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
     base.status = w.status;
 
     launch_rows_embed(w.rp, src.seqs->tokens, src.seqs->stride, src.seqs->len, src.seqs->stop_len, src.drafts, B, R, src.chunk,
-                      d.vocab, w.status, static_cast<const __nv_bfloat16*>(m->embed), m->attn_norm[0], w.x, h, w.ssq, ssq_slots,
-                      lm_head ? w.argmax : nullptr, d.d_model, TB, s);
-    for (int l = 0; l < d.n_layers; ++l) {
+                      d.vocab, w.status, static_cast<const __nv_bfloat16*>(m->embed), m->attn_norm[0], w.x, h,
+                      w.ssq, ssq_slots, lm_head ? w.argmax : nullptr, d.d_model, TB, sp.persist ? w.ssq64 : nullptr, 2 * d.n_layers + 1,
+                      w.counters, sp.persist ? COUNTER_GROUPS + sp.pp.n_units / sp.pp.splits : 0, s);
+    if (sp.persist) {
+        PersistArgs a = {};
+        a.layers = m->d_layers; a.n_layers = d.n_layers; a.M = M; a.R = R; a.TBL = TB;
+        a.d = d.d_model; a.qd = m->q_dim; a.dff = d.d_ff; a.n_q = d.n_q_heads; a.n_kv = d.n_kv_heads; a.hd = d.head_dim;
+        a.inv_d = base.inv_d; a.eps = base.eps; a.scale_log2e = 1.4426950408889634f / sqrtf((float)d.head_dim);
+        a.h = h; a.o = o; a.act = act; a.q = w.q; a.x0 = w.x; a.ssq = w.ssq64;
+        a.row_pos = w.rp.row_pos; a.seq_pos0 = w.rp.seq_pos0; a.seq_rows = w.rp.seq_rows;
+        a.block_table = kv->block_table; a.max_pages = kv->max_pages_per_seq; a.page_size = d.page_size; a.n_pages = kv->n_pages;
+        a.kv_pool = static_cast<__nv_bfloat16*>(kv->pool);
+        a.kv_half = (size_t)kv->n_pages * d.n_kv_heads * d.page_size * d.head_dim;
+        a.rope = m->rope; a.max_positions = d.max_positions;
+        a.part = w.att_part; a.bar = w.counters + COUNTER_BAR; a.unit_ctr = w.counters + COUNTER_GROUPS;
+        a.status = w.status;
+        if ((st = launch_persist(a, sp.pp, s)) != TASC_OK) return st;
+        base.ssq64 = w.ssq64 + (size_t)2 * d.n_layers * M;
+    }
+    for (int l = 0; l < d.n_layers && !sp.persist; ++l) {
         const KvView kvl = layer_kv(m, kv, l);
         FusedArgs a = base;
         a.N = m->qkv_rows; a.K = d.d_model; a.ssq_in = w.ssq;
@@ -384,6 +434,8 @@ extern "C" tasc_status tasc_model_create(const tasc_model_desc* desc, const tasc
         m->layer_mb = layer_mb;
     }
     m->rope = nullptr;
+    m->d_layers = nullptr;
+    m->aligned32 = true;
     for (int l = 0; l < d.n_layers; ++l) {
         if (!wt->attn_norm[l] || !wt->wqkv[l] || !wt->wo[l] || !wt->mlp_norm[l] || !wt->w_gate_up[l] || !wt->w_down[l]) {
             delete m;
@@ -392,6 +444,8 @@ extern "C" tasc_status tasc_model_create(const tasc_model_desc* desc, const tasc
         m->attn_norm.push_back(wt->attn_norm[l]); m->mlp_norm.push_back(wt->mlp_norm[l]);
         m->wqkv.push_back(wt->wqkv[l]); m->wo.push_back(wt->wo[l]);
         m->w_gate_up.push_back(wt->w_gate_up[l]); m->w_down.push_back(wt->w_down[l]);
+        for (const void* p : {wt->wqkv[l], wt->wo[l], wt->w_gate_up[l], wt->w_down[l]})
+            if (reinterpret_cast<uintptr_t>(p) % 32) m->aligned32 = false;
     }
     tasc_status st = TASC_OK;
     if (d.dtype == TASC_BF16) {
@@ -407,12 +461,23 @@ extern "C" tasc_status tasc_model_create(const tasc_model_desc* desc, const tasc
     }
     if (st == TASC_OK) {
         const size_t n = (size_t)d.max_positions * (d.head_dim / 2);
-        if (cudaMalloc(reinterpret_cast<void**>(&m->rope), n * sizeof(float2)) != cudaSuccess) {
+        std::vector<LayerWeights> lw;
+        auto mat = [](const void* p) { return static_cast<const __nv_bfloat16*>(p); };
+        for (int l = 0; l < d.n_layers && d.dtype == TASC_BF16; ++l)
+            lw.push_back(LayerWeights{mat(m->wqkv[l]), mat(m->wo[l]), mat(m->w_gate_up[l]), mat(m->w_down[l]), m->mlp_norm[l],
+                                      l + 1 < d.n_layers ? m->attn_norm[l + 1] : m->final_norm});
+        const size_t lw_bytes = lw.size() * sizeof(LayerWeights);
+        if (cudaMalloc(reinterpret_cast<void**>(&m->rope), n * sizeof(float2) + lw_bytes) != cudaSuccess) {
             (void)cudaGetLastError();
             st = TASC_ENOMEM;
         } else {
             launch_rope_table(m->rope, d.max_positions, d.head_dim, d.rope_base, nullptr);
-            if (cudaDeviceSynchronize() != cudaSuccess) { (void)cudaGetLastError(); st = TASC_ECUDA; }
+            m->d_layers = reinterpret_cast<LayerWeights*>(m->rope + n);
+            if ((lw_bytes && cudaMemcpyAsync(m->d_layers, lw.data(), lw_bytes, cudaMemcpyHostToDevice, nullptr) != cudaSuccess) ||
+                cudaDeviceSynchronize() != cudaSuccess) {
+                (void)cudaGetLastError();
+                st = TASC_ECUDA;
+            }
         }
     }
     if (st != TASC_OK) {

@@ -379,7 +379,8 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
             for (int t = threadIdx.x; t < TB; t += 128) {
                 const int m = t0 + t;
                 float ss = 0.f;
-                if (m < a.M)
+                if (m < a.M && a.ssq64) ss = (float)a.ssq64[m];
+                else if (m < a.M)
                     for (int j = 0; j < a.ssq_slots; ++j) ss += a.ssq_in[(size_t)m * a.ssq_slots + j];
                 s_inv[t] = 1.0f / sqrtf(ss * a.inv_d + a.eps);
             }

@@ -7,7 +7,7 @@ namespace tasc {
 
 // ------------------------------------------------------------------ launch accounting (profile.cu)
 enum Kind { K_DRAFT, K_ROWS, K_EMBED, K_GEMM, K_GEMM_LM, K_QKV_ROPE, K_ATT_SPLIT, K_ATT_COMBINE, K_RESNORM, K_SILU,
-            K_ACCEPT, K_OTHER, K_COUNT };
+            K_ACCEPT, K_OTHER, K_LAYERS, K_COUNT };
 void prof_begin(int kind, cudaStream_t s);     // counts the launch; records an event when timing is enabled
 void prof_end(int kind, cudaStream_t s);
 bool profiling_enabled();                      // per-launch event timing is on (tasc_profile_enable)
@@ -60,6 +60,7 @@ struct FusedArgs {
     int num_kb, BN, TB, TBL, stages, pair, data_bytes; // filled in by launch_gemm_fused from the plan
     int BNW, n_ft, n_tt;               // many-row kernel (gemm_wide.cu): features per MMA, feature tiles, token tiles
     int early;                         // the epilogue's global operands were complete before the preceding grid began
+    const double* ssq64;               // [M] sums of squares of the input rows (instead of ssq_in, behind the one-kernel layers)
     const float* ssq_in;               // [M][ssq_slots] partial sums of squares of the input rows (null: no scaling)
     int ssq_slots;
     float inv_d, eps;                  // rms factor = 1 / sqrt(sum(ssq) * inv_d + eps)
@@ -104,6 +105,53 @@ tasc_status launch_gemm_wide(int epi, const CUtensorMap* tmW, const CUtensorMap*
 tasc_status launch_gemm_fused(int epi, const CUtensorMap* tmW, const CUtensorMap* tmX, FusedArgs a, const FusedPlan& p,
                               cudaStream_t stream);
 
+// ------------------------------------------------------------------ all layers of a pass of few rows in one kernel (forward_persist.cu)
+constexpr int PERSIST_MAX_ROWS = 64;         // token rows of a pass
+constexpr int PERSIST_MAX_LAYERS = 64;
+constexpr int PERSIST_MAX_SPLITS = 12;       // key ranges per (sequence, KV head, slab of 16 query rows)
+constexpr int PERSIST_MAX_UNITS = 256;       // attention units of a pass whose key ranges are split
+constexpr int PERSIST_MAX_GROUPS = 4096;
+struct LayerWeights {
+    const __nv_bfloat16 *wqkv, *wo, *w_gate_up, *w_down;
+    const float *gain_mlp, *gain_next;       // norm gains of the MLP input and of the next layer's input (or the final norm)
+};
+struct PersistPlan {
+    int T;                                   // token rows per CTA / 8
+    int grid, n_tb, n_rb;                    // CTAs; token blocks x row blocks of the projections
+    int nt_res, nt_qkv;                      // 16-row tiles per row block of a residual projection, tiles of 8 row pairs of the QKV product
+    int lr[4];                               // QKV, O, gate/up, down: log2 of the row groups the warps form
+    int union_bytes, smem_bytes;
+    int splits, n_slabs, n_units;            // attention: key ranges, slabs of 16 query rows, units in all
+};
+struct PersistArgs {
+    const LayerWeights* layers;              // device, [n_layers]
+    int n_layers, M, R, TBL;
+    int d, qd, dff, n_q, n_kv, hd;
+    float inv_d, eps, scale_log2e;
+    __nv_bfloat16 *h, *o, *act;              // (hi, lo) activation buffers; h: blocks on entry, layout tiles of TBL tokens on return
+    float* q;                                // [M][qd]
+    const float* x0;                         // [M][d] embedding rows
+    double* ssq;                             // [2 n_layers + 1][M] sums of squares of the residual rows: the embedding's on entry, zeros
+                                             // behind it; the last M are the final rows' on return
+    const int *row_pos, *seq_pos0, *seq_rows;
+    const int32_t* block_table;
+    int max_pages, page_size;
+    long long n_pages;
+    __nv_bfloat16* kv_pool;
+    size_t kv_half;                          // elements of one layer's K (or V) pages
+    const float2* rope;
+    int max_positions;
+    float* part;                             // [n_units][16][hd + 2] parked key ranges
+    unsigned *unit_ctr, *bar;                // zero on entry
+    int* status;
+    unsigned r_magic, tbl_magic;             // filled in by launch_persist, like the rest
+    int page_shift;
+    int n_tb, n_rb, nt_res, nt_qkv, park_bytes, lr[4], union_bytes, splits, n_slabs, n_units;      // from the plan
+};
+// Returns false where the pass does not take this path.
+bool plan_persist(int n_layers, int M, int B, int R, int d, int qd, int n_q, int n_kv, int hd, int dff, int max_ctx, int page_size, PersistPlan& p);
+tasc_status launch_persist(PersistArgs a, const PersistPlan& p, cudaStream_t stream);
+
 // ------------------------------------------------------------------ float32 GEMM for the f32 model (gemm_simt.cu)
 // Same contract with splits = 1: P[0][m][n].
 void launch_gemm_f32(const float* X, const float* W, float* partials, int M, int N, int K,
@@ -129,11 +177,13 @@ template <typename T>
 void launch_embed_norm(const T* embed, const int* row_tok, const float* gain, float eps, float* x, T* h, int M, int d,
                        int TB, cudaStream_t stream);
 // bf16 model, first launch of a forward: row plan (chunk < 0: verify step, else prefill chunk) + embedding:
-// x[m] = embed[tok]; a_out = (hi, lo) of x * gain; ssq[m][0] = sum x^2, other slots 0; argmax[m] = 0 (if given).
+// x[m] = embed[tok]; a_out = (hi, lo) of x * gain; ssq[m][0] = sum x^2, other slots 0; argmax[m] = 0 (if given);
+// ssq64 given (the layers follow as one kernel): a_out in its blocks of 8 tokens x 64 features, ssq64[0][m] = sum x^2,
+// ssq64[1 .. n_stage)[m] = 0, and zero[0 .. n_zero) = 0 (the kernel's counters).
 void launch_rows_embed(const RowPlan& rp, const int32_t* tokens, int64_t stride, const int32_t* len, const int32_t* stop_len,
                        const int32_t* drafts, int B, int R, int chunk, int vocab, int* status, const __nv_bfloat16* embed,
                        const float* gain, float* x, __nv_bfloat16* a_out, float* ssq, int ssq_slots, unsigned long long* argmax,
-                       int d, int TB, cudaStream_t stream);
+                       int d, int TB, double* ssq64, int n_stage, unsigned* zero, int n_zero, cudaStream_t stream);
 // x += sum_s P[s]; h = RMSNorm(x) * gain  (gain == null: only the residual update)
 template <typename T>
 void launch_residual_norm(const float* partials, int splits, float* x, const float* gain, float eps, T* h, int M, int d,

@@ -12,7 +12,7 @@ namespace {
 
 const char* const KIND_NAMES[K_COUNT] = {
     "draft", "rows", "embed_norm", "gemm", "gemm_lm_head_argmax", "qkv_rope_append", "attention_split",
-    "attention_combine", "residual_norm", "silu_mul", "accept", "other"};
+    "attention_combine", "residual_norm", "silu_mul", "accept", "other", "layers"};
 
 std::atomic<unsigned long long> g_launches[K_COUNT];
 std::atomic<int> g_enabled{0};

@@ -357,6 +357,22 @@ def test_many_row_kernel_on_every_product_with_64_wide_heads():
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("hd", [64, 128])
+@pytest.mark.parametrize("B,k,P", [(1, 1, 2), (1, 7, 127), (1, 8, 128), (2, 7, 129), (3, 5, 40), (8, 3, 200), (8, 7, 33), (1, 5, 1600)])
+def test_one_kernel_for_all_layers(B, k, P, hd):
+    """Passes whose layers run as one kernel: 2 to 64 rows (one, two and four tiles of 8, full and ragged), contexts that
+    end just before, at and just behind a tile of 128 keys, one key range and as many as there can be; heads of 64 and
+    of 128.  Two layers; the oracle runs the first and the last sequence."""
+    from dataclasses import replace
+    cfg = replace(configs.shrunk(configs.get(1), n_layers=2, vocab=4096, n_docs=500), prompt_len=P)
+    if hd == 128:
+        cfg = replace(cfg, model=replace(cfg.model, d_model=512, n_q_heads=4, n_kv_heads=2, head_dim=128, d_ff=1088))
+    s = make_setup(cfg)
+    prompts = corpus.make_prompts(cfg, B, prompt_len=P)
+    check(lockstep(s, prompts, k + 3, k, oracle_rows=sorted({0, B - 1}), **BF16_TOL), f"one kernel for all layers, heads of {hd}, B={B} k={k} P={P}")
+
+
+@pytest.mark.gpu
 def test_config4_full_depth_batch1():
     """The 1.5B shape at its full depth (28 layers, vocabulary 151,936, prompt of 1,024 tokens), one sequence,
     four or more steps; the corpus tables come from the first 20,000 documents."""
