@@ -6,13 +6,13 @@
 // occurrences (left to right, non-overlapping, inside each document) before the next iteration.  The prefix-collision
 // test of the paper needs the tokens' strings; ids have none, so every candidate passes.
 //   Counting is the drafter's machinery: one open-addressing table keyed by the full packing of (n, tokens), one
-//   128-bit compare-and-swap per window, plus an atomic minimum of the window's position, which makes the argmax
-//   unique: largest reward, then the longer n-gram, then the one that occurs first.  The documents stay at their
-//   original offsets and only get shorter, so a thread per document can rewrite its document in place.
-//   All iterations are enqueued without a host round trip; an iteration that finds nothing to merge (and every later
-//   one) does nothing.
+//   128-bit compare-and-swap per new n-gram.  The table is counted in full once and then kept up to date: a merge changes
+//   the windows that overlap a replaced occurrence and no others, so only those are taken out and put back.  The argmax
+//   is unique: largest reward, then the longer n-gram, then the one that occurs first; first occurrences are looked up
+//   only in rounds where the first two tie.  The documents stay at their original offsets and only get shorter.
+//   All rounds run in one cooperative kernel without a host round trip.
 // tasc_tok_init_rows -- Section 4.2: the embedding / LM-head row of an added token is the mean of its constituents'
-//   rows (a constituent may itself be an added token).  One thread per column walks the merges in order, so a row is
+//   rows (a constituent may itself be an added token).  A thread per column walks the merges in order, so a row is
 //   always complete when a later row needs it, with no synchronisation.
 // tasc_tok_encode -- Appendix on byte-pair encoding: text is encoded with the added tokens matched first and greedily
 //   (the longest added token whose expansion into base tokens matches the upcoming base tokens).  The added tokens'
@@ -31,172 +31,657 @@ constexpr int MAX_N = TASC_TOK_MAX_N;            // longest n-gram (the key hold
 constexpr int POS_BITS = 28;                     // window positions are below 2^28
 constexpr int LEN_BITS = 3;
 
-struct Winner { int n; int tok[MAX_N]; int done; };
+// What the merge loop shares across the grid.  Words that a later round uses again exist twice: one CTA prepares the one
+// while all others still read the other.
+struct TokState {
+    int n_merges, status;
+    int rebuild;                                 // the round before which the table has to be counted again (0: the first)
+    unsigned int bar;                            // arrivals at the grid barrier
+    unsigned int first[2];                       // first position of the n-grams that tie
+    unsigned long long used[2];                  // slots claimed
+};
+// The best n-gram of a part of the table: its rank (reward and length), one slot that has it, and how many have it.
+struct __align__(16) Best { unsigned long long rank; unsigned int slot, ties; };
 
-// One window (n tokens starting at i) per thread and n-gram length; rem[i] = tokens after i inside its document.
-__global__ void tok_count_kernel(const int32_t* __restrict__ cur, const uint8_t* __restrict__ rem, int64_t T, int n,
-                                 uint64_t* keys, uint32_t* counts, uint32_t* first, uint64_t mask, const Winner* w, int* status) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (w->done || i >= T || rem[i] < n - 1) return;
-    Key key = key_make(n);
-    for (int j = 0; j < n; ++j) key_put(key, j, (uint32_t)cur[i + j]);
-    const uint64_t slot = table_upsert(keys, mask, key);
-    if (slot == ~0ull) { set_status(status, TASC_ECAPACITY); return; }
-    atomicAdd(&counts[slot], 1u);
-    atomicMin(&first[slot], (uint32_t)i);
+// A slot's word: n-gram length (3 bits) and count (29 bits; positions are below 2^28).
+constexpr uint32_t CNT_BITS = 29, CNT_MASK = (1u << CNT_BITS) - 1u;
+// (reward, length) of a word, 0 for a count of zero: reward = count * (length - 1)
+__device__ __forceinline__ unsigned long long tok_rank(uint32_t w) {
+    const uint32_t c = w & CNT_MASK, n = w >> CNT_BITS;
+    return c ? (((unsigned long long)c * (n - 1u)) << LEN_BITS) | n : 0ull;
 }
 
-// reward (33 bits) | n (3 bits) | 2^28 - 1 - first position (28 bits): one unsigned maximum picks the largest
-// reward, then the longer n-gram, then the earlier first occurrence
-__device__ __forceinline__ unsigned long long tok_rank(uint32_t count, int n, uint32_t first) {
-    const unsigned long long reward = (unsigned long long)count * (unsigned long long)(n - 1);
-    return (reward << (LEN_BITS + POS_BITS)) | ((unsigned long long)n << POS_BITS) |
-           (unsigned long long)(((1u << POS_BITS) - 1u) - first);
-}
-__device__ __forceinline__ int key_order(const Key& k) { return (int)((k.hi >> 56) & 0x7Full); }
+constexpr int TOK_THREADS = 1024, TOK_WARPS = TOK_THREADS / 32;
+constexpr int CHUNK_BITS = 7;                    // slots whose best n-gram is kept: 512 bytes of words, one load of a warp
+constexpr long long TOK_BARRIER_CYCLES = 20000000000ll;           // (a document of millions of tokens is one warp's work)
 
-__global__ void tok_best_kernel(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ counts,
-                                const uint32_t* __restrict__ first, uint64_t cap, unsigned long long* best, const Winner* w) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned long long r = 0;
-    if (!w->done && i < cap && counts[i]) {
-        const Key k = {keys[2 * i], keys[2 * i + 1]};
-        r = tok_rank(counts[i], key_order(k), first[i]);
+struct TokArgs {
+    int32_t* cur;                                // tokens at the documents' original offsets; -1 behind a document's end
+    uint8_t* rem;                                // tokens that follow in the document (255 = more)
+    uint8_t* mark;
+    const int32_t* doc_of;
+    const int64_t* offsets;
+    int32_t *doc_len, *doc_round;                // length now; last round + 1 in which the n-gram was found
+    int64_t n_docs, T;
+    uint64_t* keys;
+    uint32_t* words;
+    uint8_t* dirty;                              // per chunk of slots: its best has to be looked up again
+    Best *chunk_best, *cta_best;
+    uint64_t cap;
+    TokState* st;
+    int32_t* merges;
+    int base_vocab, budget, n_max;
+};
+
+// The table's slots come in pairs of one 32-byte sector; a key is in the first pair of its own sequence that had room.  (With
+// single slots one behind the other, the longest of the tens of thousands of look-ups of a round took over 30 trips to
+// L2, 18 us; now about four.)
+struct Probe {
+    uint64_t pair, step, mask;
+    __device__ __forceinline__ Probe(const TokArgs& a, const Key& key) {
+        const uint64_t h = key_hash(key);
+        mask = a.cap / 2 - 1;
+        pair = h & mask;
+        step = (h >> 36) | 1ull;
     }
+    __device__ __forceinline__ void next() { pair = (pair + step) & mask; }
+};
+struct KeyPair { ulonglong2 k[2]; };
+__device__ __forceinline__ KeyPair tok_pair(const TokArgs& a, uint64_t pair) {
+    KeyPair v;
+    asm volatile("ld.global.cg.v2.u64 {%0, %1}, [%2];" : "=l"(v.k[0].x), "=l"(v.k[0].y) : "l"(a.keys + 4 * pair) : "memory");
+    asm volatile("ld.global.cg.v2.u64 {%0, %1}, [%2];" : "=l"(v.k[1].x), "=l"(v.k[1].y) : "l"(a.keys + 4 * pair + 2) : "memory");
+    return v;
+}
+// Adds an occurrence of a window, or takes one out that was counted before this round.  1 if that claimed a slot.  (One loop
+// for both: the lanes of a warp make their trips to the table together.)
+__device__ __forceinline__ int tok_change(const TokArgs& a, const Key& key, int n, bool add, int round) {
+    Probe p(a, key);
+    for (uint64_t probe = 0; probe <= p.mask; ++probe, p.next()) {
+        const KeyPair v = tok_pair(a, p.pair);
+        Key k0 = {v.k[0].x, v.k[0].y}, k1 = {v.k[1].x, v.k[1].y};
+        bool claimed = false;
+        // (a half that is still zero may belong to a key that is being written)
+        if (add && (k0.lo == 0 || k0.hi == 0)) {
+            k0 = cas128(a.keys + 4 * p.pair, Key{0ull, 0ull}, key);
+            if (k0.lo == 0 && k0.hi == 0) { k0 = key; claimed = true; }
+        }
+        bool at0 = k0.lo == key.lo && k0.hi == key.hi;
+        if (add && !at0 && (k1.lo == 0 || k1.hi == 0)) {
+            k1 = cas128(a.keys + 4 * p.pair + 2, Key{0ull, 0ull}, key);
+            if (k1.lo == 0 && k1.hi == 0) { k1 = key; claimed = true; }
+        }
+        if (at0 || (k1.lo == key.lo && k1.hi == key.hi)) {
+            const uint64_t slot = 2 * p.pair + (at0 ? 0 : 1);
+            atomicAdd(&a.words[slot], !add ? 0xFFFFFFFFu : claimed ? ((uint32_t)n << CNT_BITS) + 1u : 1u);
+            a.dirty[slot >> CHUNK_BITS] = 1;
+            return claimed;
+        }
+        if (!add && k1.lo == 0 && k1.hi == 0) break;
+    }
+    a.st->rebuild = round + 1;                   // the table is full: all is counted again before the next round
+    return 0;
+}
+// Rank of a window's n-gram while no window is being added or taken out.
+__device__ __forceinline__ unsigned long long tok_rank_of(const TokArgs& a, const Key& key) {
+    Probe p(a, key);
+    for (uint64_t probe = 0; probe <= p.mask; ++probe, p.next()) {
+        const KeyPair v = tok_pair(a, p.pair);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (v.k[i].x == key.lo && v.k[i].y == key.hi) return tok_rank(__ldcg(a.words + 2 * p.pair + i));
+        if (v.k[1].x == 0 && v.k[1].y == 0) break;
+    }
+    return 0ull;
+}
+
+__device__ __forceinline__ void best_merge(Best& a, const Best& b) {
+    if (b.rank > a.rank) a = b;
+    else if (b.rank == a.rank && b.rank) { a.ties += b.ties; a.slot = min(a.slot, b.slot); }
+}
+__device__ __forceinline__ Best best_warp(Best v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long x = __shfl_xor_sync(0xFFFFFFFFu, r, o);
-        r = x > r ? x : r;
+        Best x;
+        x.rank = __shfl_xor_sync(0xFFFFFFFFu, v.rank, o);
+        x.slot = __shfl_xor_sync(0xFFFFFFFFu, v.slot, o);
+        x.ties = __shfl_xor_sync(0xFFFFFFFFu, v.ties, o);
+        best_merge(v, x);
     }
-    if ((threadIdx.x & 31) == 0 && r) atomicMax(best, r);
+    return v;
+}
+__device__ __forceinline__ Best best_load(const Best* p) {
+    const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(p));
+    return Best{v.x, (unsigned int)v.y, (unsigned int)(v.y >> 32)};
 }
 
-// The slot whose rank equals the maximum is the iteration's n-gram t*: recorded as merge number *n_merges.
-__global__ void tok_winner_kernel(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ counts,
-                                  const uint32_t* __restrict__ first, uint64_t cap, const unsigned long long* best,
-                                  Winner* w, int32_t* merges, int* n_merges) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (w->done) return;
-    const unsigned long long b = *best;
-    if (b == 0ull) {                                   // no n-gram left: this and every later iteration is empty
-        if (i == 0) { w->n = 0; }
-        return;
+constexpr int DOC_SMEM = 256;                    // documents up to this length are rewritten in shared memory
+constexpr int LIST_MAX = 512;                    // windows to take out or put in that a warp collects before it looks them up
+constexpr int HIT_MAX = 1024;                    // documents of one CTA that are handed out to its warps in a round
+struct TokWarp {
+    int old_tok[DOC_SMEM], new_tok[DOC_SMEM];
+    uint16_t list[LIST_MAX];                     // start (8 bits), length - 2 (3 bits), put in (1 bit)
+    uint8_t old_mark[DOC_SMEM], new_mark[DOC_SMEM];
+};
+struct TokShared {
+    Best red[TOK_WARPS];
+    int n, tok[MAX_N];                           // this round's n-gram
+    int stop;
+    int n_hits, next_hit;
+    int hits[HIT_MAX];
+    TokWarp warp[TOK_WARPS];
+};
+
+// Grid barrier; false when the wait ran out (a cooperative launch: all CTAs are resident).
+__device__ __forceinline__ bool tok_barrier(TokState* st, unsigned int& epoch, TokShared& sh) {
+    ++epoch;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&st->bar) : "memory");
+        const unsigned int target = epoch * gridDim.x;
+        const long long t0 = clock64();
+        for (;;) {
+            unsigned int v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&st->bar) : "memory");
+            if ((int)(v - target) >= 0) break;
+            if (clock64() - t0 > TOK_BARRIER_CYCLES) { set_status(&st->status, TASC_ETIMEOUT); sh.stop = 1; break; }
+        }
     }
-    if (i >= cap || !counts[i]) return;
-    const Key k = {keys[2 * i], keys[2 * i + 1]};
-    const int n = key_order(k);
-    if (tok_rank(counts[i], n, first[i]) != b) return;
-    const int at = *n_merges;                           // one thread gets here
-    w->n = n;
-    for (int j = 0; j < MAX_N; ++j) {
-        const int t = j < n ? (int)key_get(k, j) : -1;
-        w->tok[j] = t;
-        merges[(size_t)at * MAX_N + j] = t;
-    }
+    __syncthreads();
+    return sh.stop == 0;
 }
 
-// After the search: close the iteration (count the merge, or mark the procedure as finished).
-__global__ void tok_commit_kernel(Winner* w, int* n_merges, unsigned long long* best) {
-    if (w->done) return;
-    if (*best == 0ull || w->n == 0) w->done = 1;
-    else *n_merges += 1;
-    *best = 0ull;
-}
-
-// One thread per document: replaces the occurrences of t* (left to right, non-overlapping) by the new id, in place,
-// and rewrites the document's remaining-token counts.  new_id = base_vocab + (*n_merges - 1) after the commit.
-__global__ void tok_rewrite_kernel(int32_t* cur, uint8_t* rem, const int64_t* __restrict__ doc_start, int32_t* doc_len,
-                                   int64_t n_docs, const Winner* w, const int* n_merges, int base_vocab) {
-    const int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (d >= n_docs || w->done) return;
-    const int n = w->n;
-    const int new_id = base_vocab + *n_merges - 1;
-    int t[MAX_N];
+// A warp's list of windows: all lanes call everything.
+struct TokList {
+    TokWarp& w;
+    const int32_t *old_tok, *new_tok;            // what the starts in the list count from
+    int total;
+    // the windows of the 32 positions from c on that hold a mark; starts are relative to `base`
+    __device__ __forceinline__ void collect(const TokArgs& a, const uint8_t* mk, int L, int c, int base, bool add) {
+        const int lane = threadIdx.x & 31, i = c + lane;
+        // lengths of this position's windows that hold a mark: all from the first marked token on
+        int from = MAX_N + 1;
+        const int lim = min(a.n_max, L - i);
 #pragma unroll
-    for (int j = 0; j < MAX_N; ++j) t[j] = w->tok[j];
-    int32_t* doc = cur + doc_start[d];
-    uint8_t* r = rem + doc_start[d];
-    const int L = doc_len[d];
-    int rd = 0, wr = 0;
-    while (rd < L) {
-        bool hit = rd + n <= L;
-        for (int j = 0; hit && j < n; ++j) hit = doc[rd + j] == t[j];
-        if (hit) { doc[wr++] = new_id; rd += n; }
-        else { doc[wr++] = doc[rd++]; }
+        for (int j = MAX_N - 1; j >= 0; --j) if (j < lim && mk[i + j]) from = j + 1;
+        from = max(from, 2);
+        const int cnt = max(0, lim - from + 1);
+        int at = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, at, o);
+            if (lane >= o) at += y;
+        }
+        const int sum = __shfl_sync(0xFFFFFFFFu, at, 31);
+        at += total - cnt;
+        for (int j = 0; j < cnt; ++j) w.list[at + j] = (uint16_t)((i - base) | ((from + j - 2) << 8) | (add ? 1 << 11 : 0));
+        total += sum;
     }
-    if (wr == L) return;                                // nothing replaced: counts unchanged
-    doc_len[d] = wr;
-    for (int j = 0; j < L; ++j) {
-        const int left = wr - 1 - j;
-        r[j] = (uint8_t)(left < 0 ? 0 : (left > 255 ? 255 : left));
+    __device__ __forceinline__ bool full() const { return total + 32 * (MAX_N - 1) > LIST_MAX; }
+    // looks the windows up; returns the slots this lane has claimed
+    __device__ __forceinline__ int flush(const TokArgs& a, int round) {
+        int claimed = 0;
+        __syncwarp();
+        for (int p = threadIdx.x & 31; p < total; p += 32) {
+            const int e = w.list[p], m = ((e >> 8) & 7) + 2;
+            const bool add = (e >> 11) & 1;
+            const int32_t* tok = (add ? new_tok : old_tok) + (e & 255);
+            Key key = key_make(m);
+#pragma unroll
+            for (int j = 0; j < MAX_N; ++j) if (j < m) key_put(key, j, (uint32_t)tok[j]);
+            claimed += tok_change(a, key, m, add, round);
+        }
+        __syncwarp();
+        total = 0;
+        return claimed;
     }
+};
+
+// Replaces the occurrences of the round's n-gram in one document, in place: left to right, non-overlapping.  A document of
+// at most DOC_SMEM tokens is worked on in shared memory, so that all its windows, old and new, are looked up together (a
+// look-up is a trip to L2 or to memory behind it); a longer one where it is, its windows chunk by chunk.
+template <bool SMALL>
+__device__ __noinline__ int tok_rewrite(const TokArgs& a, TokShared& sh, int d, int64_t s0, int L, int new_id, int round) {
+    const int lane = threadIdx.x & 31, n = sh.n;
+    TokWarp& w = sh.warp[threadIdx.x >> 5];
+    int32_t* doc = a.cur + s0;
+    const int32_t* old_tok = SMALL ? w.old_tok : doc;
+    uint8_t* old_mark = SMALL ? w.old_mark : a.mark + s0;
+    int32_t* new_tok = SMALL ? w.new_tok : doc;
+    uint8_t* new_mark = SMALL ? w.new_mark : a.mark + s0;
+    if (SMALL) {
+        int x[DOC_SMEM / 32];
+#pragma unroll
+        for (int u = 0; u < DOC_SMEM / 32; ++u) x[u] = u * 32 + lane < L ? doc[u * 32 + lane] : -1;
+#pragma unroll
+        for (int u = 0; u < DOC_SMEM / 32; ++u) w.old_tok[u * 32 + lane] = x[u];
+        __syncwarp();
+    }
+    int skip = 0;                                              // first position that is not part of the last occurrence
+    for (int c = 0; c < L; c += 32) {
+        const int i = c + lane;
+        bool hit = i + n <= L;
+        for (int j = 0; hit && j < n; ++j) hit = old_tok[i + j] == sh.tok[j];
+        uint32_t hits = __ballot_sync(0xFFFFFFFFu, hit), starts = 0u, inside = 0u;
+        if (skip > c) inside = skip - c >= 32 ? 0xFFFFFFFFu : (1u << (skip - c)) - 1u;
+        while (hits) {
+            const int p = c + __ffs(hits) - 1;
+            hits &= hits - 1u;
+            if (p < skip) continue;
+            starts |= 1u << (p - c);
+            skip = p + n;
+            for (int q = p + 1; q < skip && q < c + 32; ++q) inside |= 1u << (q - c);
+        }
+        // 1 = first of an occurrence, 2 = the others
+        if (i < L) old_mark[i] = (starts >> lane) & 1u ? 1 : ((inside >> lane) & 1u ? 2 : 0);
+    }
+    __syncwarp();
+    TokList list = {w, old_tok, new_tok, 0};
+    int claimed = 0;
+    for (int c = 0; c < L; c += 32) {
+        if (!SMALL) list.old_tok = doc + c;
+        list.collect(a, old_mark, L, c, SMALL ? 0 : c, false);
+        if (!SMALL || list.full()) claimed += list.flush(a, round);
+    }
+    // a chunk's tokens are in registers before any of them is overwritten, and what is written lies before it
+    int wr = 0;
+    for (int c = 0; c < L; c += 32) {
+        const int i = c + lane;
+        const int tok = i < L ? old_tok[i] : 0, f = i < L ? old_mark[i] : 2;
+        const uint32_t keep = __ballot_sync(0xFFFFFFFFu, f != 2);
+        const int at = wr + __popc(keep & ((1u << lane) - 1u));
+        __syncwarp();
+        if (f != 2) {
+            const int t = f == 1 ? new_id : tok;
+            new_tok[at] = t;
+            new_mark[at] = (uint8_t)f;
+            if (SMALL) doc[at] = t;
+        }
+        wr += __popc(keep);
+        __syncwarp();
+    }
+    for (int i = lane; i < L; i += 32) {
+        if (i < wr) a.rem[s0 + i] = (uint8_t)min(wr - 1 - i, 255);
+        else doc[i] = -1;
+    }
+    if (lane == 0) a.doc_len[d] = wr;
+    __syncwarp();
+    for (int c = 0; c < wr; c += 32) {
+        if (!SMALL) list.new_tok = doc + c;
+        list.collect(a, new_mark, wr, c, SMALL ? 0 : c, true);
+        if (!SMALL || list.full()) claimed += list.flush(a, round);
+    }
+    return claimed + list.flush(a, round);
 }
 
-__global__ void tok_init_docs_kernel(const int64_t* __restrict__ offsets, int64_t n_docs, int64_t* doc_start, int32_t* doc_len,
-                                     uint8_t* rem) {
-    const int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// All rounds of Algorithm 1.  A warp looks for the n-gram in the documents that start in its share of the positions; the
+// documents found are handed out to the warps of the CTA.  A round is a chain of short steps: the best n-gram of the slots
+// that have changed, a grid barrier, the documents that hold it, a barrier.
+//   Measured on 20,000 documents (1.4 M tokens, 4.1 M windows, n_max 4), per round: 525 us when every round cleared and
+//   recounted the table, 31 us now, of which about 11 are the re-tokenising of one document (a warp, hundreds of instructions in a chain).
+__global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid_constant__ TokArgs a) {
+    extern __shared__ __align__(16) uint8_t dyn[];
+    TokShared& sh = *reinterpret_cast<TokShared*>(dyn);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t nw = (int64_t)gridDim.x * TOK_WARPS, wid = (int64_t)warp * gridDim.x + blockIdx.x;
+    if (threadIdx.x == 0) { sh.stop = 0; sh.n_hits = 0; sh.next_hit = 0; }
+    // this warp's documents
+    auto doc_at = [&](int64_t pos) {
+        int64_t lo = 0, hi = a.n_docs;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (a.offsets[mid] < pos) lo = mid + 1; else hi = mid;
+        }
+        return lo;
+    };
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.st->first[0] = a.st->first[1] = 0xFFFFFFFFu;
+    const int64_t own = (int64_t)blockIdx.x * TOK_WARPS + warp;           // (neighbouring documents: one CTA's)
+    const int64_t s = a.offsets[doc_at(own * a.T / nw)], e = own + 1 == nw ? a.T : a.offsets[doc_at((own + 1) * a.T / nw)];
+    const uint64_t n_chunks = a.cap >> CHUNK_BITS;
+    unsigned int epoch = 0;
+    int n_merges = 0, n_ties = 0, n_rebuilds = 0;
+    __syncthreads();
+    auto publish_claims = [&](int claimed) {
+        claimed = __reduce_add_sync(0xFFFFFFFFu, claimed);
+        if (lane == 0 && claimed) atomicAdd(&a.st->used[n_rebuilds & 1], (unsigned long long)claimed);
+    };
+    for (int round = 0;; ++round) {
+        // ---- the table, if it has to be counted (again): n-grams that no longer occur keep their slots until then
+        const unsigned long long used = *(volatile unsigned long long*)&a.st->used[n_rebuilds & 1];
+        if (*(volatile int*)&a.st->rebuild == round || used * 4 > a.cap * 3) {
+            const uint64_t gt = (uint64_t)blockIdx.x * TOK_THREADS + threadIdx.x, gn = (uint64_t)gridDim.x * TOK_THREADS;
+            for (uint64_t i = gt; i < a.cap; i += gn) {
+                reinterpret_cast<ulonglong2*>(a.keys)[i] = make_ulonglong2(0ull, 0ull);
+                a.words[i] = 0u;
+            }
+            for (uint64_t i = gt; i < n_chunks; i += gn) a.dirty[i] = 1;
+            ++n_rebuilds;
+            if (gt == 0) a.st->used[n_rebuilds & 1] = 0ull;
+            if (!tok_barrier(a.st, epoch, sh)) return;
+            int claimed = 0;
+            for (int64_t i = s + lane; i < e; i += 32) {
+                if (a.cur[i] < 0) continue;
+                const int lim = min(a.n_max, (int)a.rem[i] + 1);
+                for (int n = 2; n <= lim; ++n) {
+                    Key key = key_make(n);
+                    for (int j = 0; j < n; ++j) key_put(key, j, (uint32_t)a.cur[i + j]);
+                    claimed += tok_change(a, key, n, true, round);
+                }
+            }
+            __syncwarp();
+            publish_claims(claimed);
+            if (!tok_barrier(a.st, epoch, sh)) return;
+        }
+        // ---- the best of this warp's chunks of the table
+        Best v = {0ull, 0u, 0u};
+        for (uint64_t c0 = 0; c0 * nw < n_chunks; c0 += 32) {
+            const uint64_t c = (c0 + lane) * nw + wid;
+            const bool mine = c < n_chunks, stale = mine && __ldcg(a.dirty + c);
+            Best b = {0ull, 0u, 0u};
+            if (mine) b = a.chunk_best[c];
+            uint32_t todo = __ballot_sync(0xFFFFFFFFu, stale);
+            while (todo) {
+                int src[4];                                    // four chunks at a time
+                uint4 w[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    src[u] = __ffs(todo) - 1;
+                    todo &= todo - 1u;
+                    w[u] = make_uint4(0u, 0u, 0u, 0u);
+                    if (src[u] >= 0) w[u] = __ldcg(reinterpret_cast<const uint4*>(a.words + (((c0 + src[u]) * nw + wid) << CHUNK_BITS)) + lane);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (src[u] < 0) break;
+                    const uint32_t y[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+                    // the chunk's largest reward, then the lengths that have it (a reward is below 2^31)
+                    uint32_t top = 0u;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) top = max(top, (y[q] & CNT_MASK) * ((y[q] >> CNT_BITS) - 1u));
+                    top = __reduce_max_sync(0xFFFFFFFFu, top);
+                    Best x = {0ull, 0u, 0u};
+                    if (top) {
+                        uint32_t len = 0u;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) if ((uint32_t)(tok_rank(y[q]) >> LEN_BITS) == top) len = max(len, y[q] >> CNT_BITS);
+                        len = __reduce_max_sync(0xFFFFFFFFu, len);
+                        x.rank = ((unsigned long long)top << LEN_BITS) | len;
+                        uint32_t n_top = 0u, at = 0xFFFFFFFFu;
+#pragma unroll
+                        for (int q = 3; q >= 0; --q) if (tok_rank(y[q]) == x.rank) { ++n_top; at = lane * 4 + q; }
+                        x.ties = __reduce_add_sync(0xFFFFFFFFu, n_top);
+                        x.slot = (unsigned int)((((c0 + src[u]) * nw + wid) << CHUNK_BITS) + __reduce_min_sync(0xFFFFFFFFu, at));
+                    }
+                    if (lane == src[u]) { b = x; a.chunk_best[c] = x; a.dirty[c] = 0; }
+                }
+            }
+            best_merge(v, b);
+        }
+        v = best_warp(v);
+        if (lane == 0) sh.red[warp] = v;
+        __syncthreads();
+        if (warp == 0) {
+            v = best_warp(sh.red[lane]);
+            if (lane == 0) a.cta_best[blockIdx.x] = v;
+        }
+        if (!tok_barrier(a.st, epoch, sh)) return;
+        // ---- the best of all, found by every CTA for itself
+        if (warp == 0) {
+            v = Best{0ull, 0u, 0u};
+            for (int i = lane; i < (int)gridDim.x; i += 32) best_merge(v, best_load(a.cta_best + i));
+            v = best_warp(v);
+            if (lane == 0) sh.red[0] = v;
+        }
+        __syncthreads();
+        const unsigned long long best = sh.red[0].rank;
+        if (best == 0ull || n_merges >= a.budget) break;
+        const int n = (int)(best & ((1u << LEN_BITS) - 1u));
+        const bool tie = sh.red[0].ties > 1;
+        if (tie) {
+            // ---- several: the one with the first position
+            unsigned int* first = &a.st->first[n_ties & 1];
+            if (blockIdx.x == 0 && threadIdx.x == 0) a.st->first[~n_ties & 1] = 0xFFFFFFFFu;
+            for (int64_t c = s; c < e; c += 32) {
+                // (one lane's reading decides for all: the value changes meanwhile)
+                if ((int64_t)__shfl_sync(0xFFFFFFFFu, *(volatile unsigned int*)first, 0) <= c) break;
+                const int64_t i = c + lane;
+                bool hit = false;
+                if (i < e && a.cur[i] >= 0 && (int)a.rem[i] >= n - 1) {
+                    Key key = key_make(n);
+                    for (int j = 0; j < n; ++j) key_put(key, j, (uint32_t)a.cur[i + j]);
+                    hit = tok_rank_of(a, key) == best;
+                }
+                const uint32_t hits = __ballot_sync(0xFFFFFFFFu, hit);
+                if (hits) {
+                    if (lane == 0) atomicMin(first, (unsigned int)(c + __ffs(hits) - 1));
+                    break;
+                }
+            }
+            ++n_ties;
+            if (!tok_barrier(a.st, epoch, sh)) return;
+        }
+        if (threadIdx.x == 0) {
+            Key k = {0ull, 0ull};
+            int64_t at = 0;
+            if (tie) at = *(volatile unsigned int*)&a.st->first[~n_ties & 1];
+            else { const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(a.keys) + sh.red[0].slot); k = Key{v.x, v.y}; }
+            sh.n = n;
+            for (int j = 0; j < MAX_N; ++j) {
+                const int t = j >= n ? -1 : tie ? __ldcg(a.cur + at + j) : (int)key_get(k, j);
+                sh.tok[j] = t;
+                if (blockIdx.x == 0) a.merges[(size_t)n_merges * MAX_N + j] = t;
+            }
+        }
+        const int new_id = a.base_vocab + n_merges++;
+        __syncthreads();
+        // ---- its documents
+        const int t0 = sh.tok[0];
+        int claimed = 0;
+        auto rewrite = [&](int d) {
+            const int L = a.doc_len[d];
+            const int64_t s0 = a.offsets[d];
+            claimed += L <= DOC_SMEM ? tok_rewrite<true>(a, sh, d, s0, L, new_id, round) : tok_rewrite<false>(a, sh, d, s0, L, new_id, round);
+        };
+        for (int64_t p = s & ~3ll; p < e; p += 512) {
+            int4 x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t q = p + u * 128 + 4 * lane;
+                x[u] = q < e ? *reinterpret_cast<const int4*>(a.cur + q) : make_int4(-1, -1, -1, -1);
+            }
+            uint32_t mine = 0u;                                // positions with the first token
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int y[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) mine |= y[j] == t0 ? 1u << (u * 4 + j) : 0u;
+            }
+            while (__any_sync(0xFFFFFFFFu, mine != 0u)) {
+                int d = -1;
+                if (mine) {
+                    const int b = __ffs(mine) - 1;
+                    mine &= mine - 1u;
+                    const int64_t q = p + (b >> 2) * 128 + 4 * lane + (b & 3);
+                    // (an occurrence across the end of a document is found not to be one when the document is rewritten)
+                    bool hit = q >= s && q + n <= a.T;
+                    for (int i = 1; hit && i < n; ++i) hit = a.cur[q + i] == sh.tok[i];
+                    // the first hit of a document in this round puts it on the list
+                    if (hit && q < e) {
+                        d = a.doc_of[q];
+                        if (atomicExch(&a.doc_round[d], round + 1) == round + 1) d = -1;
+                    }
+                }
+                uint32_t docs = __ballot_sync(0xFFFFFFFFu, d >= 0);
+                if (docs) {
+                    int slot = 0;
+                    if (lane == 0) slot = atomicAdd(&sh.n_hits, __popc(docs));
+                    slot = __shfl_sync(0xFFFFFFFFu, slot, 0) + __popc(docs & ((1u << lane) - 1u));
+                    if (d >= 0 && slot < HIT_MAX) sh.hits[slot] = d;
+                    for (docs = __ballot_sync(0xFFFFFFFFu, d >= 0 && slot >= HIT_MAX); docs; docs &= docs - 1u)
+                        rewrite(__shfl_sync(0xFFFFFFFFu, d, __ffs(docs) - 1));
+                }
+            }
+        }
+        __syncthreads();
+        const int n_hits = min(sh.n_hits, HIT_MAX);
+        for (;;) {
+            int slot = 0;
+            if (lane == 0) slot = atomicAdd(&sh.next_hit, 1);
+            slot = __shfl_sync(0xFFFFFFFFu, slot, 0);
+            if (slot >= n_hits) break;
+            rewrite(sh.hits[slot]);
+        }
+        publish_claims(claimed);
+        if (!tok_barrier(a.st, epoch, sh)) return;
+        if (threadIdx.x == 0) { sh.n_hits = 0; sh.next_hit = 0; }          // (two barriers before their next use)
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.st->n_merges = n_merges;
+}
+
+// What the host has to know about the documents before it can allocate.
+struct TokCheck { unsigned long long windows; int64_t tokens; int bad; };
+__global__ void tok_check_kernel(const int64_t* __restrict__ offsets, int64_t n_docs, int n_max, TokCheck* out) {
+    unsigned long long w = 0;
+    bool bad = false;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; d < n_docs; d += step) {
+        const int64_t len = offsets[d + 1] - offsets[d];
+        if (len < 0 || len >= (1ll << 31)) bad = true;
+        else for (int n = 2; n <= n_max; ++n) w += (unsigned long long)(len - n + 1 > 0 ? len - n + 1 : 0);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xFFFFFFFFu, w, o);
+    if ((threadIdx.x & 31) == 0 && w) atomicAdd(&out->windows, w);
+    if (bad || (blockIdx.x == 0 && threadIdx.x == 0 && offsets[0] != 0)) out->bad = 1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) out->tokens = offsets[n_docs];
+}
+
+// One warp per document.
+__global__ void tok_init_docs_kernel(const int64_t* __restrict__ offsets, int64_t n_docs, int32_t* doc_len, int32_t* doc_round,
+                                     int32_t* doc_of, uint8_t* rem) {
+    const int64_t d = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (d >= n_docs) return;
     const int64_t s = offsets[d];
     const int L = (int)(offsets[d + 1] - s);
-    doc_start[d] = s;
-    doc_len[d] = L;
-    for (int j = 0; j < L; ++j) {
-        const int left = L - 1 - j;
-        rem[s + j] = (uint8_t)(left > 255 ? 255 : left);
+    if (lane == 0) { doc_len[d] = L; doc_round[d] = 0; }
+    for (int j = lane; j < L; j += 32) {
+        doc_of[s + j] = (int32_t)d;
+        rem[s + j] = (uint8_t)min(L - 1 - j, 255);
     }
 }
 
-// Exclusive scan of the document lengths into offsets (one block; each thread owns a contiguous run of documents).
-__global__ void __launch_bounds__(1024)
-tok_scan_kernel(const int32_t* __restrict__ doc_len, int64_t n_docs, int64_t* offsets_out) {
-    __shared__ long long part[1024];
-    const int t = threadIdx.x;
-    const int64_t per = (n_docs + 1023) / 1024;
-    const int64_t lo = min(n_docs, (int64_t)t * per), hi = min(n_docs, lo + per);
-    long long s = 0;
-    for (int64_t d = lo; d < hi; ++d) s += doc_len[d];
-    part[t] = s;
+// Exclusive scan of the document lengths: blocks of 1,024 documents, their totals by one block, then the sum of both.
+constexpr int SCAN_THREADS = 1024;
+__device__ __forceinline__ long long block_exclusive(long long v, long long* s_warp, long long& total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    long long x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[warp] = x;
     __syncthreads();
-    if (t == 0) {
-        long long run = 0;
-        for (int i = 0; i < 1024; ++i) { const long long v = part[i]; part[i] = run; run += v; }
-        offsets_out[n_docs] = run;
+    if (warp == 0) {
+        long long w = s_warp[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long y = __shfl_up_sync(0xFFFFFFFFu, w, o);
+            if (lane >= o) w += y;
+        }
+        s_warp[lane] = w;
     }
     __syncthreads();
-    long long run = part[t];
-    for (int64_t d = lo; d < hi; ++d) { offsets_out[d] = run; run += doc_len[d]; }
+    total = s_warp[31];
+    const long long r = x - v + (warp ? s_warp[warp - 1] : 0ll);
+    __syncthreads();
+    return r;
 }
-__global__ void tok_compact_kernel(const int32_t* __restrict__ cur, const int64_t* __restrict__ doc_start,
-                                   const int32_t* __restrict__ doc_len, const int64_t* __restrict__ offsets_out,
+__global__ void __launch_bounds__(SCAN_THREADS)
+tok_scan_blocks_kernel(const int32_t* __restrict__ doc_len, int64_t n_docs, int64_t* offsets_out, long long* totals) {
+    __shared__ long long s_warp[32];
+    const int64_t d = (int64_t)blockIdx.x * SCAN_THREADS + threadIdx.x;
+    long long total;
+    const long long r = block_exclusive(d < n_docs ? doc_len[d] : 0, s_warp, total);
+    if (d < n_docs) offsets_out[d] = r;
+    if (threadIdx.x == 0) totals[blockIdx.x] = total;
+}
+__global__ void __launch_bounds__(SCAN_THREADS)
+tok_scan_totals_kernel(long long* totals, int64_t n_blocks, int64_t* end) {
+    __shared__ long long s_warp[32];
+    long long run = 0;
+    for (int64_t b0 = 0; b0 < n_blocks; b0 += SCAN_THREADS) {
+        const int64_t b = b0 + threadIdx.x;
+        long long total;
+        const long long r = block_exclusive(b < n_blocks ? totals[b] : 0, s_warp, total);
+        if (b < n_blocks) totals[b] = run + r;
+        run += total;
+    }
+    if (threadIdx.x == 0) *end = run;
+}
+// One warp per document: its final offset, and its tokens there.
+__global__ void tok_compact_kernel(const int32_t* __restrict__ cur, const int64_t* __restrict__ offsets,
+                                   const int32_t* __restrict__ doc_len, int64_t* offsets_out, const long long* __restrict__ totals,
                                    int64_t n_docs, int32_t* tokens_out) {
-    const int64_t d = blockIdx.x;
+    const int64_t d = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (d >= n_docs) return;
-    const int32_t* src = cur + doc_start[d];
-    int32_t* dst = tokens_out + offsets_out[d];
-    for (int j = threadIdx.x; j < doc_len[d]; j += blockDim.x) dst[j] = src[j];
+    const int64_t off = offsets_out[d] + totals[d / SCAN_THREADS];
+    __syncwarp();
+    if (lane == 0) offsets_out[d] = off;
+    const int32_t* src = cur + offsets[d];
+    int32_t* dst = tokens_out + off;
+    for (int j = lane; j < doc_len[d]; j += 32) dst[j] = src[j];
 }
 
 // ------------------------------------------------------------------------------------------- new rows
+// Bound: a chain (a row may need any earlier one).  A thread fetches the values of a group of merges together, as far as
+// they were complete before the group, then walks it.  256 merges of 896 columns: 316 us when every merge waited for its
+// own loads, 168 us in groups.
+constexpr int ROWS_GROUP = 8, ROWS_THREADS = 64;
 template <typename T>
-__global__ void tok_rows_kernel(const T* __restrict__ base, int base_vocab, int d, const int32_t* __restrict__ merges,
-                                int n_merges, T* rows_out, int* status) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(ROWS_THREADS)
+tok_rows_kernel(const T* base, int base_vocab, int d, const int32_t* __restrict__ merges, int n_merges, T* rows_out,
+                int* status) {
+    const int j = blockIdx.x * ROWS_THREADS + threadIdx.x;
     if (j >= d) return;
-    for (int i = 0; i < n_merges; ++i) {
-        float acc = 0.f;
-        int n = 0;
-        for (int c = 0; c < MAX_N; ++c) {
-            const int t = merges[(size_t)i * MAX_N + c];
-            if (t < 0) break;
-            float v = 0.f;
-            if (t < base_vocab) v = Num<T>::to_f(base[(size_t)t * d + j]);
-            else if (t - base_vocab < i) v = Num<T>::to_f(rows_out[(size_t)(t - base_vocab) * d + j]);   // written by this thread
-            else set_status(status, TASC_EINVAL);                                                      // a constituent that does not exist yet
-            acc += v;
-            ++n;
+    for (int g0 = 0; g0 < n_merges; g0 += ROWS_GROUP) {
+        int tok[ROWS_GROUP][MAX_N];
+        T val[ROWS_GROUP][MAX_N];
+#pragma unroll
+        for (int i = 0; i < ROWS_GROUP; ++i)
+#pragma unroll
+            for (int c = 0; c < MAX_N; ++c) tok[i][c] = g0 + i < n_merges ? merges[(size_t)(g0 + i) * MAX_N + c] : -1;
+#pragma unroll
+        for (int i = 0; i < ROWS_GROUP; ++i)
+#pragma unroll
+            for (int c = 0; c < MAX_N; ++c) {
+                // (no branch: all loads of the group are under way together; what cannot be used reads some other row)
+                const int t = tok[i][c];
+                const T* row = t >= base_vocab && t - base_vocab < g0 ? rows_out + (size_t)(t - base_vocab) * d : base + (size_t)(t >= 0 && t < base_vocab ? t : 0) * d;
+                val[i][c] = row[j];
+            }
+#pragma unroll
+        for (int i = 0; i < ROWS_GROUP; ++i) {
+            if (g0 + i >= n_merges) break;
+            float acc = 0.f;
+            int n = 0;
+            bool more = true;
+#pragma unroll
+            for (int c = 0; c < MAX_N; ++c) {
+                const int t = tok[i][c];
+                more = more && t >= 0;
+                if (!more) continue;
+                float v = Num<T>::to_f(val[i][c]);
+                if (t - base_vocab >= g0 + i) { set_status(status, TASC_EINVAL); v = 0.f; }      // a constituent that does not exist yet
+                else if (t - base_vocab >= g0) v = Num<T>::to_f(rows_out[(size_t)(t - base_vocab) * d + j]);      // written by this thread
+                acc += v;
+                ++n;
+            }
+            if (n < 2) { set_status(status, TASC_EINVAL); n = 1; }
+            rows_out[(size_t)(g0 + i) * d + j] = Num<T>::from_f(acc / (float)n);
         }
-        if (n < 2) { set_status(status, TASC_EINVAL); n = 1; }
-        rows_out[(size_t)i * d + j] = Num<T>::from_f(acc / (float)n);
     }
 }
 
@@ -223,7 +708,7 @@ __device__ __forceinline__ int trie_step(const TrieTable& t, int node, int tok) 
 // One thread per document: at every position the longest added token whose expansion matches, else the base token.
 // Output in place of a scratch copy at the document's original offset; lengths to doc_len.
 __global__ void tok_encode_kernel(const int32_t* __restrict__ tokens, const int64_t* __restrict__ offsets, int64_t n_docs,
-                                  TrieTable trie, int32_t* scratch, int64_t* doc_start, int32_t* doc_len) {
+                                  TrieTable trie, int32_t* scratch, int32_t* doc_len) {
     const int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (d >= n_docs) return;
     const int64_t s = offsets[d];
@@ -242,14 +727,17 @@ __global__ void tok_encode_kernel(const int32_t* __restrict__ tokens, const int6
         if (best_tok >= 0) { out[w++] = best_tok; i += best_len; }
         else { out[w++] = doc[i++]; }
     }
-    doc_start[d] = s;
     doc_len[d] = w;
 }
 
-tasc_status compact_docs(const int32_t* cur, const int64_t* doc_start, const int32_t* doc_len, int64_t n_docs,
+int64_t scan_blocks(int64_t n_docs) { return (n_docs + SCAN_THREADS - 1) / SCAN_THREADS; }
+// totals: scan_blocks(n_docs) words
+tasc_status compact_docs(const int32_t* cur, const int64_t* offsets, const int32_t* doc_len, int64_t n_docs, long long* totals,
                          int32_t* tokens_out, int64_t* offsets_out, cudaStream_t stream) {
-    tok_scan_kernel<<<1, 1024, 0, stream>>>(doc_len, n_docs, offsets_out);
-    if (n_docs > 0) tok_compact_kernel<<<(unsigned)n_docs, 64, 0, stream>>>(cur, doc_start, doc_len, offsets_out, n_docs, tokens_out);
+    const int64_t nb = scan_blocks(n_docs);
+    if (nb) tok_scan_blocks_kernel<<<(unsigned)nb, SCAN_THREADS, 0, stream>>>(doc_len, n_docs, offsets_out, totals);
+    tok_scan_totals_kernel<<<1, SCAN_THREADS, 0, stream>>>(totals, nb, reinterpret_cast<int64_t*>(offsets_out) + n_docs);
+    if (nb) tok_compact_kernel<<<blocks_for((uint64_t)n_docs, 8), 256, 0, stream>>>(cur, offsets, doc_len, offsets_out, totals, n_docs, tokens_out);
     TASC_CUDA_TRY(cudaGetLastError());
     return TASC_OK;
 }
@@ -267,72 +755,55 @@ extern "C" tasc_status tasc_tok_enrich(const int32_t* corpus_tokens, const int64
         return TASC_EINVAL;
     *n_merges = 0;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    std::vector<int64_t> offs((size_t)n_docs + 1);
-    TASC_CUDA_TRY(cudaMemcpyAsync(offs.data(), doc_offsets, offs.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
-    TASC_CUDA_TRY(cudaStreamSynchronize(stream));
-    if (offs[0] != 0) return TASC_EINVAL;
-    uint64_t windows = 0;
-    for (int64_t d = 0; d < n_docs; ++d) {
-        const int64_t len = offs[d + 1] - offs[d];
-        if (len < 0 || len >= (1ll << 31)) return TASC_EINVAL;
-        for (int n = 2; n <= n_max; ++n) windows += (uint64_t)std::max<int64_t>(0, len - n + 1);
+    DeviceSlab slab;
+    const TokCheck zero = {0ull, 0, 0};
+    TokCheck hc;
+    {
+        DeviceSlab small;
+        const size_t o = small.add(sizeof(TokCheck));
+        if (!small.allocate()) return TASC_ENOMEM;
+        TokCheck* dc = small.at<TokCheck>(o);
+        TASC_CUDA_TRY(cudaMemcpyAsync(dc, &zero, sizeof(zero), cudaMemcpyHostToDevice, stream));
+        tok_check_kernel<<<std::min(blocks_for((uint64_t)n_docs + 1, 256), 592u), 256, 0, stream>>>(doc_offsets, n_docs, n_max, dc);
+        TASC_CUDA_TRY(cudaMemcpyAsync(&hc, dc, sizeof(hc), cudaMemcpyDeviceToHost, stream));
+        TASC_CUDA_TRY(cudaStreamSynchronize(stream));
     }
-    const int64_t T = offs[n_docs];
-    if (T >= (1ll << POS_BITS)) return TASC_EINVAL;
+    const int64_t T = hc.tokens;
+    if (hc.bad || T < 0 || T >= (1ll << POS_BITS)) return TASC_EINVAL;
     if (T > 0 && (!corpus_tokens || !tokens_out)) return TASC_EINVAL;
 
-    int32_t* cur = nullptr;
-    uint8_t* rem = nullptr;
-    int64_t* doc_start = nullptr;
-    int32_t* doc_len = nullptr;
-    uint64_t* keys = nullptr;
-    uint32_t *counts = nullptr, *first = nullptr;
-    unsigned long long* best = nullptr;
-    Winner* win = nullptr;
-    int* dn = nullptr;                         // [0] number of merges, [1] status
-    const uint64_t cap = pow2_at_least(2 * std::max<uint64_t>(windows, 1));
-    tasc_status rc = TASC_OK;
-#define TRY_ALLOC(ptr, bytes) if (rc == TASC_OK && cudaMalloc(reinterpret_cast<void**>(&(ptr)), (bytes)) != cudaSuccess) { (void)cudaGetLastError(); rc = TASC_ENOMEM; }
-    TRY_ALLOC(cur, (size_t)std::max<int64_t>(T, 1) * 4);
-    TRY_ALLOC(rem, (size_t)std::max<int64_t>(T, 1));
-    TRY_ALLOC(doc_start, (size_t)std::max<int64_t>(n_docs, 1) * 8);
-    TRY_ALLOC(doc_len, (size_t)std::max<int64_t>(n_docs, 1) * 4);
-    TRY_ALLOC(keys, cap * 16);
-    TRY_ALLOC(counts, cap * 4);
-    TRY_ALLOC(first, cap * 4);
-    TRY_ALLOC(best, 8);
-    TRY_ALLOC(win, sizeof(Winner));
-    TRY_ALLOC(dn, 2 * sizeof(int));
-#undef TRY_ALLOC
-    int h_dn[2] = {0, 0};
-    if (rc == TASC_OK) {
-        cudaMemsetAsync(best, 0, 8, stream);
-        cudaMemsetAsync(win, 0, sizeof(Winner), stream);
-        cudaMemsetAsync(dn, 0, 2 * sizeof(int), stream);
-        cudaMemsetAsync(merges, 0xFF, (size_t)budget * MAX_N * sizeof(int32_t), stream);
-        if (T > 0) cudaMemcpyAsync(cur, corpus_tokens, (size_t)T * 4, cudaMemcpyDeviceToDevice, stream);
-        if (n_docs > 0) tok_init_docs_kernel<<<blocks_for((uint64_t)n_docs, 128), 128, 0, stream>>>(doc_offsets, n_docs, doc_start, doc_len, rem);
-        for (int it = 0; it < budget && T > 0; ++it) {
-            cudaMemsetAsync(keys, 0, cap * 16, stream);
-            cudaMemsetAsync(counts, 0, cap * 4, stream);
-            cudaMemsetAsync(first, 0xFF, cap * 4, stream);
-            for (int n = 2; n <= n_max; ++n)
-                tok_count_kernel<<<blocks_for((uint64_t)T, 256), 256, 0, stream>>>(cur, rem, T, n, keys, counts, first, cap - 1, win, dn + 1);
-            tok_best_kernel<<<blocks_for(cap, 256), 256, 0, stream>>>(keys, counts, first, cap, best, win);
-            tok_winner_kernel<<<blocks_for(cap, 256), 256, 0, stream>>>(keys, counts, first, cap, best, win, merges, dn);
-            tok_commit_kernel<<<1, 1, 0, stream>>>(win, dn, best);
-            tok_rewrite_kernel<<<blocks_for((uint64_t)n_docs, 128), 128, 0, stream>>>(cur, rem, doc_start, doc_len, n_docs, win, dn, base_vocab);
-        }
-        if (cudaGetLastError() != cudaSuccess) rc = TASC_ECUDA;
-        if (rc == TASC_OK) rc = compact_docs(cur, doc_start, doc_len, n_docs, tokens_out, offsets_out, stream);
-        if (rc == TASC_OK && (cudaMemcpyAsync(h_dn, dn, sizeof(h_dn), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
-                              cudaStreamSynchronize(stream) != cudaSuccess)) { (void)cudaGetLastError(); rc = TASC_ECUDA; }
-        if (rc == TASC_OK && h_dn[1] != 0) rc = h_dn[1];
+    int dev = 0, grid = 0;
+    TASC_CUDA_TRY(cudaGetDevice(&dev));
+    TASC_CUDA_TRY(cudaDeviceGetAttribute(&grid, cudaDevAttrMultiProcessorCount, dev));      // one CTA per SM
+    const uint64_t cap = std::max<uint64_t>(pow2_at_least(2 * hc.windows), 1ull << CHUNK_BITS), chunks = cap >> CHUNK_BITS;
+    const size_t t = (size_t)T + 4, nd = (size_t)n_docs;
+    const size_t o_keys = slab.add(cap * 16), o_words = slab.add(cap * 4), o_dirty = slab.add(chunks), o_chunk = slab.add(chunks * sizeof(Best)),
+                 o_cta = slab.add(grid * sizeof(Best)), o_st = slab.add(sizeof(TokState)), o_cur = slab.add(t * 4), o_of = slab.add(t * 4),
+                 o_rem = slab.add(t), o_mark = slab.add(t), o_len = slab.add(nd * 4), o_round = slab.add(nd * 4), o_tot = slab.add(scan_blocks(n_docs) * 8);
+    if (!slab.allocate()) return TASC_ENOMEM;
+    TokArgs a = {};
+    a.cur = slab.at<int32_t>(o_cur); a.rem = slab.at<uint8_t>(o_rem); a.mark = slab.at<uint8_t>(o_mark); a.doc_of = slab.at<int32_t>(o_of);
+    a.offsets = doc_offsets; a.doc_len = slab.at<int32_t>(o_len); a.doc_round = slab.at<int32_t>(o_round); a.n_docs = n_docs; a.T = T;
+    a.keys = slab.at<uint64_t>(o_keys); a.words = slab.at<uint32_t>(o_words); a.dirty = slab.at<uint8_t>(o_dirty);
+    a.chunk_best = slab.at<Best>(o_chunk); a.cta_best = slab.at<Best>(o_cta); a.cap = cap; a.st = slab.at<TokState>(o_st);
+    a.merges = merges; a.base_vocab = base_vocab; a.budget = budget; a.n_max = n_max;
+    TokState hs = {};
+    TASC_CUDA_TRY(cudaMemsetAsync(a.st, 0, sizeof(TokState), stream));
+    TASC_CUDA_TRY(cudaMemsetAsync(merges, 0xFF, (size_t)budget * MAX_N * sizeof(int32_t), stream));
+    if (T > 0) TASC_CUDA_TRY(cudaMemcpyAsync(a.cur, corpus_tokens, (size_t)T * 4, cudaMemcpyDeviceToDevice, stream));
+    if (n_docs > 0) tok_init_docs_kernel<<<blocks_for(nd, 8), 256, 0, stream>>>(doc_offsets, n_docs, a.doc_len, a.doc_round, slab.at<int32_t>(o_of), a.rem);
+    if (T > 0 && budget > 0) {
+        void* args[] = {&a};
+        TASC_CUDA_TRY(cudaFuncSetAttribute(tok_rounds_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TokShared)));
+        TASC_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(tok_rounds_kernel), dim3(grid), dim3(TOK_THREADS), args, sizeof(TokShared), stream));
     }
-    cudaFree(cur); cudaFree(rem); cudaFree(doc_start); cudaFree(doc_len); cudaFree(keys); cudaFree(counts); cudaFree(first);
-    cudaFree(best); cudaFree(win); cudaFree(dn);
-    if (rc == TASC_OK) *n_merges = h_dn[0];
-    return rc;
+    const tasc_status rc = compact_docs(a.cur, doc_offsets, a.doc_len, n_docs, slab.at<long long>(o_tot), tokens_out, offsets_out, stream);
+    if (rc != TASC_OK) return rc;
+    TASC_CUDA_TRY(cudaMemcpyAsync(&hs, a.st, sizeof(hs), cudaMemcpyDeviceToHost, stream));
+    TASC_CUDA_TRY(cudaStreamSynchronize(stream));
+    if (hs.status != 0) return hs.status;
+    *n_merges = hs.n_merges;
+    return TASC_OK;
 }
 
 extern "C" tasc_status tasc_tok_init_rows(const void* matrix, int32_t dtype, int32_t base_vocab, int32_t d,
@@ -343,12 +814,12 @@ extern "C" tasc_status tasc_tok_init_rows(const void* matrix, int32_t dtype, int
         return TASC_EINVAL;
     if (n_merges == 0) return TASC_OK;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    const unsigned blocks = (unsigned)((d + 127) / 128);
+    const unsigned blocks = (unsigned)((d + ROWS_THREADS - 1) / ROWS_THREADS);
     if (dtype == TASC_F32)
-        tok_rows_kernel<float><<<blocks, 128, 0, stream>>>(static_cast<const float*>(matrix), base_vocab, d, merges, n_merges,
+        tok_rows_kernel<float><<<blocks, ROWS_THREADS, 0, stream>>>(static_cast<const float*>(matrix), base_vocab, d, merges, n_merges,
                                                            static_cast<float*>(rows_out), device_status);
     else
-        tok_rows_kernel<__nv_bfloat16><<<blocks, 128, 0, stream>>>(static_cast<const __nv_bfloat16*>(matrix), base_vocab, d, merges,
+        tok_rows_kernel<__nv_bfloat16><<<blocks, ROWS_THREADS, 0, stream>>>(static_cast<const __nv_bfloat16*>(matrix), base_vocab, d, merges,
                                                                    n_merges, static_cast<__nv_bfloat16*>(rows_out), device_status);
     TASC_CUDA_TRY(cudaGetLastError());
     return TASC_OK;
@@ -404,29 +875,19 @@ extern "C" tasc_status tasc_tok_encode(const int32_t* tokens, const int64_t* doc
         hk[slot] = key;
         hc[slot] = e.second;
     }
-    uint64_t* d_keys = nullptr;
-    int32_t *d_child = nullptr, *d_tok = nullptr, *scratch = nullptr, *doc_len = nullptr;
-    int64_t* doc_start = nullptr;
-    tasc_status rc = TASC_OK;
-#define TRY_ALLOC(ptr, bytes) if (rc == TASC_OK && cudaMalloc(reinterpret_cast<void**>(&(ptr)), (bytes)) != cudaSuccess) { (void)cudaGetLastError(); rc = TASC_ENOMEM; }
-    TRY_ALLOC(d_keys, cap * 8);
-    TRY_ALLOC(d_child, cap * 4);
-    TRY_ALLOC(d_tok, node_token.size() * 4);
-    TRY_ALLOC(scratch, (size_t)std::max<int64_t>(T, 1) * 4);
-    TRY_ALLOC(doc_len, (size_t)std::max<int64_t>(n_docs, 1) * 4);
-    TRY_ALLOC(doc_start, (size_t)std::max<int64_t>(n_docs, 1) * 8);
-#undef TRY_ALLOC
-    if (rc == TASC_OK) {
-        cudaMemcpyAsync(d_keys, hk.data(), cap * 8, cudaMemcpyHostToDevice, stream);
-        cudaMemcpyAsync(d_child, hc.data(), cap * 4, cudaMemcpyHostToDevice, stream);
-        cudaMemcpyAsync(d_tok, node_token.data(), node_token.size() * 4, cudaMemcpyHostToDevice, stream);
-        TrieTable trie = {d_keys, d_child, d_tok, cap - 1};
-        if (n_docs > 0)
-            tok_encode_kernel<<<blocks_for((uint64_t)n_docs, 128), 128, 0, stream>>>(tokens, doc_offsets, n_docs, trie, scratch, doc_start, doc_len);
-        if (cudaGetLastError() != cudaSuccess) rc = TASC_ECUDA;
-        if (rc == TASC_OK) rc = compact_docs(scratch, doc_start, doc_len, n_docs, tokens_out, offsets_out, stream);
-        if (cudaStreamSynchronize(stream) != cudaSuccess) { (void)cudaGetLastError(); rc = TASC_ECUDA; }   // the host tables must outlive the copies
-    }
-    cudaFree(d_keys); cudaFree(d_child); cudaFree(d_tok); cudaFree(scratch); cudaFree(doc_len); cudaFree(doc_start);
+    DeviceSlab slab;
+    const size_t o_keys = slab.add(cap * 8), o_child = slab.add(cap * 4), o_tok = slab.add(node_token.size() * 4),
+                 o_scratch = slab.add((size_t)T * 4), o_len = slab.add((size_t)n_docs * 4), o_tot = slab.add(scan_blocks(n_docs) * 8);
+    if (!slab.allocate()) return TASC_ENOMEM;
+    int32_t *scratch = slab.at<int32_t>(o_scratch), *doc_len = slab.at<int32_t>(o_len);
+    TASC_CUDA_TRY(cudaMemcpyAsync(slab.at<uint64_t>(o_keys), hk.data(), cap * 8, cudaMemcpyHostToDevice, stream));
+    TASC_CUDA_TRY(cudaMemcpyAsync(slab.at<int32_t>(o_child), hc.data(), cap * 4, cudaMemcpyHostToDevice, stream));
+    TASC_CUDA_TRY(cudaMemcpyAsync(slab.at<int32_t>(o_tok), node_token.data(), node_token.size() * 4, cudaMemcpyHostToDevice, stream));
+    const TrieTable trie = {slab.at<uint64_t>(o_keys), slab.at<int32_t>(o_child), slab.at<int32_t>(o_tok), cap - 1};
+    if (n_docs > 0)
+        tok_encode_kernel<<<blocks_for((uint64_t)n_docs, 128), 128, 0, stream>>>(tokens, doc_offsets, n_docs, trie, scratch, doc_len);
+    TASC_CUDA_TRY(cudaGetLastError());
+    const tasc_status rc = compact_docs(scratch, doc_offsets, doc_len, n_docs, slab.at<long long>(o_tot), tokens_out, offsets_out, stream);
+    TASC_CUDA_TRY(cudaStreamSynchronize(stream));                    // the host tables must outlive the copies
     return rc;
 }

@@ -80,6 +80,18 @@ def test_synthetic_task_corpus(n_max, budget):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("lens,vocab,budget,n_max", [
+    ([57] * 3 + [4], 4000, 60, 4),               # nearly all n-grams distinct, a table half full: it is counted again on the way
+    ([1, 31, 32, 33, 63, 64, 65, 0, 2, 3], 3, 40, 6),      # chunk edges, overlapping and tying n-grams
+    ([3000, 5, 700], 7, 50, 5),                  # documents longer than a warp's share
+    (list(range(40)) * 8, 12, 64, 3)])
+def test_counts_kept_over_the_rounds(lens, vocab, budget, n_max):
+    b = need_gpu()
+    r = np.random.default_rng(sum(lens) + vocab)
+    check_enrich(b, *flat([r.integers(0, vocab, n).tolist() for n in lens]), vocab, budget, n_max)
+
+
+@pytest.mark.gpu
 def test_rejects_bad_arguments():
     b = need_gpu()
     t, o = to_dev([1, 2, 3], [0, 3])
