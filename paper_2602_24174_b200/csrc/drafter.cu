@@ -1,12 +1,13 @@
 // On-device n-gram drafter (TASC-draft): corpus tables p_corp, context model p_prompt, exact mixture argmax.
 //
-// Build (once per task): for each order n = 1..n_max every window (n context tokens, next token) of
-// every document is counted in an open-addressing scratch table keyed by the full 128-bit packing of
-// (n, tokens) -- one 128-bit compare-and-swap claims or finds a slot, so there is no fingerprint
-// matching and counts are exact.  Elements with count >= p_min are then moved into the final
-// per-order structure: a context table (packed context -> offset, number of successors, total count)
-// plus a flat successor array of (next, count).  Slot placement depends on thread timing, results do
-// not: lookups return the same sets, and the export sorts canonically.
+// Build (once per task): the windows (n context tokens, next token) of every order n = 1..n_max are counted exactly, in an
+// open-addressing table whose 16-byte slots hold key, count and one position of the n-gram: a window's whole update is one
+// 32-byte sector.  Order 1 is keyed by its two tokens, order n by the slot of its prefix in order n - 1's table and its
+// last token, which is as exact and half as long.  A window can only reach p_min if the two windows of order n - 1 inside
+// it have, so each order counts only what the order before left over.  Elements with count >= p_min are listed and moved
+// into the final per-order structure: a context table (packed context -> offset, number of successors, total count) plus
+// a flat successor array of (next, count).  Slot placement depends on thread timing, results do not: lookups return the
+// same sets, and the export sorts canonically.
 //
 // Draft (every step): one CTA per sequence.  For each of the k drafts: warp-cooperative probes of the
 // context tables of all orders at once (one warp per order, 32 slots per probe round; longest hit wins), a scan of the sequence's committed tokens for the
@@ -46,98 +47,295 @@ struct DeviceTables {
 
 struct tasc_drafter {
     DeviceTables dt;
+    tasc::DeviceSlab slab[TASC_MAX_ORDER + 1];      // the memory of dt.t[n]
     int p_min, vocab, device;
 };
 
 namespace tasc {
 namespace {
 
-// remaining[i] = number of tokens after position i inside its document, clamped to 255
-__global__ void mark_remaining_kernel(const int64_t* __restrict__ offsets, int64_t n_docs, int64_t T, uint8_t* remaining) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T) return;
-    int64_t lo = 0, hi = n_docs;           // last doc with offsets[doc] <= i
-    while (hi - lo > 1) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (offsets[mid] <= i) lo = mid; else hi = mid;
+// ------------------------------------------------------------------------------------------- corpus
+// What the host has to know about the documents before it can allocate.
+struct CorpusCheck { unsigned long long pairs; long long tokens; int bad; };
+__global__ void corpus_check_kernel(const int64_t* __restrict__ offsets, int64_t n_docs, CorpusCheck* out) {
+    unsigned long long w = 0;
+    bool bad = false;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; d < n_docs; d += step) {
+        const int64_t len = offsets[d + 1] - offsets[d];
+        if (len < 0) bad = true;
+        else if (len > 1) w += (unsigned long long)(len - 1);
     }
-    const int64_t rem = offsets[lo + 1] - i - 1;
-    remaining[i] = (uint8_t)(rem > 255 ? 255 : (rem < 0 ? 0 : rem));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xFFFFFFFFu, w, o);
+    if ((threadIdx.x & 31) == 0 && w) atomicAdd(&out->pairs, w);
+    if (bad || (blockIdx.x == 0 && threadIdx.x == 0 && offsets[0] != 0)) out->bad = 1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) out->tokens = offsets[n_docs];
+}
+tasc_status check_corpus(const int64_t* offsets, int64_t n_docs, CorpusCheck& h, cudaStream_t stream) {
+    DeviceSlab slab;
+    const size_t o = slab.add(sizeof(CorpusCheck));
+    if (!slab.allocate(stream)) return TASC_ENOMEM;
+    TASC_CUDA_TRY(cudaMemsetAsync(slab.at<CorpusCheck>(o), 0, sizeof(h), stream));
+    corpus_check_kernel<<<std::min(blocks_for((uint64_t)n_docs + 1, 256), 592u), 256, 0, stream>>>(offsets, n_docs, slab.at<CorpusCheck>(o));
+    TASC_CUDA_TRY(cudaMemcpyAsync(&h, slab.at<CorpusCheck>(o), sizeof(h), cudaMemcpyDeviceToHost, stream));
+    TASC_CUDA_TRY(cudaStreamSynchronize(stream));
+    return h.bad || h.tokens < 0 ? TASC_EINVAL : TASC_OK;
 }
 
-__global__ void token_hist_kernel(const int32_t* __restrict__ tokens, int64_t T, int vocab, uint32_t* hist, int* status) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T) return;
-    const int t = tokens[i];
-    if (t < 0 || t >= vocab) { set_status(status, TASC_EINVAL); return; }
-    atomicAdd(&hist[t], 1u);
+// remaining[i] = number of tokens after position i inside its document, clamped to 255; and the histogram of the tokens.
+// A block searches the offsets for the documents of its SCAN_POS positions, a thread among those only.
+constexpr int SCAN_THREADS = 256, SCAN_PER = 8, SCAN_POS = SCAN_THREADS * SCAN_PER;
+__global__ void __launch_bounds__(SCAN_THREADS)
+corpus_scan_kernel(const int32_t* __restrict__ tokens, const int64_t* __restrict__ offsets, int64_t n_docs, int64_t T, int vocab,
+                   uint8_t* __restrict__ remaining, uint32_t* hist, int* status) {
+    __shared__ int64_t s_doc[2];
+    const int64_t p0 = (int64_t)blockIdx.x * SCAN_POS;
+    auto doc_of = [&](int64_t i, int64_t lo, int64_t hi) {       // last doc in [lo, hi) with offsets[doc] <= i
+        while (hi - lo > 1) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (offsets[mid] <= i) lo = mid; else hi = mid;
+        }
+        return lo;
+    };
+    if (threadIdx.x < 2) s_doc[threadIdx.x] = doc_of(threadIdx.x ? min(p0 + SCAN_POS, T) - 1 : p0, 0, n_docs);
+    __syncthreads();
+    const int64_t d0 = s_doc[0], d1 = s_doc[1] + 1;
+#pragma unroll
+    for (int u = 0; u < SCAN_PER; ++u) {
+        const int64_t i = p0 + u * SCAN_THREADS + threadIdx.x;
+        if (i >= T) break;
+        const int64_t rem = offsets[doc_of(i, d0, d1) + 1] - i - 1;
+        remaining[i] = (uint8_t)(rem > 255 ? 255 : (rem < 0 ? 0 : rem));
+        const int t = tokens[i];
+        if (t < 0 || t >= vocab) set_status(status, TASC_EINVAL);
+        else atomicAdd(&hist[t], 1u);
+    }
 }
 __global__ void hist_argmax_kernel(const uint32_t* __restrict__ hist, int vocab, unsigned long long* best) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= vocab) return;
-    atomicMax(best, ((unsigned long long)hist[i] << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)i));
+    unsigned long long v = i < vocab ? ((unsigned long long)hist[i] << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)i) : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(best, v);
 }
 
-__global__ void count_kernel(const int32_t* __restrict__ tokens, const uint8_t* __restrict__ remaining, int64_t T, int n,
-                             uint64_t* keys, uint32_t* counts, uint64_t mask, int* status) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T || remaining[i] < n) return;
-    Key key = key_make(n);
-    for (int j = 0; j <= n; ++j) key_put(key, j, (uint32_t)tokens[i + j]);   // context 0..n-1, next in field n
-    const uint64_t slot = table_upsert(keys, mask, key);
-    if (slot == ~0ull) { set_status(status, TASC_ECAPACITY); return; }
-    atomicAdd(&counts[slot], 1u);
-}
+// ------------------------------------------------------------------------------------------- counting
+// Two slots to a sector; a key is in the first pair from its home pair on that had room.  (Memory goes by sectors: one per
+// window here, against two when keys of 16 bytes and counts were arrays of their own.  Filled to 4/5 at most, 1.25 slots per
+// window: a table of a power of two had 2 to 4.)
+struct __align__(16) CountSlot { unsigned long long key; uint32_t count, pos; };
+struct CountTable { CountSlot* slots; uint32_t pairs; };
+constexpr uint32_t NO_SLOT = 0xFFFFFFFFu;
+inline uint64_t count_pairs(uint64_t windows) { return (windows + windows / 4) / 2 + 32; }
 
-__global__ void survivors_kernel(const uint32_t* __restrict__ counts, uint64_t cap, uint32_t p_min, unsigned long long* n_surv) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool s = i < cap && counts[i] >= p_min;
-    const uint32_t b = __ballot_sync(0xFFFFFFFFu, s);
-    if ((threadIdx.x & 31) == 0 && b) atomicAdd(n_surv, (unsigned long long)__popc(b));
-}
-
-__device__ __forceinline__ Key context_of(Key entry, int n) {
-    // clear the `next` field (field n)
-    Key k = entry;
-    const int bit = n * TOK_BITS;
-    const uint64_t m = (uint64_t)TOK_MASK;
-    if (bit + TOK_BITS <= 64) k.lo &= ~(m << bit);
-    else if (bit >= 64) k.hi &= ~(m << (bit - 64));
-    else { k.lo &= ~(m << bit); k.hi &= ~(m >> (64 - bit)); }
+__device__ __forceinline__ uint64_t mix64(uint64_t k) {
+    k ^= k >> 32; k *= 0xD6E8FEB86659FD93ull; k ^= k >> 29; k *= 0x9E3779B97F4A7C15ull; k ^= k >> 32;
     return k;
 }
+// Counts one window; its slot, or NO_SLOT when the table is full.
+__device__ __forceinline__ uint32_t count_window(const CountTable& t, unsigned long long key, uint32_t pos) {
+    uint32_t pair = (uint32_t)__umul64hi(mix64(key), (uint64_t)t.pairs);
+    for (uint32_t probe = 0; probe < t.pairs; ++probe) {
+        CountSlot* s = t.slots + 2 * (size_t)pair;
+        unsigned long long k0 = __ldcg(&s[0].key), k1 = __ldcg(&s[1].key);
+        bool claimed = false;
+        if (k0 == 0ull) {
+            k0 = atomicCAS(&s[0].key, 0ull, key);
+            if (k0 == 0ull) { k0 = key; claimed = true; }
+        }
+        if (k0 != key && k1 == 0ull) {
+            k1 = atomicCAS(&s[1].key, 0ull, key);
+            if (k1 == 0ull) { k1 = key; claimed = true; }
+        }
+        if (k0 == key || k1 == key) {
+            const int i = k0 == key ? 0 : 1;
+            if (claimed) s[i].pos = pos;
+            atomicAdd(&s[i].count, 1u);
+            return 2 * pair + i;
+        }
+        pair = pair + 1 == t.pairs ? 0 : pair + 1;
+    }
+    return NO_SLOT;
+}
+// Order 1: all windows of two tokens.  id[i] = the slot of the one that starts at i (id may be null).
+__global__ void __launch_bounds__(256)
+count_pairs_kernel(const int32_t* __restrict__ tokens, const uint8_t* __restrict__ remaining, int64_t T, CountTable t, uint32_t* __restrict__ id, int* status) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= T) return;
+    uint32_t slot = NO_SLOT;
+    if (remaining[i] >= 1) {
+        const unsigned long long key = VALID_BIT | ((unsigned long long)((uint32_t)tokens[i] & TOK_MASK) << TOK_BITS) | ((uint32_t)tokens[i + 1] & TOK_MASK);
+        slot = count_window(t, key, (uint32_t)i);
+        if (slot == NO_SLOT) set_status(status, TASC_ECAPACITY);
+    }
+    if (id) id[i] = slot;
+}
+// Order n >= 2: prev[i] = slot of the order n - 1 window at i, NO_SLOT if there is none or it is too rare.
+__global__ void __launch_bounds__(256)
+count_next_kernel(const int32_t* __restrict__ tokens, const uint8_t* __restrict__ remaining, int64_t T, int n,
+                  const uint32_t* __restrict__ prev, CountTable t, uint32_t* __restrict__ id, int* status) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= T) return;
+    uint32_t slot = NO_SLOT;
+    if (remaining[i] >= n && prev[i] != NO_SLOT && prev[i + 1] != NO_SLOT) {
+        slot = count_window(t, VALID_BIT | ((unsigned long long)prev[i] << TOK_BITS) | ((uint32_t)tokens[i + n] & TOK_MASK), (uint32_t)i);
+        if (slot == NO_SLOT) set_status(status, TASC_ECAPACITY);
+    }
+    id[i] = slot;
+}
+// Takes the windows that stay below p_min out of id, and counts the positions where the next order has to look
+// (id[i + 1] is judged by its count: the neighbour may not have been taken out yet).
+__global__ void __launch_bounds__(256)
+prune_kernel(uint32_t* __restrict__ id, const uint8_t* __restrict__ remaining, int64_t T, int n, CountTable t, uint32_t p_min, unsigned long long* n_next) {
+    __shared__ uint32_t s_id[257];
+    __shared__ uint32_t s_n;
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (threadIdx.x == 0) s_n = 0;
+    auto keep = [&](int64_t p) {
+        const uint32_t v = p < T ? id[p] : NO_SLOT;
+        return v != NO_SLOT && t.slots[v].count >= p_min ? v : NO_SLOT;
+    };
+    const uint32_t v = keep(i);
+    s_id[threadIdx.x] = v;
+    __syncthreads();
+    // the last position of a block may count one window too many: the next block's first position is not looked up again
+    const bool next = v != NO_SLOT && remaining[i] >= n + 1 && (threadIdx.x == 255 || s_id[threadIdx.x + 1] != NO_SLOT);
+    const uint32_t b = __ballot_sync(0xFFFFFFFFu, next);
+    if ((threadIdx.x & 31) == 0 && b) atomicAdd(&s_n, (uint32_t)__popc(b));
+    if (i < T) id[i] = v;
+    __syncthreads();
+    if (threadIdx.x == 0 && s_n) atomicAdd(n_next, (unsigned long long)s_n);
+}
 
-__global__ void ctx_insert_kernel(const uint64_t* __restrict__ skeys, const uint32_t* __restrict__ counts, uint64_t cap,
-                                  uint32_t p_min, int n, OrderTable t, int* status) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cap || counts[i] < p_min) return;
-    const Key e = {skeys[2 * i], skeys[2 * i + 1]};
-    const uint64_t slot = table_upsert(t.keys, t.mask, context_of(e, n));
-    if (slot == ~0ull) { set_status(status, TASC_ECAPACITY); return; }
-    atomicAdd(&t.vals[slot].n_succ, 1u);
-    atomicAdd(&t.vals[slot].total, counts[i]);
+// ------------------------------------------------------------------------------------------- tables
+struct Survivor { uint32_t pos, count; };
+// Lists the n-grams that occur at least p_min times.  One reservation per block of LIST_SLOTS slots.
+constexpr int LIST_PER = 16, LIST_SLOTS = 256 * LIST_PER;
+__global__ void __launch_bounds__(256)
+list_kernel(CountTable t, uint32_t p_min, Survivor* __restrict__ list, unsigned long long* n_list) {
+    __shared__ uint32_t s_n;
+    __shared__ unsigned long long s_base;
+    const uint64_t n_slots = 2 * (uint64_t)t.pairs, s0 = (uint64_t)blockIdx.x * LIST_SLOTS + threadIdx.x;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    Survivor v[LIST_PER];
+    uint32_t at[LIST_PER];
+#pragma unroll
+    for (int u = 0; u < LIST_PER; ++u) {
+        const uint64_t s = s0 + u * 256;
+        v[u] = Survivor{0u, 0u};
+        if (s < n_slots) {
+            const uint4 x = *reinterpret_cast<const uint4*>(t.slots + s);
+            v[u] = Survivor{x.w, x.z};
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < LIST_PER; ++u) {
+        const bool yes = v[u].count >= p_min;
+        const uint32_t b = __ballot_sync(0xFFFFFFFFu, yes);
+        uint32_t base = 0;
+        if ((threadIdx.x & 31) == 0 && b) base = atomicAdd(&s_n, (uint32_t)__popc(b));
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        at[u] = yes ? base + __popc(b & ((1u << (threadIdx.x & 31)) - 1u)) : NO_SLOT;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && s_n) s_base = atomicAdd(n_list, (unsigned long long)s_n);
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < LIST_PER; ++u)
+        if (at[u] != NO_SLOT) list[s_base + at[u]] = v[u];
 }
-__global__ void assign_offsets_kernel(OrderTable t, unsigned long long* cursor) {
+
+// The elements of one order: from the corpus (a list of positions), or packed (tasc_drafter_import).
+struct CorpusElements {
+    const int32_t* tokens;
+    const Survivor* list;
+    __device__ __forceinline__ void get(uint64_t i, int n, Key& ctx, int& next, uint32_t& count) const {
+        const Survivor s = list[i];
+        ctx = key_make(n);
+        for (int j = 0; j < n; ++j) key_put(ctx, j, (uint32_t)tokens[(size_t)s.pos + j]);
+        next = (int)((uint32_t)tokens[(size_t)s.pos + n] & TOK_MASK);
+        count = s.count;
+    }
+};
+struct PackedElements {
+    const uint64_t* keys;
+    const uint32_t* counts;
+    __device__ __forceinline__ void get(uint64_t i, int n, Key& ctx, int& next, uint32_t& count) const {
+        const Key e = {keys[2 * i], keys[2 * i + 1]};
+        ctx = key_make(n);
+        for (int j = 0; j < n; ++j) key_put(ctx, j, key_get(e, j));
+        next = (int)key_get(e, n);
+        count = counts[i];
+    }
+};
+// place[i] = (slot of the element's context, its number among the context's successors)
+template <typename Elements>
+__global__ void __launch_bounds__(256) ctx_insert_kernel(Elements el, uint64_t n_el, int n, OrderTable t, uint2* __restrict__ place, int* status) {
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > t.mask) return;
-    const uint32_t n = t.vals[i].n_succ;
-    if (n) t.vals[i].offset = atomicAdd(cursor, (unsigned long long)n);
+    if (i >= n_el) return;
+    Key ctx;
+    int next;
+    uint32_t count;
+    el.get(i, n, ctx, next, count);
+    const uint64_t slot = table_upsert(t.keys, t.mask, ctx);
+    if (slot == ~0ull) { set_status(status, TASC_ECAPACITY); place[i] = make_uint2(NO_SLOT, 0u); return; }
+    // (n_succ, total) as one word: n_succ stays below 2^32, so nothing is carried into the total
+    const unsigned long long old = atomicAdd(reinterpret_cast<unsigned long long*>(&t.vals[slot].n_succ), ((unsigned long long)count << 32) | 1ull);
+    place[i] = make_uint2((uint32_t)slot, (uint32_t)old);
 }
-__global__ void succ_fill_kernel(const uint64_t* __restrict__ skeys, const uint32_t* __restrict__ counts, uint64_t cap,
-                                 uint32_t p_min, int n, OrderTable t, uint32_t* fill, int* status) {
+// Every context's share of the successor array; one reservation per block.
+__global__ void __launch_bounds__(256) assign_offsets_kernel(OrderTable t, unsigned long long* cursor) {
+    __shared__ uint32_t s_warp[8];
+    __shared__ unsigned long long s_base;
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cap || counts[i] < p_min) return;
-    const Key e = {skeys[2 * i], skeys[2 * i + 1]};
-    const uint64_t slot = table_upsert(t.keys, t.mask, context_of(e, n));     // always found
-    if (slot == ~0ull) { set_status(status, TASC_ECAPACITY); return; }
-    const unsigned long long pos = t.vals[slot].offset + atomicAdd(&fill[slot], 1u);
-    if (pos >= (unsigned long long)t.n_succ) { set_status(status, TASC_ECAPACITY); return; }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t n = i <= t.mask ? t.vals[i].n_succ : 0u;
+    uint32_t x = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[warp] = x;
+    __syncthreads();
+    uint32_t before = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) { if (w < warp) before += s_warp[w]; total += s_warp[w]; }
+    if (threadIdx.x == 0 && total) s_base = atomicAdd(cursor, (unsigned long long)total);
+    __syncthreads();
+    if (n) t.vals[i].offset = s_base + before + x - n;
+}
+template <typename Elements>
+__global__ void __launch_bounds__(256) succ_fill_kernel(Elements el, uint64_t n_el, int n, OrderTable t, const uint2* __restrict__ place, int* status) {
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_el || place[i].x == NO_SLOT) return;
+    Key ctx;
     Succ s;
-    s.next = (int32_t)key_get(e, n);
-    s.count = counts[i];
+    el.get(i, n, ctx, s.next, s.count);
+    const unsigned long long pos = t.vals[place[i].x].offset + place[i].y;
+    if (pos >= (unsigned long long)t.n_succ) { set_status(status, TASC_ECAPACITY); return; }
     t.succ[pos] = s;
 }
-
+// The table of one order from its elements.  contexts: an upper bound of how many there are.
+template <typename Elements>
+tasc_status build_order(tasc_drafter* d, int n, const Elements& el, uint64_t n_el, uint64_t contexts, uint2* place, unsigned long long* cursor,
+                        int* status, cudaStream_t stream) {
+    OrderTable& t = d->dt.t[n];
+    DeviceSlab& slab = d->slab[n];
+    const uint64_t ccap = pow2_at_least(2 * std::min(n_el, contexts));
+    const size_t o_keys = slab.add(ccap * 16), o_vals = slab.add(ccap * sizeof(CtxVal)), o_succ = slab.add(n_el * sizeof(Succ));
+    if (!slab.allocate(stream)) return TASC_ENOMEM;
+    t = OrderTable{slab.at<uint64_t>(o_keys), slab.at<CtxVal>(o_vals), slab.at<Succ>(o_succ), ccap - 1, (long long)n_el};
+    TASC_CUDA_TRY(cudaMemsetAsync(t.keys, 0, o_succ, stream));         // keys and values
+    TASC_CUDA_TRY(cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), stream));
+    ctx_insert_kernel<<<blocks_for(n_el, 256), 256, 0, stream>>>(el, n_el, n, t, place, status);
+    assign_offsets_kernel<<<blocks_for(ccap, 256), 256, 0, stream>>>(t, cursor);
+    succ_fill_kernel<<<blocks_for(n_el, 256), 256, 0, stream>>>(el, n_el, n, t, place, status);
+    TASC_CUDA_TRY(cudaGetLastError());
+    return TASC_OK;
+}
 
 // Order-1 model with one successor of count 1 per context: context token c -> table[c].
 __global__ void bigram_insert_kernel(const int32_t* __restrict__ table, int vocab, OrderTable t, int* status) {
@@ -158,23 +356,33 @@ __global__ void bigram_insert_kernel(const int32_t* __restrict__ table, int voca
 }
 
 // ------------------------------------------------------------------------------------------- corpus statistics
-// The statistics are functions of the multiset of counts only, so the device first turns the count table into a
-// histogram of count VALUES (how many bigrams occur c times), which is exact integer work whose result does not
-// depend on where the hash table put anything; one block then walks that histogram in a fixed order.
+// The statistics are functions of the multiset of counts only, so the device first turns the counts into a histogram of
+// count VALUES (how many bigrams occur c times), which is exact integer work whose result does not depend on where the
+// hash table put anything; that histogram is then added up in a fixed order, from the largest count value down.
 constexpr int CC_BITS = 20;                       // count values below 2^20 have a histogram bin of their own
 constexpr uint32_t CC_BINS = 1u << CC_BITS;
 constexpr int CC_OVERFLOW = 4096;                 // larger count values are listed individually
-constexpr int STATS_THREADS = 1024;
+constexpr int CC_LOW = 1024;                      // ... and nearly all counts are below this: binned in shared memory first
+constexpr int STATS_THREADS = 256, BIN_PER = 16, BIN_CHUNK = STATS_THREADS * BIN_PER, BIN_CHUNKS = (int)(CC_BINS / BIN_CHUNK);
 
-// [0] distinct keys, [1] overflow entries, [2] sum of squared counts
-__global__ void count_values_kernel(const uint32_t* __restrict__ counts, uint64_t n, uint32_t* __restrict__ bins,
-                                    uint32_t* __restrict__ overflow, unsigned long long* __restrict__ scal, int* status) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t c = i < n ? counts[i] : 0u;
-    unsigned long long sq = (unsigned long long)c * c;
-    unsigned int nz = c ? 1u : 0u;
-    if (c) {
-        if (c < CC_BINS) atomicAdd(&bins[c], 1u);
+// counts[i * stride], i < n.  scal: [0] distinct keys, [1] overflow entries, [2] sum of squared counts
+__global__ void __launch_bounds__(STATS_THREADS)
+count_values_kernel(const uint32_t* __restrict__ counts, int stride, uint64_t n, uint32_t* __restrict__ bins,
+                    uint32_t* __restrict__ overflow, unsigned long long* __restrict__ scal, int* status) {
+    __shared__ uint32_t low[CC_LOW];
+    for (int i = threadIdx.x; i < CC_LOW; i += STATS_THREADS) low[i] = 0u;
+    __syncthreads();
+    unsigned long long sq = 0ull;
+    unsigned int nz = 0u;
+    const uint64_t step = (uint64_t)gridDim.x * STATS_THREADS;
+#pragma unroll 8
+    for (uint64_t i = (uint64_t)blockIdx.x * STATS_THREADS + threadIdx.x; i < n; i += step) {
+        const uint32_t c = counts[i * stride];
+        if (!c) continue;
+        sq += (unsigned long long)c * c;
+        ++nz;
+        if (c < CC_LOW) atomicAdd(&low[c], 1u);
+        else if (c < CC_BINS) atomicAdd(&bins[c], 1u);
         else {
             const unsigned long long at = atomicAdd(&scal[1], 1ull);
             if (at < CC_OVERFLOW) overflow[at] = c; else set_status(status, TASC_ECAPACITY);
@@ -189,6 +397,9 @@ __global__ void count_values_kernel(const uint32_t* __restrict__ counts, uint64_
         atomicAdd(&scal[0], (unsigned long long)nz);
         atomicAdd(&scal[2], sq);                   // integer sums: the order of the additions does not matter
     }
+    __syncthreads();
+    for (int i = threadIdx.x; i < CC_LOW; i += STATS_THREADS)
+        if (low[i]) atomicAdd(&bins[i], low[i]);
 }
 
 struct CountSummary {
@@ -198,20 +409,57 @@ struct CountSummary {
     unsigned long long n_for_cdf;    // smallest number of the largest counts that reach cdf_num / cdf_den of n_total
     double sum_c_log2_c;             // sum over all keys of c log2 c
 };
+struct BinSum { unsigned long long mass, keys; double lg; };
 
-// One block.  bins[c] = number of keys with count c (c < 2^20), overflow[] = the counts >= 2^20.  Walks the count
-// values from the largest down: thread t owns a contiguous range of bins, an exclusive scan over the threads
-// gives the mass and the number of keys above its range, and the thread whose range holds the crossing of the
-// coverage target finishes the count by itself.  Sums are taken in a fixed order, so the result is reproducible.
+// A thread's BIN_PER bins of chunk `chunk` (chunk 0 has the largest count values, thread 0 the largest of a chunk).
+__device__ __forceinline__ uint32_t bin_top(int chunk) { return CC_BINS - 1u - (uint32_t)chunk * BIN_CHUNK - (uint32_t)threadIdx.x * BIN_PER; }
+// Sum of the block's values in thread 0, added in a fixed order.
+__device__ __forceinline__ BinSum bin_reduce(BinSum v, BinSum* red) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        v.mass += __shfl_down_sync(0xFFFFFFFFu, v.mass, o);
+        v.keys += __shfl_down_sync(0xFFFFFFFFu, v.keys, o);
+        v.lg += __shfl_down_sync(0xFFFFFFFFu, v.lg, o);
+    }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int i = 1; i < STATS_THREADS / 32; ++i) { v.mass += red[i].mass; v.keys += red[i].keys; v.lg += red[i].lg; }
+    return v;
+}
+// grid (BIN_CHUNKS, 2): the sums of a chunk of bins of the bigrams (y = 0) and the tokens (y = 1).  (One block that walked all
+// bins of one histogram: 0.75 ms.)
+__global__ void __launch_bounds__(STATS_THREADS) bin_sums_kernel(const uint32_t* __restrict__ bins, BinSum* __restrict__ sums) {
+    __shared__ BinSum red[STATS_THREADS / 32];
+    const uint32_t* b = bins + (size_t)blockIdx.y * CC_BINS;
+    const uint32_t top = bin_top(blockIdx.x);
+    uint32_t m[BIN_PER];
+#pragma unroll
+    for (int i = 0; i < BIN_PER; ++i) m[i] = b[top - i];
+    BinSum v = {0ull, 0ull, 0.0};
+#pragma unroll
+    for (int i = 0; i < BIN_PER; ++i) {
+        const uint32_t c = top - i;
+        if (c && m[i]) { v.mass += (unsigned long long)m[i] * c; v.keys += m[i]; v.lg += (double)m[i] * ((double)c * log2((double)c)); }
+    }
+    v = bin_reduce(v, red);
+    if (threadIdx.x == 0) sums[blockIdx.y * BIN_CHUNKS + blockIdx.x] = v;
+}
+// One block per histogram: adds up the overflow list and the chunks, and finds where the counts, from the largest down,
+// reach the coverage target: in the list, or in one chunk, where the thread whose bins hold the crossing finishes the count.
 __global__ void __launch_bounds__(STATS_THREADS)
-count_summary_kernel(const uint32_t* __restrict__ bins, uint32_t* __restrict__ overflow, const unsigned long long* __restrict__ scal,
-                     unsigned long long cdf_num, unsigned long long cdf_den, CountSummary* out) {
+count_summary_kernel(const uint32_t* __restrict__ bins, const BinSum* __restrict__ sums, const uint32_t* __restrict__ overflow_,
+                     const unsigned long long* __restrict__ scal_, unsigned long long cdf_num_, unsigned long long cdf_den_, CountSummary* out_) {
+    __shared__ BinSum s_sum[BIN_CHUNKS];
     __shared__ unsigned long long s_mass[STATS_THREADS], s_keys[STATS_THREADS];
-    __shared__ double s_log[STATS_THREADS];
     __shared__ uint32_t s_over[CC_OVERFLOW];
-    __shared__ unsigned long long s_result, s_over_mass;
-    __shared__ double s_over_log;
-    const int t = threadIdx.x;
+    __shared__ unsigned long long s_need, s_above, s_k;
+    __shared__ int s_chunk;
+    const int set = blockIdx.x, t = threadIdx.x;
+    const uint32_t *b = bins + (size_t)set * CC_BINS, *overflow = overflow_ + (size_t)set * CC_OVERFLOW;
+    const unsigned long long* scal = scal_ + 4 * set;
+    const unsigned long long cdf_num = set ? 1ull : cdf_num_, cdf_den = set ? 1ull : cdf_den_;
+    CountSummary* out = out_ + set;
     const int n_over = (int)min(scal[1], (unsigned long long)CC_OVERFLOW);
     // the overflow list, largest first: rank by counting (a few thousand entries at most)
     for (int i = t; i < n_over; i += STATS_THREADS) {
@@ -223,70 +471,53 @@ count_summary_kernel(const uint32_t* __restrict__ bins, uint32_t* __restrict__ o
         }
         s_over[rank] = c;
     }
+    for (int i = t; i < BIN_CHUNKS; i += STATS_THREADS) s_sum[i] = sums[set * BIN_CHUNKS + i];
     __syncthreads();
     if (t == 0) {
-        unsigned long long m = 0;
+        unsigned long long m = 0, k = (unsigned long long)n_over;
         double l = 0.0;
         for (int i = 0; i < n_over; ++i) { m += s_over[i]; l += (double)s_over[i] * log2((double)s_over[i]); }
-        s_over_mass = m; s_over_log = l; s_result = 0ull;
-    }
-    // thread t owns bins hi, hi - 1, ..., lo (descending count values)
-    constexpr uint32_t PER = CC_BINS / STATS_THREADS;
-    const uint32_t hi = CC_BINS - 1u - (uint32_t)t * PER, lo = hi - (PER - 1u);
-    unsigned long long mass = 0, keys = 0;
-    double lg = 0.0;
-    for (uint32_t c = hi; ; --c) {
-        const uint32_t m = c ? bins[c] : 0u;
-        if (m) { mass += (unsigned long long)m * c; keys += m; lg += (double)m * ((double)c * log2((double)c)); }
-        if (c == lo) break;
-    }
-    s_mass[t] = mass; s_keys[t] = keys; s_log[t] = lg;
-    __syncthreads();
-    if (t == 0) {
-        // serial exclusive scan over the 1,024 partial sums (fixed order)
-        unsigned long long m = s_over_mass, k = (unsigned long long)n_over;
-        double l = s_over_log;
-        for (int i = 0; i < STATS_THREADS; ++i) {
-            const unsigned long long mi = s_mass[i], ki = s_keys[i];
-            l += s_log[i];
-            s_mass[i] = m; s_keys[i] = k;
-            m += mi; k += ki;
-        }
+        for (int i = 0; i < BIN_CHUNKS; ++i) { m += s_sum[i].mass; k += s_sum[i].keys; l += s_sum[i].lg; }
         out->n_total = m; out->n_distinct = k; out->sum_sq = scal[2]; out->sum_c_log2_c = l;
-        s_over_mass = m;                                     // total mass, for the threads below
-    }
-    __syncthreads();
-    const unsigned long long total = s_over_mass;
-    if (total == 0) { if (t == 0) out->n_for_cdf = 0; return; }
-    // target: smallest run with run * den >= num * total.  128-bit products are not needed: total < 2^40, num, den <= 2^16.
-    const unsigned long long need = (cdf_num * total + cdf_den - 1) / cdf_den;
-    if (t == 0) {
-        // crossing inside the overflow list?
+        out->n_for_cdf = 0;
+        s_chunk = -1;
+        // target: smallest run with run * den >= num * total.  128-bit products are not needed: total < 2^40, num, den <= 2^16.
+        const unsigned long long need = (cdf_num * m + cdf_den - 1) / cdf_den;
         unsigned long long run = 0;
-        for (int i = 0; i < n_over; ++i) {
+        k = 0;
+        bool found = m == 0;
+        for (int i = 0; i < n_over && !found; ++i) {
             run += s_over[i];
-            if (run >= need) { s_result = (unsigned long long)i + 1; break; }
+            ++k;
+            if (run >= need) { out->n_for_cdf = k; found = true; }
+        }
+        for (int i = 0; i < BIN_CHUNKS && !found; ++i) {
+            if (run + s_sum[i].mass >= need) { s_chunk = i; s_need = need; s_above = run; s_k = k; found = true; }
+            run += s_sum[i].mass;
+            k += s_sum[i].keys;
         }
     }
     __syncthreads();
-    const unsigned long long above = s_mass[t];
-    if (s_result == 0 && above < need && above + mass >= need) {
-        unsigned long long run = above, k = s_keys[t];
-        for (uint32_t c = hi; ; --c) {
-            const uint32_t m = c ? bins[c] : 0u;
-            if (m) {
-                if (run + (unsigned long long)m * c >= need) {
-                    k += (need - run + c - 1) / c;
-                    break;
-                }
-                run += (unsigned long long)m * c; k += m;
-            }
-            if (c == lo) break;
-        }
-        s_result = k;
+    if (s_chunk < 0) return;
+    const uint32_t top = bin_top(s_chunk);
+    unsigned long long mass = 0, keys = 0;
+    for (int i = 0; i < BIN_PER; ++i) {
+        const uint32_t c = top - i, m = c ? b[c] : 0u;
+        mass += (unsigned long long)m * c;
+        keys += m;
     }
+    s_mass[t] = mass; s_keys[t] = keys;
     __syncthreads();
-    if (t == 0) out->n_for_cdf = s_result;
+    unsigned long long run = s_above, k = s_k;
+    for (int i = 0; i < t; ++i) { run += s_mass[i]; k += s_keys[i]; }
+    if (run >= s_need || run + mass < s_need) return;
+    for (int i = 0; i < BIN_PER; ++i) {
+        const uint32_t c = top - i, m = c ? b[c] : 0u;
+        if (!m) continue;
+        if (run + (unsigned long long)m * c >= s_need) { out->n_for_cdf = k + (s_need - run + c - 1) / c; return; }
+        run += (unsigned long long)m * c;
+        k += m;
+    }
 }
 
 // ------------------------------------------------------------------------------------------- draft
@@ -470,13 +701,79 @@ draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t 
     }
 }
 
-void free_tables(DeviceTables& dt) {
-    for (int n = 0; n <= TASC_MAX_ORDER; ++n) {
-        if (dt.t[n].keys) cudaFree(dt.t[n].keys);
-        if (dt.t[n].vals) cudaFree(dt.t[n].vals);
-        if (dt.t[n].succ) cudaFree(dt.t[n].succ);
-        dt.t[n] = OrderTable{nullptr, nullptr, nullptr, 0, 0};
+tasc_drafter* new_drafter(int n_max, int fallback, int p_min, int vocab) {
+    tasc_drafter* d = new (std::nothrow) tasc_drafter();
+    if (!d) return nullptr;
+    for (int n = 0; n <= TASC_MAX_ORDER; ++n) d->dt.t[n] = OrderTable{nullptr, nullptr, nullptr, 0, 0};
+    d->dt.n_max = n_max; d->dt.fallback = fallback; d->p_min = p_min; d->vocab = vocab;
+    if (cudaGetDevice(&d->device) != cudaSuccess) (void)cudaGetLastError();
+    return d;
+}
+// Frees the handle when nothing on its device reads the tables any more.
+void free_drafter(tasc_drafter* d) {
+    int dev = d->device;
+    if (cudaGetDevice(&dev) != cudaSuccess) (void)cudaGetLastError();
+    if (dev != d->device) cudaSetDevice(d->device);
+    if (cudaDeviceSynchronize() != cudaSuccess) (void)cudaGetLastError();
+    for (DeviceSlab& s : d->slab) s.release(nullptr);
+    if (dev != d->device) cudaSetDevice(dev);
+    delete d;
+}
+
+// Everything of tasc_drafter_build that can fail once the handle exists.
+tasc_status build_from_corpus(tasc_drafter* d, const int32_t* tokens, const int64_t* offsets, int64_t n_docs, const CorpusCheck& c, cudaStream_t stream) {
+    const int64_t T = c.tokens;
+    if (T == 0) return TASC_OK;                  // (the fallback stays 0)
+    if (T >= (1ll << 32) - 1 || count_pairs(c.pairs) >= (1ull << 31)) return TASC_ENOMEM;
+    const int n_max = d->dt.n_max, p_min = d->p_min, vocab = d->vocab;
+    // scalars: [0] histogram argmax, [1] n-grams listed, [2] positions left for the next order, [3] cursor, [4] status
+    DeviceSlab slab;
+    const uint64_t pairs1 = count_pairs(c.pairs), list_max = c.pairs / (uint64_t)p_min + 1;
+    const size_t o_scal = slab.add(64), o_hist = slab.add((size_t)vocab * 4), o_slots = slab.add(pairs1 * 2 * sizeof(CountSlot)),
+                 o_id0 = slab.add((size_t)T * 4), o_id1 = slab.add((size_t)T * 4), o_rem = slab.add((size_t)T),
+                 o_list = slab.add(list_max * sizeof(Survivor)), o_place = slab.add(list_max * sizeof(uint2));
+    if (!slab.allocate(stream)) return TASC_ENOMEM;
+    unsigned long long* scal = slab.at<unsigned long long>(o_scal);
+    int* status = reinterpret_cast<int*>(scal + 4);
+    uint32_t *hist = slab.at<uint32_t>(o_hist), *id = slab.at<uint32_t>(o_id0), *prev = slab.at<uint32_t>(o_id1);
+    uint8_t* remaining = slab.at<uint8_t>(o_rem);
+    Survivor* list = slab.at<Survivor>(o_list);
+    TASC_CUDA_TRY(cudaMemsetAsync(scal, 0, o_hist + (size_t)vocab * 4, stream));
+    corpus_scan_kernel<<<blocks_for(T, SCAN_POS), SCAN_THREADS, 0, stream>>>(tokens, offsets, n_docs, T, vocab, remaining, hist, status);
+    hist_argmax_kernel<<<blocks_for(vocab, 256), 256, 0, stream>>>(hist, vocab, scal);
+    unsigned long long h[5];
+    uint64_t windows = c.pairs, contexts = (uint64_t)vocab;
+    for (int n = 1; n <= n_max && windows; ++n) {
+        const CountTable t = {slab.at<CountSlot>(o_slots), (uint32_t)count_pairs(windows)};
+        TASC_CUDA_TRY(cudaMemsetAsync(t.slots, 0, (size_t)t.pairs * 2 * sizeof(CountSlot), stream));
+        TASC_CUDA_TRY(cudaMemsetAsync(scal + 1, 0, 2 * sizeof(*scal), stream));
+        if (n == 1) count_pairs_kernel<<<blocks_for(T, 256), 256, 0, stream>>>(tokens, remaining, T, t, id, status);
+        else count_next_kernel<<<blocks_for(T, 256), 256, 0, stream>>>(tokens, remaining, T, n, prev, t, id, status);
+        list_kernel<<<blocks_for(2 * (uint64_t)t.pairs, LIST_SLOTS), 256, 0, stream>>>(t, (uint32_t)p_min, list, scal + 1);
+        if (n < n_max) prune_kernel<<<blocks_for(T, 256), 256, 0, stream>>>(id, remaining, T, n, t, (uint32_t)p_min, scal + 2);
+        TASC_CUDA_TRY(cudaGetLastError());
+        TASC_CUDA_TRY(cudaMemcpyAsync(h, scal, sizeof(h), cudaMemcpyDeviceToHost, stream));
+        TASC_CUDA_TRY(cudaStreamSynchronize(stream));
+        if ((int)h[4] != 0) return (int)h[4];                    // a token id outside [0, vocab)
+        if (n == 1) d->dt.fallback = (int)(0xFFFFFFFFu - (uint32_t)(h[0] & 0xFFFFFFFFull));
+        if (h[1] == 0) break;                                    // nor can anything longer be frequent
+        const tasc_status rc = build_order(d, n, CorpusElements{tokens, list}, h[1], contexts, slab.at<uint2>(o_place), scal + 3, status, stream);
+        if (rc != TASC_OK) return rc;
+        windows = h[2];
+        contexts = h[1];                                         // every context of the next order is one of these
+        std::swap(id, prev);
     }
+    if (c.pairs == 0) {
+        TASC_CUDA_TRY(cudaMemcpyAsync(h, scal, sizeof(h), cudaMemcpyDeviceToHost, stream));
+        TASC_CUDA_TRY(cudaStreamSynchronize(stream));
+        if ((int)h[4] != 0) return (int)h[4];
+        d->dt.fallback = (int)(0xFFFFFFFFu - (uint32_t)(h[0] & 0xFFFFFFFFull));
+        return TASC_OK;
+    }
+    int st = 0;
+    TASC_CUDA_TRY(cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, stream));
+    TASC_CUDA_TRY(cudaStreamSynchronize(stream));
+    return st;
 }
 
 }  // namespace
@@ -493,110 +790,14 @@ extern "C" tasc_status tasc_drafter_build(const int32_t* corpus_tokens, const in
         vocab > (1 << TASC_VOCAB_BITS))
         return TASC_EINVAL;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    std::vector<int64_t> offs((size_t)n_docs + 1);
-    TASC_CUDA_TRY(cudaMemcpyAsync(offs.data(), doc_offsets, offs.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
-    TASC_CUDA_TRY(cudaStreamSynchronize(stream));
-    if (offs[0] != 0) return TASC_EINVAL;
-    uint64_t windows[TASC_MAX_ORDER + 1] = {0};
-    for (int64_t d = 0; d < n_docs; ++d) {
-        const int64_t len = offs[d + 1] - offs[d];
-        if (len < 0) return TASC_EINVAL;
-        for (int n = 1; n <= n_max; ++n) windows[n] += (uint64_t)std::max<int64_t>(0, len - n);
-    }
-    const int64_t T = offs[n_docs];
-    if (T > 0 && !corpus_tokens) return TASC_EINVAL;
-
-    tasc_drafter* d = new (std::nothrow) tasc_drafter();
+    CorpusCheck c;
+    tasc_status rc = check_corpus(doc_offsets, n_docs, c, stream);
+    if (rc != TASC_OK) return rc;
+    if (c.tokens > 0 && !corpus_tokens) return TASC_EINVAL;
+    tasc_drafter* d = new_drafter(n_max, 0, p_min, vocab);
     if (!d) return TASC_ENOMEM;
-    for (int n = 0; n <= TASC_MAX_ORDER; ++n) d->dt.t[n] = OrderTable{nullptr, nullptr, nullptr, 0, 0};
-    d->dt.n_max = n_max; d->dt.fallback = 0; d->p_min = p_min; d->vocab = vocab;
-    cudaGetDevice(&d->device);
-
-    // scratch shared by all orders
-    uint8_t* remaining = nullptr;
-    uint32_t* hist = nullptr;
-    unsigned long long* scalars = nullptr;     // [0] histogram argmax, [1] survivors, [2] cursor
-    int* status = nullptr;
-    uint64_t* skeys = nullptr;
-    uint32_t* scounts = nullptr;
-    uint32_t* fill = nullptr;
-    const uint64_t scap = pow2_at_least(2 * std::max<uint64_t>(windows[1], 1));
-    tasc_status rc = TASC_OK;
-    auto fail = [&](tasc_status s) { rc = s; };
-#define TRY_ALLOC(ptr, bytes) if (rc == TASC_OK && cudaMalloc(reinterpret_cast<void**>(&(ptr)), (bytes)) != cudaSuccess) { (void)cudaGetLastError(); fail(TASC_ENOMEM); }
-    TRY_ALLOC(remaining, (size_t)std::max<int64_t>(T, 1));
-    TRY_ALLOC(hist, (size_t)vocab * sizeof(uint32_t));
-    TRY_ALLOC(scalars, 4 * sizeof(unsigned long long));
-    TRY_ALLOC(status, sizeof(int));
-    TRY_ALLOC(skeys, scap * 16);
-    TRY_ALLOC(scounts, scap * 4);
-    if (rc == TASC_OK) {
-        cudaMemsetAsync(hist, 0, (size_t)vocab * sizeof(uint32_t), stream);
-        cudaMemsetAsync(scalars, 0, 4 * sizeof(unsigned long long), stream);
-        cudaMemsetAsync(status, 0, sizeof(int), stream);
-        if (T > 0) {
-            mark_remaining_kernel<<<blocks_for(T, 256), 256, 0, stream>>>(doc_offsets, n_docs, T, remaining);
-            token_hist_kernel<<<blocks_for(T, 256), 256, 0, stream>>>(corpus_tokens, T, vocab, hist, status);
-        }
-        hist_argmax_kernel<<<blocks_for(vocab, 256), 256, 0, stream>>>(hist, vocab, scalars);
-        int st = 0;
-        unsigned long long best = 0;
-        if (cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
-            cudaMemcpyAsync(&best, scalars, sizeof(best), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
-            cudaStreamSynchronize(stream) != cudaSuccess) { (void)cudaGetLastError(); fail(TASC_ECUDA); }
-        else if (st != 0) fail(st);               // a token id outside [0, vocab)
-        else d->dt.fallback = T > 0 ? (int)(0xFFFFFFFFu - (uint32_t)(best & 0xFFFFFFFFull)) : 0;
-    }
-    for (int n = 1; n <= n_max && rc == TASC_OK; ++n) {
-        if (windows[n] == 0) continue;
-        const uint64_t cap = pow2_at_least(2 * windows[n]);      // <= scap
-        cudaMemsetAsync(skeys, 0, cap * 16, stream);
-        cudaMemsetAsync(scounts, 0, cap * 4, stream);
-        cudaMemsetAsync(scalars + 1, 0, 2 * sizeof(unsigned long long), stream);
-        count_kernel<<<blocks_for(T, 256), 256, 0, stream>>>(corpus_tokens, remaining, T, n, skeys, scounts, cap - 1, status);
-        survivors_kernel<<<blocks_for(cap, 256), 256, 0, stream>>>(scounts, cap, (uint32_t)p_min, scalars + 1);
-        unsigned long long n_surv = 0;
-        if (cudaMemcpyAsync(&n_surv, scalars + 1, sizeof(n_surv), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
-            cudaStreamSynchronize(stream) != cudaSuccess) { (void)cudaGetLastError(); fail(TASC_ECUDA); break; }
-        if (n_surv == 0) continue;
-        OrderTable& t = d->dt.t[n];
-        const uint64_t ccap = pow2_at_least(2 * n_surv);
-        t.mask = ccap - 1;
-        t.n_succ = (long long)n_surv;
-        TRY_ALLOC(t.keys, ccap * 16);
-        TRY_ALLOC(t.vals, ccap * sizeof(CtxVal));
-        TRY_ALLOC(t.succ, n_surv * sizeof(Succ));
-        TRY_ALLOC(fill, ccap * sizeof(uint32_t));
-        if (rc != TASC_OK) break;
-        cudaMemsetAsync(t.keys, 0, ccap * 16, stream);
-        cudaMemsetAsync(t.vals, 0, ccap * sizeof(CtxVal), stream);
-        cudaMemsetAsync(fill, 0, ccap * sizeof(uint32_t), stream);
-        ctx_insert_kernel<<<blocks_for(cap, 256), 256, 0, stream>>>(skeys, scounts, cap, (uint32_t)p_min, n, t, status);
-        assign_offsets_kernel<<<blocks_for(ccap, 256), 256, 0, stream>>>(t, scalars + 2);
-        succ_fill_kernel<<<blocks_for(cap, 256), 256, 0, stream>>>(skeys, scounts, cap, (uint32_t)p_min, n, t, fill, status);
-        if (cudaStreamSynchronize(stream) != cudaSuccess) { (void)cudaGetLastError(); fail(TASC_ECUDA); break; }
-        cudaFree(fill);
-        fill = nullptr;
-    }
-    if (rc == TASC_OK) {
-        int st = 0;
-        if (cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
-            cudaStreamSynchronize(stream) != cudaSuccess) { (void)cudaGetLastError(); fail(TASC_ECUDA); }
-        else if (st != 0) fail(st);
-    }
-#undef TRY_ALLOC
-    if (fill) cudaFree(fill);
-    if (remaining) cudaFree(remaining);
-    if (hist) cudaFree(hist);
-    if (scalars) cudaFree(scalars);
-    if (status) cudaFree(status);
-    if (skeys) cudaFree(skeys);
-    if (scounts) cudaFree(scounts);
-    if (rc != TASC_OK) {
-        free_tables(d->dt);
-        delete d;
-        return rc;
-    }
+    rc = build_from_corpus(d, corpus_tokens, doc_offsets, n_docs, c, stream);
+    if (rc != TASC_OK) { free_drafter(d); return rc; }
     *out = d;
     return TASC_OK;
 }
@@ -606,37 +807,25 @@ extern "C" tasc_status tasc_drafter_from_bigram(const int32_t* table, int32_t vo
     *out = nullptr;
     if (!table || vocab < 1 || vocab > (1 << TASC_VOCAB_BITS)) return TASC_EINVAL;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    tasc_drafter* d = new (std::nothrow) tasc_drafter();
+    tasc_drafter* d = new_drafter(1, 0, 1, vocab);
     if (!d) return TASC_ENOMEM;
-    for (int n = 0; n <= TASC_MAX_ORDER; ++n) d->dt.t[n] = OrderTable{nullptr, nullptr, nullptr, 0, 0};
-    d->dt.n_max = 1; d->dt.fallback = 0; d->p_min = 1; d->vocab = vocab;
-    cudaGetDevice(&d->device);
     OrderTable& t = d->dt.t[1];
+    DeviceSlab& slab = d->slab[1];
     const uint64_t cap = pow2_at_least(2 * (uint64_t)vocab);
-    t.mask = cap - 1;
-    t.n_succ = vocab;
-    int* status = nullptr;
+    const size_t o_status = slab.add(sizeof(int)), o_keys = slab.add(cap * 16), o_vals = slab.add(cap * sizeof(CtxVal)), o_succ = slab.add((size_t)vocab * sizeof(Succ));
     tasc_status rc = TASC_OK;
-    if (cudaMalloc(reinterpret_cast<void**>(&t.keys), cap * 16) != cudaSuccess ||
-        cudaMalloc(reinterpret_cast<void**>(&t.vals), cap * sizeof(CtxVal)) != cudaSuccess ||
-        cudaMalloc(reinterpret_cast<void**>(&t.succ), (size_t)vocab * sizeof(Succ)) != cudaSuccess ||
-        cudaMalloc(reinterpret_cast<void**>(&status), sizeof(int)) != cudaSuccess) { (void)cudaGetLastError(); rc = TASC_ENOMEM; }
+    if (!slab.allocate(stream)) rc = TASC_ENOMEM;
     if (rc == TASC_OK) {
-        cudaMemsetAsync(t.keys, 0, cap * 16, stream);
-        cudaMemsetAsync(t.vals, 0, cap * sizeof(CtxVal), stream);
-        cudaMemsetAsync(status, 0, sizeof(int), stream);
+        int* status = slab.at<int>(o_status);
+        t = OrderTable{slab.at<uint64_t>(o_keys), slab.at<CtxVal>(o_vals), slab.at<Succ>(o_succ), cap - 1, vocab};
+        cudaMemsetAsync(status, 0, o_succ, stream);                    // status, keys and values
         bigram_insert_kernel<<<blocks_for((uint64_t)vocab, 256), 256, 0, stream>>>(table, vocab, t, status);
         int st = 0;
         if (cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
             cudaStreamSynchronize(stream) != cudaSuccess) { (void)cudaGetLastError(); rc = TASC_ECUDA; }
         else if (st != 0) rc = st;
     }
-    if (status) cudaFree(status);
-    if (rc != TASC_OK) {
-        free_tables(d->dt);
-        delete d;
-        return rc;
-    }
+    if (rc != TASC_OK) { free_drafter(d); return rc; }
     *out = d;
     return TASC_OK;
 }
@@ -648,66 +837,49 @@ extern "C" tasc_status tasc_corpus_stats(const int32_t* corpus_tokens, const int
         return TASC_EINVAL;
     *out = tasc_corpus_statistics{};
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    std::vector<int64_t> offs((size_t)n_docs + 1);
-    TASC_CUDA_TRY(cudaMemcpyAsync(offs.data(), doc_offsets, offs.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
-    TASC_CUDA_TRY(cudaStreamSynchronize(stream));
-    if (offs[0] != 0) return TASC_EINVAL;
-    uint64_t pairs = 0;
-    for (int64_t d = 0; d < n_docs; ++d) {
-        const int64_t len = offs[d + 1] - offs[d];
-        if (len < 0) return TASC_EINVAL;
-        pairs += (uint64_t)std::max<int64_t>(0, len - 1);
-    }
-    const int64_t T = offs[n_docs];
+    CorpusCheck c;
+    const tasc_status rc = check_corpus(doc_offsets, n_docs, c, stream);
+    if (rc != TASC_OK) return rc;
+    const int64_t T = c.tokens;
     if (T > 0 && !corpus_tokens) return TASC_EINVAL;
     if ((uint64_t)T >= (1ull << 40)) return TASC_EINVAL;
+    if (T >= (1ll << 32) - 1 || count_pairs(c.pairs) >= (1ull << 31)) return TASC_ENOMEM;
 
-    uint8_t* remaining = nullptr;
-    uint32_t *hist = nullptr, *bins = nullptr, *overflow = nullptr, *scounts = nullptr;
-    unsigned long long* scal = nullptr;      // [0..2] bigram scalars, [4..6] token scalars
-    CountSummary* summ = nullptr;            // [0] bigrams, [1] tokens
-    int* status = nullptr;
-    uint64_t* skeys = nullptr;
-    const uint64_t cap = pow2_at_least(2 * std::max<uint64_t>(pairs, 1));
-    tasc_status rc = TASC_OK;
-#define TRY_ALLOC(ptr, bytes) if (rc == TASC_OK && cudaMalloc(reinterpret_cast<void**>(&(ptr)), (bytes)) != cudaSuccess) { (void)cudaGetLastError(); rc = TASC_ENOMEM; }
-    TRY_ALLOC(remaining, (size_t)std::max<int64_t>(T, 1));
-    TRY_ALLOC(hist, (size_t)vocab * sizeof(uint32_t));
-    TRY_ALLOC(bins, 2 * (size_t)CC_BINS * sizeof(uint32_t));
-    TRY_ALLOC(overflow, 2 * (size_t)CC_OVERFLOW * sizeof(uint32_t));
-    TRY_ALLOC(scal, 8 * sizeof(unsigned long long));
-    TRY_ALLOC(summ, 2 * sizeof(CountSummary));
-    TRY_ALLOC(status, sizeof(int));
-    TRY_ALLOC(skeys, cap * 16);
-    TRY_ALLOC(scounts, cap * 4);
-#undef TRY_ALLOC
-    CountSummary h[2] = {};
-    if (rc == TASC_OK) {
-        cudaMemsetAsync(hist, 0, (size_t)vocab * sizeof(uint32_t), stream);
-        cudaMemsetAsync(bins, 0, 2 * (size_t)CC_BINS * sizeof(uint32_t), stream);
-        cudaMemsetAsync(scal, 0, 8 * sizeof(unsigned long long), stream);
-        cudaMemsetAsync(status, 0, sizeof(int), stream);
-        cudaMemsetAsync(skeys, 0, cap * 16, stream);
-        cudaMemsetAsync(scounts, 0, cap * 4, stream);
-        if (T > 0) {
-            mark_remaining_kernel<<<blocks_for(T, 256), 256, 0, stream>>>(doc_offsets, n_docs, T, remaining);
-            token_hist_kernel<<<blocks_for(T, 256), 256, 0, stream>>>(corpus_tokens, T, vocab, hist, status);
-            // bigrams = the windows of the order-1 model before pruning: (token, next) inside one document
-            count_kernel<<<blocks_for(T, 256), 256, 0, stream>>>(corpus_tokens, remaining, T, 1, skeys, scounts, cap - 1, status);
-        }
-        count_values_kernel<<<blocks_for(cap, 256), 256, 0, stream>>>(scounts, cap, bins, overflow, scal, status);
-        count_values_kernel<<<blocks_for(vocab, 256), 256, 0, stream>>>(hist, (uint64_t)vocab, bins + CC_BINS, overflow + CC_OVERFLOW, scal + 4, status);
-        count_summary_kernel<<<1, STATS_THREADS, 0, stream>>>(bins, overflow, scal, (unsigned long long)cdf_num, (unsigned long long)cdf_den, summ);
-        count_summary_kernel<<<1, STATS_THREADS, 0, stream>>>(bins + CC_BINS, overflow + CC_OVERFLOW, scal + 4, 1ull, 1ull, summ + 1);
-        int st = 0;
-        if (cudaMemcpyAsync(h, summ, sizeof(h), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
-            cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
-            cudaStreamSynchronize(stream) != cudaSuccess) { (void)cudaGetLastError(); rc = TASC_ECUDA; }
-        else if (st != 0) rc = st;
+    // scal: [0..2] bigram scalars, [4..6] token scalars, [8] status; behind it everything that starts as zero
+    DeviceSlab slab;
+    const CountTable empty = {nullptr, (uint32_t)count_pairs(c.pairs)};
+    const size_t table_bytes = (size_t)empty.pairs * 2 * sizeof(CountSlot);
+    const size_t o_scal = slab.add(9 * sizeof(unsigned long long)), o_hist = slab.add((size_t)vocab * 4), o_bins = slab.add(2 * (size_t)CC_BINS * 4),
+                 o_slots = slab.add(table_bytes), o_over = slab.add(2 * (size_t)CC_OVERFLOW * 4), o_sums = slab.add(2 * BIN_CHUNKS * sizeof(BinSum)),
+                 o_summ = slab.add(2 * sizeof(CountSummary)), o_rem = slab.add((size_t)T);
+    if (!slab.allocate(stream)) return TASC_ENOMEM;
+    unsigned long long* scal = slab.at<unsigned long long>(o_scal);
+    int* status = reinterpret_cast<int*>(scal + 8);
+    uint32_t *hist = slab.at<uint32_t>(o_hist), *bins = slab.at<uint32_t>(o_bins), *overflow = slab.at<uint32_t>(o_over);
+    uint8_t* remaining = slab.at<uint8_t>(o_rem);
+    const CountTable table = {slab.at<CountSlot>(o_slots), empty.pairs};
+    const uint64_t n_slots = 2 * (uint64_t)table.pairs;
+    TASC_CUDA_TRY(cudaMemsetAsync(scal, 0, o_slots + table_bytes, stream));
+    if (T > 0) {
+        corpus_scan_kernel<<<blocks_for(T, SCAN_POS), SCAN_THREADS, 0, stream>>>(corpus_tokens, doc_offsets, n_docs, T, vocab, remaining, hist, status);
+        // bigrams = the windows of the order-1 model before pruning: (token, next) inside one document
+        count_pairs_kernel<<<blocks_for(T, 256), 256, 0, stream>>>(corpus_tokens, remaining, T, table, nullptr, status);
     }
-    cudaFree(remaining); cudaFree(hist); cudaFree(bins); cudaFree(overflow); cudaFree(scal); cudaFree(summ);
-    cudaFree(status); cudaFree(skeys); cudaFree(scounts);
-    if (rc != TASC_OK) return rc;
+    constexpr unsigned VALUE_BLOCKS = 148 * 8;           // all resident
+    count_values_kernel<<<std::min(blocks_for(n_slots, STATS_THREADS), VALUE_BLOCKS), STATS_THREADS, 0, stream>>>(
+        &table.slots->count, (int)(sizeof(CountSlot) / 4), n_slots, bins, overflow, scal, status);
+    count_values_kernel<<<std::min(blocks_for(vocab, STATS_THREADS), VALUE_BLOCKS), STATS_THREADS, 0, stream>>>(
+        hist, 1, (uint64_t)vocab, bins + CC_BINS, overflow + CC_OVERFLOW, scal + 4, status);
+    bin_sums_kernel<<<dim3(BIN_CHUNKS, 2), STATS_THREADS, 0, stream>>>(bins, slab.at<BinSum>(o_sums));
+    count_summary_kernel<<<2, STATS_THREADS, 0, stream>>>(bins, slab.at<BinSum>(o_sums), overflow, scal, (unsigned long long)cdf_num,
+                                                          (unsigned long long)cdf_den, slab.at<CountSummary>(o_summ));
+    TASC_CUDA_TRY(cudaGetLastError());
+    CountSummary h[2] = {};
+    int st = 0;
+    TASC_CUDA_TRY(cudaMemcpyAsync(h, slab.at<CountSummary>(o_summ), sizeof(h), cudaMemcpyDeviceToHost, stream));
+    TASC_CUDA_TRY(cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, stream));
+    TASC_CUDA_TRY(cudaStreamSynchronize(stream));
+    if (st != 0) return st;
     // the closing arithmetic on a handful of scalars: H = log2 N - (sum c log2 c) / N;  H_2 = 2 log2 N - log2 sum c^2
     auto entropy = [](const CountSummary& c) { return c.n_total ? log2((double)c.n_total) - c.sum_c_log2_c / (double)c.n_total : 0.0; };
     out->n_tokens = T;
@@ -789,58 +961,35 @@ extern "C" tasc_status tasc_drafter_import(const tasc_ngram_entry* entries, int6
         keys[e.n].push_back(k.hi);
         counts[e.n].push_back(e.count);
     }
-    tasc_drafter* d = new (std::nothrow) tasc_drafter();
+    tasc_drafter* d = new_drafter(n_max, fallback_token, 1, vocab);
     if (!d) return TASC_ENOMEM;
-    for (int n = 0; n <= TASC_MAX_ORDER; ++n) d->dt.t[n] = OrderTable{nullptr, nullptr, nullptr, 0, 0};
-    d->dt.n_max = n_max; d->dt.fallback = fallback_token; d->p_min = 1; d->vocab = vocab;
-    cudaGetDevice(&d->device);
-    tasc_status rc = TASC_OK;
-    int* status = nullptr;
-    unsigned long long* cursor = nullptr;
-    if (cudaMalloc(reinterpret_cast<void**>(&status), sizeof(int)) != cudaSuccess ||
-        cudaMalloc(reinterpret_cast<void**>(&cursor), sizeof(unsigned long long)) != cudaSuccess) { (void)cudaGetLastError(); rc = TASC_ENOMEM; }
-    if (rc == TASC_OK) cudaMemsetAsync(status, 0, sizeof(int), stream);
-    for (int n = 1; n <= n_max && rc == TASC_OK; ++n) {
-        const uint64_t cnt = counts[n].size();
-        if (cnt == 0) continue;
-        uint64_t* skeys = nullptr;
-        uint32_t *scounts = nullptr, *fill = nullptr;
-        OrderTable& t = d->dt.t[n];
-        const uint64_t ccap = pow2_at_least(2 * cnt);
-        t.mask = ccap - 1;
-        t.n_succ = (long long)cnt;
-        if (cudaMalloc(reinterpret_cast<void**>(&skeys), cnt * 16) != cudaSuccess ||
-            cudaMalloc(reinterpret_cast<void**>(&scounts), cnt * 4) != cudaSuccess ||
-            cudaMalloc(reinterpret_cast<void**>(&fill), ccap * 4) != cudaSuccess ||
-            cudaMalloc(reinterpret_cast<void**>(&t.keys), ccap * 16) != cudaSuccess ||
-            cudaMalloc(reinterpret_cast<void**>(&t.vals), ccap * sizeof(CtxVal)) != cudaSuccess ||
-            cudaMalloc(reinterpret_cast<void**>(&t.succ), cnt * sizeof(Succ)) != cudaSuccess) { (void)cudaGetLastError(); rc = TASC_ENOMEM; }
-        if (rc == TASC_OK) {
-            cudaMemcpyAsync(skeys, keys[n].data(), cnt * 16, cudaMemcpyHostToDevice, stream);
-            cudaMemcpyAsync(scounts, counts[n].data(), cnt * 4, cudaMemcpyHostToDevice, stream);
-            cudaMemsetAsync(t.keys, 0, ccap * 16, stream);
-            cudaMemsetAsync(t.vals, 0, ccap * sizeof(CtxVal), stream);
-            cudaMemsetAsync(fill, 0, ccap * 4, stream);
-            cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), stream);
-            ctx_insert_kernel<<<blocks_for(cnt, 256), 256, 0, stream>>>(skeys, scounts, cnt, 1u, n, t, status);
-            assign_offsets_kernel<<<blocks_for(ccap, 256), 256, 0, stream>>>(t, cursor);
-            succ_fill_kernel<<<blocks_for(cnt, 256), 256, 0, stream>>>(skeys, scounts, cnt, 1u, n, t, fill, status);
-            if (cudaStreamSynchronize(stream) != cudaSuccess) { (void)cudaGetLastError(); rc = TASC_ECUDA; }
+    uint64_t most = 0;
+    for (const auto& v : counts) most = std::max<uint64_t>(most, v.size());
+    DeviceSlab slab;
+    const size_t o_scal = slab.add(16), o_keys = slab.add(most * 16), o_counts = slab.add(most * 4), o_place = slab.add(most * sizeof(uint2));
+    auto fill = [&]() -> tasc_status {
+        if (!slab.allocate(stream)) return TASC_ENOMEM;
+        unsigned long long* scal = slab.at<unsigned long long>(o_scal);          // [0] cursor, [1] status
+        int* status = reinterpret_cast<int*>(scal + 1);
+        TASC_CUDA_TRY(cudaMemsetAsync(scal, 0, 16, stream));
+        for (int n = 1; n <= n_max; ++n) {
+            const uint64_t cnt = counts[n].size();
+            if (cnt == 0) continue;
+            const PackedElements el = {slab.at<uint64_t>(o_keys), slab.at<uint32_t>(o_counts)};
+            TASC_CUDA_TRY(cudaMemcpyAsync(slab.at<uint64_t>(o_keys), keys[n].data(), cnt * 16, cudaMemcpyHostToDevice, stream));
+            TASC_CUDA_TRY(cudaMemcpyAsync(slab.at<uint32_t>(o_counts), counts[n].data(), cnt * 4, cudaMemcpyHostToDevice, stream));
+            const tasc_status rc = build_order(d, n, el, cnt, cnt, slab.at<uint2>(o_place), scal, status, stream);
+            if (rc != TASC_OK) return rc;
         }
-        if (skeys) cudaFree(skeys);
-        if (scounts) cudaFree(scounts);
-        if (fill) cudaFree(fill);
-    }
-    if (rc == TASC_OK) {
         int st = 0;
-        if (cudaMemcpy(&st, status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) { (void)cudaGetLastError(); rc = TASC_ECUDA; }
-        else if (st != 0) rc = st;
-    }
-    if (status) cudaFree(status);
-    if (cursor) cudaFree(cursor);
+        TASC_CUDA_TRY(cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, stream));
+        TASC_CUDA_TRY(cudaStreamSynchronize(stream));
+        return st;
+    };
+    const tasc_status rc = fill();
     if (rc != TASC_OK) {
-        free_tables(d->dt);
-        delete d;
+        cudaStreamSynchronize(stream);                               // the host arrays must outlive the copies
+        free_drafter(d);
         return rc;
     }
     *out = d;
@@ -849,8 +998,7 @@ extern "C" tasc_status tasc_drafter_import(const tasc_ngram_entry* entries, int6
 
 extern "C" tasc_status tasc_drafter_destroy(tasc_drafter* d) {
     if (!d) return TASC_EINVAL;
-    free_tables(d->dt);
-    delete d;
+    free_drafter(d);
     return TASC_OK;
 }
 

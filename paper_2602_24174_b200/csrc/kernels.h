@@ -17,6 +17,42 @@ struct ProfScope {
     ~ProfScope() { prof_end(kind, s); }
 };
 
+// ------------------------------------------------------------------ device memory of the set-up calls (scratch.cu)
+// Memory for work on `stream`; a block is freed in that stream's order, or after it on any stream of an idle device.
+bool scratch_alloc(void** p, size_t bytes, cudaStream_t stream, bool* pooled);
+void scratch_free(void* p, cudaStream_t stream, bool pooled);
+void scratch_trim();                           // gives back what the current device's pool holds
+
+// Parts laid out one behind the other in one block, which is freed with the object (on the stream given then).
+class DeviceSlab {
+public:
+    DeviceSlab() = default;
+    DeviceSlab(const DeviceSlab&) = delete;
+    DeviceSlab& operator=(const DeviceSlab&) = delete;
+    ~DeviceSlab() { release(stream_); }
+    size_t add(size_t bytes) {                   // offset of a new part
+        const size_t o = bytes_;
+        bytes_ += (bytes + 255) / 256 * 256;
+        return o;
+    }
+    bool allocate(cudaStream_t stream) {
+        stream_ = stream;
+        return scratch_alloc(reinterpret_cast<void**>(&base_), bytes_ ? bytes_ : 256, stream, &pooled_);
+    }
+    void release(cudaStream_t stream) {
+        scratch_free(base_, stream, pooled_);
+        base_ = nullptr;
+        bytes_ = 0;
+    }
+    template <typename T> T* at(size_t offset) const { return reinterpret_cast<T*>(base_ + offset); }
+
+private:
+    uint8_t* base_ = nullptr;
+    size_t bytes_ = 0;
+    cudaStream_t stream_ = nullptr;
+    bool pooled_ = false;
+};
+
 // ------------------------------------------------------------------ tensor-core GEMM with split-K partial sums in global memory (gemm_tcgen05.cu)
 // The exported building block tasc_gemm_bf16 / tasc_gemm_bf16_static; the forward uses gemm_fused.cu.
 // Computes partial sums P[s][m][n] = sum over the k-range of split s of X[m][k] * W[n][k]

@@ -77,32 +77,6 @@ inline uint64_t pow2_at_least(uint64_t v) {
     return p;
 }
 
-// Device memory of one call: parts laid out one behind the other in one allocation (an allocation and its release cost more
-// than many of the kernels that use them), freed with the object.
-class DeviceSlab {
-public:
-    DeviceSlab() = default;
-    DeviceSlab(const DeviceSlab&) = delete;
-    DeviceSlab& operator=(const DeviceSlab&) = delete;
-    ~DeviceSlab() { if (base_) cudaFree(base_); }
-    size_t add(size_t bytes) {                   // offset of a new part
-        const size_t o = bytes_;
-        bytes_ += (bytes + 255) / 256 * 256;
-        return o;
-    }
-    bool allocate() {
-        if (cudaMalloc(reinterpret_cast<void**>(&base_), bytes_ ? bytes_ : 256) == cudaSuccess) return true;
-        (void)cudaGetLastError();
-        base_ = nullptr;
-        return false;
-    }
-    template <typename T> T* at(size_t offset) const { return reinterpret_cast<T*>(base_ + offset); }
-
-private:
-    uint8_t* base_ = nullptr;
-    size_t bytes_ = 0;
-};
-
 inline unsigned blocks_for(uint64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
 }  // namespace

@@ -761,7 +761,7 @@ extern "C" tasc_status tasc_tok_enrich(const int32_t* corpus_tokens, const int64
     {
         DeviceSlab small;
         const size_t o = small.add(sizeof(TokCheck));
-        if (!small.allocate()) return TASC_ENOMEM;
+        if (!small.allocate(stream)) return TASC_ENOMEM;
         TokCheck* dc = small.at<TokCheck>(o);
         TASC_CUDA_TRY(cudaMemcpyAsync(dc, &zero, sizeof(zero), cudaMemcpyHostToDevice, stream));
         tok_check_kernel<<<std::min(blocks_for((uint64_t)n_docs + 1, 256), 592u), 256, 0, stream>>>(doc_offsets, n_docs, n_max, dc);
@@ -780,7 +780,7 @@ extern "C" tasc_status tasc_tok_enrich(const int32_t* corpus_tokens, const int64
     const size_t o_keys = slab.add(cap * 16), o_words = slab.add(cap * 4), o_dirty = slab.add(chunks), o_chunk = slab.add(chunks * sizeof(Best)),
                  o_cta = slab.add(grid * sizeof(Best)), o_st = slab.add(sizeof(TokState)), o_cur = slab.add(t * 4), o_of = slab.add(t * 4),
                  o_rem = slab.add(t), o_mark = slab.add(t), o_len = slab.add(nd * 4), o_round = slab.add(nd * 4), o_tot = slab.add(scan_blocks(n_docs) * 8);
-    if (!slab.allocate()) return TASC_ENOMEM;
+    if (!slab.allocate(stream)) return TASC_ENOMEM;
     TokArgs a = {};
     a.cur = slab.at<int32_t>(o_cur); a.rem = slab.at<uint8_t>(o_rem); a.mark = slab.at<uint8_t>(o_mark); a.doc_of = slab.at<int32_t>(o_of);
     a.offsets = doc_offsets; a.doc_len = slab.at<int32_t>(o_len); a.doc_round = slab.at<int32_t>(o_round); a.n_docs = n_docs; a.T = T;
@@ -878,7 +878,7 @@ extern "C" tasc_status tasc_tok_encode(const int32_t* tokens, const int64_t* doc
     DeviceSlab slab;
     const size_t o_keys = slab.add(cap * 8), o_child = slab.add(cap * 4), o_tok = slab.add(node_token.size() * 4),
                  o_scratch = slab.add((size_t)T * 4), o_len = slab.add((size_t)n_docs * 4), o_tot = slab.add(scan_blocks(n_docs) * 8);
-    if (!slab.allocate()) return TASC_ENOMEM;
+    if (!slab.allocate(stream)) return TASC_ENOMEM;
     int32_t *scratch = slab.at<int32_t>(o_scratch), *doc_len = slab.at<int32_t>(o_len);
     TASC_CUDA_TRY(cudaMemcpyAsync(slab.at<uint64_t>(o_keys), hk.data(), cap * 8, cudaMemcpyHostToDevice, stream));
     TASC_CUDA_TRY(cudaMemcpyAsync(slab.at<int32_t>(o_child), hc.data(), cap * 4, cudaMemcpyHostToDevice, stream));

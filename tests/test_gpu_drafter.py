@@ -143,6 +143,19 @@ def test_drafts_do_not_depend_on_table_layout():
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("lens,vocab,p_min", [
+    ([255, 1, 256, 0, 257, 2, 2047, 2048, 2049], 6, 3),        # documents that end at, before and behind the blocks' edges
+    ([7] * 700, 40, 5), ([1] * 50 + [2], 9, 1),
+    ([300, 300], 500, 2)])                                     # hardly anything occurs twice
+def test_orders_counted_from_what_the_order_before_left(lens, vocab, p_min):
+    r = np.random.default_rng(sum(lens))
+    tokens = (r.random(sum(lens)) ** 2 * vocab).astype(np.int32)
+    offsets = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    b, dr, ng = build_both(tokens, offsets, 5, p_min, vocab)
+    assert_tables_equal(dr, ng)
+
+
+@pytest.mark.gpu
 def test_config2_full_corpus_tables():
     """All 200,000 documents (14 M tokens) of configuration 2's corpus, n_max 4, p_min 5: export bit-exact."""
     cfg = configs.get(2)
