@@ -30,14 +30,14 @@ struct tasc_model {
     std::vector<const float*> attn_norm, mlp_norm;
     std::vector<const void*> wqkv, wo, w_gate_up, w_down;
     float2* rope;                                   // [max_positions][head_dim / 2] (cos, sin), library-owned
-    tasc::LayerWeights* d_layers;                   // bf16 models: device copy of the layers' weight pointers, behind the rope table
+    void* d_layers;                                 // device copy of the layers' weight pointers (LayerWeights, LayerWeightsF32), behind the rope table
     // tensor maps of the weight matrices (bf16 models): box = 64 columns x 128 rows (gate/up: 64 rows, see EPI_SWIGLU)
     std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
     CUtensorMap tm_lm;
     int qkv_rows, q_dim, kv_dim;
     int few_tiles;                                  // token tiles for 49..128 rows (see gemm_token_tile), from the layer's weight bytes
-    double layer_mb;                                // projection weights of one layer, MB
-    bool aligned32;                                 // every layer matrix starts on a 32-byte boundary (forward_persist.cu)
+    double layer_mb;                                // projection weights of one layer, MB (two bytes each)
+    bool aligned32;                                 // every layer matrix starts on a 32-byte boundary (forward_persist.cu, forward_f32.cu)
     mutable std::mutex plan_mu;
     mutable std::vector<StepPlans> plans;           // most recently used last; a handful of (B, k, workspace) combinations
 };
@@ -176,12 +176,30 @@ struct RowSource {
     int chunk;
 };
 
-// float32 model (the tiny configuration): one launch per stage, float32 SIMT kernels.
+// float32 model (the tiny configuration): the whole pass in one kernel if one cluster can hold it, otherwise one launch per
+// stage, float32 SIMT kernels.
 tasc_status forward_f32(const tasc_model* m, const tasc_kv* kv, const Workspace& w, const RowSource& src, int B, int R, bool lm_head,
                         float* logits, cudaStream_t s) {
     const tasc_model_desc& d = m->desc;
     const int M = B * R;
     const tasc_seqs* sq = src.seqs;
+    if (m->aligned32 && plan_forward_f32(M, d.d_model, d.n_q_heads, d.n_kv_heads, d.head_dim, d.d_ff, kv->max_pages_per_seq * d.page_size, 2.0 * m->layer_mb)) {
+        ForwardF32Args a = {};
+        a.layers = static_cast<const LayerWeightsF32*>(m->d_layers);
+        a.embed = static_cast<const float*>(m->embed); a.final_norm = m->final_norm;
+        a.lm_head = lm_head ? static_cast<const float*>(m->lm_head) : nullptr;
+        a.n_layers = d.n_layers; a.M = M; a.R = R; a.d = d.d_model; a.n_q = d.n_q_heads; a.n_kv = d.n_kv_heads; a.hd = d.head_dim;
+        a.dff = d.d_ff; a.vocab = d.vocab; a.eps = d.rms_eps;
+        a.rp = w.rp; a.tokens = sq->tokens; a.stride = sq->stride; a.len = sq->len; a.stop_len = sq->stop_len; a.drafts = src.drafts;
+        a.chunk = src.chunk;
+        a.x = w.x; a.q = w.q; a.o = static_cast<float*>(w.o); a.act = static_cast<float*>(w.act);
+        a.rope = m->rope; a.max_positions = d.max_positions;
+        a.block_table = kv->block_table; a.max_pages = kv->max_pages_per_seq; a.page_size = d.page_size; a.n_pages = kv->n_pages;
+        a.kv_pool = static_cast<float*>(kv->pool);
+        a.kv_half = (size_t)kv->n_pages * d.n_kv_heads * d.page_size * d.head_dim;
+        a.argmax = lm_head ? w.argmax : nullptr; a.logits = lm_head ? logits : nullptr; a.status = w.status;
+        return launch_forward_f32(a, s);
+    }
     if (src.chunk < 0) launch_rows_verify(w.rp, sq->tokens, sq->stride, sq->len, sq->stop_len, src.drafts, B, R, d.vocab, w.status, s);
     else launch_rows_prefill(w.rp, sq->tokens, sq->stride, sq->len, B, R, src.chunk, d.vocab, w.status, s);
     const int max_ctx = kv->max_pages_per_seq * d.page_size;
@@ -303,7 +321,7 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
                       w.counters, sp.persist ? COUNTER_GROUPS + sp.pp.n_units / sp.pp.splits : 0, s);
     if (sp.persist) {
         PersistArgs a = {};
-        a.layers = m->d_layers; a.n_layers = d.n_layers; a.M = M; a.R = R; a.TBL = TB;
+        a.layers = static_cast<const LayerWeights*>(m->d_layers); a.n_layers = d.n_layers; a.M = M; a.R = R; a.TBL = TB;
         a.d = d.d_model; a.qd = m->q_dim; a.dff = d.d_ff; a.n_q = d.n_q_heads; a.n_kv = d.n_kv_heads; a.hd = d.head_dim;
         a.inv_d = base.inv_d; a.eps = base.eps; a.scale_log2e = 1.4426950408889634f / sqrtf((float)d.head_dim);
         a.h = h; a.o = o; a.act = act; a.q = w.q; a.x0 = w.x; a.ssq = w.ssq64;
@@ -436,7 +454,8 @@ extern "C" tasc_status tasc_model_create(const tasc_model_desc* desc, const tasc
     }
     m->rope = nullptr;
     m->d_layers = nullptr;
-    m->aligned32 = true;
+    m->aligned32 = d.dtype == TASC_BF16 || (reinterpret_cast<uintptr_t>(wt->embed) % 16 == 0 && reinterpret_cast<uintptr_t>(wt->lm_head) % 16 == 0 &&
+                                            reinterpret_cast<uintptr_t>(wt->final_norm) % 16 == 0);
     for (int l = 0; l < d.n_layers; ++l) {
         if (!wt->attn_norm[l] || !wt->wqkv[l] || !wt->wo[l] || !wt->mlp_norm[l] || !wt->w_gate_up[l] || !wt->w_down[l]) {
             delete m;
@@ -447,6 +466,8 @@ extern "C" tasc_status tasc_model_create(const tasc_model_desc* desc, const tasc
         m->w_gate_up.push_back(wt->w_gate_up[l]); m->w_down.push_back(wt->w_down[l]);
         for (const void* p : {wt->wqkv[l], wt->wo[l], wt->w_gate_up[l], wt->w_down[l]})
             if (reinterpret_cast<uintptr_t>(p) % 32) m->aligned32 = false;
+        for (const float* p : {wt->attn_norm[l], wt->mlp_norm[l]})
+            if (d.dtype == TASC_F32 && reinterpret_cast<uintptr_t>(p) % 16) m->aligned32 = false;
     }
     tasc_status st = TASC_OK;
     if (d.dtype == TASC_BF16) {
@@ -462,19 +483,25 @@ extern "C" tasc_status tasc_model_create(const tasc_model_desc* desc, const tasc
     }
     if (st == TASC_OK) {
         const size_t n = (size_t)d.max_positions * (d.head_dim / 2);
-        std::vector<LayerWeights> lw;
+        std::vector<uint8_t> lw;
+        auto add = [&](const auto& w) { lw.insert(lw.end(), reinterpret_cast<const uint8_t*>(&w), reinterpret_cast<const uint8_t*>(&w + 1)); };
         auto mat = [](const void* p) { return static_cast<const __nv_bfloat16*>(p); };
-        for (int l = 0; l < d.n_layers && d.dtype == TASC_BF16; ++l)
-            lw.push_back(LayerWeights{mat(m->wqkv[l]), mat(m->wo[l]), mat(m->w_gate_up[l]), mat(m->w_down[l]), m->mlp_norm[l],
-                                      l + 1 < d.n_layers ? m->attn_norm[l + 1] : m->final_norm});
-        const size_t lw_bytes = lw.size() * sizeof(LayerWeights);
+        auto matf = [](const void* p) { return static_cast<const float*>(p); };
+        for (int l = 0; l < d.n_layers; ++l) {
+            if (d.dtype == TASC_BF16)
+                add(LayerWeights{mat(m->wqkv[l]), mat(m->wo[l]), mat(m->w_gate_up[l]), mat(m->w_down[l]), m->mlp_norm[l],
+                                 l + 1 < d.n_layers ? m->attn_norm[l + 1] : m->final_norm});
+            else
+                add(LayerWeightsF32{m->attn_norm[l], matf(m->wqkv[l]), matf(m->wo[l]), m->mlp_norm[l], matf(m->w_gate_up[l]), matf(m->w_down[l])});
+        }
+        const size_t lw_bytes = lw.size();
         if (cudaMalloc(reinterpret_cast<void**>(&m->rope), n * sizeof(float2) + lw_bytes) != cudaSuccess) {
             (void)cudaGetLastError();
             st = TASC_ENOMEM;
         } else {
             launch_rope_table(m->rope, d.max_positions, d.head_dim, d.rope_base, nullptr);
-            m->d_layers = reinterpret_cast<LayerWeights*>(m->rope + n);
-            if ((lw_bytes && cudaMemcpyAsync(m->d_layers, lw.data(), lw_bytes, cudaMemcpyHostToDevice, nullptr) != cudaSuccess) ||
+            m->d_layers = m->rope + n;
+            if (cudaMemcpyAsync(m->d_layers, lw.data(), lw_bytes, cudaMemcpyHostToDevice, nullptr) != cudaSuccess ||
                 cudaDeviceSynchronize() != cudaSuccess) {
                 (void)cudaGetLastError();
                 st = TASC_ECUDA;

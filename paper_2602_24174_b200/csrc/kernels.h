@@ -256,6 +256,42 @@ void launch_min_generated(const int32_t* len, const int32_t* prompt_len, int B, 
 void launch_bigram_rows(int32_t* tokens, int32_t* len, int t0, int vocab, int B, cudaStream_t stream);
 void launch_bigram_store(const unsigned long long* argmax, int32_t* table, int t0, int vocab, int B, cudaStream_t stream);
 
+// ------------------------------------------------------------------ the whole forward of a small float32 model (forward_f32.cu)
+struct LayerWeightsF32 { const float *attn_norm, *wqkv, *wo, *mlp_norm, *w_gate_up, *w_down; };
+struct ForwardF32Args {
+    const LayerWeightsF32* layers;                 // device array
+    const float *embed, *final_norm, *lm_head;     // lm_head null: no LM head in this pass
+    int n_layers, M, R, d, n_q, n_kv, hd, dff, vocab;
+    float eps;
+    // rows, as in launch_rows_embed
+    RowPlan rp;
+    const int32_t* tokens;
+    int64_t stride;
+    const int32_t *len, *stop_len, *drafts;
+    int chunk;
+    float *x, *q, *o, *act;                        // [M][d], [M][n_q * hd], same, [M][dff]
+    const float2* rope;
+    int max_positions;
+    const int32_t* block_table;
+    int max_pages, page_size;
+    long long n_pages;
+    float* kv_pool;                                // a layer's keys, then its values: kv_half elements each
+    size_t kv_half;
+    unsigned long long* argmax;
+    float* logits;
+    int* status;
+    int width;                                     // (set by the launch)
+    float scale;
+};
+// What one cluster runs: four-layer models, a step in us as one launch per stage / in the cluster: 1 MB per layer 323 / 100 at
+// 5 rows and 426 / 376 at 72, 13 MB 653 / 192 at 5 and 900 / 521 at 24, 47 MB 1056 / 470 at 5; the rows are also limited by
+// its shared memory.  Its attention has 16 SMs: at 2^18 (row, query head, key) triples about 80 us per layer, as long as
+// the split kernel's few CTAs for one sequence.
+constexpr double F32_CLUSTER_LAYER_MB = 48.0;
+constexpr long long F32_CLUSTER_SCORES = 1ll << 18;
+bool plan_forward_f32(int M, int d, int n_q, int n_kv, int hd, int dff, int max_ctx, double layer_mb);
+tasc_status launch_forward_f32(ForwardF32Args a, cudaStream_t stream);
+
 // ------------------------------------------------------------------ attention (attention.cu)
 // Verify attention of R query rows per sequence over the paged KV cache (grouped-query, causal within the rows).
 template <typename T>

@@ -373,6 +373,23 @@ def test_one_kernel_for_all_layers(B, k, P, hd):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("B,k,P,shape", [(1, 3, 2, {}), (1, 8, 300, {}), (3, 4, 33, {}), (8, 8, 70, {}),
+                                         (2, 6, 40, dict(n_layers=3, d_model=136, n_q_heads=6, n_kv_heads=2, head_dim=40, d_ff=200, vocab=333)),
+                                         (1, 2, 40, dict(d_model=768, n_q_heads=3, n_kv_heads=3, head_dim=256, d_ff=1024)),
+                                         (2, 2, 40, dict(d_model=1024, n_q_heads=8, n_kv_heads=8, head_dim=128, d_ff=4096)),  # per stage: a layer too large
+                                         (40, 8, 20, {})])                                                                    # ... too many rows
+def test_float32_forward_in_one_cluster(B, k, P, shape):
+    """Rows that are no multiple of the eight multiplied at a time, keys below, at and over the blocks of 32 and the eight
+    warps that share them, an odd vocabulary and heads that are no multiple of 32; and either side of the dispatch."""
+    from dataclasses import replace
+    cfg = replace(configs.shrunk(configs.get(0), n_docs=200), prompt_len=P)
+    cfg = replace(cfg, model=replace(cfg.model, **shape))
+    s = make_setup(cfg)
+    prompts = corpus.make_prompts(cfg, B, prompt_len=P)
+    check(lockstep(s, prompts, k + 3, k, oracle_rows=sorted({0, B - 1}), **F32_TOL), f"float32, B={B} k={k} P={P} {shape}")
+
+
+@pytest.mark.gpu
 def test_config4_full_depth_batch1():
     """The 1.5B shape at its full depth (28 layers, vocabulary 151,936, prompt of 1,024 tokens), one sequence,
     four or more steps; the corpus tables come from the first 20,000 documents."""
