@@ -15,6 +15,18 @@
 // the epilogue owns one token row (its TMEM lane) and 32 consecutive features per tcgen05.ld, so the
 // row-wise consumers (RMS factor, RoPE pairs, sum of squares, row arg-max) need no exchange between threads.
 //
+// Pairs.  What bounds a tile is not the MMAs but what the SMs take in: a k-block of a 128 x 256 tile brings 64 KB (32 KB of
+// token rows, hi and lo, and 32 KB of weights) for 1,024 cycles of MMA.  So where a product has 256-feature tiles for two token tiles or more, two CTAs form a pair
+// (cta_group::2): one MMA of 256 token rows on both SMs' tensor cores, each CTA loading its own token rows and HALF of the
+// weight rows, 48 KB per k-block.  The even CTA issues the MMAs and counts both CTAs' bytes on its barriers; the commits
+// release stages and announce accumulators in both.
+//   2,048 rows, 1,536 -> 17,920 features: 164 us before, 147 in pairs (tensor pipes 87 % busy), 140 with the epilogue below.
+//
+// Epilogue.  A thread holds 32 features of one row; 32 threads that each touch their own row make every access 32 lines, and
+// at 2,048 rows the residual epilogue (nothing hides it in a grid of one wave) was longer than the MMAs of the O product.  A
+// warp turns its 32 x 32 values around in shared memory first, so that eight lanes share a row: O and down together 162 ->
+// 138 us, QKV 37 -> 34.
+//
 // Split-K.  A product with few output tiles and a long reduction (the down-projection, the narrow QKV and
 // O matrices) runs as clusters of S CTAs instead: one tile per cluster, CTA r takes the r-th share of the
 // k-blocks, parks its accumulator in its own shared memory (the ring is idle by then), and after a cluster
@@ -41,12 +53,16 @@ constexpr int EPI_WARPS = 8;                 // two per TMEM lane quarter: they 
 constexpr int THREADS = (EPI_WARPS + 2) * 32;
 constexpr int MAX_STAGES = 8;
 constexpr int MAX_DYN_SMEM = 226 * 1024;
+constexpr int STAGING_BYTES = EPI_WARPS * 32 * 32 * 4;        // behind the ring: the epilogue warps turn their rows around there
 
+// CLUSTER: the arrivals may be another CTA's.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool wait_or_fail(uint32_t bar, uint32_t parity, volatile int* failed) {
-    if (mbar_try_wait(bar, parity)) return true;
+    auto ready = [&]() { return CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
+    if (ready()) return true;
     const long long t0 = clock64();
     for (;;) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (ready()) return true;
         if (*failed) return false;
         if (clock64() - t0 > 1000000000ll) return false;
     }
@@ -55,40 +71,21 @@ __device__ __forceinline__ bool wait_or_fail(uint32_t bar, uint32_t parity, vola
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
     return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(a)) | ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
 }
-// 32 consecutive values of one row -> bf16, 64 bytes.
-__device__ __forceinline__ void store_bf16x32(__nv_bfloat16* p, const float (&v)[32]) {
-#pragma unroll
-    for (int e = 0; e < 32; e += 8)
-        *reinterpret_cast<uint4*>(p + e) = make_uint4(pack_bf16x2(v[e], v[e + 1]), pack_bf16x2(v[e + 2], v[e + 3]),
-                                                      pack_bf16x2(v[e + 4], v[e + 5]), pack_bf16x2(v[e + 6], v[e + 7]));
-}
-// 32 consecutive values of one row -> (hi, lo) bf16, 64 bytes each.
-__device__ __forceinline__ void store_hilo32(__nv_bfloat16* hi_ptr, __nv_bfloat16* lo_ptr, const float (&v)[32]) {
-#pragma unroll
-    for (int e = 0; e < 32; e += 8) {
-        uint32_t h[4], l[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            __nv_bfloat16 h0, l0, h1, l1;
-            split_bf16(v[e + 2 * q], h0, l0);
-            split_bf16(v[e + 2 * q + 1], h1, l1);
-            h[q] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-            l[q] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
-        }
-        *reinterpret_cast<uint4*>(hi_ptr + e) = make_uint4(h[0], h[1], h[2], h[3]);
-        *reinterpret_cast<uint4*>(lo_ptr + e) = make_uint4(l[0], l[1], l[2], l[3]);
-    }
+// four consecutive values -> bf16; -> (hi, lo) bf16
+__device__ __forceinline__ uint2 bf16x4(const float4& v) { return make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w)); }
+__device__ __forceinline__ void hilo4(const float4& v, uint2& hi, uint2& lo) {
+    __nv_bfloat16 h[4], l[4];
+    split_bf16(v.x, h[0], l[0]);
+    split_bf16(v.y, h[1], l[1]);
+    split_bf16(v.z, h[2], l[2]);
+    split_bf16(v.w, h[3], l[3]);
+    auto two = [](const __nv_bfloat16* p) { return (uint32_t)__bfloat16_as_ushort(p[0]) | ((uint32_t)__bfloat16_as_ushort(p[1]) << 16); };
+    hi = make_uint2(two(h), two(h + 2));
+    lo = make_uint2(two(l), two(l + 2));
 }
 __device__ __forceinline__ void store_f32x32(float* p, const float (&v)[32]) {
 #pragma unroll
     for (int e = 0; e < 32; e += 4) *reinterpret_cast<float4*>(p + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-}
-__device__ __forceinline__ void load_f32x32(const float* p, float (&v)[32]) {
-#pragma unroll
-    for (int e = 0; e < 32; e += 4) {
-        const float4 t = *reinterpret_cast<const float4*>(p + e);
-        v[e] = t.x; v[e + 1] = t.y; v[e + 2] = t.z; v[e + 3] = t.w;
-    }
 }
 // 32 accumulator columns of this thread's TMEM lane, as floats.
 __device__ __forceinline__ void acc32(uint32_t taddr, float (&v)[32]) {
@@ -99,7 +96,7 @@ __device__ __forceinline__ void acc32(uint32_t taddr, float (&v)[32]) {
     for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(r[e]);
 }
 
-template <int EPI>
+template <int EPI, bool PAIR>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const FusedArgs a) {
     extern __shared__ uint8_t smem_raw[];
@@ -113,7 +110,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 
     const int BNW = a.BNW, TBL = a.TBL, stages = a.stages, num_kb = a.num_kb;
     const uint32_t a_bytes = (uint32_t)(2 * TBL) * 128u;        // one k-block of the token tile: TBL hi rows, TBL lo rows
-    const uint32_t w_bytes = (uint32_t)BNW * 128u;
+    const uint32_t w_bytes = (uint32_t)(PAIR ? BNW / 2 : BNW) * 128u;   // (a pair's CTAs load half of the weight rows each)
     const uint32_t stage_bytes = a_bytes + w_bytes;
     const uint32_t bar_full = smem_u32(s_bars);
     const uint32_t bar_empty = bar_full + 8u * MAX_STAGES;
@@ -121,20 +118,23 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     const uint32_t bar_acc_empty = bar_acc_full + 16u;          // [2]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_tiles = a.n_ft * a.n_tt;
+    const int rank = (int)cluster_ctarank();
+    const int n_tt = PAIR ? (a.n_tt + 1) / 2 : a.n_tt;          // token tiles, or pairs of them
+    const int n_tiles = a.n_ft * n_tt;
     // S = 1: persistent, tiles blockIdx.x, + gridDim.x, ...   S > 1: the grid is S * n_tiles CTAs, one tile per cluster
-    const int S = (int)cluster_nctarank(), rank = (int)cluster_ctarank();
-    const int tile0 = S > 1 ? (int)blockIdx.x / S : (int)blockIdx.x;
-    const int tstep = S > 1 ? n_tiles : (int)gridDim.x;
+    const int S = PAIR ? 1 : (int)cluster_nctarank();
+    const int tile0 = PAIR ? (int)blockIdx.x / 2 : S > 1 ? (int)blockIdx.x / S : (int)blockIdx.x;
+    const int tstep = PAIR ? (int)gridDim.x / 2 : S > 1 ? n_tiles : (int)gridDim.x;
     const int my_tiles = tile0 < n_tiles ? (n_tiles - tile0 + tstep - 1) / tstep : 0;
-    const int kb0 = (int)(((long long)num_kb * rank) / S);
-    const int nkb = (int)(((long long)num_kb * (rank + 1)) / S) - kb0;      // k-blocks of this CTA (all of them when S = 1)
+    const int kb0 = PAIR ? 0 : (int)(((long long)num_kb * rank) / S);
+    const int nkb = PAIR ? num_kb : (int)(((long long)num_kb * (rank + 1)) / S) - kb0;      // k-blocks of this CTA (all of them when S = 1)
     constexpr int XPAD = 4;                                                 // floats: rows of the parked tile fall on distinct banks
     float* xch = reinterpret_cast<float*>(smem);                            // [128][BNW + XPAD], split-K only
     constexpr int FLD = 4 * 32 + XPAD;                                      // a CTA finishes at most four 32-column chunks of a split tile
     float* fin = xch + 128 * (BNW + XPAD);                                  // [128][FLD] the S copies of this CTA's chunks, added up
     uint32_t own_mask = 0u;                                                 // split-K: the tile's 32-column chunks that this CTA finishes
     const int FT = EPI == EPI_SWIGLU ? BNW / 2 : BNW;           // output features per tile
+    float* stage = reinterpret_cast<float*>(smem + (size_t)stages * stage_bytes) + warp * 1024;      // the epilogue warps' 32 x 32 values (S = 1)
     auto fail = [&]() { set_status(a.status, TASC_ETIMEOUT); *failed = 1; };
 #ifdef TASC_TIMELINE
     const unsigned long long g_t0 = global_ns();
@@ -149,18 +149,19 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar_acc_full + 8u * b, 1);
-            mbar_init(bar_acc_empty + 8u * b, EPI_WARPS * 32);
+            mbar_init(bar_acc_empty + 8u * b, EPI_WARPS * 32 * (PAIR ? 2 : 1));
         }
         fence_barrier_init();
         tma_prefetch_desc(&tmW);
         tma_prefetch_desc(&tmX);
     }
     if (warp == EPI_WARPS + 1) {
-        tmem_alloc(smem_u32(&s_tmem), (uint32_t)(2 * BNW));
-        tmem_relinquish();
+        if (PAIR) { tmem_alloc_pair(smem_u32(&s_tmem), (uint32_t)(2 * BNW)); tmem_relinquish_pair(); }
+        else { tmem_alloc(smem_u32(&s_tmem), (uint32_t)(2 * BNW)); tmem_relinquish(); }
     }
     tc_fence_before();
     __syncthreads();
+    if (PAIR) { cluster_arrive(); cluster_wait(); }              // both CTAs' barriers are set up before either is signalled
     tc_fence_after();
     const uint32_t tmem_base = s_tmem;
 
@@ -170,12 +171,21 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             const uint64_t pol_w = a.n_tt > 1 ? policy_evict_last() : policy_evict_first();   // a weight tile is read once per token tile
             const uint64_t pol_x = policy_evict_last();                                       // token rows are read by every feature tile
             const int total = my_tiles * nkb;
+            const uint32_t full0 = PAIR ? cluster_map(bar_full, 0u) : bar_full;      // a pair's bytes are counted by its even CTA
+            auto expect = [&](int s) {
+                if (!PAIR) mbar_expect_tx(bar_full + 8u * s, stage_bytes);
+                else if (rank == 0) mbar_expect_tx(bar_full + 8u * s, 2u * stage_bytes);
+            };
             auto load_w = [&](int i) {
                 const int tile = tile0 + (i / nkb) * tstep;
-                const int f0 = (tile / a.n_tt) * FT, kc = (kb0 + i % nkb) * BK;
+                const int f0 = (tile / n_tt) * FT, kc = (kb0 + i % nkb) * BK;
                 const int s = i % stages;
-                const uint32_t dst = smem_u32(smem + (size_t)s * stage_bytes) + a_bytes, bar = bar_full + 8u * s;
-                if (EPI == EPI_SWIGLU) {                   // FT gate rows, then the FT matching up rows (boxes of 64 rows)
+                const uint32_t dst = smem_u32(smem + (size_t)s * stage_bytes) + a_bytes, bar = full0 + 8u * s;
+                if (PAIR) {                                // 128 of the 256 weight rows: the gate rows or the up rows; the lower or the upper half
+                    if (EPI == EPI_SWIGLU)
+                        for (int r = 0; r < FT; r += 64) tma_load_2d_pair(dst + (uint32_t)r * 128u, &tmW, kc, rank * a.N + f0 + r, bar, pol_w);
+                    else tma_load_2d_pair(dst, &tmW, kc, f0 + rank * 128, bar, pol_w);
+                } else if (EPI == EPI_SWIGLU) {                   // FT gate rows, then the FT matching up rows (boxes of 64 rows)
                     for (int r = 0; r < FT; r += 64) {
                         tma_load_2d_hint(dst + (uint32_t)r * 128u, &tmW, kc, f0 + r, bar, pol_w);
                         tma_load_2d_hint(dst + (uint32_t)(FT + r) * 128u, &tmW, kc, a.N + f0 + r, bar, pol_w);
@@ -187,22 +197,23 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             auto load_x = [&](int i) {
                 const int tile = tile0 + (i / nkb) * tstep;
                 const int s = i % stages;
-                tma_load_2d_hint(smem_u32(smem + (size_t)s * stage_bytes), &tmX, (kb0 + i % nkb) * BK, (tile % a.n_tt) * 2 * TBL,
-                                 bar_full + 8u * s, pol_x);
+                const uint32_t dst = smem_u32(smem + (size_t)s * stage_bytes);
+                if (PAIR) tma_load_2d_pair(dst, &tmX, (i % nkb) * BK, (2 * (tile % n_tt) + rank) * 2 * TBL, full0 + 8u * s, pol_x);
+                else tma_load_2d_hint(dst, &tmX, (kb0 + i % nkb) * BK, (tile % n_tt) * 2 * TBL, bar_full + 8u * s, pol_x);
             };
             // The weights of the first stages depend on no earlier kernel: they are requested before the
             // preceding grid has finished, the token rows after it.
             const int pre = total < stages ? total : stages;
             for (int i = 0; i < pre; ++i) {
-                mbar_expect_tx(bar_full + 8u * (i % stages), stage_bytes);
+                expect(i % stages);
                 load_w(i);
             }
             griddep_wait();
             for (int i = 0; i < pre; ++i) load_x(i);
             for (int i = pre; i < total; ++i) {
                 const int s = i % stages;
-                if (!wait_or_fail(bar_empty + 8u * s, (((uint32_t)(i / stages)) & 1u) ^ 1u, failed)) { fail(); break; }
-                mbar_expect_tx(bar_full + 8u * s, stage_bytes);
+                if (!wait_or_fail<PAIR>(bar_empty + 8u * s, (((uint32_t)(i / stages)) & 1u) ^ 1u, failed)) { fail(); break; }
+                expect(s);
                 load_w(i);
                 load_x(i);
             }
@@ -211,32 +222,35 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         __syncwarp();
     } else if (warp == EPI_WARPS + 1) {
         // ------------------------------------------------------------ MMA issue
-        if (lane == 0) {
-            const uint32_t idesc = umma_idesc_bf16_f32(128, BNW);
+        if (lane == 0 && (!PAIR || rank == 0)) {
+            const uint32_t idesc = umma_idesc_bf16_f32(PAIR ? 256 : 128, BNW);
+            auto mma = [&](uint32_t d, uint32_t sa, uint32_t sb, uint32_t acc) {
+                if (PAIR) umma_bf16_pair(d, umma_desc_k_sw128(sa), umma_desc_k_sw128(sb), idesc, acc);
+                else umma_bf16(d, umma_desc_k_sw128(sa), umma_desc_k_sw128(sb), idesc, acc);
+            };
+            auto commit = [&](uint32_t bar) { if (PAIR) umma_commit_pair(bar); else umma_commit(bar); };
             int it = 0;
             bool ok = true;
             for (int j = 0; j < my_tiles && ok; ++j) {
                 const int b = j & 1;
-                if (!wait_or_fail(bar_acc_empty + 8u * b, (((uint32_t)(j >> 1)) & 1u) ^ 1u, failed)) { fail(); break; }
+                if (!wait_or_fail<PAIR>(bar_acc_empty + 8u * b, (((uint32_t)(j >> 1)) & 1u) ^ 1u, failed)) { fail(); break; }
                 tc_fence_after();
                 const uint32_t d = tmem_base + (uint32_t)(b * BNW);
                 for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = it % stages;
-                    if (!wait_or_fail(bar_full + 8u * s, ((uint32_t)(it / stages)) & 1u, failed)) { fail(); ok = false; break; }
+                    if (!wait_or_fail<PAIR>(bar_full + 8u * s, ((uint32_t)(it / stages)) & 1u, failed)) { fail(); ok = false; break; }
                     tc_fence_after();
                     const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes);
                     const uint32_t sb = sa + a_bytes;
 #pragma unroll
                     for (int kk = 0; kk < BK / UMMA_K; ++kk)
-                        umma_bf16(d, umma_desc_k_sw128(sa + kk * UMMA_K * 2), umma_desc_k_sw128(sb + kk * UMMA_K * 2), idesc,
-                                  (kb > 0 || kk > 0) ? 1u : 0u);
+                        mma(d, sa + kk * UMMA_K * 2, sb + kk * UMMA_K * 2, (kb > 0 || kk > 0) ? 1u : 0u);
 #pragma unroll
                     for (int kk = 0; kk < BK / UMMA_K; ++kk)
-                        umma_bf16(d, umma_desc_k_sw128(sa + (uint32_t)TBL * 128u + kk * UMMA_K * 2),
-                                  umma_desc_k_sw128(sb + kk * UMMA_K * 2), idesc, 1u);
-                    umma_commit(bar_empty + 8u * s);
+                        mma(d, sa + (uint32_t)TBL * 128u + kk * UMMA_K * 2, sb + kk * UMMA_K * 2, 1u);
+                    commit(bar_empty + 8u * s);
                 }
-                if (ok) umma_commit(bar_acc_full + 8u * b);
+                if (ok) commit(bar_acc_full + 8u * b);
             }
         }
         __syncwarp();
@@ -254,11 +268,10 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     // Finishes tile `tile`.  `acc` = TMEM address of this thread's lane in the tile's accumulator.  With split-K the
     // 32-column units come from the S parked copies instead, added in rank order, and this CTA takes every S-th unit.
     auto finish_tile = [&](int tile, uint32_t acc) {
-        const int ft = tile / a.n_tt, tt = tile % a.n_tt;
+        const int ft = tile / n_tt, tt = PAIR ? 2 * (tile % n_tt) + rank : tile % n_tt;
         const int f0 = ft * FT;
         const int m = tt * TBL + rowl;
         const bool rowok = rowl < TBL && m < a.M;
-        const size_t orow = (size_t)tt * (2 * TBL) + rowl;            // row of the (hi, lo) output layout; lo at + TBL
         auto get32 = [&](int col, float (&v)[32]) {
             if (S == 1) {
                 acc32(acc + (uint32_t)col, v);
@@ -273,10 +286,34 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 }
             }
         };
+        // A thread has 32 values of ONE row; memory wants rows.  The 32 x 32 values of a warp go through shared memory (its own
+        // swizzled 4 KB, or with split-K the reduced chunk they came from), and come back as emit(row within the quarter, column,
+        // four values) with eight lanes to a row: 4 lines per access, where a thread per row touched 32.
+        auto staged = [&](int col, int r, int c4) {
+            return S == 1 ? reinterpret_cast<float4*>(stage + r * 32 + ((c4 ^ (r & 7)) << 2))
+                          : reinterpret_cast<float4*>(fin + (size_t)(quarter * 32 + r) * FLD + __popc(own_mask & ((1u << (col >> 5)) - 1u)) * 32 + 4 * c4);
+        };
+        auto rows_out = [&](int col, const float (&v)[32], auto&& emit) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) *staged(col, lane, e) = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) emit(4 * i + (lane >> 3), 4 * (lane & 7), *staged(col, 4 * i + (lane >> 3), lane & 7));
+            __syncwarp();
+        };
+        const int q_row0 = quarter * 32, m0 = tt * TBL + q_row0;        // first row of the quarter in the tile, in the pass
+        auto row_ok = [&](int r) { return q_row0 + r < TBL && m0 + r < a.M; };
+        const size_t orow0 = (size_t)tt * (2 * TBL) + q_row0;
+        auto store_hilo = [&](int r, int f, const float4& x) {
+            uint2 h, l;
+            hilo4(x, h, l);
+            *reinterpret_cast<uint2*>(a.a_out + (orow0 + r) * a.N + f) = h;
+            *reinterpret_cast<uint2*>(a.a_out + (orow0 + r + TBL) * a.N + f) = l;
+        };
         int unit = 0;                                                 // running index of the tile's work units
         int owned = 0;                                                // ... of those of this CTA (every S-th)
         auto mine = [&]() {                                           // the quarter's two warps alternate over the CTA's units
-            const bool own = (unit++ % S) == rank;
+            const bool own = PAIR || (unit++ % S) == rank;
             return own && (owned++ & 1) == wq;
         };
         float sc = 1.0f;
@@ -304,32 +341,40 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     const float g0 = g[e] * sc, u0 = u[e] * sc;
                     g[e] = __fdividef(g0, 1.0f + __expf(-g0)) * u0;
                 }
-                if (rowok) store_hilo32(a.a_out + orow * a.N + f0 + c, a.a_out + (orow + TBL) * a.N + f0 + c, g);
+                rows_out(c, g, [&](int r, int e, const float4& x) { if (row_ok(r)) store_hilo(r, f0 + c + e, x); });
             }
         } else if (EPI == EPI_RESID) {
             // ssq_out has one slot per 32 features here (a.ssq_out_slots of them, a multiple of four per 128 features)
             for (int c = 0; c < BNW && f0 + c < a.N; c += 32) {
                 if (!mine()) continue;
                 const int f = f0 + c;
-                float v[32], x[32];
-                get32(c, v);
-                if (rowok) {
-                    float* xrow = a.x + (size_t)m * a.N + f;
-                    load_f32x32(xrow, x);
-                    float ss = 0.f;
+                float v[32];
+                float4 x[8];
+                const int e0 = f + 4 * (lane & 7);
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) { x[e] += v[e]; ss += x[e] * x[e]; }
-                    store_f32x32(xrow, x);
-#pragma unroll
-                    for (int e = 0; e < 32; e += 4) {
-                        const float4 g4 = __ldg(reinterpret_cast<const float4*>(a.gain + f + e));
-                        x[e] *= g4.x; x[e + 1] *= g4.y; x[e + 2] *= g4.z; x[e + 3] *= g4.w;
-                    }
-                    store_hilo32(a.a_out + orow * a.N + f, a.a_out + (orow + TBL) * a.N + f, x);
-                    a.ssq_out[(size_t)m * a.ssq_out_slots + f / 32] = ss;
-                    if (f + 32 >= a.N)                                // the slots past the last 32 features
-                        for (int q = f / 32 + 1; q < a.ssq_out_slots; ++q) a.ssq_out[(size_t)m * a.ssq_out_slots + q] = 0.f;
+                for (int i = 0; i < 8; ++i) {
+                    const int r = 4 * i + (lane >> 3);
+                    x[i] = row_ok(r) ? *reinterpret_cast<const float4*>(a.x + (size_t)(m0 + r) * a.N + e0) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
+                const float4 g4 = __ldg(reinterpret_cast<const float4*>(a.gain + e0));
+                get32(c, v);
+                int i = 0;
+                rows_out(c, v, [&](int r, int, const float4& y) {
+                    float4 t = x[i++];
+                    t.x += y.x; t.y += y.y; t.z += y.z; t.w += y.w;
+                    float ss = (t.x * t.x + t.y * t.y) + (t.z * t.z + t.w * t.w);
+                    ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 1);
+                    ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 2);
+                    ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 4);
+                    if (!row_ok(r)) return;
+                    *reinterpret_cast<float4*>(a.x + (size_t)(m0 + r) * a.N + e0) = t;
+                    store_hilo(r, e0, make_float4(t.x * g4.x, t.y * g4.y, t.z * g4.z, t.w * g4.w));
+                    if ((lane & 7) == 0) {
+                        a.ssq_out[(size_t)(m0 + r) * a.ssq_out_slots + f / 32] = ss;
+                        if (f + 32 >= a.N)                            // the slots past the last 32 features
+                            for (int q = f / 32 + 1; q < a.ssq_out_slots; ++q) a.ssq_out[(size_t)(m0 + r) * a.ssq_out_slots + q] = 0.f;
+                    }
+                });
             }
         } else if (EPI == EPI_QKV) {
             const int hd = a.hd, half = hd >> 1;
@@ -349,9 +394,8 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 if (fh < qd + kvd) {
                     // a query or key head: rotate the pairs (i, i + half); a unit is 32 pairs
                     const bool is_q = fh < qd;
-                    __nv_bfloat16* kdst = nullptr;
-                    if (!is_q && pos >= 0 && page >= 0)
-                        kdst = a.k_pages + (((size_t)page * a.n_kv + (fh - qd) / hd) * a.page_size + pos % a.page_size) * hd;
+                    const long long kdst = !is_q && pos >= 0 && page >= 0
+                        ? (long long)((((size_t)page * a.n_kv + (fh - qd) / hd) * a.page_size + pos % a.page_size) * hd) : -1ll;
                     for (int jj = 0; jj < half; jj += 32) {
                         if (!mine()) continue;
                         float lo[32], hi[32];
@@ -371,28 +415,30 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 #pragma unroll
                             for (int e = 0; e < 32; ++e) { lo[e] = 0.f; hi[e] = 0.f; }
                         }
-                        if (is_q) {
-                            if (rowok) {
-                                store_f32x32(a.qbuf + (size_t)m * qd + fh + jj, lo);
-                                store_f32x32(a.qbuf + (size_t)m * qd + fh + half + jj, hi);
-                            }
-                        } else if (kdst) {
-                            store_bf16x32(kdst + jj, lo);
-                            store_bf16x32(kdst + half + jj, hi);
-                        }
+                        auto put = [&](int col, int at, const float (&v)[32]) {
+                            rows_out(col, v, [&](int r, int e, const float4& x) {
+                                const long long dst = __shfl_sync(0xFFFFFFFFu, kdst, r);
+                                if (is_q) { if (row_ok(r)) *reinterpret_cast<float4*>(a.qbuf + (size_t)(m0 + r) * qd + fh + at + e) = x; }
+                                else if (dst >= 0) *reinterpret_cast<uint2*>(a.k_pages + dst + at + e) = bf16x4(x);
+                            });
+                        };
+                        put(hc + jj, jj, lo);
+                        put(hc + half + jj, half + jj, hi);
                     }
                 } else {
                     // a value head
-                    __nv_bfloat16* vdst = nullptr;
-                    if (pos >= 0 && page >= 0)
-                        vdst = a.v_pages + (((size_t)page * a.n_kv + (fh - qd - kvd) / hd) * a.page_size + pos % a.page_size) * hd;
+                    const long long vdst = pos >= 0 && page >= 0
+                        ? (long long)((((size_t)page * a.n_kv + (fh - qd - kvd) / hd) * a.page_size + pos % a.page_size) * hd) : -1ll;
                     for (int c = 0; c < hd; c += 32) {
                         if (!mine()) continue;
                         float v[32];
                         get32(hc + c, v);
 #pragma unroll
                         for (int e = 0; e < 32; ++e) v[e] *= sc;
-                        if (vdst) store_bf16x32(vdst + c, v);
+                        rows_out(hc + c, v, [&](int r, int e, const float4& x) {
+                            const long long dst = __shfl_sync(0xFFFFFFFFu, vdst, r);
+                            if (dst >= 0) *reinterpret_cast<uint2*>(a.v_pages + dst + c + e) = bf16x4(x);
+                        });
                     }
                 }
             }
@@ -426,10 +472,11 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         g_ta = global_ns();
 #endif
         const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        const uint32_t acc_empty0 = PAIR ? cluster_map(bar_acc_empty, 0u) : bar_acc_empty;      // the MMAs are issued by the even CTA
         if (S == 1) {
             for (int j = 0; j < my_tiles; ++j) {
                 const int b = j & 1;
-                bool ok = wait_or_fail(bar_acc_full + 8u * b, ((uint32_t)(j >> 1)) & 1u, failed);
+                bool ok = wait_or_fail<PAIR>(bar_acc_full + 8u * b, ((uint32_t)(j >> 1)) & 1u, failed);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) { if (lane == 0) fail(); break; }
 #ifdef TASC_TIMELINE
@@ -439,7 +486,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 tc_fence_after();
                 finish_tile(tile0 + j * tstep, lane_base + (uint32_t)(b * BNW));
                 tc_fence_before();
-                mbar_arrive(bar_acc_empty + 8u * b);
+                if (PAIR) mbar_arrive_cluster(acc_empty0 + 8u * b); else mbar_arrive(bar_acc_empty + 8u * b);
             }
         } else if (my_tiles > 0) {
             // split-K, part 1: this CTA's partial tile -> its shared memory (zeros after a failed wait, so that the
@@ -480,7 +527,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             // quarter (32 rows x 32 columns); eight consecutive lanes cover the 128 bytes of a row, so a warp-wide
             // remote read touches 4 rows, and the reads of all copies are in flight together.
             {
-                const int f0 = (tile0 / a.n_tt) * FT;
+                const int f0 = (tile0 / n_tt) * FT;
                 int unit = 0;
                 auto take = [&](int c0, int c1) {
                     if ((unit++ % S) == rank) { own_mask |= 1u << (c0 >> 5); if (c1 >= 0) own_mask |= 1u << (c1 >> 5); }
@@ -541,16 +588,17 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         while (clock64() - t0 < 2000000ll) { }
     }
     __syncthreads();
+    if (PAIR) { cluster_arrive(); cluster_wait(); }              // neither CTA leaves while the other may signal or read it
     if (warp == EPI_WARPS + 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, (uint32_t)(2 * BNW));
+        if (PAIR) tmem_dealloc_pair(tmem_base, (uint32_t)(2 * BNW)); else tmem_dealloc(tmem_base, (uint32_t)(2 * BNW));
     }
 #ifdef TASC_TIMELINE
     if (threadIdx.x == 0) ctalog_put(g_t0, g_ta, g_tb, 20 + EPI, g_tc, g_td, g_te, g_tf);
 #endif
 }
 
-template <int EPI>
+template <int EPI, bool PAIR>
 tasc_status prepare_wide() {
     static std::mutex mu;
     static bool attr_done[64] = {false};
@@ -559,16 +607,16 @@ tasc_status prepare_wide() {
     if (dev < 0 || dev >= 64) return TASC_EINVAL;
     std::lock_guard<std::mutex> lk(mu);
     if (!attr_done[dev]) {
-        TASC_CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
+        TASC_CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel<EPI, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
         attr_done[dev] = true;
     }
     return TASC_OK;
 }
 
-template <int EPI>
+template <int EPI, bool PAIR>
 tasc_status launch_wide(const CUtensorMap* tmW, const CUtensorMap* tmX, const FusedArgs& a, const FusedPlan& p, int kind,
                         cudaStream_t stream) {
-    tasc_status pst = prepare_wide<EPI>();
+    tasc_status pst = prepare_wide<EPI, PAIR>();
     if (pst != TASC_OK) return pst;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)p.grid, 1, 1);
@@ -580,9 +628,9 @@ tasc_status launch_wide(const CUtensorMap* tmW, const CUtensorMap* tmX, const Fu
     at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[n].val.programmaticStreamSerializationAllowed = 1;
     ++n;
-    if (p.S > 1) {
+    if (PAIR || p.S > 1) {
         at[n].id = cudaLaunchAttributeClusterDimension;
-        at[n].val.clusterDim.x = (unsigned)p.S;
+        at[n].val.clusterDim.x = PAIR ? 2u : (unsigned)p.S;
         at[n].val.clusterDim.y = 1;
         at[n].val.clusterDim.z = 1;
         ++n;
@@ -590,14 +638,14 @@ tasc_status launch_wide(const CUtensorMap* tmW, const CUtensorMap* tmX, const Fu
     cfg.attrs = at;
     cfg.numAttrs = n;
     ProfScope ps(kind, stream);
-    TASC_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_wide_kernel<EPI>, *tmW, *tmX, a));
+    TASC_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_wide_kernel<EPI, PAIR>, *tmW, *tmX, a));
     return TASC_OK;
 }
 
 // Clusters of S CTAs with `smem` bytes each that the device can hold at once (0 if the query fails).
 template <int EPI>
 int wide_clusters(int S, int smem) {
-    if (prepare_wide<EPI>() != TASC_OK) return 0;
+    if (prepare_wide<EPI, false>() != TASC_OK) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)S, 1, 1);
     cfg.blockDim = dim3(THREADS, 1, 1);
@@ -610,7 +658,7 @@ int wide_clusters(int S, int smem) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_wide_kernel<EPI>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_wide_kernel<EPI, false>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
     return n;
 }
 
@@ -659,6 +707,7 @@ bool plan_wide(int M, int N, int K, int epi, int hd, FusedPlan& p, int token_til
     p.m_tiles = (M + p.TBL - 1) / p.TBL;
     p.num_kb = (K + BK - 1) / BK;
     p.wide = 1;
+    p.cta_pair = 0;
     const int sms = sm_count();
     // Tile width and k-splits, by a cost in SM cycles.  A k-block of a tile of `bnw` features is 8 MMAs of bnw / 2 cycles
     // and brings (2 TBL + bnw) rows of 128 bytes into shared memory, which an SM takes in at about 40 bytes per cycle
@@ -670,8 +719,8 @@ bool plan_wide(int M, int N, int K, int epi, int hd, FusedPlan& p, int token_til
         const int ft = epi == EPI_SWIGLU ? bnw / 2 : bnw;
         const int tiles = ((N + ft - 1) / ft) * p.m_tiles;
         const int stage_bytes = (2 * p.TBL + bnw) * 128;
-        const int st = std::max(2, std::min((200 * 1024) / stage_bytes, MAX_STAGES));
-        const int data = std::max(st * stage_bytes, 128 * (bnw + 4) * 4 + 128 * (4 * 32 + 4) * 4);
+        const int st = std::max(2, std::min((192 * 1024) / stage_bytes, MAX_STAGES));
+        const int data = std::max(st * stage_bytes + STAGING_BYTES, 128 * (bnw + 4) * 4 + 128 * (4 * 32 + 4) * 4);
         const int smem = std::min(std::max(1024 + data, 120 * 1024), MAX_DYN_SMEM);
         const double per_kb = std::max(4.0 * bnw, (2.0 * p.TBL + bnw) * 128.0 / 40.0);
         for (int S = 1; S <= (may_split ? 8 : 1); ++S) {
@@ -684,9 +733,25 @@ bool plan_wide(int M, int N, int K, int epi, int hd, FusedPlan& p, int token_til
             const double cost = (double)waves * ((p.num_kb + S - 1) / S) * per_kb + (S > 1 ? 6000.0 + 10.0 * bnw : 12.0 * bnw);
             if (best_cost < 0. || cost < best_cost) {
                 best_cost = cost;
-                p.BNW = bnw; p.S = S; p.out_tiles = (N + ft - 1) / ft; p.stages = st; p.data_bytes = data; p.smem_bytes = smem;
+                p.BNW = bnw; p.S = S; p.cta_pair = 0; p.out_tiles = (N + ft - 1) / ft; p.stages = st; p.data_bytes = data; p.smem_bytes = smem;
                 p.grid = S > 1 ? tiles * S : std::min(tiles, sms);
             }
+        }
+    }
+    // Pairs of CTAs on 256 features and two token tiles: half the weight rows per CTA.
+    if (p.m_tiles >= 2 && sms % 2 == 0) {
+        const int ft = epi == EPI_SWIGLU ? 128 : 256;
+        const int out_tiles = (N + ft - 1) / ft, tiles = out_tiles * ((p.m_tiles + 1) / 2), pairs = sms / 2;
+        const int stage_bytes = (2 * p.TBL + 128) * 128;
+        const int st = std::min((192 * 1024) / stage_bytes, MAX_STAGES);
+        // (a k-block takes a pair 0.92 of the time of a CTA alone, measured on 448 rows x 151,936 features; a lone last token
+        // tile wastes half a pair: at 288 rows x 160,128 features, three token tiles, 174 us in pairs against 140)
+        const double per_kb = std::max(4.0 * 256, 0.92 * (2.0 * p.TBL + 256) * 128.0 / 40.0);
+        const double cost = (double)((tiles + pairs - 1) / pairs) * p.num_kb * per_kb + 12.0 * 256;
+        if (cost < best_cost) {
+            p.BNW = 256; p.S = 1; p.cta_pair = 1; p.out_tiles = out_tiles; p.stages = st; p.data_bytes = st * stage_bytes + STAGING_BYTES;
+            p.smem_bytes = std::min(std::max(1024 + p.data_bytes, 120 * 1024), MAX_DYN_SMEM);
+            p.grid = 2 * std::min(tiles, pairs);
         }
     }
     return best_cost >= 0.;
@@ -697,10 +762,10 @@ tasc_status launch_gemm_wide(int epi, const CUtensorMap* tmW, const CUtensorMap*
     a.num_kb = p.num_kb; a.BN = p.BN; a.TB = p.TB; a.TBL = p.TBL; a.stages = p.stages; a.pair = 1; a.data_bytes = p.data_bytes;
     a.BNW = p.BNW; a.n_ft = p.out_tiles; a.n_tt = p.m_tiles;
     switch (epi) {
-        case EPI_QKV:    return launch_wide<EPI_QKV>(tmW, tmX, a, p, K_GEMM, stream);
-        case EPI_RESID:  return launch_wide<EPI_RESID>(tmW, tmX, a, p, K_GEMM, stream);
-        case EPI_SWIGLU: return launch_wide<EPI_SWIGLU>(tmW, tmX, a, p, K_GEMM, stream);
-        case EPI_LM:     return launch_wide<EPI_LM>(tmW, tmX, a, p, K_GEMM_LM, stream);
+        case EPI_QKV:    return p.cta_pair ? launch_wide<EPI_QKV, true>(tmW, tmX, a, p, K_GEMM, stream) : launch_wide<EPI_QKV, false>(tmW, tmX, a, p, K_GEMM, stream);
+        case EPI_RESID:  return p.cta_pair ? launch_wide<EPI_RESID, true>(tmW, tmX, a, p, K_GEMM, stream) : launch_wide<EPI_RESID, false>(tmW, tmX, a, p, K_GEMM, stream);
+        case EPI_SWIGLU: return p.cta_pair ? launch_wide<EPI_SWIGLU, true>(tmW, tmX, a, p, K_GEMM, stream) : launch_wide<EPI_SWIGLU, false>(tmW, tmX, a, p, K_GEMM, stream);
+        case EPI_LM:     return p.cta_pair ? launch_wide<EPI_LM, true>(tmW, tmX, a, p, K_GEMM_LM, stream) : launch_wide<EPI_LM, false>(tmW, tmX, a, p, K_GEMM_LM, stream);
         default: return TASC_EINVAL;
     }
 }

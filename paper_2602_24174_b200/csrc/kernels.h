@@ -126,6 +126,7 @@ struct FusedPlan {
     int stages, data_bytes, smem_bytes;
     int wide;          // 1: the many-row kernel of gemm_wide.cu (M > 128) with BNW weight rows per MMA and `grid` persistent CTAs
     int BNW, grid;
+    int cta_pair;      // ... which work in pairs (cta_group::2) on two token tiles
     int threads;       // few-row kernel: 192, or 384 (six more warps that only finish columns) where a CTA finishes many token columns
 };
 // hd: head_dim, for EPI_QKV.  wide_min_mb: < 0 for a pass whose products all take the few-row kernel; otherwise the

@@ -340,6 +340,18 @@ def test_config4_geometry_between_one_and_two_full_token_tiles(B):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("B,P", [(37, 9), (55, 40), (75, 129)])
+def test_many_row_kernel_on_pairs_of_token_tiles(B, P):
+    """Configuration 4's geometry (one layer, an 8,200-token vocabulary: a feature tile of eight) at 259, 385 and 525 rows of
+    7 per sequence, after prefills in passes of 1,184 to 2,040: an even and an odd number of token tiles for the kernel's
+    pairs, ragged last tiles.  The oracle runs the first, a middle and the last sequence."""
+    cfg = configs.shrunk(configs.get(4), n_layers=1, vocab=8200, n_docs=500)
+    s = make_setup(cfg)
+    prompts = corpus.make_prompts(cfg, B, prompt_len=P)
+    check(lockstep(s, prompts, cfg.k + 1, cfg.k, oracle_rows=[0, B // 2, B - 1], **BF16_TOL), f"pairs of token tiles, B={B} P={P}")
+
+
+@pytest.mark.gpu
 def test_many_row_kernel_on_every_product_with_64_wide_heads():
     """A one-layer shape whose five weight matrices are all large enough for the many-row GEMM kernel (d_model 2,048,
     32 query / 8 KV heads of 64, d_ff 2,048, vocabulary 8,192: 8 to 34 MB each) at 40 sequences x 7 rows = 280 rows
