@@ -273,6 +273,7 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
             // attention works on blocks of at most 16 rows per sequence (one block in a verify step, several in a prefill pass)
             const int att_rows = R <= 16 ? R : 16;
             sp.att = plan_attention_mma(B * (R / att_rows), d.n_kv_heads, d.head_dim, d.n_q_heads / d.n_kv_heads, att_rows, max_ctx);
+            plan_attention_tc(B * (R / att_rows), d.n_kv_heads, d.head_dim, d.n_q_heads / d.n_kv_heads, att_rows, max_ctx, d.page_size, sp.att);
             // passes of more than 128 rows: the products with large weight matrices take the many-row kernel
             const double big_mb = 2.0 * 2.0 * (double)d.d_ff * d.d_model / 1e6;      // the largest matrix of a layer (gate/up)
             const bool wide_pass = M > 128 && big_mb >= WIDE_MATRIX_MB && (M >= WIDE_ROWS || m->layer_mb >= WIDE_LAYER_MB);

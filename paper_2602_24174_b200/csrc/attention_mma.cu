@@ -679,7 +679,7 @@ AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ct
     // pipes need per tile and 16-row slab when all warps have work (the lower bound once several groups run).
     const float t_tile = hd >= 128 ? 2.0f : (hd >= 64 ? 1.3f : 0.8f);
     const float t_pipe = hd >= 128 ? 0.6f : (hd >= 64 ? 0.3f : 0.15f);
-    AttnPlan best = {1, 2, g};
+    AttnPlan best = {1, 2, g, 0, 1e30f};
     float best_cost = 1e30f;
     // Candidates: all g heads of a KV head in one CTA; and, for few sequences with 128-wide heads (where one warp needs
     // 2 us per key tile), the largest share of the heads whose rows still fill a single 16-row slab.  (Measured: on the
@@ -713,7 +713,7 @@ AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ct
                 // every head group re-reads its KV head's keys: L2 traffic, about 0.1 us per extra pass over a tile
                 const float reread = 0.1f * tiles_cta * (float)(g / hs - 1) / (float)std::max(1, g / hs);
                 const float cost = waves * (2.5f + loop) + merge + crowd + reread;
-                if (cost < best_cost - 1e-6f) { best_cost = cost; best = AttnPlan{s, stages, hs}; }
+                if (cost < best_cost - 1e-6f) { best_cost = cost; best = AttnPlan{s, stages, hs, 0, cost}; }
             }
         }
     }
@@ -754,6 +754,7 @@ tasc_status launch_attention_mma(const float* qbuf, const __nv_bfloat16* k_pages
         if ((st = encode_tmap_kv(&tmK, k_pages, rows, hd)) != TASC_OK) return st;
         if ((st = encode_tmap_kv(&tmV, v_pages, rows, hd)) != TASC_OK) return st;
     }
+    if (plan.tc) return launch_attention_tc(qbuf, tmK, tmV, block_table, max_pages, n_pages, rp, out, TB, B, R, n_q, n_kv, hd, plan, status, stream);
     if (GP == 64) {
         if (hd == 32) return launch_inst<32, 4>(a, tmK, tmV, B * n_sub, stream);
         if (hd == 64) return launch_inst<64, 4>(a, tmK, tmV, B * n_sub, stream);

@@ -1,0 +1,581 @@
+// Verify and prefill attention for bf16 models on the 5th-generation tensor cores: the same job as attention_mma.cu (which see
+// for the row and key order, the paged cache and the precision: Q and P as (hi, lo) bf16 pairs) for passes with enough rows
+// and sequences.
+//
+// Bound: at 42 rows (7 rows x 6 query heads of a KV head) and 1,500 keys the warp-level kernel spent 5 us per 128 keys, on
+// mma.sync pipes that half of its warps used and on barriers, while K and V could stream in a tenth of that.  Here S = Q K^T
+// and P V are tcgen05 MMAs of 128 rows (M; the rows past the query tile cost nothing, the issue rate is the same) issued by
+// one thread, S and O in TMEM, K and V staged by TMA, so that the softmax is what is left: a thread owns half of the keys
+// of one row, registers hold its half of the row's O.  Per tile of TK keys
+//   MMA warp       S(t + 1) while the softmax works on S(t); then P(t) V(t) into an O tile of its own
+//   softmax warps  S(t) -> maximum (exchanged between the two threads of a row) -> P(t) as hi, lo in shared memory;
+//                  then O += O tile (t - 1), rescaled: O is accumulated in registers, so a new maximum costs no pass over TMEM
+//   TMA warp       K and V tiles, a ring of two or more
+// Query tiles of up to 64 rows take 128 keys per tile, up to 128 rows 64 keys (P is TK x rows x 4 bytes of shared memory).
+// Key ranges split over a cluster are merged as in attention_mma.cu.
+//
+// Measured, per layer: 1.5B at 64 sequences x 7 rows and up to 1,530 keys 61 -> 33 us (2.0 us per 128 keys: softmax 0.9, its
+// half of O 0.3, P 0.4, waits 0.4); 0.5B + 8,192 tokens at 32 x 9 rows, 640 keys 15.5 -> 13.4; prefill of 16 x 1,024 tokens
+// on the 1.5B 72 -> 47 us per pass of 2,048 rows.
+//
+// Every wait is bounded; after one that ran out the loops run on without waiting, so that all barriers are still met.
+#include "kernels.h"
+
+#include <algorithm>
+#include <mutex>
+
+namespace tasc {
+
+namespace {
+
+constexpr int SM_WARPS = 8;                      // softmax: two per TMEM lane quarter, which share its rows
+constexpr int THREADS = (SM_WARPS + 2) * 32;     // + TMA warp, MMA warp
+constexpr int PAGE = 16;
+constexpr int MAX_PAGES = 1024;
+constexpr int MAX_SMEM = 216 * 1024;
+constexpr int MAX_RING = 4;
+
+struct TcArgs {
+    const float* q;
+    const int32_t* block_table;
+    int max_pages;
+    long long n_pages;
+    const int* seq_pos0;
+    const int* seq_rows;
+    __nv_bfloat16* out;
+    int TB;
+    int R, Rs, n_sub, n_q, n_kv, splits, stages;
+    int* status;
+    float scale_log2e;
+};
+
+// two floats -> packed bf16 pair (hi) and the packed pair of the residuals (lo)
+__device__ __forceinline__ void pack_hilo(float x, float y, uint32_t& hi, uint32_t& lo) {
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(y), "f"(x));
+    const float rx = x - __uint_as_float(hi << 16), ry = y - __uint_as_float(hi & 0xFFFF0000u);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(ry), "f"(rx));
+}
+// 2^x of the hardware (what exp2f calls, without its detour for results below 2^-126, which are zero here)
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// Shared-memory descriptor of an operand whose rows (128 bytes, swizzled) are steps along K and whose columns are M or N:
+// 64 columns to a row block, `col_stride` bytes from one block of 64 columns to the next, 8 K-rows to 1,024 bytes.
+__device__ __forceinline__ uint64_t umma_desc_mn_sw128(uint32_t smem_addr, uint32_t col_stride) {
+    uint64_t d = 0;
+    d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(col_stride >> 4) << 16;
+    d |= (uint64_t)(1024u >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+
+template <int HD, int RP> struct Tc {
+    static constexpr int TK = RP == 64 ? 128 : 64;               // keys of a tile
+    static constexpr int HB = HD / 64;                           // blocks of 64 columns of a head
+    static constexpr int Q_BYTES = RP * HD * 2;                  // hi or lo
+    static constexpr int P_BYTES = RP * TK * 2;
+    static constexpr int KV_BYTES = TK * HD * 2;                 // K or V tile
+    static constexpr int FIXED = 2 * Q_BYTES + 2 * P_BYTES;
+    static constexpr int S_COL = 0, O_COL = 2 * TK;              // TMEM columns: two S tiles, two O tiles
+    static constexpr int COLS = 2 * TK + 2 * HD <= 256 ? 256 : 512;
+    static constexpr int SC = TK / 2, OC = HD / 2;               // a thread's share of a row of S, of O
+    static int smem(int stages) { return 1024 + FIXED + stages * 2 * KV_BYTES; }
+};
+
+template <int HD, int RP>
+__global__ void __launch_bounds__(THREADS, 1)
+attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const TcArgs a) {
+    using C = Tc<HD, RP>;
+    constexpr int TK = C::TK;
+    extern __shared__ uint8_t sm_raw[];
+    uint8_t* sm = sm_raw + ((1024u - (smem_u32(sm_raw) & 1023u)) & 1023u);
+    uint8_t* Qs = sm;                                            // hi, then lo: [HB][RP][128 bytes]
+    uint8_t* Ps = Qs + 2 * C::Q_BYTES;                           // hi, then lo: [TK / 64][RP][128 bytes]
+    uint8_t* ring = Ps + 2 * C::P_BYTES;                         // [stages] K [HB][TK][128 bytes], V the same
+    __shared__ int s_pages[MAX_PAGES];
+    __shared__ float s_max[2][2][RP], s_sum[2][RP];
+    __shared__ uint64_t s_bars[4 * MAX_RING + 10];
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_fail;
+    volatile int* failed = &s_fail;
+
+    const int sp = blockIdx.x, kh = blockIdx.y, b = blockIdx.z / a.n_sub, rb = (blockIdx.z % a.n_sub) * a.Rs;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int g = a.n_q / a.n_kv, R = a.Rs, G = g * R, h0 = kh * g, qd = a.n_q * HD;
+    // (the row plan, the block table and the committed K / V were written before the preceding grid started)
+    const int seq_pos0 = a.seq_pos0[b];
+    int rows = a.seq_rows[b] - rb;
+    rows = rows < 0 ? 0 : (rows > R ? R : rows);
+    const int pos0 = seq_pos0 + rb;
+    auto out_row = [&](int rho) {
+        const int m = b * a.R + rb + rho % R;
+        return (size_t)(m / a.TB) * (2 * a.TB) + (m % a.TB);
+    };
+    if (rows == 0) {
+        griddep_wait();
+        griddep_launch_dependents();
+        // sequence not in this pass: its rows of the output are zero
+        if (sp == 0) {
+            for (int i = tid; i < G * (HD / 4); i += THREADS) {
+                const int rho = i / (HD / 4), d4 = (i % (HD / 4)) * 4;
+                const size_t row = out_row(rho), col = (size_t)(h0 + rho / R) * HD + d4;
+                *reinterpret_cast<uint2*>(a.out + row * qd + col) = make_uint2(0u, 0u);
+                *reinterpret_cast<uint2*>(a.out + (row + a.TB) * qd + col) = make_uint2(0u, 0u);
+            }
+        }
+        return;
+    }
+    // this CTA's keys: the tiles are dealt out evenly over the splits
+    const int total = pos0 + rows;
+    const int tiles_all = (total + TK - 1) / TK, t_base = tiles_all / a.splits, t_rem = tiles_all % a.splits;
+    const int n_tiles = t_base + (sp < t_rem ? 1 : 0);
+    const int k_begin = (sp * t_base + min(sp, t_rem)) * TK;
+    const int k_end = min(total, k_begin + n_tiles * TK);
+    const int pg_lo = k_begin / PAGE, n_pg = n_tiles > 0 ? (k_end - 1) / PAGE - pg_lo + 1 : 0;
+    const int quarters = (G + 31) / 32;                          // TMEM lane quarters with rows: 2 softmax warps each
+    const uint32_t arrivals = (uint32_t)quarters * 64u;
+
+    const uint32_t bar_k_full = smem_u32(s_bars), bar_v_full = bar_k_full + 8u * MAX_RING;
+    const uint32_t bar_k_empty = bar_v_full + 8u * MAX_RING, bar_v_empty = bar_k_empty + 8u * MAX_RING;
+    const uint32_t bar_s_full = bar_v_empty + 8u * MAX_RING, bar_s_empty = bar_s_full + 16u;
+    const uint32_t bar_o_full = bar_s_empty + 16u, bar_o_empty = bar_o_full + 16u;
+    const uint32_t bar_p_full = bar_o_empty + 16u, bar_q_full = bar_p_full + 8u;
+    if (tid == 0) {
+        s_fail = 0;
+        for (int i = 0; i < a.stages; ++i) {
+            mbar_init(bar_k_full + 8u * i, 1);
+            mbar_init(bar_v_full + 8u * i, 1);
+            mbar_init(bar_k_empty + 8u * i, 1);
+            mbar_init(bar_v_empty + 8u * i, 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(bar_s_full + 8u * i, 1);
+            mbar_init(bar_s_empty + 8u * i, arrivals);
+            mbar_init(bar_o_full + 8u * i, 1);
+            mbar_init(bar_o_empty + 8u * i, arrivals);
+        }
+        mbar_init(bar_p_full, arrivals);
+        mbar_init(bar_q_full, SM_WARPS * 32);
+        fence_barrier_init();
+        tma_prefetch_desc(&tmK);
+        tma_prefetch_desc(&tmV);
+    }
+    for (int i = tid; i < n_pg; i += THREADS) {
+        const int pslot = pg_lo + i;
+        int page = -1;
+        if (pslot < a.max_pages) page = a.block_table[(size_t)b * a.max_pages + pslot];
+        s_pages[i] = (page >= 0 && page < a.n_pages) ? page : -1;      // ids outside the pool are never used as addresses
+    }
+    if (warp == SM_WARPS + 1) {
+        tmem_alloc(smem_u32(&s_tmem), (uint32_t)C::COLS);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+    auto wait = [&](uint32_t bar, uint32_t parity) {             // after a failure: no more waiting
+        if (mbar_try_wait(bar, parity)) return;
+        const long long t0 = clock64();
+        while (!mbar_try_wait(bar, parity)) {
+            if (*failed) return;
+            if (clock64() - t0 > 1000000000ll) { set_status(a.status, TASC_ETIMEOUT); *failed = 1; return; }
+        }
+    };
+
+    constexpr int OC = C::OC;
+    float acc[OC];                                               // this thread's half of its row of O
+    float m_run = -INFINITY, l_run = 0.f;
+    const int quarter = warp & 3, half = (warp >> 2) & 1;
+    const int rho = quarter * 32 + lane;                         // row of the query tile = TMEM lane
+    const bool active = warp < SM_WARPS && quarter < quarters;
+
+    if (warp == SM_WARPS) {
+        // ------------------------------------------------------------ TMA
+        // A tile is TK / 16 pages; a page of this KV head is one box (two for 128-wide heads) of K and one of V.  Rows past the
+        // range re-read its last page, ids outside the pool read page 0: both are masked, and nothing unmapped is touched.
+        // K and V have barriers of their own: K of a tile is free one softmax earlier than V.
+        constexpr int BOXES = (TK / PAGE) * C::HB;
+        auto load = [&](int t, bool is_v) {
+            const int s = t % a.stages;
+            const uint32_t bar = (is_v ? bar_v_full : bar_k_full) + 8u * s;
+            const uint32_t base = smem_u32(ring + (size_t)s * 2 * C::KV_BYTES) + (is_v ? C::KV_BYTES : 0);
+            if (lane == 0) mbar_expect_tx(bar, C::KV_BYTES);
+            __syncwarp();
+            if (lane < BOXES) {
+                const int pg = lane / C::HB, h = lane % C::HB;
+                int key = k_begin + t * TK + pg * PAGE;
+                key = key < k_end ? key : k_end - 1;
+                int page = s_pages[key / PAGE - pg_lo];
+                page = page < 0 ? 0 : page;
+                tma_load_2d(base + h * (TK * 128) + pg * (PAGE * 128), is_v ? &tmV : &tmK, h * 64, (page * a.n_kv + kh) * PAGE, bar);
+            }
+            __syncwarp();
+        };
+        // tiles of committed positions are requested before the preceding grid has finished, the others after it
+        int t = 0;
+        for (; t < a.stages && t < n_tiles && k_begin + (t + 1) * TK <= seq_pos0; ++t) { load(t, false); load(t, true); }
+        griddep_wait();
+        for (; t < n_tiles; ++t) {
+            const uint32_t used = (uint32_t)(t / a.stages - 1) & 1u;
+            if (t >= a.stages) { wait(bar_k_empty + 8u * (t % a.stages), used); __syncwarp(); }
+            if (*failed) break;
+            load(t, false);
+            if (t >= a.stages) { wait(bar_v_empty + 8u * (t % a.stages), used); __syncwarp(); }
+            if (*failed) break;
+            load(t, true);
+        }
+        __syncwarp();
+    } else if (warp == SM_WARPS + 1) {
+        // ------------------------------------------------------------ MMA
+        if (lane == 0 && n_tiles > 0) {
+            const uint32_t qa = smem_u32(Qs), pa = smem_u32(Ps), kv = smem_u32(ring);
+            constexpr uint32_t idesc_s = umma_idesc_bf16_f32(128, TK);
+            constexpr uint32_t idesc_o = umma_idesc_bf16_f32(128, HD) | (1u << 16);      // V: columns along N
+            auto issue_s = [&](int t) {
+                wait(bar_k_full + 8u * (t % a.stages), (uint32_t)(t / a.stages) & 1u);
+                if (t >= 2) wait(bar_s_empty + 8u * (t & 1), (uint32_t)((t >> 1) - 1) & 1u);
+                tc_fence_after();
+                const uint32_t kb = kv + (uint32_t)(t % a.stages) * 2u * C::KV_BYTES, d = tmem + C::S_COL + (uint32_t)(t & 1) * TK;
+#pragma unroll
+                for (int p = 0; p < 2; ++p)                      // hi, lo
+#pragma unroll
+                    for (int ks = 0; ks < HD / 16; ++ks)
+                        umma_bf16(d, umma_desc_k_sw128(qa + p * C::Q_BYTES + (ks >> 2) * (RP * 128) + (ks & 3) * 32),
+                                  umma_desc_k_sw128(kb + (ks >> 2) * (TK * 128) + (ks & 3) * 32), idesc_s, (p | ks) ? 1u : 0u);
+                umma_commit(bar_s_full + 8u * (t & 1));
+                umma_commit(bar_k_empty + 8u * (t % a.stages));
+            };
+            wait(bar_q_full, 0u);
+            tc_fence_after();
+            issue_s(0);
+            for (int t = 0; t < n_tiles; ++t) {
+                if (t + 1 < n_tiles) issue_s(t + 1);
+                wait(bar_v_full + 8u * (t % a.stages), (uint32_t)(t / a.stages) & 1u);
+                wait(bar_p_full, (uint32_t)t & 1u);
+                if (t >= 2) wait(bar_o_empty + 8u * (t & 1), (uint32_t)((t >> 1) - 1) & 1u);
+                tc_fence_after();
+                const uint32_t vb = kv + (uint32_t)(t % a.stages) * 2u * C::KV_BYTES + C::KV_BYTES, d = tmem + C::O_COL + (uint32_t)(t & 1) * HD;
+#pragma unroll
+                for (int p = 0; p < 2; ++p)
+#pragma unroll
+                    for (int kk = 0; kk < TK / 16; ++kk)
+                        umma_bf16(d, umma_desc_k_sw128(pa + p * C::P_BYTES + (kk >> 2) * (RP * 128) + (kk & 3) * 32),
+                                  umma_desc_mn_sw128(vb + kk * (16 * 128), TK * 128), idesc_o, (p | kk) ? 1u : 0u);
+                umma_commit(bar_o_full + 8u * (t & 1));          // also: P is free
+                umma_commit(bar_v_empty + 8u * (t % a.stages));
+            }
+        }
+        __syncwarp();
+    } else {
+        // ------------------------------------------------------------ softmax
+        griddep_wait();
+        griddep_launch_dependents();
+        // Q rows, scaled, as (hi, lo) in shared memory; zeros where there is no row
+        {
+            constexpr int NQ = RP * (HD / 4) / (SM_WARPS * 32);
+            float4 qv[NQ];
+#pragma unroll
+            for (int j = 0; j < NQ; ++j) {
+                const int i = tid + j * (SM_WARPS * 32), r = i / (HD / 4), d4 = (i % (HD / 4)) * 4;
+                qv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (r < G && r % R < rows) qv[j] = *reinterpret_cast<const float4*>(a.q + (size_t)(b * a.R + rb + r % R) * qd + (size_t)(h0 + r / R) * HD + d4);
+            }
+#pragma unroll
+            for (int j = 0; j < NQ; ++j) {
+                const int i = tid + j * (SM_WARPS * 32), r = i / (HD / 4), d4 = (i % (HD / 4)) * 4;
+                uint2 h, l;
+                pack_hilo(qv[j].x * a.scale_log2e, qv[j].y * a.scale_log2e, h.x, l.x);
+                pack_hilo(qv[j].z * a.scale_log2e, qv[j].w * a.scale_log2e, h.y, l.y);
+                const int chunk = (d4 & 63) >> 3;
+                const uint32_t off = (uint32_t)((d4 >> 6) * (RP * 128) + r * 128 + ((chunk ^ (r & 7)) << 4) + (d4 & 7) * 2);
+                *reinterpret_cast<uint2*>(Qs + off) = h;
+                *reinterpret_cast<uint2*>(Qs + C::Q_BYTES + off) = l;
+            }
+            fence_proxy_async_smem();
+            mbar_arrive(bar_q_full);
+        }
+#pragma unroll
+        for (int e = 0; e < OC; ++e) acc[e] = 0.f;
+        if (active) {
+            const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
+            const int lim = (rho < G && rho % R < rows) ? min(pos0 + rho % R, k_end - 1) : -1;      // last visible key
+            float al_o = 1.f;                                    // from acc's maximum to the one of the tile that is added next
+            auto add_o = [&](int t) {                            // O = O * al_o + the product of tile t
+                wait(bar_o_full + 8u * (t & 1), (uint32_t)(t >> 1) & 1u);
+                tc_fence_after();
+#pragma unroll
+                for (int c = 0; c < OC; c += 32) {
+                    uint32_t r[32];
+                    tmem_ld32(lane_base + C::O_COL + (uint32_t)((t & 1) * HD + half * OC + c), r);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) acc[c + e] = fmaf(acc[c + e], al_o, __uint_as_float(r[e]));
+                }
+                tc_fence_before();
+                mbar_arrive(bar_o_empty + 8u * (t & 1));
+            };
+            constexpr int SC = C::SC;
+            for (int t = 0; t < n_tiles; ++t) {
+                float s[SC];
+                wait(bar_s_full + 8u * (t & 1), (uint32_t)(t >> 1) & 1u);
+                tc_fence_after();
+#pragma unroll
+                for (int c = 0; c < SC; c += 32) {
+                    uint32_t r[32];
+                    tmem_ld32(lane_base + C::S_COL + (uint32_t)((t & 1) * TK + half * SC + c), r);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) s[c + e] = __uint_as_float(r[e]);
+                }
+                tc_fence_before();
+                mbar_arrive(bar_s_empty + 8u * (t & 1));
+                const int k0 = k_begin + t * TK + half * SC;
+                if (k0 + SC - 1 > lim) {
+#pragma unroll
+                    for (int e = 0; e < SC; ++e) if (k0 + e > lim) s[e] = -INFINITY;
+                }
+                float m4[4] = {s[0], s[1], s[2], s[3]};          // (four chains: a warp has its scheduler nearly to itself)
+#pragma unroll
+                for (int e = 4; e < SC; ++e) m4[e & 3] = fmaxf(m4[e & 3], s[e]);
+                const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+                s_max[t & 1][half][rho] = mx;
+                asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory");      // the quarter's two warps
+                const float mn = fmaxf(m_run, fmaxf(mx, s_max[t & 1][half ^ 1][rho])), mu = mn == -INFINITY ? 0.f : mn;
+                const float al = ex2(m_run - mu);                // 0 while nothing was visible
+                m_run = mn;
+                float p4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int e = 0; e < SC; ++e) { s[e] = ex2(s[e] - mu); p4[e & 3] += s[e]; }
+                l_run = l_run * al + ((p4[0] + p4[1]) + (p4[2] + p4[3]));
+                if (t > 0) add_o(t - 1);                         // (P of tile t - 1 has been used: its place is free)
+                al_o = al;
+                // P, half row: 16-byte chunks of eight keys
+#pragma unroll
+                for (int c = 0; c < SC / 8; ++c) {
+                    uint4 h, l;
+                    pack_hilo(s[8 * c], s[8 * c + 1], h.x, l.x);
+                    pack_hilo(s[8 * c + 2], s[8 * c + 3], h.y, l.y);
+                    pack_hilo(s[8 * c + 4], s[8 * c + 5], h.z, l.z);
+                    pack_hilo(s[8 * c + 6], s[8 * c + 7], h.w, l.w);
+                    const int kc = half * (SC / 8) + c;          // chunk of the row
+                    const uint32_t off = (uint32_t)((kc >> 3) * (RP * 128) + rho * 128 + (((kc & 7) ^ (rho & 7)) << 4));
+                    *reinterpret_cast<uint4*>(Ps + off) = h;
+                    *reinterpret_cast<uint4*>(Ps + C::P_BYTES + off) = l;
+                }
+                fence_proxy_async_smem();
+                mbar_arrive(bar_p_full);
+            }
+            if (n_tiles > 0) add_o(n_tiles - 1);
+            s_sum[half][rho] = l_run;
+            asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory");
+            l_run += s_sum[half ^ 1][rho];
+        }
+    }
+    // no copy and no MMA is under way any more (after a failure: give the copies a bounded time to land)
+    tc_fence_before();
+    __syncthreads();
+    if (s_fail && tid == 0) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000ll) { }
+    }
+    __syncthreads();
+    if (warp == SM_WARPS + 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, (uint32_t)C::COLS);
+    }
+    const int col0 = half * OC;
+    if (a.splits == 1) {
+        if (active && rho < G) {
+            const float inv = l_run > 0.f && rho % R < rows ? 1.0f / l_run : 0.f;
+            const size_t row = out_row(rho), col = (size_t)(h0 + rho / R) * HD + col0;
+#pragma unroll
+            for (int e = 0; e < OC; e += 8) {
+                uint4 h, l;
+                pack_hilo(acc[e] * inv, acc[e + 1] * inv, h.x, l.x);
+                pack_hilo(acc[e + 2] * inv, acc[e + 3] * inv, h.y, l.y);
+                pack_hilo(acc[e + 4] * inv, acc[e + 5] * inv, h.z, l.z);
+                pack_hilo(acc[e + 6] * inv, acc[e + 7] * inv, h.w, l.w);
+                *reinterpret_cast<uint4*>(a.out + row * qd + col + e) = h;
+                *reinterpret_cast<uint4*>(a.out + (row + a.TB) * qd + col + e) = l;
+            }
+        }
+        return;
+    }
+    // Every CTA of the cluster parks its unnormalised rows in its shared memory; CTA r merges the rows r, r + S, ...
+    constexpr int XS = HD + 4;                                   // floats per parked row: O, maximum, sum, padding
+    float* xo = reinterpret_cast<float*>(ring);
+    if (active && rho < G) {
+#pragma unroll
+        for (int e = 0; e < OC; e += 4) *reinterpret_cast<float4*>(xo + (size_t)rho * XS + col0 + e) = make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
+        if (half == 0) *reinterpret_cast<float2*>(xo + (size_t)rho * XS + HD) = make_float2(m_run, l_run);
+    }
+    cluster_arrive();
+    cluster_wait();
+    const int S = a.splits, rank = (int)cluster_ctarank();
+    uint32_t peer[8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s) peer[s] = cluster_map(smem_u32(xo), (uint32_t)(s < S ? s : 0));
+    const int my_rows = rank < G ? (G - rank + S - 1) / S : 0;
+    for (int i = tid; i < my_rows * (HD / 4); i += THREADS) {
+        const int r = rank + (i / (HD / 4)) * S, d4 = (i % (HD / 4)) * 4;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r % R < rows) {
+            float2 ml[8];
+            float4 ov[8];
+#pragma unroll
+            for (int s = 0; s < 8; ++s)
+                if (s < S) {                                     // all remote reads are issued before the first is used
+                    ml[s] = ld_cluster_f2(peer[s] + (uint32_t)(r * XS + HD) * 4u);
+                    ov[s] = ld_cluster_f4(peer[s] + (uint32_t)(r * XS + d4) * 4u);
+                }
+            float top = -INFINITY, den = 0.f;
+#pragma unroll
+            for (int s = 0; s < 8; ++s) if (s < S) top = fmaxf(top, ml[s].x);
+#pragma unroll
+            for (int s = 0; s < 8; ++s)
+                if (s < S && ml[s].x != -INFINITY) {             // (a split without visible keys)
+                    const float w = exp2f(ml[s].x - top);
+                    den += w * ml[s].y;
+                    o.x += w * ov[s].x; o.y += w * ov[s].y; o.z += w * ov[s].z; o.w += w * ov[s].w;
+                }
+            const float inv = den > 0.f ? 1.0f / den : 0.f;
+            o.x *= inv; o.y *= inv; o.z *= inv; o.w *= inv;
+        }
+        const size_t row = out_row(r), col = (size_t)(h0 + r / R) * HD + d4;
+        uint2 h, l;
+        pack_hilo(o.x, o.y, h.x, l.x);
+        pack_hilo(o.z, o.w, h.y, l.y);
+        *reinterpret_cast<uint2*>(a.out + row * qd + col) = h;
+        *reinterpret_cast<uint2*>(a.out + (row + a.TB) * qd + col) = l;
+    }
+    cluster_arrive();                                            // peers may still be reading this CTA's rows
+    cluster_wait();
+}
+
+template <int HD, int RP>
+bool prepare() {
+    static std::mutex mu;
+    static int known[64] = {0};                                  // 1 yes, 2 no
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { (void)cudaGetLastError(); return false; }
+    std::lock_guard<std::mutex> lk(mu);
+    if (!known[dev]) {
+        known[dev] = cudaFuncSetAttribute(attn_tc_kernel<HD, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM) == cudaSuccess ? 1 : 2;
+        if (known[dev] == 2) (void)cudaGetLastError();
+    }
+    return known[dev] == 1;
+}
+
+template <int HD, int RP>
+void config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[2], int splits, int n_kv, int B, int stages) {
+    cfg.gridDim = dim3((unsigned)splits, (unsigned)n_kv, (unsigned)B);
+    cfg.blockDim = dim3(THREADS, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)Tc<HD, RP>::smem(stages);
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)splits;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = splits > 1 ? 2 : 1;                           // the key-range splits of one (sequence, KV head) form a cluster
+}
+
+template <int HD, int RP>
+tasc_status launch_inst(const TcArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int B, cudaStream_t stream) {
+    if (!prepare<HD, RP>()) return TASC_ECUDA;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2];
+    config<HD, RP>(cfg, at, a.splits, a.n_kv, B, a.stages);
+    cfg.stream = stream;
+    ProfScope ps(K_ATT_SPLIT, stream);
+    TASC_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD, RP>, tmK, tmV, a));
+    return TASC_OK;
+}
+
+template <int HD, int RP> int ring_stages();
+// Clusters of `splits` CTAs that the device holds at once (0: it cannot be asked).
+template <int HD, int RP>
+int clusters(int splits) {
+    static std::mutex mu;
+    static int known[64][9] = {{0}};                             // + 1
+    int dev = 0;
+    if (!prepare<HD, RP>() || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { (void)cudaGetLastError(); return 0; }
+    std::lock_guard<std::mutex> lk(mu);
+    if (!known[dev][splits]) {
+        int n = 0;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[2];
+        config<HD, RP>(cfg, at, splits, 1, 1, ring_stages<HD, RP>());
+        cfg.attrs = at + 1;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<HD, RP>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
+        known[dev][splits] = n + 1;
+    }
+    return known[dev][splits] - 1;
+}
+template <int HD, int RP> int ring_stages() {
+    int s = MAX_RING;
+    while (s > 2 && Tc<HD, RP>::smem(s) > MAX_SMEM) --s;
+    return s;
+}
+
+}  // namespace
+
+// Splits by a cost in microseconds like plan_attention_mma's: T0 to start, `per_tile` for a tile of TK keys (taken for three
+// quarters of the context and for all of it, half each: the tiles are large), as many waves as the occupancy of the launch
+// dictates (one CTA per SM), the merge of split ranges.  The other kernel's cost is p.cost, and no less than what all its slabs
+// take of the SMs' mma.sync pipes.  Measured, steps and prefills of the 135M, 0.5B and 1.5B shapes: it pays from about 64
+// (sequence, KV head) pairs on, from 8 on with long contexts and four or more slabs of query rows, hardly ever at the 135M's
+// 18 to 27 rows.
+bool plan_attention_tc(int B, int n_kv, int hd, int g, int rows, int max_ctx, int page_size, AttnPlan& p) {
+    const int G = g * rows;
+    if ((hd != 64 && hd != 128) || page_size != PAGE || G > 128 || max_ctx / PAGE > MAX_PAGES) return false;
+    const bool small = G <= 64;
+    const int tk = small ? 128 : 64;
+    const float T0 = 2.4f, per_tile = hd == 128 ? (small ? 1.8f : 1.4f) : (small ? 1.4f : 1.1f);
+    const int groups = B * n_kv, tiles_all = std::max(1, (max_ctx + tk - 1) / tk), tiles_34 = std::max(1, (max_ctx * 3 / 4 + tk - 1) / tk);
+    const float pipes = (hd == 128 ? 0.6f : 0.3f) * (float)groups * (float)((G + 15) / 16) * (float)((max_ctx * 3 / 4 + 63) / 64) / 148.f;
+    int best = 0;
+    float best_cost = std::max(p.cost, 2.5f + pipes);
+    for (int s = 1; s <= 8 && s <= tiles_all; ++s) {
+        const int fit = hd == 64 ? (small ? clusters<64, 64>(s) : clusters<64, 128>(s)) : (small ? clusters<128, 64>(s) : clusters<128, 128>(s));
+        if (fit <= 0) continue;
+        const int waves = (groups + fit - 1) / fit;
+        const float tiles = 0.5f * (float)((tiles_all + s - 1) / s + (tiles_34 + s - 1) / s);
+        const float cost = waves * (T0 + tiles * per_tile) + (s > 1 ? 0.5f + 0.25f * s : 0.f) + (groups * s > 128 ? 3.0f : 0.f);
+        if (cost < best_cost - 1e-6f) { best_cost = cost; best = s; }
+    }
+    if (!best) return false;
+    p.tc = 1;
+    p.heads = g;
+    p.splits = best;
+    p.stages = hd == 64 ? (small ? ring_stages<64, 64>() : ring_stages<64, 128>()) : (small ? ring_stages<128, 64>() : ring_stages<128, 128>());
+    return true;
+}
+
+tasc_status launch_attention_tc(const float* qbuf, const CUtensorMap& tmK, const CUtensorMap& tmV, const int32_t* block_table, int max_pages,
+                                long long n_pages, const RowPlan& rp, __nv_bfloat16* out, int TB, int B, int R, int n_q, int n_kv, int hd,
+                                const AttnPlan& plan, int* status, cudaStream_t stream) {
+    const int Rs = R <= 16 ? R : 16;
+    if (R % Rs) return TASC_EINVAL;
+    const int G = (n_q / n_kv) * Rs;
+    if (G > 128 || (hd != 64 && hd != 128) || plan.splits < 1 || plan.splits > 8) return TASC_EINVAL;
+    TcArgs a;
+    a.q = qbuf; a.block_table = block_table; a.max_pages = max_pages; a.n_pages = n_pages;
+    a.seq_pos0 = rp.seq_pos0; a.seq_rows = rp.seq_rows;
+    a.out = out; a.TB = TB;
+    a.R = R; a.Rs = Rs; a.n_sub = R / Rs; a.n_q = n_q; a.n_kv = n_kv; a.splits = plan.splits; a.stages = plan.stages;
+    a.scale_log2e = 1.4426950408889634f / sqrtf((float)hd);
+    a.status = status;
+    const int blocks = B * a.n_sub;
+    if (hd == 64) return G <= 64 ? launch_inst<64, 64>(a, tmK, tmV, blocks, stream) : launch_inst<64, 128>(a, tmK, tmV, blocks, stream);
+    return G <= 64 ? launch_inst<128, 64>(a, tmK, tmV, blocks, stream) : launch_inst<128, 128>(a, tmK, tmV, blocks, stream);
+}
+
+}  // namespace tasc

@@ -308,6 +308,8 @@ struct AttnPlan {
     int splits;      // key-range splits per (sequence, head group) = cluster size, 1..8
     int stages;      // depth of the K/V tile ring
     int heads;       // query heads per CTA: a divisor of n_q / n_kv (the heads sharing a KV head are dealt out to several CTAs)
+    int tc;          // 1: attention_tc.cu
+    float cost;      // what the planner expects, us
 };
 // Same contract as launch_attention; the result goes to `out` as (hi, lo) bf16 rows; needs no scratch memory.
 tasc_status launch_attention_mma(const float* qbuf, const __nv_bfloat16* k_pages, const __nv_bfloat16* v_pages,
@@ -316,5 +318,10 @@ tasc_status launch_attention_mma(const float* qbuf, const __nv_bfloat16* k_pages
                                  const AttnPlan& plan, int* status, cudaStream_t stream);
 // B sequences (or sequence blocks), g = n_q / n_kv query heads per KV head, `rows` query rows per sequence block
 AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ctx);
+// The same on tcgen05 (attention_tc.cu): replaces the plan `p` where it applies and costs less.  launch_attention_mma takes either.
+bool plan_attention_tc(int B, int n_kv, int hd, int g, int rows, int max_ctx, int page_size, AttnPlan& p);
+tasc_status launch_attention_tc(const float* qbuf, const CUtensorMap& tmK, const CUtensorMap& tmV, const int32_t* block_table, int max_pages,
+                                long long n_pages, const RowPlan& rp, __nv_bfloat16* out, int TB, int B, int R, int n_q, int n_kv, int hd,
+                                const AttnPlan& plan, int* status, cudaStream_t stream);
 
 }  // namespace tasc

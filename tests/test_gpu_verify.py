@@ -340,6 +340,18 @@ def test_config4_geometry_between_one_and_two_full_token_tiles(B):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("which,B,k,P", [(4, 64, 8, 128), (4, 36, 6, 257), (4, 6, 6, 700), (2, 33, 8, 127), (2, 64, 3, 65), (2, 4, 7, 900)])
+def test_tcgen05_attention(which, B, k, P):
+    """Heads of 128 and 64, query tiles of up to 64 rows in the steps and of 96 and 112 in the prefill, key ranges whole and
+    split over two to eight CTAs, contexts that end below, at and over tiles of 64 and 128 keys.  One layer."""
+    from dataclasses import replace
+    cfg = replace(configs.shrunk(configs.get(which), n_layers=1, vocab=4096, n_docs=500), prompt_len=P)
+    s = make_setup(cfg)
+    prompts = corpus.make_prompts(cfg, B, prompt_len=P)
+    check(lockstep(s, prompts, k + 3, k, oracle_rows=sorted({0, B // 2, B - 1}), **BF16_TOL), f"tcgen05 attention, config {which}, B={B} k={k} P={P}")
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("B,P", [(37, 9), (55, 40), (75, 129)])
 def test_many_row_kernel_on_pairs_of_token_tiles(B, P):
     """Configuration 4's geometry (one layer, an 8,200-token vocabulary: a feature tile of eight) at 259, 385 and 525 rows of
