@@ -586,7 +586,14 @@ count_summary_kernel(const uint32_t* __restrict__ bins, const BinSum* __restrict
 }
 
 // ------------------------------------------------------------------------------------------- draft
+// Bound: k times a chain of look-ups (slots and their values in one trip, then the successors), about 0.4 us a trip; what
+// happens between the trips is kept short.  The suffix is matched against the context once per draft, every thread keeping the
+// lengths of its positions; the few tokens that follow the longest matches are a list that is compared with directly.  Only
+// lists beyond LIST_MAX are counted in the hash table, whose clearing and reading cost more than everything else (k = 6 behind
+// 1,530 tokens: 33 us with it, 23 without; k = 8 behind 640: 33, 25; k = 5 behind 380: 18, 15.5; k = 4 behind 64: 9.6, 8.7).
 constexpr int DRAFT_THREADS = 256;
+constexpr int LIST_MAX = 64;
+constexpr int POS_PER = 8;                       // positions whose match lengths a thread keeps; those of longer contexts are worked out again
 
 struct Best { unsigned long long score; uint32_t id; };
 __device__ __forceinline__ bool better(unsigned long long s, uint32_t id, const Best& b) {
@@ -605,8 +612,7 @@ __device__ __forceinline__ Best block_best(Best v, Best* red) {
     Best r = red[0];
     for (int i = 1; i < DRAFT_THREADS / 32; ++i)
         if (better(red[i].score, red[i].id, r)) r = red[i];
-    __syncthreads();
-    return r;
+    return r;                                    // (the caller's next barrier comes before red is written again)
 }
 
 // Warp-cooperative lookup of a packed context: each round the 32 lanes test 32 consecutive slots.
@@ -617,13 +623,14 @@ __device__ __forceinline__ bool warp_lookup(const OrderTable& t, Key key, CtxVal
     for (uint64_t round = 0; round * 32 <= t.mask; ++round) {
         const uint64_t slot = (h + round * 32 + lane) & t.mask;
         const ulonglong2 kv = *reinterpret_cast<const ulonglong2*>(t.keys + 2 * slot);
+        const uint4 v = *reinterpret_cast<const uint4*>(t.vals + slot);      // (the value of the slot that will match is among them)
         const uint32_t hit = __ballot_sync(0xFFFFFFFFu, kv.x == key.lo && kv.y == key.hi);
         const uint32_t hole = __ballot_sync(0xFFFFFFFFu, kv.x == 0 && kv.y == 0);
         if (hit) {
             const int src = __ffs(hit) - 1;
-            // all lanes read the value of the matching slot
-            const uint64_t s = (h + round * 32 + src) & t.mask;
-            out = t.vals[s];
+            out.offset = (unsigned long long)__shfl_sync(0xFFFFFFFFu, v.x, src) | ((unsigned long long)__shfl_sync(0xFFFFFFFFu, v.y, src) << 32);
+            out.n_succ = __shfl_sync(0xFFFFFFFFu, v.z, src);
+            out.total = __shfl_sync(0xFFFFFFFFu, v.w, src);
             // a hole before the hit cannot exist: insertion stops at the first free slot
             return true;
         }
@@ -638,12 +645,13 @@ draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t 
     extern __shared__ int32_t dsm[];
     int32_t* h_tok = dsm;                                          // [hs] token or -1
     uint32_t* h_cnt = reinterpret_cast<uint32_t*>(dsm + hs_mask + 1);   // [hs] count, bit 31 = seen in the corpus list
-    int32_t* s_seq = dsm + 2 * (hs_mask + 1);                      // [L] the committed tokens: every draft scans them twice
+    int32_t* s_seq = dsm + 2 * (hs_mask + 1);                      // [L] the committed tokens
     __shared__ Best red[DRAFT_THREADS / 32];
     __shared__ int s_suffix[TASC_MAX_ORDER];     // last n_max tokens of the query, newest last
-    __shared__ int s_nstar, s_tprompt;
+    __shared__ int s_best[DRAFT_THREADS / 32], s_tprompt;
     __shared__ int s_hit[TASC_MAX_ORDER];        // order n = index + 1 has a surviving context for the current suffix
     __shared__ CtxVal s_vals[TASC_MAX_ORDER];
+    __shared__ int s_list[LIST_MAX], s_seen[LIST_MAX];
 
     const int b = blockIdx.x;
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -659,6 +667,7 @@ draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t 
         const int p = L - n_max + tid;             // suffix slot tid <-> position p (only the last n_max slots are used)
         s_suffix[tid] = (tid < n_max && p >= 0) ? seq[p] : -1;
     }
+    if (tid == 0) s_tprompt = 0;
     __syncthreads();
 
     for (int j = 0; j < k; ++j) {
@@ -666,7 +675,6 @@ draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t 
         const int n_avail = Lq < n_max ? Lq : n_max;
         // ---------------------------------------------------------------- p_corp: all orders are probed at once, one warp
         // per order (warp w looks up the last w + 1 tokens); the longest order that matched wins the back-off
-        if (tid == 0) { s_nstar = 0; s_tprompt = 0; }
         if (warp < TASC_MAX_ORDER) {
             const int n = warp + 1;
             bool hit = false;
@@ -679,9 +687,8 @@ draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t 
             if ((tid & 31) == 0) { s_hit[warp] = hit ? 1 : 0; s_vals[warp] = val; }
         }
         // ---------------------------------------------------------------- p_prompt: longest suffix match in the committed tokens
-        if (use_prompt)
-            for (int i = tid; i <= hs_mask; i += DRAFT_THREADS) { h_tok[i] = -1; h_cnt[i] = 0u; }
-        __syncthreads();
+        int t_prompt_ = 0;
+        bool listed = true;                        // the successors' list holds them all
         if (use_prompt) {
             auto match_len = [&](int p) {          // tokens before successor position p that agree with the query suffix
                 int m = 0;
@@ -690,14 +697,37 @@ draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t 
                 return m;
             };
             int best = 0;
-            for (int p = 1 + tid; p < L; p += DRAFT_THREADS) best = max(best, match_len(p));
+            uint32_t kept = 0u;                    // 4 bits per position: lengths are at most TASC_MAX_ORDER
+            int i = 0;
+            for (int p = 1 + tid; p < L; p += DRAFT_THREADS, ++i) {
+                const int m = match_len(p);
+                best = max(best, m);
+                if (i < POS_PER) kept |= (uint32_t)m << (4 * i);
+            }
             best = __reduce_max_sync(0xFFFFFFFFu, best);
-            if ((tid & 31) == 0 && best > 0) atomicMax(&s_nstar, best);
+            if ((tid & 31) == 0) s_best[warp] = best;
             __syncthreads();
-            const int nstar = s_nstar;
+            int nstar = 0;
+#pragma unroll
+            for (int w = 0; w < DRAFT_THREADS / 32; ++w) nstar = max(nstar, s_best[w]);
+            auto matches = [&](int at, int p) { return (at < POS_PER ? (int)((kept >> (4 * at)) & 15u) : match_len(p)) == nstar; };
             if (nstar > 0) {
-                for (int p = 1 + tid; p < L; p += DRAFT_THREADS) {
-                    if (match_len(p) != nstar) continue;
+                i = 0;
+                for (int p = 1 + tid; p < L; p += DRAFT_THREADS, ++i) {
+                    if (!matches(i, p)) continue;
+                    const int at = atomicAdd(&s_tprompt, 1);
+                    if (at < LIST_MAX) { s_list[at] = seq[p]; s_seen[at] = 0; }
+                }
+            }
+            __syncthreads();
+            t_prompt_ = s_tprompt;
+            listed = t_prompt_ <= LIST_MAX;
+            if (!listed) {
+                for (int q = tid; q <= hs_mask; q += DRAFT_THREADS) { h_tok[q] = -1; h_cnt[q] = 0u; }
+                __syncthreads();
+                i = 0;
+                for (int p = 1 + tid; p < L; p += DRAFT_THREADS, ++i) {
+                    if (!matches(i, p)) continue;
                     const int x = seq[p];
                     uint32_t slot = ((uint32_t)x * 2654435761u) & hs_mask;
                     for (int probe = 0; probe <= hs_mask; ++probe) {
@@ -705,9 +735,10 @@ draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t 
                         if (old == -1 || old == x) { atomicAdd(&h_cnt[slot], 1u); break; }
                         slot = (slot + 1) & hs_mask;
                     }
-                    atomicAdd(&s_tprompt, 1);
                 }
+                __syncthreads();
             }
+        } else {
             __syncthreads();
         }
         int found_n = 0;
@@ -715,11 +746,14 @@ draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t 
             if (s_hit[n - 1]) found_n = n;
         const CtxVal cv = s_vals[found_n > 0 ? found_n - 1 : 0];
         const unsigned long long t_corp = cv.total;
-        const unsigned long long t_prompt = (unsigned long long)s_tprompt;
+        const unsigned long long t_prompt = (unsigned long long)t_prompt_;
         const bool has_corp = found_n > 0, has_prompt = t_prompt > 0;
         // ---------------------------------------------------------------- mixture argmax
         Best mine = {0ull, 0xFFFFFFFFu};
         bool any = false;
+        auto offer = [&](unsigned long long score, uint32_t id) {
+            if (!any || better(score, id, mine)) { mine.score = score; mine.id = id; any = true; }
+        };
         if (has_corp) {
             const Succ* sl = dt.t[found_n].succ + cv.offset;
             const unsigned long long w_c = has_prompt ? (unsigned long long)lam_num * t_prompt : 1ull;
@@ -727,7 +761,12 @@ draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t 
             for (uint32_t i = tid; i < cv.n_succ; i += DRAFT_THREADS) {
                 const Succ s = sl[i];
                 unsigned long long score = w_c * s.count;
-                if (has_prompt) {
+                if (has_prompt && listed) {
+                    uint32_t c = 0;
+                    for (int e = 0; e < t_prompt_; ++e)
+                        if (s_list[e] == s.next) { ++c; s_seen[e] = 1; }
+                    score += w_p * c;
+                } else if (has_prompt) {
                     uint32_t slot = ((uint32_t)s.next * 2654435761u) & hs_mask;
                     for (int probe = 0; probe <= hs_mask; ++probe) {
                         const int tk = h_tok[slot];
@@ -740,18 +779,26 @@ draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t 
                         slot = (slot + 1) & hs_mask;
                     }
                 }
-                if (!any || better(score, (uint32_t)s.next, mine)) { mine.score = score; mine.id = (uint32_t)s.next; any = true; }
+                offer(score, (uint32_t)s.next);
             }
+            __syncthreads();     // the corpus pass has marked the shared successors
         }
-        __syncthreads();     // corpus pass has marked the shared successors
         if (has_prompt) {
             const unsigned long long w_p = has_corp ? (unsigned long long)(lam_den - lam_num) * t_corp : 1ull;
-            for (int i = tid; i <= hs_mask; i += DRAFT_THREADS) {
-                const int tk = h_tok[i];
-                const uint32_t c = h_cnt[i];
-                if (tk < 0 || (c & 0x80000000u)) continue;      // empty, or already scored with its corpus count
-                const unsigned long long score = w_p * c;
-                if (!any || better(score, (uint32_t)tk, mine)) { mine.score = score; mine.id = (uint32_t)tk; any = true; }
+            if (listed) {
+                if (tid < t_prompt_ && !s_seen[tid]) {
+                    const int tk = s_list[tid];
+                    uint32_t c = 0;
+                    for (int e = 0; e < t_prompt_; ++e) c += s_list[e] == tk;
+                    offer(w_p * c, (uint32_t)tk);
+                }
+            } else {
+                for (int i = tid; i <= hs_mask; i += DRAFT_THREADS) {
+                    const int tk = h_tok[i];
+                    const uint32_t c = h_cnt[i];
+                    if (tk < 0 || (c & 0x80000000u)) continue;      // empty, or already scored with its corpus count
+                    offer(w_p * c, (uint32_t)tk);
+                }
             }
         }
         if (!any) { mine.score = 0ull; mine.id = 0xFFFFFFFFu; }
@@ -761,6 +808,7 @@ draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t 
             drafts[(int64_t)b * k + j] = draft;
             for (int i = 0; i + 1 < n_max; ++i) s_suffix[i] = s_suffix[i + 1];
             s_suffix[n_max - 1] = draft;
+            s_tprompt = 0;
         }
         __syncthreads();
     }
