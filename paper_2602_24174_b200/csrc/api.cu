@@ -83,16 +83,19 @@ constexpr int COUNTER_BAR = 0, COUNTER_GROUPS = 64, COUNTER_WORDS = COUNTER_GROU
 // Rows a pass may carry: TASC_MAX_ROWS per sequence for a verify step, and for bf16 models at least PREFILL_ROWS
 // in all, so that a prefill of few sequences still runs passes of hundreds of rows (weights are read once per pass).
 constexpr int PREFILL_ROWS = 2048;
-constexpr int PREFILL_ROWS_PER_SEQ = 256;
 size_t workspace_rows(const tasc_model* m, int B) {
     const size_t verify = (size_t)B * TASC_MAX_ROWS;
     return m->desc.dtype == TASC_F32 ? verify : std::max<size_t>(verify, PREFILL_ROWS);
 }
-// Rows per sequence of one prefill pass: a multiple of 16 that fits the workspace.
-int prefill_rows(const tasc_model* m, int B) {
+// Rows per sequence of a prefill pass for prompts of up to max_len tokens (all but the last are prefilled): as few passes as
+// the workspace allows, of equal length, in multiples of 16.  (Passes of 256 rows per sequence whatever the prompt: one of
+// 1,000 tokens read the 1.5B's weights four times, 10.8 ms against 6.3; four of 300 tokens ran 2,048 rows for 1,200, 11.9 ms
+// against 6.3.)
+int prefill_rows(const tasc_model* m, int B, int max_len) {
     if (m->desc.dtype == TASC_F32) return TASC_MAX_ROWS;
-    const int per = (int)(workspace_rows(m, B) / (size_t)B) / 16 * 16;
-    return std::max(TASC_MAX_ROWS, std::min(per, PREFILL_ROWS_PER_SEQ));
+    const int most = std::max(TASC_MAX_ROWS, (int)(workspace_rows(m, B) / (size_t)B) / 16 * 16);
+    const int n = std::max(max_len - 1, 1), passes = (n + most - 1) / most;
+    return std::min(most, ((n + passes - 1) / passes + 15) / 16 * 16);
 }
 
 // The layout is always made for workspace_rows() rows so that every call agrees on it.
@@ -406,7 +409,7 @@ tasc_status verify_enqueue(const tasc_model* m, const tasc_kv* kv, const tasc_se
 
 tasc_status prefill_enqueue(const tasc_model* m, const tasc_kv* kv, const tasc_seqs* seqs, const Workspace& w, int B,
                             int max_len, cudaStream_t s) {
-    const int R = prefill_rows(m, B);
+    const int R = prefill_rows(m, B, max_len);
     const int chunks = (std::max(max_len - 1, 0) + R - 1) / R;
     for (int c = 0; c < chunks; ++c) {
         tasc_status st = forward_any(m, kv, w, RowSource{seqs, nullptr, c}, B, R, false, nullptr, s);
