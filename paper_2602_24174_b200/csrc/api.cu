@@ -318,6 +318,10 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
     base.inv_d = 1.0f / (float)d.d_model;
     base.eps = d.rms_eps;
     base.status = w.status;
+    base.R = R;
+    // token tiles without rows: not with one prompt, and in a first pass only where a prompt's rows are tiles of their own
+    base.seq_rows = B > 1 && (src.chunk > 0 || (src.chunk == 0 && R >= 2 * TB)) ? w.rp.seq_rows : nullptr;
+    base.rows_early = 1;               // written by the first kernel of the pass
 
     launch_rows_embed(w.rp, src.seqs->tokens, src.seqs->stride, src.seqs->len, src.seqs->stop_len, src.drafts, B, R, src.chunk,
                       d.vocab, w.status, static_cast<const __nv_bfloat16*>(m->embed), m->attn_norm[0], w.x, h,
@@ -347,7 +351,7 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
         a.k_pages = static_cast<__nv_bfloat16*>(kvl.k); a.v_pages = static_cast<__nv_bfloat16*>(kvl.v);
         a.block_table = kv->block_table; a.max_pages = kv->max_pages_per_seq; a.page_size = d.page_size; a.n_pages = kv->n_pages;
         a.R = R; a.n_q = d.n_q_heads; a.n_kv = d.n_kv_heads; a.hd = d.head_dim; a.max_positions = d.max_positions;
-        a.early = l > 0;               // layer 0 follows the kernel that writes the row plan
+        a.early = a.rows_early = l > 0;          // layer 0 follows the kernel that writes the row plan
         if ((st = launch_gemm_fused(EPI_QKV, &m->tm_qkv[l], &tm_h, a, p_qkv, s)) != TASC_OK) return st;
 
         st = launch_attention_mma(w.q, static_cast<const __nv_bfloat16*>(kvl.k), static_cast<const __nv_bfloat16*>(kvl.v),

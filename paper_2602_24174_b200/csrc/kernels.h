@@ -96,6 +96,9 @@ struct FusedArgs {
     int num_kb, BN, TB, TBL, stages, pair, data_bytes; // filled in by launch_gemm_fused from the plan
     int BNW, n_ft, n_tt;               // many-row kernel (gemm_wide.cu): features per MMA, feature tiles, token tiles
     int early;                         // the epilogue's global operands were complete before the preceding grid began
+    const int* seq_rows;               // prefill passes: rows in use of every sequence (R rows each); the many-row kernel skips token
+                                       // tiles without any (the few-row kernel would wait longer for the counts than it gains)
+    int rows_early;                    // ... which were complete before the preceding grid began
     const double* ssq64;               // [M] sums of squares of the input rows (instead of ssq_in, behind the one-kernel layers)
     const float* ssq_in;               // [M][ssq_slots] partial sums of squares of the input rows (null: no scaling)
     int ssq_slots;
@@ -129,6 +132,12 @@ struct FusedPlan {
     int cta_pair;      // ... which work in pairs (cta_group::2) on two token tiles
     int threads;       // few-row kernel: 192, or 384 (six more warps that only finish columns) where a CTA finishes many token columns
 };
+// Whether any of the token rows m0 .. m1 - 1 is in use.
+__device__ __forceinline__ bool rows_in_use(const int* seq_rows, int R, int m0, int m1) {
+    for (int b = m0 / R; b * R < m1; ++b)
+        if (max(m0 - b * R, 0) < seq_rows[b]) return true;
+    return false;
+}
 // hd: head_dim, for EPI_QKV.  wide_min_mb: < 0 for a pass whose products all take the few-row kernel; otherwise the
 // pass lays its activations out for the many-row kernel (gemm_token_tile with many_rows) and a product takes that
 // kernel if its weight matrix has at least this many MB.

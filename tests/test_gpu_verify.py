@@ -352,6 +352,34 @@ def test_tcgen05_attention(which, B, k, P):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("lens", [[700, 2, 260, 513, 130, 131], [300, 1, 1, 33], [1100, 600]])
+def test_prefill_skips_token_tiles_without_rows(lens):
+    """Ragged prompts of configuration 4's geometry (one layer): passes in which whole token tiles, also every second one of
+    a pair, hold no row.  The verify step behind them must see the cache the oracle builds token by token."""
+    b = need_gpu()
+    cfg = configs.shrunk(configs.get(4), n_layers=1, vocab=4096, n_docs=500)
+    s = make_setup(cfg, build_drafter=False, oracle_ngrams=False)
+    B, k = len(lens), cfg.k
+    rng = np.random.default_rng(6)
+    stride = max(lens) + 4 * (k + 1)
+    host = rng.integers(0, cfg.model.vocab, (B, stride)).astype(np.int32)
+    drafts = rng.integers(0, cfg.model.vocab, (B, k)).astype(np.int32)
+    pool, bt, kv = s.model.new_kv(B, stride + b.MAX_ROWS)
+    ws = s.model.new_workspace(B, k)
+    tokens, length = torch.from_numpy(host).cuda(), torch.tensor(lens, dtype=torch.int32, device="cuda")
+    seqs = b.make_seqs(tokens, length)                       # (holds addresses only)
+    b.tasc_prefill(s.model, kv, seqs, B, max(lens), ws)
+    lg = b.tasc_verify_step(s.model, kv, seqs, torch.from_numpy(drafts).cuda(), ws, want_logits=True)[3].cpu().numpy()
+    b.tasc_poll_status(ws)
+    for i, L in enumerate(lens):
+        cache = s.oracle.new_cache(L + k + 1)
+        s.oracle.prefill(host[i, :L - 1], cache)
+        want = G.verify_step(s.oracle, cache, int(host[i, L - 1]), list(map(int, drafts[i])), keep_logits=True).logits
+        err = np.abs(lg[i] - want)
+        assert (err <= np.maximum(BF16_TOL["logit_atol"], BF16_TOL["logit_rtol"] * np.abs(want))).all(), (i, float(err.max()))
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("B,P", [(37, 9), (55, 40), (75, 129)])
 def test_many_row_kernel_on_pairs_of_token_tiles(B, P):
     """Configuration 4's geometry (one layer, an 8,200-token vocabulary: a feature tile of eight) at 259, 385 and 525 rows of
