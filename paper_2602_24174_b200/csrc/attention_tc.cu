@@ -232,7 +232,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         __syncwarp();
     } else if (warp == SM_WARPS + 1) {
         // ------------------------------------------------------------ MMA
-        if (lane == 0 && n_tiles > 0) {
+        // (the whole warp, see umma_bf16_warp)
+        if (n_tiles > 0) {
             const uint32_t qa = smem_u32(Qs), pa = smem_u32(Ps), kv = smem_u32(ring);
             constexpr uint32_t idesc_s = umma_idesc_bf16_f32(128, TK);
             constexpr uint32_t idesc_o = umma_idesc_bf16_f32(128, HD) | (1u << 16);      // V: columns along N
@@ -245,10 +246,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                 for (int p = 0; p < 2; ++p)                      // hi, lo
 #pragma unroll
                     for (int ks = 0; ks < HD / 16; ++ks)
-                        umma_bf16(d, umma_desc_k_sw128(qa + p * C::Q_BYTES + (ks >> 2) * (RP * 128) + (ks & 3) * 32),
+                        umma_bf16_warp(d, umma_desc_k_sw128(qa + p * C::Q_BYTES + (ks >> 2) * (RP * 128) + (ks & 3) * 32),
                                   umma_desc_k_sw128(kb + (ks >> 2) * (TK * 128) + (ks & 3) * 32), idesc_s, (p | ks) ? 1u : 0u);
-                umma_commit(bar_s_full + 8u * (t & 1));
-                umma_commit(bar_k_empty + 8u * (t % a.stages));
+                umma_commit_warp(bar_s_full + 8u * (t & 1));
+                umma_commit_warp(bar_k_empty + 8u * (t % a.stages));
             };
             wait(bar_q_full, 0u);
             tc_fence_after();
@@ -264,10 +265,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                 for (int p = 0; p < 2; ++p)
 #pragma unroll
                     for (int kk = 0; kk < TK / 16; ++kk)
-                        umma_bf16(d, umma_desc_k_sw128(pa + p * C::P_BYTES + (kk >> 2) * (RP * 128) + (kk & 3) * 32),
+                        umma_bf16_warp(d, umma_desc_k_sw128(pa + p * C::P_BYTES + (kk >> 2) * (RP * 128) + (kk & 3) * 32),
                                   umma_desc_mn_sw128(vb + kk * (16 * 128), TK * 128), idesc_o, (p | kk) ? 1u : 0u);
-                umma_commit(bar_o_full + 8u * (t & 1));          // also: P is free
-                umma_commit(bar_v_empty + 8u * (t % a.stages));
+                umma_commit_warp(bar_o_full + 8u * (t & 1));          // also: P is free
+                umma_commit_warp(bar_v_empty + 8u * (t % a.stages));
             }
         }
         __syncwarp();

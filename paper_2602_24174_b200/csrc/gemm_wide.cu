@@ -237,33 +237,37 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         __syncwarp();
     } else if (warp == EPI_WARPS + 1) {
         // ------------------------------------------------------------ MMA issue
-        if (lane == 0 && (!PAIR || rank == 0)) {
+        // (the whole warp, see umma_bf16_warp)
+        if (!PAIR || rank == 0) {
             const uint32_t idesc = umma_idesc_bf16_f32(PAIR ? 256 : 128, BNW);
-            auto mma = [&](uint32_t d, uint32_t sa, uint32_t sb, uint32_t acc) {
-                if (PAIR) umma_bf16_pair(d, umma_desc_k_sw128(sa), umma_desc_k_sw128(sb), idesc, acc);
-                else umma_bf16(d, umma_desc_k_sw128(sa), umma_desc_k_sw128(sb), idesc, acc);
+            const uint32_t ring = smem_u32(smem);
+            auto mma = [&](uint32_t d, uint64_t da, uint64_t db, uint32_t acc) {
+                if (PAIR) umma_bf16_pair_warp(d, da, db, idesc, acc);
+                else umma_bf16_warp(d, da, db, idesc, acc);
             };
-            auto commit = [&](uint32_t bar) { if (PAIR) umma_commit_pair(bar); else umma_commit(bar); };
-            int it = 0;
+            auto commit = [&](uint32_t bar) { if (PAIR) umma_commit_pair_warp(bar); else umma_commit_warp(bar); };
+            int s = 0;
+            uint32_t round = 0;
             bool ok = true;
             for (int j = 0; j < my_tiles && ok; ++j) {
                 const int b = j & 1;
-                if (!wait_or_fail<PAIR>(bar_acc_empty + 8u * b, (((uint32_t)(j >> 1)) & 1u) ^ 1u, failed)) { fail(); break; }
+                ok = __all_sync(0xFFFFFFFFu, wait_or_fail<PAIR>(bar_acc_empty + 8u * b, (((uint32_t)(j >> 1)) & 1u) ^ 1u, failed));
+                if (!ok) { fail(); break; }
                 tc_fence_after();
                 const uint32_t d = tmem_base + (uint32_t)(b * BNW);
-                for (int kb = 0; kb < nkb; ++kb, ++it) {
-                    const int s = it % stages;
-                    if (!wait_or_fail<PAIR>(bar_full + 8u * s, ((uint32_t)(it / stages)) & 1u, failed)) { fail(); ok = false; break; }
+                for (int kb = 0; kb < nkb; ++kb) {
+                    ok = __all_sync(0xFFFFFFFFu, wait_or_fail<PAIR>(bar_full + 8u * s, round & 1u, failed));
+                    if (!ok) { fail(); break; }
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes);
-                    const uint32_t sb = sa + a_bytes;
+                    const uint32_t sa = ring + (uint32_t)s * stage_bytes;
+                    const uint64_t hi = umma_desc_k_sw128(sa), lo = umma_desc_k_sw128(sa + (uint32_t)TBL * 128u), w = umma_desc_k_sw128(sa + a_bytes);
+                    constexpr int STEP = UMMA_K * 2 / 16;            // (addresses in units of 16 bytes)
 #pragma unroll
-                    for (int kk = 0; kk < BK / UMMA_K; ++kk)
-                        mma(d, sa + kk * UMMA_K * 2, sb + kk * UMMA_K * 2, (kb > 0 || kk > 0) ? 1u : 0u);
+                    for (int kk = 0; kk < BK / UMMA_K; ++kk) mma(d, hi + kk * STEP, w + kk * STEP, (kb > 0 || kk > 0) ? 1u : 0u);
 #pragma unroll
-                    for (int kk = 0; kk < BK / UMMA_K; ++kk)
-                        mma(d, sa + (uint32_t)TBL * 128u + kk * UMMA_K * 2, sb + kk * UMMA_K * 2, 1u);
+                    for (int kk = 0; kk < BK / UMMA_K; ++kk) mma(d, lo + kk * STEP, w + kk * STEP, 1u);
                     commit(bar_empty + 8u * s);
+                    if (++s == stages) { s = 0; ++round; }
                 }
                 if (ok) commit(bar_acc_full + 8u * b);
             }
