@@ -35,7 +35,7 @@ struct tasc_model {
     std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
     CUtensorMap tm_lm;
     int qkv_rows, q_dim, kv_dim;
-    int few_tiles;                                  // token tiles for 49..128 rows (see gemm_token_tile), from the layer's weight bytes
+    int few_tiles;                                  // 1, 2 or 3 from the layer's weight bytes (see gemm_token_tile)
     double layer_mb;                                // projection weights of one layer, MB (two bytes each)
     bool aligned32;                                 // every layer matrix starts on a 32-byte boundary (forward_persist.cu, forward_f32.cu)
     mutable std::mutex plan_mu;
@@ -164,14 +164,18 @@ KvView layer_kv(const tasc_model* m, const tasc_kv* kv, int layer) {
 }
 
 // Where the rows of a forward come from: a verify step (chunk < 0: last committed token + drafts) or prefill chunk `chunk`.
-// Which passes and products take the many-row kernel (gemm_wide.cu); see plan_fused.  Measured on the 135M, 0.5B and
-// 1.5B shapes at 192 .. 1,024 rows: a product gains from it once its weight matrix has about 7 MB (gate/up, down and
-// the LM head of the larger shapes; the narrow QKV and O matrices stay with the few-row kernel and its 128-row weight
-// tiles), and a pass of 129 .. 255 rows only on layers of 60 MB and more (its two token tiles fill three quarters of
-// the MMA's rows or less, and the few-row kernel then prefers three narrower tiles).
-constexpr double WIDE_MATRIX_MB = 7.0;
+// Which passes and products take the many-row kernel (gemm_wide.cu); see plan_fused.  Measured on the 0.5B and 1.5B shapes, a
+// step or a prefill in us with the few-row / the many-row kernel:
+//     all large products   0.5B 192 rows 1436 / 1485, 224 rows 1707 / 1563; 1.5B 140 rows 2508 / 2651, 147 rows 2745 / 2665
+//     matrices of 9 MB     0.5B 256 rows 1630 / 1766, 512 rows 1828 / 1988, 1,024 rows 2658 / 2732, 1,536 rows 4290 / 4305
+//     of 4.7 and 6.3 MB    1.5B 512 rows 3551 / 3938, 1,024 rows 6153 / 6343, 1,536 rows 9055 / 8509, 2,048 rows 97.0 / 88.4 ms
+//     of 17 MB             0.5B 256 rows 1965 / 1630
+// so by matrix: from 12 MB on, and in passes of more than 1,024 rows from 3.8 MB on (the 135M shape's 3.5 MB and less stay).
+constexpr double WIDE_MATRIX_MB = 12.0, WIDE_MATRIX_MB_1K = 3.8;
+constexpr int WIDE_1K = 1024;
+// Rows from which a pass takes it at all: more than 144 (three tiles of 48 of the few-row kernel) on layers of 60 MB and more.
 constexpr double WIDE_LAYER_MB = 60.0;
-constexpr int WIDE_ROWS = 256;
+constexpr int WIDE_ROWS = 208, WIDE_ROWS_LAYER = 145;
 
 struct RowSource {
     const tasc_seqs* seqs;
@@ -245,15 +249,15 @@ tasc_status forward_f32(const tasc_model* m, const tasc_kv* kv, const Workspace&
 // times width.  A step in us, five kernels per layer against one kernel:
 //     rows            7 MB per layer (135M)      30 MB (0.5B)             94 MB (1.5B)
 //     up to 8         798 / 578 - 818 / 591      897 / 652 - 940 / 702    1350 / 1122 - 1419 / 1172
-//     9 - 16          830 / 620 - 811 / 628      919 / 829 - 910 / 826    1412 / 1658
-//     17 - 32         857 / 770 - 868 / 789      951 / 972                -
-//     33 - 64         1006 / 814 - 945 / 819     -                        -
+//     9 - 16          782 / 620 - 811 / 628      763 / 819 - 788 / 831    1235 / 1688
+//     17 - 32         824 / 768 - 868 / 789      795 / 976                -
+//     33 - 64         857 / 810 - 884 / 818      920 / 1215               -
 //     96, 380 keys    1033 / 1077                -                        -
 // Its attention has at most one unit per SM and 12 key ranges, so the keys of a unit are bounded too (94 MB per layer, one
 // sequence of 4,000 tokens: 1559 / 1427 at 341 keys per unit).
 bool persist_pays(const tasc_model* m, int M, int max_ctx, const PersistPlan& pp) {
     if (max_ctx / pp.splits > 512) return false;
-    return M <= 8 || (M <= 16 && m->layer_mb <= 48.0) || (M <= 64 && m->layer_mb <= 12.0);
+    return M <= 8 || (M <= 64 && m->layer_mb <= 12.0);
 }
 
 // bf16 models: five launches per layer (QKV+RoPE+KV append, attention, O+residual, gate/up+SiLU*mul, down+residual),
@@ -277,10 +281,11 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
             const int att_rows = R <= 16 ? R : 16;
             sp.att = plan_attention_mma(B * (R / att_rows), d.n_kv_heads, d.head_dim, d.n_q_heads / d.n_kv_heads, att_rows, max_ctx);
             plan_attention_tc(B * (R / att_rows), d.n_kv_heads, d.head_dim, d.n_q_heads / d.n_kv_heads, att_rows, max_ctx, d.page_size, sp.att);
-            // passes of more than 128 rows: the products with large weight matrices take the many-row kernel
+            // passes of many rows: the products with large weight matrices take the many-row kernel
             const double big_mb = 2.0 * 2.0 * (double)d.d_ff * d.d_model / 1e6;      // the largest matrix of a layer (gate/up)
-            const bool wide_pass = M > 128 && big_mb >= WIDE_MATRIX_MB && (M >= WIDE_ROWS || m->layer_mb >= WIDE_LAYER_MB);
-            const double wide_min_mb = wide_pass ? WIDE_MATRIX_MB : -1.0;
+            const double matrix_mb = M > WIDE_1K ? WIDE_MATRIX_MB_1K : WIDE_MATRIX_MB;
+            const bool wide_pass = big_mb >= matrix_mb && M >= (m->layer_mb >= WIDE_LAYER_MB ? WIDE_ROWS_LAYER : WIDE_ROWS);
+            const double wide_min_mb = wide_pass ? matrix_mb : -1.0;
             sp.persist = !wide_pass && m->aligned32 &&
                          plan_persist(d.n_layers, M, B, R, d.d_model, m->q_dim, d.n_q_heads, d.n_kv_heads, d.head_dim, d.d_ff, max_ctx,
                                       d.page_size, sp.pp) &&
@@ -454,8 +459,8 @@ extern "C" tasc_status tasc_model_create(const tasc_model_desc* desc, const tasc
     m->kv_dim = d.n_kv_heads * d.head_dim;
     m->qkv_rows = m->q_dim + 2 * m->kv_dim;
     {
-        // every extra token tile streams the layer's weights once more (about 0.15 us per MB) and saves about 7 us of
-        // exchange and epilogue time per layer: below 24 MB three tiles, below 60 MB two, above that one
+        // every extra token tile streams the layer's weights once more (about 0.15 us per MB) and saves exchange and
+        // epilogue time per layer
         const double layer_mb = 2.0 * ((double)m->qkv_rows * d.d_model + (double)d.d_model * m->q_dim + 3.0 * d.d_ff * d.d_model) / 1e6;
         m->few_tiles = layer_mb < 24.0 ? 3 : (layer_mb < 60.0 ? 2 : 1);
         m->layer_mb = layer_mb;

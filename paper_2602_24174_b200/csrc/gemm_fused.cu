@@ -644,14 +644,13 @@ FusedPlan plan_fused(int M, int N, int K, int epi, int few_tiles, int hd, double
     FusedPlan p = {};
     const bool many_rows = wide_min_mb >= 0.0 && M > 128;
     const double mb = 2.0 * (double)(epi == EPI_SWIGLU ? 2 * N : N) * (double)K / 1e6;
-    // (from 512 rows on, matrices of a little more than half that size gain as well)
-    if (many_rows && (mb >= wide_min_mb || (M >= 512 && mb >= 0.55 * wide_min_mb)) && plan_wide(M, N, K, epi, hd, p)) return p;
+    if (many_rows && mb >= wide_min_mb && plan_wide(M, N, K, epi, hd, p)) return p;
     p = {};
     p.TBL = gemm_token_tile(M, true, few_tiles, many_rows);
-    // The LM head of a pass of 97 .. 128 rows in one token tile: the largest matrix of the model is tensor-bound there
+    // The LM head of a pass of 73 .. 128 rows in one token tile: the largest matrix of the model is tensor-bound there
     // (2 V d_model x 128 lanes x 2 passes), and the few-row kernel's 128-row weight tiles stream it at half the rate the
-    // many-row kernel reaches (measured on the 1.5B shape at 112 rows: 140 -> 85 us).
-    if (epi == EPI_LM && !many_rows && M > 96 && M <= 128 && p.TBL >= M && mb >= LM_WIDE_MIN_MB) {
+    // many-row kernel reaches (a step of the 1.5B shape, 112 rows 2006 -> 1980 us, 84 rows 1724 -> 1707, 70 rows 1635 -> 1634).
+    if (epi == EPI_LM && !many_rows && M > 72 && M <= 128 && p.TBL >= M && mb >= LM_WIDE_MIN_MB) {
         FusedPlan w = {};
         if (plan_wide(M, N, K, epi, hd, w, p.TBL)) return w;
     }

@@ -219,16 +219,22 @@ tasc_status encode_tmap_kv(CUtensorMap* map, const void* ptr, uint64_t rows, int
 int gemm_token_tile(int M, bool pair, int few_tiles, bool many_rows) {
     const int cap = pair ? 128 : 256;                 // tokens per tile (UMMA N <= 256)
     int m_tiles = (M + cap - 1) / cap;
-    // An MMA over a 128-row weight tile takes the same time for any number of token columns, while the split-K
-    // exchange, the accumulator read-out and the epilogue of a CTA grow with its columns -- and every token tile
-    // streams the weight tile again.  Which wins depends on the size of the weights: for narrow models (a few MB per
-    // layer) three or more token tiles per weight tile run faster than one or two wide ones above 48 rows (measured at
-    // 96, 192 and 448 rows); for a 94 MB layer one tile of 112 rows beats three of 48 by 20 % of the step, and in
-    // between two tiles are slightly ahead.  The caller passes the count for 49..128 rows (few_tiles).  Above 128 rows
-    // it stays at three or more -- unless the pass runs its large products through the many-row kernel (gemm_wide.cu),
-    // where the token rows are the MMA's M (many_rows): then as few tiles of at most 128 rows as hold them.
-    if (pair && M > 48 && M <= 128) m_tiles = std::max(m_tiles, std::max(1, std::min(few_tiles, 3)));
-    if (pair && M > 128 && !many_rows) m_tiles = std::max(m_tiles, 3);
+    // The few-row kernel's time per tile grows with its token columns (the MMA's 40 to 63 cycles per 16 of k, the split-K
+    // exchange, the accumulator read-out, the epilogue), but every token tile streams the weight tile again, from L2, and
+    // occupies more SMs.  Which wins depends on the layer's weights (few_tiles).  A step in us, by rows of a tile:
+    //     7 MB per layer    128 rows  32: 1039  48: 1079  64: 1131      256 rows  32: 1248  48: 1219  64: 1267  96: 1322
+    //                       192 rows  32: 1152  48: 1186  64: 1217      prefill of 512  32: 1565  48: 1385  64: 1400  128: 1584
+    //     30 MB             48 rows  16: 904  48: 920     45 rows  16: 917  48: 912     96 rows  32: 1112  48: 1144  96: 1183
+    //                       128 rows  32: 1355  48: 1236  64: 1267      192 rows  48: 1572  64: 1440  96: 1733
+    //     94 MB             49 rows  32: 1592  64: 1502   112 rows  64: 2002  112: 1977
+    // Passes that run their large products through the many-row kernel (many_rows; the token rows are its MMA's M) take as
+    // few tiles of at most 128 rows as hold them.
+    if (pair && !many_rows) {
+        auto tiles_of = [&](int rows) { return std::max(3, (M + rows - 1) / rows); };
+        if (few_tiles >= 3 && M > 48) m_tiles = std::max(m_tiles, tiles_of(M <= 192 ? 32 : 48));
+        else if (few_tiles == 2 && M > 45) m_tiles = std::max(m_tiles, tiles_of(64));
+        else if (M > 128) m_tiles = std::max(m_tiles, 3);
+    }
     const int per = (M + m_tiles - 1) / m_tiles;
     return std::max(16, (per + 15) / 16 * 16);
 }

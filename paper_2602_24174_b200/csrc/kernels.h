@@ -68,7 +68,7 @@ struct GemmPlan {
     int smem_bytes;
 };
 GemmPlan plan_gemm(int M, int N, int K, size_t max_partial_bytes, bool pair);
-// TB for M token rows.  few_tiles (1..3): how many token tiles 49..128 paired rows are cut into at least (see gemm_token_tile).
+// TB for M token rows.  few_tiles: 1 for layers of 60 MB and more, 2 from 24 MB on, 3 below (see gemm_token_tile).
 int gemm_token_tile(int M, bool pair, int few_tiles = 3, bool many_rows = false);
 inline size_t gemm_partial_bytes(const GemmPlan& p, int M, int N) { return (size_t)p.splits * M * N * sizeof(float); }
 

@@ -380,6 +380,18 @@ def test_prefill_skips_token_tiles_without_rows(lens):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("which,B,k", [(1, 33, 3), (1, 48, 3), (1, 49, 3), (1, 64, 7), (2, 23, 1), (2, 16, 2), (2, 52, 3), (4, 36, 3), (4, 29, 4)])
+def test_token_tiles_by_layer_size(which, B, k):
+    """Few-row kernel with token tiles of 16, 32, 48 and 64 rows, the last one full or with four rows in use (132, 192, 196 and
+    512 rows of the smallest layers, 46, 48 and 208 of the middle ones), and the rows where the largest layers change to the
+    many-row kernel (144, 145).  One layer; the oracle runs the first, a middle and the last sequence."""
+    cfg = configs.shrunk(configs.get(which), n_layers=1, vocab=4096, n_docs=500)
+    s = make_setup(cfg)
+    prompts = corpus.make_prompts(cfg, B, prompt_len=21)
+    check(lockstep(s, prompts, k + 1, k, oracle_rows=[0, B // 2, B - 1], **BF16_TOL), f"token tiles, config {which}, B={B} k={k}")
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("B,P", [(37, 9), (55, 40), (75, 129)])
 def test_many_row_kernel_on_pairs_of_token_tiles(B, P):
     """Configuration 4's geometry (one layer, an 8,200-token vocabulary: a feature tile of eight) at 259, 385 and 525 rows of
