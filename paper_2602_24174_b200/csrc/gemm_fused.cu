@@ -669,7 +669,7 @@ FusedPlan plan_fused(int M, int N, int K, int epi, int few_tiles, int hd, double
         S = std::min(S, 8);
         S = std::min(S, p.num_kb);
         // Fewer splits than fit can be faster.  Per kernel, in microseconds as measured on the 576- and 1536-wide
-        // products: a CTA's MMA chain takes about 0.46 per k-block; its epilogue about 0.5 per round of six token
+        // products: a CTA's MMA chain takes about 0.46 per k-block (0.28 to 0.46 choose the same); its epilogue about 0.5 per round of six token
         // columns (one per warp) of the columns it finishes; and a grid that takes more than about two thirds of
         // the SMs keeps the next kernel's CTAs from starting (and from fetching their weights) while this one
         // runs, about 0.035 per CTA beyond 96.  Ties go to the larger cluster.
