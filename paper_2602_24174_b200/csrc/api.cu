@@ -250,14 +250,16 @@ tasc_status forward_f32(const tasc_model* m, const tasc_kv* kv, const Workspace&
 //     rows            7 MB per layer (135M)      30 MB (0.5B)             94 MB (1.5B)
 //     up to 8         798 / 578 - 818 / 591      897 / 652 - 940 / 702    1350 / 1122 - 1419 / 1172
 //     9 - 16          782 / 620 - 811 / 628      763 / 819 - 788 / 831    1235 / 1688
-//     17 - 32         824 / 768 - 868 / 789      795 / 976                -
-//     33 - 64         857 / 810 - 884 / 818      920 / 1215               -
+//     17 - 32         784 / 773 - 823 / 796      795 / 976                -
+//     33 - 64         920 / 813 - 858 / 824      920 / 1215               -
 //     96, 380 keys    1033 / 1077                -                        -
+// Replayed from a graph the five kernels per layer follow one another more closely: 701 / 750 at 18 rows and 753 / 780 at 32
+// (7 MB), the rest as above; the one kernel's time hardly changes between 17 and 64 rows (blocks of 32).
 // Its attention has at most one unit per SM and 12 key ranges, so the keys of a unit are bounded too (94 MB per layer, one
 // sequence of 4,000 tokens: 1559 / 1427 at 341 keys per unit).
 bool persist_pays(const tasc_model* m, int M, int max_ctx, const PersistPlan& pp) {
     if (max_ctx / pp.splits > 512) return false;
-    return M <= 8 || (M <= 64 && m->layer_mb <= 12.0);
+    return M <= 8 || (m->layer_mb <= 12.0 && (M <= 16 || (M > 32 && M <= 64)));
 }
 
 // bf16 models: five launches per layer (QKV+RoPE+KV append, attention, O+residual, gate/up+SiLU*mul, down+residual),
