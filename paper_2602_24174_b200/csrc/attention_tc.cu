@@ -55,7 +55,7 @@ __device__ __forceinline__ void pack_hilo(float x, float y, uint32_t& hi, uint32
     const float rx = x - __uint_as_float(hi << 16), ry = y - __uint_as_float(hi & 0xFFFF0000u);
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(ry), "f"(rx));
 }
-// 2^x of the hardware (what exp2f calls, without its detour for results below 2^-126, which are zero here)
+// 2^x; results below 2^-126 are zero here (.ftz)
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
