@@ -222,11 +222,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         griddep_wait();
         for (; t < n_tiles; ++t) {
             const uint32_t used = (uint32_t)(t / a.stages - 1) & 1u;
-            if (t >= a.stages) { wait(bar_k_empty + 8u * (t % a.stages), used); __syncwarp(); }
-            if (*failed) break;
+            if (t >= a.stages) wait(bar_k_empty + 8u * (t % a.stages), used);
+            if (warp_failed(failed)) break;
             load(t, false);
-            if (t >= a.stages) { wait(bar_v_empty + 8u * (t % a.stages), used); __syncwarp(); }
-            if (*failed) break;
+            if (t >= a.stages) wait(bar_v_empty + 8u * (t % a.stages), used);
+            if (warp_failed(failed)) break;
             load(t, true);
         }
         __syncwarp();

@@ -146,6 +146,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long lo
     return true;
 }
 
+// Whether the CTA's fail flag is set, decided by the whole warp: another warp may set it at any time, and lanes that looked
+// for themselves could part, some leaving a loop whose next warp-wide barrier the others then wait at for good.
+__device__ __forceinline__ bool warp_failed(const volatile int* failed) { return __any_sync(0xFFFFFFFFu, *failed != 0); }
+
 // ---------------------------------------------------------------- thread-block clusters, distributed shared memory
 __device__ __forceinline__ uint32_t cluster_ctarank() {
     uint32_t r;
