@@ -72,7 +72,7 @@ struct Workspace {
     float* att_scratch;
     float* ssq;                   // [M][ceil(d / 128)] partial sums of squares of the residual rows (bf16 models)
     int ssq_slots;
-    double* ssq64;                // bf16 models, passes whose layers run as one kernel: [2 n_layers + 1][rows]
+    unsigned long long* ssq_p;    // bf16 models, passes whose layers run as one kernel: [2 n_layers + 1][rows][SSQ_WORDS]
     float* att_part;              // ... and their parked key ranges
     unsigned* counters;           // ... grid barrier, attention groups
     size_t bytes;
@@ -138,7 +138,7 @@ Workspace layout_workspace(const tasc_model* m, int B, void* base_) {
     w.ssq_slots = (d.d_model + 127) / 128;
     w.ssq = L.take<float>(base, M * w.ssq_slots * 4);      // passes of more than 128 rows keep four slots per 128 features
     const bool bf16 = d.dtype == TASC_BF16;
-    w.ssq64 = L.take<double>(base, bf16 ? (size_t)(2 * d.n_layers + 1) * PERSIST_MAX_ROWS : 1);
+    w.ssq_p = L.take<unsigned long long>(base, bf16 ? (size_t)(2 * d.n_layers + 1) * PERSIST_MAX_ROWS * SSQ_WORDS : 1);
     w.att_part = L.take<float>(base, bf16 ? (size_t)PERSIST_MAX_UNITS * 16 * (d.head_dim + 2) : 1);
     w.counters = L.take<unsigned>(base, bf16 ? COUNTER_WORDS : 1);
     w.bytes = L.off;
@@ -270,7 +270,7 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
     const int M = B * R;
     const int max_ctx = kv->max_pages_per_seq * d.page_size;
     tasc_status st;
-    StepPlans sp;
+    StepPlans sp = {};
     {
         std::lock_guard<std::mutex> lk(m->plan_mu);
         auto it = std::find_if(m->plans.begin(), m->plans.end(), [&](const StepPlans& c) {
@@ -332,14 +332,14 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
 
     launch_rows_embed(w.rp, src.seqs->tokens, src.seqs->stride, src.seqs->len, src.seqs->stop_len, src.drafts, B, R, src.chunk,
                       d.vocab, w.status, static_cast<const __nv_bfloat16*>(m->embed), m->attn_norm[0], w.x, h,
-                      w.ssq, ssq_slots, lm_head ? w.argmax : nullptr, d.d_model, TB, sp.persist ? w.ssq64 : nullptr, 2 * d.n_layers + 1,
+                      w.ssq, ssq_slots, lm_head ? w.argmax : nullptr, d.d_model, TB, sp.persist ? w.ssq_p : nullptr, 2 * d.n_layers + 1,
                       w.counters, sp.persist ? COUNTER_GROUPS + sp.pp.n_units / sp.pp.splits : 0, s);
     if (sp.persist) {
         PersistArgs a = {};
         a.layers = static_cast<const LayerWeights*>(m->d_layers); a.n_layers = d.n_layers; a.M = M; a.R = R; a.TBL = TB;
         a.d = d.d_model; a.qd = m->q_dim; a.dff = d.d_ff; a.n_q = d.n_q_heads; a.n_kv = d.n_kv_heads; a.hd = d.head_dim;
         a.inv_d = base.inv_d; a.eps = base.eps; a.scale_log2e = 1.4426950408889634f / sqrtf((float)d.head_dim);
-        a.h = h; a.o = o; a.act = act; a.q = w.q; a.x0 = w.x; a.ssq = w.ssq64;
+        a.h = h; a.o = o; a.act = act; a.q = w.q; a.x0 = w.x; a.ssq = w.ssq_p;
         a.row_pos = w.rp.row_pos; a.seq_pos0 = w.rp.seq_pos0; a.seq_rows = w.rp.seq_rows;
         a.block_table = kv->block_table; a.max_pages = kv->max_pages_per_seq; a.page_size = d.page_size; a.n_pages = kv->n_pages;
         a.kv_pool = static_cast<__nv_bfloat16*>(kv->pool);
@@ -348,7 +348,7 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
         a.part = w.att_part; a.bar = w.counters + COUNTER_BAR; a.unit_ctr = w.counters + COUNTER_GROUPS;
         a.status = w.status;
         if ((st = launch_persist(a, sp.pp, s)) != TASC_OK) return st;
-        base.ssq64 = w.ssq64 + (size_t)2 * d.n_layers * M;
+        base.ssq_exact = w.ssq_p + (size_t)2 * d.n_layers * M * SSQ_WORDS;
     }
     for (int l = 0; l < d.n_layers && !sp.persist; ++l) {
         const KvView kvl = layer_kv(m, kv, l);

@@ -106,6 +106,31 @@ __device__ __forceinline__ float warp_max(float v) {
     return v;
 }
 
+// ---------------------------------------------------------------- sums of squares that do not depend on the order
+// A sum that many CTAs add to in any order, kept exact: a float is an integer m < 2^24 times 2^(p - 149), 0 <= p < 254, and goes
+// to word p / 32 shifted by p % 32, below 2^55, so that 512 of them fit.  Infinities and NaN are p = 254 and m >= 2^23 like any
+// other number, 2^128 and more: the total is infinite as a float.
+constexpr int SSQ_WORDS = 8, SSQ_MAX_ADDS = 512;
+// v >= 0: the word it goes to and what is added there
+__device__ __forceinline__ unsigned long long ssq_word(float v, int& word) {
+    const uint32_t u = __float_as_uint(v), e = (u >> 23) & 255u;
+    const uint32_t p = e ? e - 1u : 0u;
+    word = (int)(p >> 5);
+    return (unsigned long long)((u & 0x7FFFFFu) | (e ? 0x800000u : 0u)) << (p & 31u);
+}
+__device__ __forceinline__ void ssq_add(unsigned long long* sum, float v) {
+    int word;
+    const unsigned long long w = ssq_word(v, word);
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(sum + word), "l"(w) : "memory");
+}
+// The total in all eight lanes from one word in each (lane % 8); whole warps, in a fixed order.
+__device__ __forceinline__ float ssq_total(unsigned long long w) {
+    double s = (double)w * __hiloint2double((int)(1023u - 149u + 32u * (threadIdx.x & 7u)) << 20, 0);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+    return (float)s;
+}
+
 // ---------------------------------------------------------------- shared-memory addresses, mbarrier
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 

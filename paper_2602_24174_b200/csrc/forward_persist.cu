@@ -15,6 +15,9 @@
 // accumulator.  The warps' partial tiles meet in shared memory and are added in warp order (bitwise repeatable), and
 // the stage that follows the product (RoPE + KV append, residual + next norm's input, SiLU * up) runs on the sums.
 // The residual stream of a CTA's rows stays in its shared memory from the embedding to the last layer.
+// A row's sum of squares for the RMSNorm comes from all CTAs, in any order: it is kept exact (ssq_word), so that a pass gives the
+// same bits every time.  (In one double per row the order showed: rows built for it gave other logits in 39 of 40 passes.  A
+// slot per CTA, added up in order by every reader, cost 0.3 us more per phase than eight words: 600 against 588 us at 135M, 6 rows.)
 //
 // Row pairs.  A tile's rows r and r + 8 are partners where the epilogue needs two features at once: the two halves of
 // a rotary pair (QKV), a gate row and its up row (gate/up).
@@ -154,8 +157,8 @@ struct Phase {
     int lh;                            // QKV: log2 of half a head; else 31
     int pair;                          // rows from a pair's first row to its second
     const float* gain;                 // residual phases
-    const double* ssq_in;
-    double* ssq_out;
+    const unsigned long long* ssq_in;
+    unsigned long long* ssq_out;
     bool final_rows;
     __nv_bfloat16 *kp, *vp;
 };
@@ -166,7 +169,7 @@ struct Shared {
     PersistArgs args;                  // for the routines that are not inlined (a reference to the kernel's parameters is slow there)
     long long koff[MAX_TOK];           // element offset of the token's slot in a layer's K or V pages, -1 = none
     LayerWeights layers[PERSIST_MAX_LAYERS];
-    float inv[MAX_TOK];                // RMS factors of the current input
+    float rms[MAX_TOK];                // sums of squares of the current projection's input rows, or the RMS factors
     int pos[MAX_TOK];                  // positions, -1 = unused row
     int part[3][2];                    // first and last + 1 row (pair) of this CTA in the QKV, d-wide and gate/up products
     int m0;                            // its first token row
@@ -240,8 +243,8 @@ __device__ __noinline__ void set_phase(int l, int j, Phase& ph) {
     ph.lh = j == 0 ? (HD == 64 ? 5 : 6) : 31;
     ph.pair = j == 0 ? HD / 2 : a.dff;
     ph.gain = j == 2 ? lw.gain_mlp : lw.gain_next;
-    ph.ssq_in = a.ssq + (size_t)(2 * l + (j == 3 ? 1 : 0)) * a.M;
-    ph.ssq_out = a.ssq + (size_t)(2 * l + (j == 2 ? 1 : 2)) * a.M;
+    ph.ssq_in = a.ssq + (2 * l + (j == 3 ? 1 : 0)) * (a.M * SSQ_WORDS);
+    ph.ssq_out = a.ssq + (2 * l + (j == 2 ? 1 : 2)) * (a.M * SSQ_WORDS);
     ph.final_rows = j == 4 && l + 1 == a.n_layers;
     ph.kp = a.kv_pool + (size_t)l * 2 * a.kv_half;
     ph.vp = ph.kp + a.kv_half;
@@ -267,6 +270,7 @@ struct Cta {
         return (unsigned)((m >> 3) * nch + (f >> 6)) * 1024u + (unsigned)((m & 7) * 64 + (f & 63));
     }
 
+    __device__ __forceinline__ float rms_factor(float ss) const { return 1.0f / sqrtf(ss * a.inv_d + a.eps); }
     // What one thread finishes: (row, token) of a tile -- for the pair phases both rows of the pair.
     struct Item {
         uint32_t p;            // shared address of the first parked copy this lane adds
@@ -278,11 +282,11 @@ struct Cta {
     };
     __device__ __forceinline__ Item decode(const Phase& ph, int idx, int lp, int tile0, uint32_t red, uint32_t stride, int u0, int u1, int m0) const {
         const bool resid = ph.kind == PH_RESID;
-        const int part = (idx >> 3) & ((1 << lp) - 1), rest = idx >> (3 + lp), n = rest & 7;
-        int hv = rest >> 3, row = idx & 7;
-        if (resid) { row += (hv & 1) * 8; hv >>= 1; }
+        const int lper = resid ? 4 : 3;
+        const int part = (idx >> lper) & ((1 << lp) - 1), rest = idx >> (lper + lp), n = rest & 7;
+        const int row = idx & ((1 << lper) - 1), hv = rest >> 3;
         const int tt = hv & (T - 1), tl = hv >> LT, tile = tile0 + tl, tok = tt * 8 + n;
-        const int f = u0 + tile * (resid ? 16 : 8) + row;
+        const int f = u0 + (tile << lper) + row;
         Item it;
         it.m = m0 + tok;
         it.p = red + (uint32_t)((tl * T + tt) * RED_TILE + n * RED_N + row) * 4u + (uint32_t)part * stride;
@@ -385,10 +389,21 @@ struct Cta {
                 }
             }
         };
+        // The sums of squares of the CTA's tokens, eight lanes each, for the RMS factors behind the products.  With four tiles they are
+        // requested ahead of the activations, and the factors are ready made (48 rows of the 135M: 860 -> 848 us); with one the
+        // two warps that add them up are on the critical path and do no more than that (6 rows: 588 -> 584).
+        const bool sums = kind != PH_RESID && tid < T * 64;
+        unsigned long long w8 = 0ull;
+        auto load_sums = [&]() {
+            if (sums && m0 + (tid >> 3) < a.M) asm volatile("ld.global.u64 %0, [%1];" : "=l"(w8) : "l"(ph.ssq_in + m0 * SSQ_WORDS + tid) : "memory");
+        };
+        if (T == 4) load_sums();
         for_each<D>([&](auto uc) { load_b(std::true_type{}, uc, decltype(uc)::value < n_ch); });
-        // the token's sum of squares, for the RMS factor (used after the products)
-        double ssq = 0.0;
-        if (kind != PH_RESID && it.m < a.M) asm volatile("ld.global.f64 %0, [%1];" : "=d"(ssq) : "l"(ph.ssq_in + it.m) : "memory");
+        if (T != 4) load_sums();
+        if (sums) {
+            const float ss = ssq_total(w8);
+            if ((tid & 7) == 0) sh().rms[tid >> 3] = T == 4 ? rms_factor(ss) : ss;
+        }
 #pragma unroll 1
         for (int tile0 = 0; tile0 < n_tiles; tile0 += group) {
             const int tile1 = min(n_tiles, tile0 + group);
@@ -442,7 +457,6 @@ struct Cta {
             if (tile0 > 0) it = decode(ph, tid, lp, tile0, red, stride, u0, u1, m0);
 #pragma unroll 1
             for (int idx = tid; idx < n_items;) {
-                if (tile0 + idx != tid && kind != PH_RESID && it.m < a.M) asm volatile("ld.global.f64 %0, [%1];" : "=d"(ssq) : "l"(ph.ssq_in + it.m) : "memory");
                 float v0 = 0.f, v1 = 0.f;
                 uint32_t p = it.p;
 #pragma unroll 2
@@ -450,7 +464,7 @@ struct Cta {
                     v0 += lds_f(p);
                     if (kind != PH_RESID) v1 += lds_f(p + 32);
                 }
-                if (lp >= 1) { v0 += __shfl_xor_sync(0xFFFFFFFFu, v0, 8); v1 += __shfl_xor_sync(0xFFFFFFFFu, v1, 8); }
+                if (lp >= 1) { v0 += __shfl_xor_sync(0xFFFFFFFFu, v0, per); v1 += __shfl_xor_sync(0xFFFFFFFFu, v1, per); }
                 if (lp == 2) { v0 += __shfl_xor_sync(0xFFFFFFFFu, v0, 16); v1 += __shfl_xor_sync(0xFFFFFFFFu, v1, 16); }
                 if (kind == PH_RESID) {
                     float ss = 0.f;
@@ -466,10 +480,11 @@ struct Cta {
                     ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 1);
                     ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 2);
                     ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 4);
-                    // (added in double: the order of the CTAs does not reach the 24 bits that are used)
-                    if (it.lead && (lane & 7) == 0) asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(ph.ssq_out + it.m), "d"((double)ss) : "memory");
+                    ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 8);
+                    if (it.lead && (lane & 15) == 0) ssq_add(ph.ssq_out + it.m * SSQ_WORDS, ss);
                 } else if (it.lead) {
-                    const float sc = 1.0f / sqrtf((float)ssq * a.inv_d + a.eps);
+                    float sc = sh().rms[it.m - m0];
+                    if (T != 4) sc = rms_factor(sc);
                     v0 *= sc; v1 *= sc;
                     if (kind == PH_GATEUP) {
                         const float v = v0 / (1.0f + expf(-v0)) * v1;
@@ -848,7 +863,8 @@ __global__ void __launch_bounds__(WARPS * 32, 1) layers_kernel(const __grid_cons
     if (tid == 0) { sh().stop = 0; sh().unit = Unit{}; sh().m0 = m0; }
     if (tid < 6) {
         const unsigned n = (tid >> 1) == 0 ? (unsigned)(a.qd / 2 + a.n_kv * HD) : (tid >> 1) == 1 ? (unsigned)a.d : (unsigned)a.dff;
-        sh().part[tid >> 1][tid & 1] = in_grid ? (int)(n * (unsigned)(rb + (tid & 1)) / (unsigned)a.n_rb) : 0;
+        const int blocks = (tid >> 1) == 1 ? a.n_res : a.n_rb;
+        sh().part[tid >> 1][tid & 1] = in_grid && rb < blocks ? (int)(n * (unsigned)(rb + (tid & 1)) / (unsigned)blocks) : 0;
     }
     if (tid < TOK) {
         const int m = m0 + tid;
@@ -958,7 +974,10 @@ bool plan_persist(int n_layers, int M, int B, int R, int d, int qd, int n_q, int
     p.n_tb = (M + p.T * 8 - 1) / (p.T * 8);
     p.n_rb = p.grid / p.n_tb;
     if (p.n_rb < 1) return false;
-    p.nt_res = ((d + p.n_rb - 1) / p.n_rb + 15) / 16;
+    // (blocks of a residual projection have 8 rows or more: each adds to the sums of squares of all token rows)
+    p.n_res = std::min(p.n_rb, d / 8);
+    p.nt_res = ((d + p.n_res - 1) / p.n_res + 15) / 16;
+    if (p.n_res * p.nt_res > SSQ_MAX_ADDS) return false;
     const int qkv_pairs = qd / 2 + n_kv * hd;
     p.nt_qkv = ((qkv_pairs + p.n_rb - 1) / p.n_rb + 7) / 8;
     const int x_bytes = p.nt_res * p.T * 128 * 4 + p.nt_qkv * p.T * 64 * 8;      // residual rows, rotary factors
@@ -966,9 +985,9 @@ bool plan_persist(int n_layers, int M, int B, int R, int d, int qd, int n_q, int
     p.smem_bytes = SHARED_BYTES + p.union_bytes + x_bytes;
     if (p.smem_bytes > MAX_SMEM) return false;
     // how the warps of a CTA split a projection: row groups x k groups, by the longest chain of 64-wide chunks a warp walks
-    const int rows[4] = {qkv_pairs, d, dff, d}, per[4] = {8, 16, 8, 16}, red[4] = {d, qd, d, dff};
+    const int rows[4] = {qkv_pairs, d, dff, d}, blocks[4] = {p.n_rb, p.n_res, p.n_rb, p.n_res}, per[4] = {8, 16, 8, 16}, red[4] = {d, qd, d, dff};
     for (int j = 0; j < 4; ++j) {
-        const int tiles = ((rows[j] + p.n_rb - 1) / p.n_rb + per[j] - 1) / per[j], chunks = red[j] / CHUNK;
+        const int tiles = ((rows[j] + blocks[j] - 1) / blocks[j] + per[j] - 1) / per[j], chunks = red[j] / CHUNK;
         int best = 1 << 30;
         for (int lr = 0; lr <= LW; ++lr) {
             const int rg = 1 << lr, kg = WARPS >> lr;
@@ -988,7 +1007,7 @@ bool plan_persist(int n_layers, int M, int B, int R, int d, int qd, int n_q, int
 }
 
 tasc_status launch_persist(PersistArgs a, const PersistPlan& p, cudaStream_t stream) {
-    a.n_tb = p.n_tb; a.n_rb = p.n_rb; a.nt_res = p.nt_res; a.nt_qkv = p.nt_qkv; a.park_bytes = p.union_bytes;
+    a.n_tb = p.n_tb; a.n_rb = p.n_rb; a.nt_res = p.nt_res; a.nt_qkv = p.nt_qkv; a.park_bytes = p.union_bytes; a.n_res = p.n_res;
     for (int j = 0; j < 4; ++j) a.lr[j] = p.lr[j];
     a.r_magic = (unsigned)(((1ull << 32) + a.R - 1) / a.R);        // exact for quotients of numbers below 2^16
     a.tbl_magic = (unsigned)(((1ull << 32) + a.TBL - 1) / a.TBL);

@@ -378,11 +378,18 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
 #endif
         if (!a.early) late_prefetch();
         if (EPI == EPI_QKV || EPI == EPI_SWIGLU || EPI == EPI_LM || (EPI == EPI_PLAIN && a.ssq_in)) {
+            if (EPI == EPI_LM && a.ssq_exact) {
+                for (int t = threadIdx.x >> 3; t < TB; t += 16) {        // eight lanes per row (TB is a multiple of 16)
+                    const float ss = ssq_total(t0 + t < a.M ? a.ssq_exact[(size_t)(t0 + t) * SSQ_WORDS + (threadIdx.x & 7)] : 0ull);
+                    if ((threadIdx.x & 7) == 0) s_inv[t] = 1.0f / sqrtf(ss * a.inv_d + a.eps);
+                }
+            } else
             for (int t = threadIdx.x; t < TB; t += 128) {
                 const int m = t0 + t;
                 float ss = 0.f;
-                if (m < a.M && a.ssq64) ss = (float)a.ssq64[m];
-                else if (m < a.M)
+                // (a few slots, off the critical path: unrolled, the code in front of everything else is longer, 0.5 % of a step)
+                if (m < a.M)
+#pragma unroll 1
                     for (int j = 0; j < a.ssq_slots; ++j) ss += a.ssq_in[(size_t)m * a.ssq_slots + j];
                 s_inv[t] = 1.0f / sqrtf(ss * a.inv_d + a.eps);
             }
@@ -727,7 +734,7 @@ FusedPlan plan_fused(int M, int N, int K, int epi, int few_tiles, int hd, double
 tasc_status launch_gemm_fused(int epi, const CUtensorMap* tmW, const CUtensorMap* tmX, FusedArgs a, const FusedPlan& p,
                               cudaStream_t stream) {
     if (a.M <= 0 || a.N <= 0 || a.K <= 0) return TASC_EINVAL;
-    if (p.wide) return launch_gemm_wide(epi, tmW, tmX, a, p, stream);
+    if (p.wide) return a.ssq_exact ? TASC_EINVAL : launch_gemm_wide(epi, tmW, tmX, a, p, stream);
     a.num_kb = p.num_kb; a.BN = p.BN; a.TB = p.TB; a.TBL = p.TBL; a.stages = p.stages; a.pair = 1; a.data_bytes = p.data_bytes;
     switch (epi) {
         case EPI_PLAIN:  return launch_epi<EPI_PLAIN>(tmW, tmX, a, p, K_GEMM, stream);

@@ -338,9 +338,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         float sc = 1.0f;
         if (a.ssq_in && rowok) {
             float ss = 0.f;
-            if (a.ssq64) {
-                ss = (float)a.ssq64[m];
-            } else if (a.ssq_slots % 4 == 0) {
+            if (a.ssq_slots % 4 == 0) {
                 const float4* sp = reinterpret_cast<const float4*>(a.ssq_in + (size_t)m * a.ssq_slots);
                 for (int q = 0; q < a.ssq_slots / 4; ++q) { const float4 t = sp[q]; ss += (t.x + t.y) + (t.z + t.w); }
             } else {

@@ -99,9 +99,9 @@ struct FusedArgs {
     const int* seq_rows;               // prefill passes: rows in use of every sequence (R rows each); the many-row kernel skips token
                                        // tiles without any (the few-row kernel would wait longer for the counts than it gains)
     int rows_early;                    // ... which were complete before the preceding grid began
-    const double* ssq64;               // [M] sums of squares of the input rows (instead of ssq_in, behind the one-kernel layers)
     const float* ssq_in;               // [M][ssq_slots] partial sums of squares of the input rows (null: no scaling)
     int ssq_slots;
+    const unsigned long long* ssq_exact;   // [M][SSQ_WORDS], instead of ssq_in behind the one-kernel layers
     float inv_d, eps;                  // rms factor = 1 / sqrt(sum(ssq) * inv_d + eps)
     float* y;                          // EPI_PLAIN
     const int* row_pos;                // EPI_QKV: position of each row, -1 = unused
@@ -168,6 +168,7 @@ struct PersistPlan {
     int lr[4];                               // QKV, O, gate/up, down: log2 of the row groups the warps form
     int union_bytes, smem_bytes;
     int splits, n_slabs, n_units;            // attention: key ranges, slabs of 16 query rows, units in all
+    int n_res;                               // row blocks of a residual projection
 };
 struct PersistArgs {
     const LayerWeights* layers;              // device, [n_layers]
@@ -177,8 +178,8 @@ struct PersistArgs {
     __nv_bfloat16 *h, *o, *act;              // (hi, lo) activation buffers; h: blocks on entry, layout tiles of TBL tokens on return
     float* q;                                // [M][qd]
     const float* x0;                         // [M][d] embedding rows
-    double* ssq;                             // [2 n_layers + 1][M] sums of squares of the residual rows: the embedding's on entry, zeros
-                                             // behind it; the last M are the final rows' on return
+    unsigned long long* ssq;                 // [2 n_layers + 1][M][SSQ_WORDS] sums of squares of the residual rows: the embedding's on entry,
+                                             // zeros behind it; the last M are the final rows' on return
     const int *row_pos, *seq_pos0, *seq_rows;
     const int32_t* block_table;
     int max_pages, page_size;
@@ -192,7 +193,7 @@ struct PersistArgs {
     int* status;
     unsigned r_magic, tbl_magic;             // filled in by launch_persist, like the rest
     int page_shift;
-    int n_tb, n_rb, nt_res, nt_qkv, park_bytes, lr[4], union_bytes, splits, n_slabs, n_units;      // from the plan
+    int n_tb, n_rb, nt_res, nt_qkv, park_bytes, lr[4], union_bytes, splits, n_slabs, n_units, n_res;      // from the plan
 };
 // Returns false where the pass does not take this path.
 bool plan_persist(int n_layers, int M, int B, int R, int d, int qd, int n_q, int n_kv, int hd, int dff, int max_ctx, int page_size, PersistPlan& p);
@@ -224,12 +225,12 @@ void launch_embed_norm(const T* embed, const int* row_tok, const float* gain, fl
                        int TB, cudaStream_t stream);
 // bf16 model, first launch of a forward: row plan (chunk < 0: verify step, else prefill chunk) + embedding:
 // x[m] = embed[tok]; a_out = (hi, lo) of x * gain; ssq[m][0] = sum x^2, other slots 0; argmax[m] = 0 (if given);
-// ssq64 given (the layers follow as one kernel): a_out in its blocks of 8 tokens x 64 features, ssq64[0][m] = sum x^2,
-// ssq64[1 .. n_stage)[m] = 0, and zero[0 .. n_zero) = 0 (the kernel's counters).
+// ssq_p given (the layers follow as one kernel): a_out in its blocks of 8 tokens x 64 features, ssq_p[0][m] = sum x^2,
+// ssq_p[1 .. n_stage)[m] = 0 (SSQ_WORDS words each), and zero[0 .. n_zero) = 0 (the kernel's counters).
 void launch_rows_embed(const RowPlan& rp, const int32_t* tokens, int64_t stride, const int32_t* len, const int32_t* stop_len,
                        const int32_t* drafts, int B, int R, int chunk, int vocab, int* status, const __nv_bfloat16* embed,
                        const float* gain, float* x, __nv_bfloat16* a_out, float* ssq, int ssq_slots, unsigned long long* argmax,
-                       int d, int TB, double* ssq64, int n_stage, unsigned* zero, int n_zero, cudaStream_t stream);
+                       int d, int TB, unsigned long long* ssq_p, int n_stage, unsigned* zero, int n_zero, cudaStream_t stream);
 // x += sum_s P[s]; h = RMSNorm(x) * gain  (gain == null: only the residual update)
 template <typename T>
 void launch_residual_norm(const float* partials, int splits, float* x, const float* gain, float eps, T* h, int M, int d,

@@ -91,7 +91,7 @@ rows_embed_kernel(RowPlan rp, const int32_t* __restrict__ tokens, int64_t stride
                   const int32_t* __restrict__ stop_len, const int32_t* __restrict__ drafts, int R, int chunk, int vocab,
                   int* status, const __nv_bfloat16* __restrict__ embed, const float* __restrict__ gain, float* __restrict__ x,
                   __nv_bfloat16* __restrict__ a_out, float* __restrict__ ssq, int ssq_slots, unsigned long long* argmax, int d,
-                  int TB, double* __restrict__ ssq64, int n_stage, unsigned* __restrict__ zero, int n_zero) {
+                  int TB, unsigned long long* __restrict__ ssq_p, int n_stage, unsigned* __restrict__ zero, int n_zero) {
     __shared__ float red[4];
     __shared__ int s_tok;
     const int m = blockIdx.x;
@@ -132,14 +132,17 @@ rows_embed_kernel(RowPlan rp, const int32_t* __restrict__ tokens, int64_t stride
         const float v = __bfloat162float(e[j]);
         x[(size_t)m * d + j] = v;
         ss += v * v;
-        if (ssq64) {
+        if (ssq_p) {
             const size_t at = (size_t)((m >> 3) * (d >> 6) + (j >> 6)) * 1024 + (m & 7) * 64 + (j & 63);
             split_bf16(v * gain[j], a_out[at], a_out[at + 512]);
         } else ActStore<__nv_bfloat16>::put(a_out, m, j, d, TB, v * gain[j]);
     }
     ss = block_sum(ss, red);
-    if (ssq64) {
-        for (int j = threadIdx.x; j < n_stage; j += blockDim.x) ssq64[(size_t)j * gridDim.x + m] = j == 0 ? (double)ss : 0.0;
+    if (ssq_p) {
+        int at;
+        const unsigned long long word = ssq_word(ss, at);
+        for (int j = threadIdx.x; j < n_stage * SSQ_WORDS; j += blockDim.x)
+            ssq_p[((size_t)(j / SSQ_WORDS) * gridDim.x + m) * SSQ_WORDS + j % SSQ_WORDS] = j == at ? word : 0ull;
     } else
     for (int j = threadIdx.x; j < ssq_slots; j += blockDim.x) ssq[(size_t)m * ssq_slots + j] = j == 0 ? ss : 0.f;
     if (threadIdx.x == 0 && argmax) argmax[m] = 0ull;
@@ -376,10 +379,10 @@ void launch_embed_norm(const T* embed, const int* row_tok, const float* gain, fl
 void launch_rows_embed(const RowPlan& rp, const int32_t* tokens, int64_t stride, const int32_t* len, const int32_t* stop_len,
                        const int32_t* drafts, int B, int R, int chunk, int vocab, int* status, const __nv_bfloat16* embed,
                        const float* gain, float* x, __nv_bfloat16* a_out, float* ssq, int ssq_slots, unsigned long long* argmax,
-                       int d, int TB, double* ssq64, int n_stage, unsigned* zero, int n_zero, cudaStream_t stream) {
+                       int d, int TB, unsigned long long* ssq_p, int n_stage, unsigned* zero, int n_zero, cudaStream_t stream) {
     ProfScope ps(K_EMBED, stream);
     rows_embed_kernel<<<B * R, 128, 0, stream>>>(rp, tokens, stride, len, stop_len, drafts, R, chunk, vocab, status, embed, gain,
-                                                 x, a_out, ssq, ssq_slots, argmax, d, TB, ssq64, n_stage, zero, n_zero);
+                                                 x, a_out, ssq, ssq_slots, argmax, d, TB, ssq_p, n_stage, zero, n_zero);
 }
 template <typename T>
 void launch_residual_norm(const float* partials, int splits, float* x, const float* gain, float eps, T* h, int M, int d,

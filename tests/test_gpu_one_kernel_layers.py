@@ -1,0 +1,74 @@
+"""Passes whose decoder layers run as one cooperative kernel (forward_persist.cu): what its sums of squares have to
+guarantee whatever the order of the CTAs."""
+import numpy as np
+import pytest
+import torch
+
+from tests.gpu_harness import make_setup, need_gpu
+from workload import configs, weights as W
+
+
+def layers_launches(b):
+    return b.tasc_launch_counts()["layers"]
+
+
+def a_step(b, s, host_tokens, drafts_h):
+    """A function that runs one verify step from the same committed state and returns its logits, and the workspace."""
+    B, P = host_tokens.shape
+    k = drafts_h.shape[1]
+    tokens = torch.zeros((B, P + 2 * (k + 1)), dtype=torch.int32, device="cuda")
+    length0 = torch.full((B,), P, dtype=torch.int32, device="cuda")
+    length = length0.clone()
+    pool, bt, kv = s.model.new_kv(B, tokens.shape[1] + b.MAX_ROWS)
+    ws = s.model.new_workspace(B, k)
+    tokens[:, :P] = torch.from_numpy(host_tokens).cuda()
+    drafts = torch.from_numpy(drafts_h).cuda()
+    seqs = b.make_seqs(tokens, length)
+    b.tasc_prefill(s.model, kv, seqs, B, P, ws)
+    b.tasc_poll_status(ws)
+
+    def step(keep=(pool, bt, tokens, length, drafts)):
+        length.copy_(length0)
+        return b.tasc_verify_step(s.model, kv, seqs, drafts, ws, want_logits=True)[3]
+    return step, ws
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,k", [(1, 5), (4, 3), (8, 5)])
+def test_sums_of_squares_do_not_depend_on_the_order_of_the_ctas(B, k):
+    """A residual row whose squares make any change of the order of the additions visible: one feature's square is a^2 in
+    [2^24, 2^25), one 1 (the middle between two floats), the other hundreds are 2^-34.  Added behind a^2 in double a CTA's few of
+    these vanish, among themselves they do not, and a^2 + 1 then rounds to the next float instead of back to a^2.  (The residual
+    projections are zero, so the row stays what it is.)  The step's logits must be the same bits every time -- and for the same
+    row times a power of two, which reaches every part of the sum's range, as long as the squares do not overflow."""
+    b = need_gpu()
+    cfg = configs.shrunk(configs.get(1), n_layers=4, vocab=512, n_docs=200)
+    d = cfg.model.d_model
+    f32 = np.float32
+
+    def factor(ss):
+        return f32(1) / np.sqrt(f32(f32(ss) * f32(f32(1) / f32(d)) + f32(cfg.model.rms_eps)))
+    a = next(v for v in range(4096, 5760, 32) if factor(v * v) != factor(v * v + 2))
+    w = W.make_weights(cfg.model, 0, gain_jitter=0.1)
+    row = np.full(d, 2.0 ** -17, dtype=f32)
+    row[:12] = 0.0
+    row[0], row[5] = a, 1.0
+    w["lm_head"] = w["lm_head"].copy()
+    for layer in w["layers"]:
+        layer["wo"] = np.zeros_like(layer["wo"])
+        layer["w_down"] = np.zeros_like(layer["w_down"])
+    rng = np.random.default_rng(2)
+    prompts, drafts = rng.integers(0, 512, (B, 3)).astype(np.int32), rng.integers(0, 512, (B, k)).astype(np.int32)
+    want = None
+    for power in (0, 7, 23, 40, 56):
+        w["embed"] = np.tile(row * f32(2.0) ** power, (cfg.model.vocab, 1))
+        s = make_setup(cfg, build_drafter=False, oracle_ngrams=False, host_w=w)
+        step, ws = a_step(b, s, prompts, drafts)
+        before = layers_launches(b)
+        first = step().clone()
+        assert layers_launches(b) == before + 1
+        different = sum(int(not torch.equal(step(), first)) for _ in range(40))
+        b.tasc_poll_status(ws)
+        assert different == 0, f"2^{power}: {different} of 40 repetitions differ"
+        want = first if want is None else want
+        assert bool((first == 0).all()) if power == 56 else torch.equal(first, want), f"2^{power}"
