@@ -1,5 +1,5 @@
-"""Passes whose decoder layers run as one cooperative kernel (forward_persist.cu): what its sums of squares have to
-guarantee whatever the order of the CTAs."""
+"""Passes whose decoder layers run as one cooperative kernel (forward_persist.cu): what its grid barriers and its sums of
+squares have to guarantee whatever else the GPU does."""
 import numpy as np
 import pytest
 import torch
@@ -31,6 +31,26 @@ def a_step(b, s, host_tokens, drafts_h):
         length.copy_(length0)
         return b.tasc_verify_step(s.model, kv, seqs, drafts, ws, want_logits=True)[3]
     return step, ws
+
+
+@pytest.mark.gpu
+def test_a_kernel_of_another_stream_that_holds_an_sm_is_waited_for():
+    """The layers need an SM each to themselves, all at once.  While another stream's kernel holds one for about 1.3 s (longer
+    than a barrier's limit within a pass), the step has to wait for it like any other launch: no time-out, same logits."""
+    b = need_gpu()
+    cfg = configs.shrunk(configs.get(1), n_layers=2, vocab=4096, n_docs=200)
+    s = make_setup(cfg, build_drafter=False, oracle_ngrams=False)
+    rng = np.random.default_rng(1)
+    step, ws = a_step(b, s, rng.integers(0, 4096, (1, 40)).astype(np.int32), rng.integers(0, 4096, (1, 5)).astype(np.int32))
+    before = layers_launches(b)
+    want = step().cpu().numpy()
+    assert layers_launches(b) == before + 1
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(2_500_000_000)
+    got = step()
+    b.tasc_poll_status(ws)
+    assert np.array_equal(got.cpu().numpy(), want)
 
 
 @pytest.mark.gpu
