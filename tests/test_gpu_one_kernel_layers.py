@@ -1,11 +1,14 @@
-"""Passes whose decoder layers run as one cooperative kernel (forward_persist.cu): what its grid barriers and its sums of
-squares have to guarantee whatever else the GPU does."""
+"""Passes whose decoder layers run as one cooperative kernel (forward_persist.cu): which ones those are, parity at the sizes of its
+token blocks, and what its grid barriers and its sums of squares have to guarantee whatever else the GPU does."""
+from dataclasses import replace
+
 import numpy as np
 import pytest
 import torch
 
-from tests.gpu_harness import make_setup, need_gpu
-from workload import configs, weights as W
+from tests.gpu_harness import lockstep, make_setup, need_gpu
+from tests.test_gpu_verify import BF16_TOL, check
+from workload import configs, corpus, weights as W
 
 
 def layers_launches(b):
@@ -92,3 +95,72 @@ def test_sums_of_squares_do_not_depend_on_the_order_of_the_ctas(B, k):
         assert different == 0, f"2^{power}: {different} of 40 repetitions differ"
         want = first if want is None else want
         assert bool((first == 0).all()) if power == 56 else torch.equal(first, want), f"2^{power}"
+
+
+def shape_of(hd, n_layers):
+    """Configuration 1's shape, or one with heads of 128."""
+    cfg = configs.shrunk(configs.get(1), n_layers=n_layers, vocab=4096, n_docs=500)
+    if hd == 128:
+        cfg = replace(cfg, model=replace(cfg.model, d_model=512, n_q_heads=4, n_kv_heads=2, head_dim=128, d_ff=1088))
+    return cfg
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("hd", [64, 128])
+@pytest.mark.parametrize("B,k,P", [(11, 2, 40), (5, 6, 130), (8, 5, 200), (7, 8, 33), (16, 3, 70)])
+def test_two_blocks_of_32_rows(B, k, P, hd):
+    """33, 35, 48, 63 and 64 rows: a second block of token rows with one row, some, or all of them in use.  Two layers; the oracle
+    runs the first, a middle and the last sequence."""
+    b = need_gpu()
+    cfg = replace(shape_of(hd, 2), prompt_len=P)
+    s = make_setup(cfg)
+    prompts = corpus.make_prompts(cfg, B, prompt_len=P)
+    before = layers_launches(b)
+    rep = lockstep(s, prompts, k + 3, k, oracle_rows=sorted({0, B // 2, B - 1}), **BF16_TOL)
+    assert layers_launches(b) - before >= rep.steps
+    check(rep, f"two blocks of 32 rows, heads of {hd}, B={B} k={k} P={P}")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,k", [(1, 5), (4, 3), (7, 8)])
+def test_a_step_is_bitwise_repeatable(B, k):
+    """6, 16 and 63 rows behind 300 tokens, four layers: split key ranges and their merge included."""
+    b = need_gpu()
+    s = make_setup(shape_of(64, 4), build_drafter=False, oracle_ngrams=False)
+    rng = np.random.default_rng(4)
+    step, ws = a_step(b, s, rng.integers(0, 4096, (B, 300)).astype(np.int32), rng.integers(0, 4096, (B, k)).astype(np.int32))
+    before = layers_launches(b)
+    want = step().clone()
+    assert layers_launches(b) == before + 1
+    for _ in range(10):
+        assert torch.equal(step(), want)
+    b.tasc_poll_status(ws)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,k", [(2, 5), (7, 6)])
+def test_generate_graph_replay_equals_plain_enqueue(B, k):
+    """tasc_generate with its step replayed from a graph (a side stream) and enqueued (the default stream), steps of 12 and 49
+    rows: the same tokens and statistics."""
+    b = need_gpu()
+    cfg = shape_of(64, 4)
+    s = make_setup(cfg, oracle_ngrams=False)
+    max_new = 30
+    prompts = corpus.make_prompts(cfg, B, prompt_len=100)
+    results = []
+    for side in (False, True):
+        tokens = torch.zeros((B, 100 + max_new + k + 2), dtype=torch.int32, device="cuda")
+        tokens[:, :100] = torch.from_numpy(prompts).cuda()
+        length = torch.full((B,), 100, dtype=torch.int32, device="cuda")
+        pool, bt, kv = s.model.new_kv(B, tokens.shape[1] + b.MAX_ROWS)
+        ws = s.model.new_workspace(B, k)
+        stream = torch.cuda.Stream() if side else torch.cuda.current_stream()
+        stream.wait_stream(torch.cuda.current_stream())
+        before = layers_launches(b)
+        with torch.cuda.stream(stream):
+            out, st = b.tasc_generate(s.model, s.drafter, kv, b.make_seqs(tokens, length), B, max_new, k, ws)
+        torch.cuda.current_stream().wait_stream(stream)
+        assert layers_launches(b) > before
+        results.append((out.cpu().numpy(), st.steps, list(st.accepted_hist)))
+    assert np.array_equal(results[0][0], results[1][0])
+    assert results[0][1:] == results[1][1:]

@@ -424,9 +424,10 @@ def test_many_row_kernel_on_every_product_with_64_wide_heads():
 @pytest.mark.parametrize("hd", [64, 128])
 @pytest.mark.parametrize("B,k,P", [(1, 1, 2), (1, 7, 127), (1, 8, 128), (2, 7, 129), (3, 5, 40), (8, 3, 200), (8, 7, 33), (1, 5, 1600)])
 def test_one_kernel_for_all_layers(B, k, P, hd):
-    """Passes whose layers run as one kernel: 2 to 64 rows (one, two and four tiles of 8, full and ragged), contexts that
-    end just before, at and just behind a tile of 128 keys, one key range and as many as there can be; heads of 64 and
-    of 128.  Two layers; the oracle runs the first and the last sequence."""
+    """Passes whose layers run as one kernel: 2, 6, 8, 9, 16 and 64 rows (one, two and four tiles of 8, full and ragged; more of
+    them in test_gpu_one_kernel_layers.py), contexts that end just before, at and just behind a tile of 128 keys, one key range
+    and as many as there can be; heads of 64 and of 128.  The 18 and 32 rows next to them run as five kernels per layer.  Two
+    layers; the oracle runs the first and the last sequence."""
     from dataclasses import replace
     cfg = replace(configs.shrunk(configs.get(1), n_layers=2, vocab=4096, n_docs=500), prompt_len=P)
     if hd == 128:
