@@ -244,22 +244,31 @@ tasc_status forward_f32(const tasc_model* m, const tasc_kv* kv, const Workspace&
     return TASC_OK;
 }
 
-// Whether the layers of a pass run as one persistent kernel (forward_persist.cu).  Its phases cost about 2.5 us less than
-// kernels of their own, but a CTA reads the activations of all its token rows itself, so what it loses grows with rows
-// times width.  A step in us, five kernels per layer against one kernel:
-//     rows            7 MB per layer (135M)      30 MB (0.5B)             94 MB (1.5B)
-//     up to 8         798 / 578 - 818 / 591      897 / 652 - 940 / 702    1350 / 1122 - 1419 / 1172
-//     9 - 16          782 / 620 - 811 / 628      763 / 819 - 788 / 831    1235 / 1688
-//     17 - 32         784 / 773 - 823 / 796      795 / 976                -
-//     33 - 64         920 / 813 - 858 / 824      920 / 1215               -
-//     96, 380 keys    1033 / 1077                -                        -
-// Replayed from a graph the five kernels per layer follow one another more closely: 701 / 750 at 18 rows and 753 / 780 at 32
-// (7 MB), the rest as above; the one kernel's time hardly changes between 17 and 64 rows (blocks of 32).
-// Its attention has at most one unit per SM and 12 key ranges, so the keys of a unit are bounded too (94 MB per layer, one
-// sequence of 4,000 tokens: 1559 / 1427 at 341 keys per unit).
+// Whether the layers of a pass that forward_persist.cu can take run as its one persistent kernel.  Its phases cost about 2.5 us
+// less than kernels of their own, but a CTA reads the activations of all its token rows itself, so what it loses grows with rows
+// times width.  A step in us, enqueued / replayed from a graph (where the five kernels per layer follow one another more closely):
+//     rows   7 MB per layer (135M)            30 MB (0.5B)                     94 MB (1.5B)
+//            five kernels   one kernel        five kernels   one kernel        five kernels   one kernel
+//       7                                                                      1213 / 1140    1144 / 1137
+//       6    747 / 669      594 / 586         746 / 689      650 / 640
+//       8    768 / 681      601 / 592         740 / 662      643 / 635         1223 / 1141    1132 / 1123
+//      12    791 / 694      622 / 613         762 / 686      804 / 793         1226 / 1151    1665 / 1657
+//      16    791 / 691      624 / 614         759 / 698      804 / 794         1259 / 1190    1681 / 1672
+//      18    816 / 709      758 / 749
+//      24    801 / 731      758 / 748
+//      32    822 / 744      769 / 761         795 / 729      955 / 948 (28)
+//      33    883 / 802      795 / 787
+//      48    936 / 869      849 / 838         905 / 850      1197 / 1187
+//      64    889 / 818      830 / 819
+//      96    965 / 898      1052 / 1042
+// (270 - 380, 560 and 1,071 keys).  The one kernel's time hardly changes between 17 and 32 rows and between 33 and 64 (blocks of
+// 32); a generation replays, so 17 to 32 rows are not its (plan_persist).
+// Its attention has at most one unit per SM and 12 key ranges, so the bytes of a unit's keys are bounded too, by 512 keys of 64:
+//     1.5B, 7 rows    1,500 keys 1235 / 1155, 1160 / 1150   3,000 (250 per unit) 1357 / 1273, 1296 / 1288   3,600 1340 / 1266, 1357 / 1348
+//     135M, 48 rows   1,500 (500 per unit) 1100 / 1010, 1070 / 1061                                         4,000 1385 / 1290, 1676 / 1666
 bool persist_pays(const tasc_model* m, int M, int max_ctx, const PersistPlan& pp) {
-    if (max_ctx / pp.splits > 512) return false;
-    return M <= 8 || (m->layer_mb <= 12.0 && (M <= 16 || (M > 32 && M <= 64)));
+    if (max_ctx / pp.splits * m->desc.head_dim > 512 * 64) return false;
+    return M <= 8 || m->layer_mb <= 12.0;
 }
 
 // bf16 models: five launches per layer (QKV+RoPE+KV append, attention, O+residual, gate/up+SiLU*mul, down+residual),

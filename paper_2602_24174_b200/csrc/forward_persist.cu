@@ -27,8 +27,8 @@
 // the warps splitting the head's columns.  K and V are staged by cp.async; the committed positions' are requested before
 // the barrier.  Key ranges of one group are merged by the CTA that finishes last, in range order.
 //
-// Measured (one verify step, five kernels per layer before, this kernel now): 135M at 6 rows 797 -> 583 us, 0.5B at 6 rows
-// 897 -> 652, 1.5B at 7 rows 1415 -> 1172.  What is left is the barrier and the first fresh read behind it, about 2.4 us
+// Measured (one verify step, five kernels per layer / this kernel): 135M at 6 rows 747 / 594 us, 0.5B at 6 rows 746 / 650, 1.5B
+// at 7 rows 1213 / 1144; more of it at persist_pays.  What is left is the barrier and the first fresh read behind it, about 2.4 us
 // for each of the five phases (of 3.0 per phase at 135M, of 6.9 at 1.5B, where streaming the weights is the larger part).
 //
 // Every wait is bounded: a barrier that is not reached in about half a second records TASC_ETIMEOUT and the CTA
@@ -971,6 +971,7 @@ bool plan_persist(int n_layers, int M, int B, int R, int d, int qd, int n_q, int
         }
         p.grid = sms[dev];
     }
+    if (M > 16 && M <= 32) return false;             // (one block of four tiles: slower than kernels per phase, see persist_pays)
     p.T = M <= 8 ? 1 : (M <= 16 ? 2 : 4);
     p.n_tb = (M + p.T * 8 - 1) / (p.T * 8);
     p.n_rb = p.grid / p.n_tb;

@@ -122,6 +122,23 @@ def test_two_blocks_of_32_rows(B, k, P, hd):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("which,B,k,P,one", [(1, 1, 1, 20, 1), (1, 2, 7, 20, 1), (1, 3, 5, 20, 0), (1, 8, 3, 20, 0), (1, 11, 2, 20, 1), (1, 16, 3, 20, 1),
+                                             (1, 13, 4, 20, 0), (2, 2, 3, 20, 1), (2, 3, 2, 20, 0), (4, 1, 6, 3030, 1), (4, 1, 6, 3100, 0)])
+def test_which_steps_run_their_layers_as_one_kernel(which, B, k, P, one):
+    """2, 16, 18, 32, 33, 64 and 65 rows of the small layers, 8 and 9 of larger ones, and heads of 128 with 12 key ranges of 256 and
+    of more keys."""
+    b = need_gpu()
+    cfg = replace(configs.shrunk(configs.get(which), n_layers=1, vocab=512, n_docs=100), prompt_len=P)
+    s = make_setup(cfg, build_drafter=False, oracle_ngrams=False)
+    rng = np.random.default_rng(3)
+    step, ws = a_step(b, s, rng.integers(0, 512, (B, P)).astype(np.int32), rng.integers(0, 512, (B, k)).astype(np.int32))
+    before = layers_launches(b)
+    step()
+    b.tasc_poll_status(ws)
+    assert layers_launches(b) - before == one
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("B,k", [(1, 5), (4, 3), (7, 8)])
 def test_a_step_is_bitwise_repeatable(B, k):
     """6, 16 and 63 rows behind 300 tokens, four layers: split key ranges and their merge included."""
