@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
     float* part = xs + (size_t)((M + ROWS - 1) / ROWS * ROWS) * a.width;                      // [WARPS][hd + 4] attention states
     int* s_pos = reinterpret_cast<int*>(part + WARPS * (hd + 4));
     int* s_tok = s_pos + M;
-    unsigned long long* s_best = reinterpret_cast<unsigned long long*>(s_tok + M + ((M + M) & 1));
+    unsigned long long* s_best = reinterpret_cast<unsigned long long*>(s_tok + M);
 
     // ---- row plan: every CTA for itself, CTA 0 for the kernels behind
     for (int m = threadIdx.x; m < M; m += THREADS) {
