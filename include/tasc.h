@@ -14,8 +14,10 @@
  *     in a status word inside the caller's workspace and read by
  *     tasc_poll_status, which synchronises the stream.
  *   - The caller owns weights, KV pool, block table, token buffers and the
- *     workspace.  The library owns only what tasc_drafter_build and
- *     tasc_model_create allocate, released by the matching destroy call.
+ *     workspace.  The library owns what the calls that return a tasc_drafter and
+ *     tasc_model_create allocate, released by the matching destroy call, and per
+ *     device up to 2 GB that the set-up calls (corpus tables, statistics,
+ *     tokenizer) keep for the next one: see tasc_scratch_release.
  *   - Token ids are int32, document offsets int64.
  */
 #ifndef TASC_H
@@ -71,8 +73,9 @@ typedef struct {
  *   vocab          <= 2^TASC_VOCAB_BITS
  *   out            host; receives a handle owning device tables (tasc_drafter_destroy)
  * Device memory: the tables the handle owns (about 40 bytes per surviving element), and, while the call runs,
- * a counting table of 2^ceil(log2(2 W)) slots of 20 bytes, W = the windows of order 1 (tokens minus documents), plus
- * one byte per token -- about 5.4 GB for a corpus of 110 M tokens; freed before the call returns.
+ * a counting table of 1.25 W slots of 16 bytes, W = the windows of order 1 (tokens minus documents), 9 bytes per
+ * token and 16 bytes for every p_min-th window -- about 3.5 GB for a corpus of 110 M tokens with p_min = 5; given back
+ * before the call returns (blocks of up to 1 GB to the library's pool, see tasc_scratch_release).
  * Synchronises the stream before returning.  Errors: EINVAL, ENOMEM, ECUDA,
  * ECAPACITY (internal table overflow; not expected for valid input).
  */
@@ -162,8 +165,8 @@ typedef struct {
  *   cdf_num / cdf_den   coverage target of bigrams_for_cdf (the paper's 80 % = 4 / 5); 1 <= cdf_num <= cdf_den <= 65536
  *   out                 host (written)
  * Counting and the reductions run on the device; the integer fields are exact and, like the entropies, do not depend
- * on thread timing.  Allocates transient device memory (about 40 bytes per bigram occurrence plus 8 MiB) and frees it
- * before returning; synchronises the stream.  The corpus must hold fewer than 2^40 tokens.
+ * on thread timing.  Allocates transient device memory (about 21 bytes per bigram occurrence plus 8 MiB) and gives it
+ * back before returning; synchronises the stream.  A corpus of 2^32 - 1 tokens or more, or of 3.4e9 bigrams: ENOMEM.
  * Errors: EINVAL, ENOMEM, ECUDA, ECAPACITY (more than 4,096 distinct bigrams or tokens occurring 2^20 times or more).
  */
 tasc_status tasc_corpus_stats(const int32_t* corpus_tokens, const int64_t* doc_offsets, int64_t n_docs, int32_t vocab,
@@ -187,8 +190,9 @@ tasc_status tasc_corpus_stats(const int32_t* corpus_tokens, const int64_t* doc_o
  *   n_merges      host (written): additions made
  *   tokens_out    device, int32[doc_offsets[n_docs]] (written): the corpus in the enriched vocabulary, compacted
  *   offsets_out   device, int64[n_docs + 1] (written)
- * Every round recounts the whole corpus: the cost is budget x corpus size, so select on a sample of the corpus.
- * Allocates transient device memory (about 50 bytes per n-gram window) and frees it; synchronises the stream.
+ * The counts are kept over the rounds: a round reads the corpus once for the new token's occurrences, recounts the windows
+ * around them, and looks again at the parts of the count table that this changed.
+ * Allocates transient device memory (40 to 80 bytes per n-gram window, 14 per token) and gives it back; synchronises the stream.
  * Errors: EINVAL, ENOMEM, ECUDA, ECAPACITY.
  */
 tasc_status tasc_tok_enrich(const int32_t* corpus_tokens, const int64_t* doc_offsets, int64_t n_docs, int32_t base_vocab,
@@ -366,6 +370,14 @@ tasc_status tasc_bigram_table(const tasc_model* m, const tasc_kv* kv, int32_t B,
 
 /* Synchronise the stream and return the device status word of the workspace (TASC_OK if clean); clears it. */
 tasc_status tasc_poll_status(void* workspace, tasc_stream stream);
+
+/*
+ * Gives back to the device what the library's pool on the current device holds beyond the blocks in use.  The set-up calls
+ * take their transient memory, and the tables of a drafter, from that pool in blocks of up to 1 GB; between calls it keeps
+ * up to 2 GB (a first allocation from the driver costs more than most of these calls).  tasc_model_create and
+ * tasc_model_destroy do the same.  Synchronises the device; not during a stream capture.  Errors: ECUDA.
+ */
+tasc_status tasc_scratch_release(void);
 
 /*
  * Failure-path self-test.  Every device-side wait of the library (TMA arrival, MMA completion, ring slots) is

@@ -447,7 +447,7 @@ extern "C" tasc_status tasc_model_create(const tasc_model_desc* desc, const tasc
     if (!out) return TASC_EINVAL;
     *out = nullptr;
     if (!desc || !wt) return TASC_EINVAL;
-    scratch_trim();                                  // a program that makes a model has better uses for the memory
+    (void)scratch_trim();                            // a program that makes a model has better uses for the memory
     const tasc_model_desc& d = *desc;
     if (d.n_layers < 1 || d.d_model < 8 || d.n_q_heads < 1 || d.n_kv_heads < 1 || d.n_q_heads % d.n_kv_heads ||
         d.head_dim < 8 || d.head_dim > 256 || d.head_dim % 8 || d.d_ff < 8 || d.vocab < 2 ||
@@ -543,7 +543,7 @@ extern "C" tasc_status tasc_model_create(const tasc_model_desc* desc, const tasc
 
 extern "C" tasc_status tasc_model_destroy(tasc_model* m) {
     if (!m) return TASC_EINVAL;
-    scratch_trim();
+    (void)scratch_trim();
     if (m->rope) cudaFree(m->rope);
     delete m;
     return TASC_OK;

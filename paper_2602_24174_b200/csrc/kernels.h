@@ -21,7 +21,7 @@ struct ProfScope {
 // Memory for work on `stream`; a block is freed in that stream's order, or after it on any stream of an idle device.
 bool scratch_alloc(void** p, size_t bytes, cudaStream_t stream, bool* pooled);
 void scratch_free(void* p, cudaStream_t stream, bool pooled);
-void scratch_trim();                           // gives back what the current device's pool holds
+tasc_status scratch_trim();                    // gives back what the current device's pool holds
 
 // Parts laid out one behind the other in one block, which is freed with the object (on the stream given then).
 class DeviceSlab {

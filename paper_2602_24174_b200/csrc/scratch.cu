@@ -53,7 +53,7 @@ bool scratch_alloc(void** p, size_t bytes, cudaStream_t stream, bool* pooled) {
     *pooled = false;
     if (cudaMalloc(p, bytes) == cudaSuccess) return true;
     (void)cudaGetLastError();
-    scratch_trim();                                  // what the pool holds may be what is missing
+    (void)scratch_trim();                            // what the pool holds may be what is missing
     if (cudaMalloc(p, bytes) == cudaSuccess) return true;
     (void)cudaGetLastError();
     *p = nullptr;
@@ -65,11 +65,17 @@ void scratch_free(void* p, cudaStream_t stream, bool pooled) {
     if (!(pooled ? cudaFreeAsync(p, stream) == cudaSuccess : cudaFree(p) == cudaSuccess)) (void)cudaGetLastError();
 }
 
-void scratch_trim() {
+tasc_status scratch_trim() {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) { (void)cudaGetLastError(); return; }
+    TASC_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= MAX_DEVICES) return TASC_OK;
     std::lock_guard<std::mutex> lk(pool_mu);
-    if (pools[dev] && cudaMemPoolTrimTo(pools[dev], 0) != cudaSuccess) (void)cudaGetLastError();
+    if (!pools[dev]) return TASC_OK;
+    TASC_CUDA_TRY(cudaDeviceSynchronize());          // a block whose turn to be freed has not come is one in use
+    TASC_CUDA_TRY(cudaMemPoolTrimTo(pools[dev], 0));
+    return TASC_OK;
 }
 
 }  // namespace tasc
+
+extern "C" tasc_status tasc_scratch_release(void) { return tasc::scratch_trim(); }
