@@ -106,6 +106,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     const int sp = blockIdx.x, kh = blockIdx.y, b = blockIdx.z / a.n_sub, rb = (blockIdx.z % a.n_sub) * a.Rs;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = a.n_q / a.n_kv, R = a.Rs, G = g * R, h0 = kh * g, qd = a.n_q * HD;
+#ifdef TASC_TIMELINE
+    struct LogAtExit { unsigned long long t0, ta, tb, tc, td; __device__ ~LogAtExit() { if (threadIdx.x == 0) ctalog_put(t0, ta, tb, 11, tc, td); } } log_at_exit{global_ns(), 0, 0, 0, 0};
+#endif
     // (the row plan, the block table and the committed K / V were written before the preceding grid started)
     const int seq_pos0 = a.seq_pos0[b];
     int rows = a.seq_rows[b] - rb;
@@ -275,6 +278,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     } else {
         // ------------------------------------------------------------ softmax
         griddep_wait();
+#ifdef TASC_TIMELINE
+        log_at_exit.ta = global_ns();
+#endif
         griddep_launch_dependents();
         // Q rows, scaled, as (hi, lo) in shared memory; zeros where there is no row
         {
@@ -300,6 +306,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
             fence_proxy_async_smem();
             mbar_arrive(bar_q_full);
         }
+#ifdef TASC_TIMELINE
+        log_at_exit.tc = global_ns();
+#endif
 #pragma unroll
         for (int e = 0; e < OC; ++e) acc[e] = 0.f;
         if (active) {
@@ -324,6 +333,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
             for (int t = 0; t < n_tiles; ++t) {
                 float s[SC];
                 wait(bar_s_full + 8u * (t & 1), (uint32_t)(t >> 1) & 1u);
+#ifdef TASC_TIMELINE
+                if (t == 0) log_at_exit.td = global_ns();
+#endif
                 tc_fence_after();
 #pragma unroll
                 for (int c = 0; c < SC; c += 32) {
@@ -377,6 +389,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
             l_run += s_sum[half ^ 1][rho];
         }
     }
+#ifdef TASC_TIMELINE
+    log_at_exit.tb = global_ns();
+#endif
     // no copy and no MMA is under way any more (after a failure: give the copies a bounded time to land)
     tc_fence_before();
     __syncthreads();

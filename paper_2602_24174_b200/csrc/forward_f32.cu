@@ -32,6 +32,15 @@ constexpr int MAX_HD = 256;
 constexpr int MAX_SMEM = 220 * 1024;
 
 __device__ __forceinline__ void cluster_sync_all() { cluster_arrive(); cluster_wait(); }
+#ifdef TASC_TIMELINE
+// A stage of a CTA: start, rows staged, work done, behind the barrier.
+#define TL_STAGED() (tl_a = global_ns())
+#define TL_END(tag) do { if (threadIdx.x == 0) ctalog_put(tl_0, tl_a, tl_b, tag); tl_0 = tl_a = global_ns(); } while (0)
+#define TL_SYNC(tag) do { tl_b = global_ns(); cluster_sync_all(); TL_END(tag); } while (0)
+#else
+#define TL_STAGED() do { } while (0)
+#define TL_SYNC(tag) cluster_sync_all()
+#endif
 
 // Sums of eight values over the warp's lanes; lane l gets the sum of value l / 4.
 __device__ __forceinline__ float sum8(float (&v)[ROWS]) {
@@ -83,6 +92,9 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
     int* s_tok = s_pos + M;
     unsigned long long* s_best = reinterpret_cast<unsigned long long*>(s_tok + M);
 
+#ifdef TASC_TIMELINE
+    unsigned long long tl_0 = global_ns(), tl_a = tl_0, tl_b = tl_0;
+#endif
     // ---- row plan: every CTA for itself, CTA 0 for the kernels behind
     for (int m = threadIdx.x; m < M; m += THREADS) {
         const int b = m / a.R, r = m % a.R, L = a.len[b];
@@ -139,10 +151,12 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
             }
         }
         __syncthreads();
+        TL_STAGED();
     };
     auto stage_rows = [&](const float* src, int K) {
         for (int i = threadIdx.x; i < M * (K / 4); i += THREADS) *reinterpret_cast<float4*>(xs + 4 * (size_t)i) = ldg_fresh(src + 4 * (size_t)i);
         __syncthreads();
+        TL_STAGED();
     };
     // n_pairs pairs of weight rows; emit(pair, token row, dot with the first, dot with the second), one lane per value
     auto product = [&](int n_pairs, int K, auto row0, auto row1, auto emit) {
@@ -203,7 +217,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
                     dst[i] = v0;
                     dst[i + half] = v1;
                 });
-        cluster_sync_all();
+        TL_SYNC(40);
         // ---- attention: unit = (token row, query head)
         const int n_units = M * a.n_q, g = a.n_q / a.n_kv, sub = warp / UNIT_WARPS, sw = warp % UNIT_WARPS;
         for (int u0 = cta; u0 < n_units; u0 += CTAS * (WARPS / UNIT_WARPS)) {
@@ -271,20 +285,20 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
             }
             __syncthreads();
         }
-        cluster_sync_all();
+        TL_SYNC(41);
         // ---- O
         stage_rows(a.o, qd);
         residual(lw.wo, qd);
-        cluster_sync_all();
+        TL_SYNC(42);
         // ---- gate / up
         stage_norm(lw.mlp_norm, false);
         product(a.dff, d, [&](int p) { return lw.w_gate_up + (size_t)p * d; }, [&](int p) { return lw.w_gate_up + (size_t)(a.dff + p) * d; },
                 [&](int p, int m, float g0, float u) { a.act[(size_t)m * a.dff + p] = g0 / (1.0f + expf(-g0)) * u; });
-        cluster_sync_all();
+        TL_SYNC(43);
         // ---- down
         stage_rows(a.act, a.dff);
         residual(lw.w_down, a.dff);
-        cluster_sync_all();
+        TL_SYNC(44);
     }
     if (!a.lm_head) return;
     stage_norm(a.final_norm, false);
@@ -300,7 +314,13 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
                 }
             });
     __syncthreads();
+#ifdef TASC_TIMELINE
+    tl_b = global_ns();
+#endif
     for (int m = threadIdx.x; m < M; m += THREADS) atomicMax(&a.argmax[m], s_best[m]);
+#ifdef TASC_TIMELINE
+    TL_END(45);
+#endif
 }
 
 size_t smem_bytes(int M, int width, int hd) {

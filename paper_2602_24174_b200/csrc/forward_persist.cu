@@ -178,12 +178,30 @@ struct Shared {
     int stop;                          // a wait ran out
     int last;                          // this CTA merges the key ranges
     Unit unit;                         // the current attention unit
+#ifdef TASC_TIMELINE
+    unsigned long long tl[3];          // a phase of this CTA: start, past the barrier, products or key tiles done
+#endif
     int pg[MAX_PAGES];                 // first pool rows of the pages of its key range, -1 outside the pool
 };
 constexpr int SHARED_BYTES = (sizeof(Shared) + 1023) / 1024 * 1024;
 extern __shared__ __align__(1024) uint8_t dyn_smem[];
 __device__ __forceinline__ Shared& sh() { return *reinterpret_cast<Shared*>(dyn_smem); }
 __device__ __forceinline__ uint8_t* un() { return dyn_smem + SHARED_BYTES; }       // union: parked tiles / attention buffers
+
+#ifdef TASC_TIMELINE
+__device__ __forceinline__ void tl_stamp(int i) { if (threadIdx.x == 0) sh().tl[i] = global_ns(); }
+__device__ __forceinline__ void tl_phase(int j) {
+    if (threadIdx.x != 0) return;
+    ctalog_put(sh().tl[0], sh().tl[1], sh().tl[2] ? sh().tl[2] : sh().tl[1], 30 + j);
+    sh().tl[2] = 0;
+    sh().tl[0] = global_ns();
+}
+#define TL_STAMP(i) tl_stamp(i)
+#define TL_PHASE(j) tl_phase(j)
+#else
+#define TL_STAMP(i) do { } while (0)
+#define TL_PHASE(j) do { } while (0)
+#endif
 
 // Grid barrier: arrival number `epoch` of every CTA completes barrier `epoch`.
 __device__ __forceinline__ void grid_arrive(const PersistArgs& a) {
@@ -376,6 +394,7 @@ struct Cta {
             }
         }
         if (!grid_wait(a, epoch)) return false;
+        TL_STAMP(1);
         if (n_tiles == 0) return true;
         auto load_b = [&](auto first, auto uc, bool ok) {
             constexpr int u = decltype(uc)::value;
@@ -454,6 +473,7 @@ struct Cta {
                 }
             }
             __syncthreads();
+            TL_STAMP(2);
             const int n_items = items_of(tile1 - tile0) << lp;
             if (tile0 > 0) it = decode(ph, tid, lp, tile0, red, stride, u0, u1, m0);
 #pragma unroll 1
@@ -612,6 +632,7 @@ struct Cta {
         };
         place();
         if (!grid_wait(a, epoch)) { cp_async_wait<0>(); return false; }
+        TL_STAMP(1);
 #pragma unroll 1
         for (; u < a.n_units; u += gridDim.x) {
             if (u != (int)blockIdx.x) { prepare_unit(u); from = q.k0; place(); }        // (its barriers: the previous unit's tiles are no longer read)
@@ -783,6 +804,7 @@ struct Cta {
                     if (warp == 0 && t == 0) *reinterpret_cast<float2*>(part + 16 * HD + row * 2) = make_float2(m_run[hf], L);
                 }
             }
+            TL_STAMP(2);
             if (a.splits > 1) merge();
         }
         return true;
@@ -901,6 +923,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) layers_kernel(const __grid_cons
         const int f = sh().part[1][0] + tile * 16 + row, m = m0 + tt * 8 + n;
         c.xs()[i] = f < sh().part[1][1] && m < a.M ? a.x0[(size_t)m * a.d + f] : 0.f;
     }
+#ifdef TASC_TIMELINE
+    if (tid == 0) { sh().tl[0] = global_ns(); sh().tl[2] = 0; }
+#endif
     grid_arrive(a);                                               // (also makes the shared arrays visible to the CTA)
     // (one call of each routine: the layer loop has to stay within the instruction caches -- measured, an SM fetches code
     // that is not in its 32 KB cache at about five cycles per instruction, which is more than a phase's work)
@@ -914,10 +939,11 @@ __global__ void __launch_bounds__(WARPS * 32, 1) layers_kernel(const __grid_cons
                 if (!c.attention(kp, kp + a.kv_half)) return;
             } else {
                 if (!c.project(sh().phase[slot], l + (j == 4), j == 0 ? 2 : j == 4 ? 0 : j + 1, sh().phase[slot ^ 1])) return;
-                if (l + 1 == a.n_layers && j == 4) return;
+                if (l + 1 == a.n_layers && j == 4) { TL_PHASE(j); return; }
                 slot ^= 1;
             }
             grid_arrive(a);
+            TL_PHASE(j);
             ++c.epoch;
         }
     }

@@ -3,11 +3,12 @@
     python -m paper_2602_24174_b200.build --timeline
     python -m paper_2602_24174_b200.timeline --config 1 --batch 16
 
-The instrumented library (same sources, -DTASC_TIMELINE) appends one record per CTA of the fused GEMM and the
-attention kernels: start, end and up to six intermediate stamps on the GPU's global nanosecond timer.  One step
-(draft + verify) is captured in a CUDA graph, replayed, and the records are grouped into kernels; for every kind
-of kernel the table gives the time from the end of its predecessor to its own end ("period", the kernel's share
-of the step's critical path) and where it goes.  Synthetic seeded inputs; a development aid, not a benchmark.
+The instrumented library (same sources, -DTASC_TIMELINE) appends one record per CTA of the GEMM and the attention
+kernels, and one per CTA and phase where all layers are one kernel: start, end and up to six intermediate stamps on the
+GPU's global nanosecond timer.  One step (draft + verify) is captured in a CUDA graph, replayed, and the records are
+grouped into kernels (or phases); for every kind the table gives the time from the end of its predecessor to its own
+end ("period", the kernel's share of the step's critical path) and where it goes.  The stamps cost time themselves,
+about 1 us per kernel or phase.  Synthetic seeded inputs; a development aid, not a benchmark.
 """
 from __future__ import annotations
 
@@ -24,7 +25,10 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
-NAMES = {0: "plain", 1: "qkv", 2: "resid", 3: "swiglu", 4: "lm", 10: "attn"}
+NAMES = {0: "plain", 1: "qkv", 2: "resid", 3: "swiglu", 4: "lm", 10: "attn", 11: "attn tc",
+         20: "wide plain", 21: "wide qkv", 22: "wide resid", 23: "wide swiglu", 24: "wide lm",
+         30: "1k qkv", 31: "1k attn", 32: "1k o", 33: "1k gate/up", 34: "1k down",
+         40: "f32 qkv", 41: "f32 attn", 42: "f32 o", 43: "f32 gate/up", 44: "f32 down", 45: "f32 lm"}
 
 
 def main():
@@ -109,20 +113,28 @@ def main():
         a["period"] += end - us(prev_end); a["lag"] += wait - us(prev_end); a["main"] += acc - wait; a["tail"] += end - acc
         a["lead_first"] += us(prev_end) - us(t0[ix].min()); a["lead_last"] += us(prev_end) - us(t0[ix].max())
         st = [us(x[ix].max()) for x in tx]
-        if tg == 10:
+        if tg in (10, 11):
             a["p0"] += st[0] - wait; a["p1"] += st[1] - st[0]; a["p2"] += acc - st[1]
-        else:
+        elif tg < 30 and all((x[ix] > 0).all() for x in tx):       # (the persistent tiles of the many-row kernel have no such phases)
+            a["detail"] = 1
             a["p0"] += st[0] - acc; a["p1"] += st[1] - st[0]; a["p2"] += st[2] - st[1]; a["p3"] += st[3] - st[2]; a["p4"] += end - st[3]
         prev_end = t1[ix].max()
-    print("kind     n   CTAs | period = wait lag + main + tail   (us, means)   | detail")
+    print("kind          n   CTAs | period = wait lag + main + tail   (us, means)   | detail")
     for name, a in agg.items():
         c = a["n"]
-        if name == "attn":
-            det = f"Q staged {a['p0']/c:.2f}, first tiles landed {a['p1']/c:.2f}, tile loop {a['p2']/c:.2f}; tail = merge/write + exit"
-        else:
+        if name in ("attn", "attn tc"):
+            first = "first tiles landed" if name == "attn" else "first scores"
+            det = f"Q staged {a['p0']/c:.2f}, {first} {a['p1']/c:.2f}, tile loop {a['p2']/c:.2f}; tail = merge/write + exit"
+        elif name.startswith("1k"):
+            det = "lag = barrier; main = products or key tiles; tail = epilogue or merge, and arrival"
+        elif name.startswith("f32"):
+            det = "lag = rows staged; main = products or keys; tail = cluster barrier"
+        elif a["detail"]:
             det = (f"tail: TMEM->smem {a['p0']/c:.2f}, cluster barrier {a['p1']/c:.2f}, split-K pull {a['p2']/c:.2f}, "
                    f"epilogue {a['p3']/c:.2f}, leave {a['p4']/c:.2f}")
-        print(f"{name:7s} {int(c):3d} {int(a['ctas']/c):5d} | {a['period']/c:6.2f} = {a['lag']/c:5.2f} + {a['main']/c:5.2f} + {a['tail']/c:5.2f} | "
+        else:
+            det = "main = to the first tile's accumulator; tail = the other tiles and the epilogues"
+        print(f"{name:11s} {int(c):3d} {int(a['ctas']/c):5d} | {a['period']/c:6.2f} = {a['lag']/c:5.2f} + {a['main']/c:5.2f} + {a['tail']/c:5.2f} | "
               f"started {a['lead_first']/c:.1f} .. {a['lead_last']/c:.1f} before | {det}")
     print("wait lag: predecessor's end -> last CTA past griddepcontrol.wait; main: -> accumulator complete (GEMM) / key tiles done "
           "(attention); tail: -> last CTA gone; started: first .. last CTA start, microseconds before the predecessor's end")
