@@ -328,7 +328,7 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
     FusedArgs base = {};
     base.M = M;
     const int ssq_sub = M > 128 ? 4 : 1;
-    const int ssq_slots = w.ssq_slots * ssq_sub;
+    const int ssq_slots = (w.ssq_slots * ssq_sub + 3) / 4 * 4;      // read four at a time; what no product writes stays zero
     base.ssq_slots = ssq_slots;
     base.ssq_sub = ssq_sub;
     base.inv_d = 1.0f / (float)d.d_model;

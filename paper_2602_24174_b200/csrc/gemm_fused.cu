@@ -387,10 +387,14 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
             for (int t = threadIdx.x; t < TB; t += 128) {
                 const int m = t0 + t;
                 float ss = 0.f;
-                // (a few slots, off the critical path: unrolled, the code in front of everything else is longer, 0.5 % of a step)
-                if (m < a.M)
-#pragma unroll 1
-                    for (int j = 0; j < a.ssq_slots; ++j) ss += a.ssq_in[(size_t)m * a.ssq_slots + j];
+                // (in front of the products: longer code is fetched late, a slot at a time waits for L2 every time.  A step or prefill of
+                // the 0.5B with loads of four slots, unrolled 1, 2, 4 times: 28 rows 789, 795, 790 us, 192 rows 1442, 1431, 1430, 200
+                // prompt tokens 1344, 1327, 1325; a slot at a time 796, 1447, 1350)
+                if (m < a.M) {
+                    const float4* p = reinterpret_cast<const float4*>(a.ssq_in + (size_t)m * a.ssq_slots);
+#pragma unroll 4
+                    for (int j = 0; j < a.ssq_slots / 4; ++j) { const float4 q = p[j]; ss += q.x; ss += q.y; ss += q.z; ss += q.w; }
+                }
                 s_inv[t] = 1.0f / sqrtf(ss * a.inv_d + a.eps);
             }
         }

@@ -10,7 +10,7 @@
 // something else; a lane's result depends on its own row only, and those lanes are never stored.)
 //
 // Persistent CTAs.  One CTA per SM walks the (feature tile, token tile) pairs blockIdx.x, + gridDim.x, ...
-// with two accumulators in TMEM: while the four epilogue warps drain tile j, the MMA warp already
+// with two accumulators in TMEM: while the eight epilogue warps drain tile j, the MMA warp already
 // works on tile j + 1 in the other accumulator, and the TMA ring never stops between tiles.  A thread of
 // the epilogue owns one token row (its TMEM lane) and 32 consecutive features per tcgen05.ld, so the
 // row-wise consumers (RMS factor, RoPE pairs, sum of squares, row arg-max) need no exchange between threads.
@@ -338,12 +338,8 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         float sc = 1.0f;
         if (a.ssq_in && rowok) {
             float ss = 0.f;
-            if (a.ssq_slots % 4 == 0) {
-                const float4* sp = reinterpret_cast<const float4*>(a.ssq_in + (size_t)m * a.ssq_slots);
-                for (int q = 0; q < a.ssq_slots / 4; ++q) { const float4 t = sp[q]; ss += (t.x + t.y) + (t.z + t.w); }
-            } else {
-                for (int q = 0; q < a.ssq_slots; ++q) ss += a.ssq_in[(size_t)m * a.ssq_slots + q];
-            }
+            const float4* sp = reinterpret_cast<const float4*>(a.ssq_in + (size_t)m * a.ssq_slots);
+            for (int q = 0; q < a.ssq_slots / 4; ++q) { const float4 t = sp[q]; ss += (t.x + t.y) + (t.z + t.w); }
             sc = 1.0f / sqrtf(ss * a.inv_d + a.eps);
         }
 

@@ -100,7 +100,7 @@ struct FusedArgs {
                                        // tiles without any (the few-row kernel would wait longer for the counts than it gains)
     int rows_early;                    // ... which were complete before the preceding grid began
     const float* ssq_in;               // [M][ssq_slots] partial sums of squares of the input rows (null: no scaling)
-    int ssq_slots;
+    int ssq_slots;                     // a multiple of 4
     const unsigned long long* ssq_exact;   // [M][SSQ_WORDS], instead of ssq_in behind the one-kernel layers
     float inv_d, eps;                  // rms factor = 1 / sqrt(sum(ssq) * inv_d + eps)
     float* y;                          // EPI_PLAIN
