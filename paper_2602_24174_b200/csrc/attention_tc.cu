@@ -5,7 +5,7 @@
 // Bound: at 42 rows (7 rows x 6 query heads of a KV head) and 1,500 keys the warp-level kernel spent 5 us per 128 keys, on
 // mma.sync pipes that half of its warps used and on barriers, while K and V could stream in a tenth of that.  Here S = Q K^T
 // and P V are tcgen05 MMAs of 128 rows (M; the rows past the query tile cost nothing, the issue rate is the same) issued by
-// one thread, S and O in TMEM, K and V staged by TMA, so that the softmax is what is left: a thread owns half of the keys
+// one warp, S and O in TMEM, K and V staged by TMA, so that the softmax is what is left: a thread owns half of the keys
 // of one row, registers hold its half of the row's O.  Per tile of TK keys
 //   MMA warp       S(t + 1) while the softmax works on S(t); then P(t) V(t) into an O tile of its own
 //   softmax warps  S(t) -> maximum (exchanged between the two threads of a row) -> P(t) as hi, lo in shared memory;

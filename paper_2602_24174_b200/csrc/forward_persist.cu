@@ -3,8 +3,8 @@
 // What bounds such a pass is not its bytes but its chain of dependent phases: QKV, attention, O, gate/up, down, five
 // per layer, each of which needs the whole output of the one before.  As separate kernels (gemm_fused.cu,
 // attention_mma.cu) a phase costs 4 - 8 us of launch hand-over, cluster exchange and tails around well under 1 us of
-// work.  Here every SM runs one CTA for the whole pass and the phases are separated by a grid barrier (about 1.3 us:
-// one release increment per CTA on a counter in L2, one polling thread per CTA).
+// work.  Here every SM runs one CTA for the whole pass and the phases are separated by a grid barrier (about 0.85 us
+// from the last CTA's arrival until the last one is past it: one release increment per CTA on a counter in L2, one polling thread per CTA).
 //
 // Projections.  A CTA owns a block of output rows (1 / n_rb of them) for a block of T * 8 token rows and computes them
 // over the whole reduction, so no partial sum leaves the CTA.  Its warps split the reduction; weights go from global
@@ -28,8 +28,10 @@
 // the barrier.  Key ranges of one group are merged by the CTA that finishes last, in range order.
 //
 // Measured (one verify step, five kernels per layer / this kernel): 135M at 6 rows 747 / 594 us, 0.5B at 6 rows 746 / 650, 1.5B
-// at 7 rows 1213 / 1144; more of it at persist_pays.  What is left is the barrier and the first fresh read behind it, about 2.4 us
-// for each of the five phases (of 3.0 per phase at 135M, of 6.9 at 1.5B, where streaming the weights is the larger part).
+// at 7 rows 1213 / 1144; more of it at persist_pays.  What is left, by stamps (which add about 0.3 us a phase): at 135M 3.1 - 3.3 us per
+// projection, 0.8 - 1.0 of it the barrier, 0.7 - 1.0 the products behind their first fresh read, 1.5 the epilogue and the arrival;
+// attention 6.9, 2.5 of it the merge of the key ranges.  At 1.5B the weights: gate/up 12.0 (products 8.2), down 7.9 (5.3), QKV 6.5 (CTAs
+// start it 1.4 us apart), O 3.6, attention 9.8 (merge 4.1).
 //
 // Every wait is bounded: a barrier that is not reached in about half a second records TASC_ETIMEOUT and the CTA
 // leaves.  The limit holds for the first barrier too: a cooperative grid starts when all its CTAs can be resident, not one by

@@ -679,11 +679,12 @@ FusedPlan plan_fused(int M, int N, int K, int epi, int few_tiles, int hd, double
         S = std::max(1, 148 / tiles);
         S = std::min(S, 8);
         S = std::min(S, p.num_kb);
-        // Fewer splits than fit can be faster.  Per kernel, in microseconds as measured on the 576- and 1536-wide
-        // products: a CTA's MMA chain takes about 0.46 per k-block (0.28 to 0.46 choose the same); its epilogue about 0.5 per round of six token
-        // columns (one per warp) of the columns it finishes; and a grid that takes more than about two thirds of
-        // the SMs keeps the next kernel's CTAs from starting (and from fetching their weights) while this one
-        // runs, about 0.035 per CTA beyond 96.  Ties go to the larger cluster.
+        // Fewer splits than fit can be faster.  Per kernel, in microseconds: a CTA's epilogue takes about 0.5 per round of six token
+        // columns (one per warp) of the columns it finishes; a grid that takes more than about two thirds of the SMs keeps the next
+        // kernel's CTAs from starting (and from fetching their weights) while this one runs, about 0.035 per CTA beyond 96; and a
+        // k-block of a CTA's chain counts 0.46.  That is more than its MMAs take (160 to 250 cycles, 0.13): with 0.13 in its place some
+        // passes gain and others lose (135M 128 rows 1031 -> 1010 us a step, 0.5B 128 rows 1255 -> 1236, 144 rows 1301 -> 1294, 96 rows
+        // 1114 -> 1118, 0.5B + 8,192 tokens 288 rows 1562 -> 1568).  Ties go to the larger cluster.
         // (With a single token tile the chain's kernels are narrow and the largest cluster stays the best.)
         const int cols = std::min(p.TB, M);
         int best = S;
