@@ -39,21 +39,23 @@ METRIC = "generated tokens/s with n-gram spec decode @1 B200; verify-step HBM GB
 UNIT = "tokens/s"
 
 
-# DRAM traffic of the fused GEMM kernel from an ncu capture (dram__bytes_read.sum + dram__bytes_write.sum summed
-# over the step's launches of that kernel, per launch), keyed by (configuration, batch, k).  A figure is valid for
-# the kernel source whose digest is stored with it; after any change of gemm_fused.cu `traffic` reads null.
+# DRAM traffic of the dominant kernels from an ncu capture (dram__bytes_read.sum + dram__bytes_write.sum of the one-kernel
+# layers and the LM head, per launch), keyed by (configuration, batch, k).  A figure is valid for the kernel sources whose
+# digest is stored with it; after any change of them `traffic` reads null.
 NCU_TRAFFIC = {
-    # configuration 4, B = 1, k = 6: per layer 6.48 + 4.92 + 55.21 + 28.20 MB (QKV, O, gate/up, down) and 469.8 MB for the LM
-    # head, captured on the same kernels with the model cut to 2 layers (--layers 2) and summed for 28 layers, over the
-    # step's 113 launches (algorithmic: 27.55 MB per launch)
-    (4, 1, 6): {"bytes_per_launch": (28 * 94798336 + 470330624) / 113, "kernel_sha256_16": "73c53c5da55f6b57"},
+    # configuration 4, B = 1, k = 6: the model cut to 2 and 4 layers (--layers), 208.5 and 416.8 MB in the layers' launch, so 2,916 MB
+    # at 28, and 467.2 MB in the LM head's (algorithmic: 1,557 MB per launch)
+    (4, 1, 6): {"bytes_per_launch": (208545152 + 26 * 104150016 + 467210240) / 2, "kernel_sha256_16": "641d0621fcad257a"},
 }
 
 
 def kernel_digest():
     import hashlib
-    path = os.path.join(ROOT, "paper_2602_24174_b200", "csrc", "gemm_fused.cu")
-    return hashlib.sha256(open(path, "rb").read()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for name in ("forward_persist.cu", "gemm_fused.cu"):
+        with open(os.path.join(ROOT, "paper_2602_24174_b200", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 def load_peaks():
