@@ -108,19 +108,20 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
     const uint32_t bar_acc = bar_full + 16u * stages;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * stages + 1);
     float* s_inv = reinterpret_cast<float*>(bars + 2 * stages + 2);                       // [128]
+    long long* s_kv = reinterpret_cast<long long*>(s_inv + 128);                          // [128] EPI_QKV: element offsets of the columns' slots in the K and V pages
 
     const int S = (int)cluster_nctarank();
     const int rank = (int)cluster_ctarank();
     const int out_tile = blockIdx.y, m_tile = blockIdx.z;
-    const int kb_begin = (int)(((long long)a.num_kb * rank) / S);
-    const int kb_end = (int)(((long long)a.num_kb * (rank + 1)) / S);
+    const int kb_begin = (int)((unsigned)(a.num_kb * rank) / (unsigned)S);
+    const int kb_end = (int)((unsigned)(a.num_kb * (rank + 1)) / (unsigned)S);
     const int n_kb = kb_end - kb_begin;
     const int f0 = out_tile * (EPI == EPI_SWIGLU ? 64 : BM);   // first output feature of the tile
     const int m0 = m_tile * BN;                                // first row of the tile in the activation buffer
     const int t0 = m_tile * TB;                                // first token of the tile
     int valid = a.M - t0;                                      // token columns in use
     valid = valid > TB ? TB : valid;
-    const int per = (valid + S - 1) / S;                       // token columns reduced and finished by each CTA of the cluster
+    const int per = (int)((unsigned)(valid + S - 1) / (unsigned)S);                       // token columns reduced and finished by each CTA of the cluster
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #ifdef TASC_TIMELINE
@@ -129,8 +130,7 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
     __shared__ unsigned long long g_ta, g_tb, g_tc, g_td, g_te, g_tf;
     const int cta_lin = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
 #endif
-    uint32_t ncols = 32;
-    while ((int)ncols < BN) ncols <<= 1;
+    const uint32_t ncols = BN <= 32 ? 32u : 1u << (32 - __clz(BN - 1));
     __shared__ int s_fail;              // a bounded wait ran out somewhere in this CTA
     auto fail = [&]() { set_status(a.status, TASC_ETIMEOUT); s_fail = 1; };
 
@@ -150,39 +150,69 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
     // Token columns this CTA reduces and finishes: [rank * per, rank * per + count).
     int count = valid - rank * per;
     count = count < 0 ? 0 : (count > per ? per : count);
-    // Global operands of the epilogue of one column (position, rotary factors, KV page, residual row).  The
-    // first NPF columns of every warp are fetched while the MMAs run, so their latency is off the tail.
-    struct Pre { float4 x, cs01, cs23; int pos, page; };
+    // Global operands of the epilogue of one column (rotary factors, residual values).  The first NPF columns of every warp are
+    // fetched while the MMAs run, so their latency is off the tail.  Every warp reduces and finishes columns: column tl belongs to
+    // warp tl % EW.
+    // One copy of this code for all warp roles, and of the finishing code for all columns, no loops unrolled by the compiler, no 64-bit
+    // divisions: a kernel of a few microseconds waits for instructions it executes once (under ncu a third of the QKV kernel's
+    // instruction-cache requests missed, and 8 of 18 warps-cycles per issue stalled for want of an instruction).  With 18 copies
+    // of the one and 4 of the other the QKV kernel had 94 - 109 KB of code, now 29; O and down 42 -> 20, gate/up 39 -> 26.  A step of
+    // the 135M at 96 rows 968 -> 928 us, of the 0.5B at 28 rows 794 -> 756, at 288 rows 1551 -> 1484, 255 prompt tokens 1066 -> 958.
+    struct Pre { float4 u, v; };
     constexpr int NPF = 3;
-    // every warp reduces and finishes columns: column tl belongs to warp tl % EW
+    const int f = f0 + 4 * lane;                               // this lane's four features
+    const int hd = a.hd, half = hd >> 1, qd = a.n_q * hd, kvd = a.n_kv * hd;
+    const int in_head = f & (hd - 1);                          // (head_dim is 32, 64 or 128)
+    auto row_position = [&](int m) {
+        const int pos = a.row_pos[m];
+        return pos < a.max_positions ? pos : -1;
+    };
     auto prefetch = [&](int tl) -> Pre {
         Pre q;
-        q.x = q.cs01 = q.cs23 = make_float4(0.f, 0.f, 0.f, 0.f);
-        q.pos = -1; q.page = -1;
+        q.u = q.v = make_float4(0.f, 0.f, 0.f, 0.f);
         const int m = t0 + rank * per + tl;
-        const int f = f0 + 4 * lane;
         if (EPI == EPI_QKV) {
-            const int hd = a.hd, half = hd >> 1;
-            const int qd = a.n_q * hd, kvd = a.n_kv * hd;
-            int pos = a.row_pos[m];
-            if (pos >= a.max_positions) { set_status(a.status, TASC_EINVAL); pos = -1; }
-            q.pos = pos;
+            const int pos = row_position(m);
             if (pos >= 0 && f < qd + kvd) {
-                const float4* cs = reinterpret_cast<const float4*>(a.rope + (size_t)pos * half + ((f % hd) % half));
-                q.cs01 = cs[0];                                  // (cos, sin) of four consecutive pair indices
-                q.cs23 = cs[1];
-            }
-            if (pos >= 0 && f >= qd && f < qd + 2 * kvd) {
-                const int pslot = pos / a.page_size;
-                if (pslot < a.max_pages) q.page = a.block_table[(size_t)(m / a.R) * a.max_pages + pslot];
-                if (q.page < 0 || q.page >= a.n_pages) { set_status(a.status, TASC_ENOKV); q.page = -1; }
+                const float4* cs = reinterpret_cast<const float4*>(a.rope + (size_t)pos * half + (in_head & (half - 1)));
+                q.u = cs[0];                                   // (cos, sin) of four consecutive pair indices
+                q.v = cs[1];
             }
         } else if (EPI == EPI_RESID) {
-            if (f < a.N) q.x = *reinterpret_cast<const float4*>(a.x + (size_t)m * a.N + f);
+            if (f < a.N) q.u = *reinterpret_cast<const float4*>(a.x + (size_t)m * a.N + f);
         }
         return q;
     };
     float4 gain4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    Pre pf[NPF];
+    auto operands = [&]() {
+#pragma unroll
+        for (int i = 0; i < NPF; ++i)
+            if (warp + EW * i < count) pf[i] = prefetch(warp + EW * i);
+        if (EPI == EPI_RESID && f < a.N) gain4 = *reinterpret_cast<const float4*>(a.gain + f);
+        // where the keys and values of the CTA's columns go: a thread per column (read behind the cluster barrier)
+        if (EPI == EPI_QKV)
+#pragma unroll 1
+            for (int tl = threadIdx.x; tl < count; tl += EW * 32) {
+                const int m = t0 + rank * per + tl, pos = row_position(m);
+                if (pos < 0 && a.row_pos[m] >= 0) set_status(a.status, TASC_EINVAL);
+                long long off = pos < 0 ? -2 : -1;             // -2: not in use, -1: no page
+                if (pos >= 0 && f0 + BM > qd) {
+                    const int pslot = pos / a.page_size;
+                    int page = -1;
+                    if (pslot < a.max_pages) page = a.block_table[(size_t)(m / a.R) * a.max_pages + pslot];
+                    if (page < 0 || page >= a.n_pages) set_status(a.status, TASC_ENOKV);
+                    else off = ((long long)page * a.n_kv * a.page_size + (pos - pslot * a.page_size)) * hd;
+                }
+                s_kv[tl] = off;
+            }
+    };
+    __nv_bfloat16* kv_base = nullptr;                          // this lane's place in the first slot of the first page
+    if (EPI == EPI_QKV && f >= qd && f < qd + 2 * kvd) {
+        const bool is_k = f < qd + kvd;
+        const int kh = (f - in_head - qd - (is_k ? 0 : kvd)) / hd;
+        kv_base = (is_k ? a.k_pages : a.v_pages) + (size_t)kh * a.page_size * hd + in_head;
+    }
     auto finish = [&](int tl, const Pre& q) {
         const int t = rank * per + tl;
         const float4 acc = *reinterpret_cast<const float4*>((S > 1 ? fin + (size_t)tl * BM : xch + (size_t)t * BM) + 4 * lane);
@@ -191,53 +221,42 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
             const float sc = a.ssq_in ? s_inv[t] : 1.0f;
             const float v[4] = {acc.x * sc, acc.y * sc, acc.z * sc, acc.w * sc};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int f = f0 + 4 * lane + e;
-                if (f < a.N) a.y[(size_t)m * a.N + f] = v[e];
-            }
+            for (int e = 0; e < 4; ++e)
+                if (f + e < a.N) a.y[(size_t)m * a.N + f + e] = v[e];
         } else if (EPI == EPI_QKV) {
             const float sc = s_inv[t];
-            const float4 sacc = make_float4(acc.x * sc, acc.y * sc, acc.z * sc, acc.w * sc);
-            const int hd = a.hd, half = hd >> 1;
-            const float4 partner = shfl_xor4(sacc, half >> 2);
-            const int f = f0 + 4 * lane;
-            const int qd = a.n_q * hd, kvd = a.n_kv * hd;
-            const int pos = q.pos;
-            float v[4] = {sacc.x, sacc.y, sacc.z, sacc.w};
-            if (f < qd + kvd && pos >= 0) {
-                const float co[4] = {q.cs01.x, q.cs01.z, q.cs23.x, q.cs23.z};
-                const float si[4] = {q.cs01.y, q.cs01.w, q.cs23.y, q.cs23.w};
+            float v[4] = {acc.x * sc, acc.y * sc, acc.z * sc, acc.w * sc};
+            const float4 partner = shfl_xor4(make_float4(v[0], v[1], v[2], v[3]), half >> 2);
+            const long long off = s_kv[tl];
+            if (f < qd + kvd && off > -2) {
+                const float co[4] = {q.u.x, q.u.z, q.v.x, q.v.z};
+                const float si[4] = {q.u.y, q.u.w, q.v.y, q.v.w};
                 const float pv[4] = {partner.x, partner.y, partner.z, partner.w};
-                const float sgn = (f % hd) < half ? -1.0f : 1.0f;   // first half: a c - b s; second half: b c + a s
+                const float sgn = in_head < half ? -1.0f : 1.0f;    // first half: a c - b s; second half: b c + a s
 #pragma unroll
                 for (int e = 0; e < 4; ++e) v[e] = v[e] * co[e] + sgn * pv[e] * si[e];
             }
             if (f < qd) {
-                if (pos < 0) { v[0] = v[1] = v[2] = v[3] = 0.f; }
+                if (off == -2) { v[0] = v[1] = v[2] = v[3] = 0.f; }
                 *reinterpret_cast<float4*>(a.qbuf + (size_t)m * qd + f) = make_float4(v[0], v[1], v[2], v[3]);
-            } else if (f < qd + 2 * kvd && pos >= 0 && q.page >= 0) {
-                const bool is_k = f < qd + kvd;
-                const int gidx = f - qd - (is_k ? 0 : kvd);
-                const int kh = gidx / hd, i = gidx % hd;
-                __nv_bfloat16* base = is_k ? a.k_pages : a.v_pages;
-                store_bf16x4(base + (((size_t)q.page * a.n_kv + kh) * a.page_size + pos % a.page_size) * hd + i, v);
+            } else if (kv_base && off >= 0) {
+                store_bf16x4(kv_base + off, v);
             }
         } else if (EPI == EPI_RESID) {
-            const int f = f0 + 4 * lane;
             float ss = 0.f;
             if (f < a.N) {
-                const float4 xv = make_float4(q.x.x + acc.x, q.x.y + acc.y, q.x.z + acc.z, q.x.w + acc.w);
+                const float4 xv = make_float4(q.u.x + acc.x, q.u.y + acc.y, q.u.z + acc.z, q.u.w + acc.w);
                 *reinterpret_cast<float4*>(a.x + (size_t)m * a.N + f) = xv;
                 ss = xv.x * xv.x + xv.y * xv.y + xv.z * xv.z + xv.w * xv.w;
                 const float v[4] = {xv.x * gain4.x, xv.y * gain4.y, xv.z * gain4.z, xv.w * gain4.w};
-                const size_t row = (size_t)(m / TBL) * (2 * TBL) + m % TBL;
+                const size_t row = (size_t)m0 + t;              // (one layout tile per CTA)
                 store_hilo4(a.a_out + row * a.N + f, a.a_out + (row + TBL) * a.N + f, v);
             }
             ss = warp_sum(ss);
             if (lane == 0) {
                 float* slot = a.ssq_out + (size_t)m * a.ssq_out_slots + (size_t)out_tile * a.ssq_sub;
-                slot[0] = ss;
-                for (int j = 1; j < a.ssq_sub; ++j) slot[j] = 0.f;
+                if (a.ssq_sub == 4) *reinterpret_cast<float4*>(slot) = make_float4(ss, 0.f, 0.f, 0.f);
+                else slot[0] = ss;
             }
         } else if (EPI == EPI_SWIGLU) {
             const float sc = s_inv[t];
@@ -254,7 +273,7 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
                 __nv_bfloat16 h0, l0, h1, l1;
                 split_bf16(v0, h0, l0);
                 split_bf16(v1, h1, l1);
-                const size_t row = (size_t)(m / TBL) * (2 * TBL) + m % TBL;
+                const size_t row = (size_t)m0 + t;
                 *reinterpret_cast<uint32_t*>(a.a_out + row * a.N + j) =
                     (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
                 *reinterpret_cast<uint32_t*>(a.a_out + (row + TBL) * a.N + j) =
@@ -262,31 +281,16 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
             }
         }
     };
-    Pre pf[NPF];
-    // Where the epilogue's operands were complete before the preceding grid began (a.early: the row plan, rotary
-    // table and page ids of a QKV launch that does not follow the row-plan kernel; the residual rows and gain of a
-    // RESID launch), they are requested ahead of griddepcontrol.wait, otherwise after it.
-    auto late_prefetch = [&]() {
-        if (EPI != EPI_LM) {
-#pragma unroll
-            for (int i = 0; i < NPF; ++i)
-                if (warp + EW * i < count) pf[i] = prefetch(warp + EW * i);
-            if (EPI == EPI_RESID && f0 + 4 * lane < a.N) gain4 = *reinterpret_cast<const float4*>(a.gain + f0 + 4 * lane);
-        }
-    };
 
     if (warp == 4) {
-        if (lane == 0) {
+        if (lane < 2 * stages) mbar_init(bar_full + 8u * lane, 1);        // (at most eight stages; the empty ones follow the full ones)
+        if (lane == 31) {
             s_fail = 0;
-            for (int s = 0; s < stages; ++s) {
-                mbar_init(bar_full + 8u * s, 1);
-                mbar_init(bar_empty + 8u * s, 1);
-            }
             mbar_init(bar_acc, 1);
-            fence_barrier_init();
             tma_prefetch_desc(&tmW);
             tma_prefetch_desc(&tmX);
         }
+        fence_barrier_init();
         __syncwarp();
         // The weights of the first stages depend on no earlier kernel: their loads start before the rest of
         // the CTA is set up and before the preceding grid has finished.  One lane per stage: a lane that has
@@ -307,11 +311,20 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     if (threadIdx.x == 0) TL(0);
+    // Where the epilogue's operands were complete before the preceding grid began (a.early: the row plan, rotary
+    // table and page ids of a QKV launch that does not follow the row-plan kernel; the residual rows and gain of a
+    // RESID launch), they are requested ahead of griddepcontrol.wait, otherwise after it.
+    if (EPI == EPI_QKV || EPI == EPI_RESID) {
+        if (!a.early) griddep_wait();
+        operands();
+    }
+    griddep_wait();
+#ifdef TASC_TIMELINE
+    if (threadIdx.x == 0) g_ta = global_ns();
+#endif
 
     if (warp == 4) {
         // ------------------------------------------------------------ TMA producer
-        if (a.early) late_prefetch();
-        griddep_wait();                 // every lane: the token rows below, and the epilogue operands later
         if (lane < pre) {
             const uint32_t dstB = smem_u32(smem + (size_t)lane * stage_bytes) + A_STAGE_BYTES;
             mbar_expect_tx(bar_full + 8u * lane, b_stage_bytes);
@@ -322,6 +335,7 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
             TL(2);
             int s = 0;
             uint32_t parity = 0;                                     // of the stage's previous use
+#pragma unroll 1
             for (int i = pre; i < n_kb; ++i) {
                 if (!mbar_wait(bar_empty + 8u * s, parity)) { fail(); break; }
                 const uint32_t dstA = smem_u32(smem + (size_t)s * stage_bytes);
@@ -334,10 +348,8 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
             TL(3);
         }
         __syncwarp();
-        if (!a.early) late_prefetch();
     } else if (warp == 5) {
         // ------------------------------------------------------------ MMA issue
-        if (a.early) late_prefetch();
         // (the whole warp, see umma_bf16_warp: a k-block of 96 columns 376 -> 225 cycles)
         {
             const uint32_t idesc = umma_idesc_bf16_f32(BM, BN);
@@ -345,6 +357,7 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
             bool ok = true;
             int s = 0;
             uint32_t round = 0;
+#pragma unroll 1
             for (int i = 0; i < n_kb; ++i) {
                 ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar_full + 8u * s, round & 1u));
                 if (!ok) { fail(); break; }
@@ -362,23 +375,12 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
             if (lane == 0) TL(5);
         }
         __syncwarp();
-        griddep_wait();
-        if (!a.early) late_prefetch();
-    } else if (warp >= 6) {
-        // ------------------------------------------------------------ the additional column finishers: nothing to do before part 2
-        if (a.early) late_prefetch();
-        griddep_wait();
-        if (!a.early) late_prefetch();
-    } else {
+    } else if (warp < 4) {
         // ------------------------------------------------------------ epilogue, part 1: accumulator -> shared memory
-        if (a.early) late_prefetch();
-        griddep_wait();
-#ifdef TASC_TIMELINE
-        if (threadIdx.x == 0) g_ta = global_ns();
-#endif
-        if (!a.early) late_prefetch();
+        // (the additional column finishers have nothing to do before part 2)
         if (EPI == EPI_QKV || EPI == EPI_SWIGLU || EPI == EPI_LM || (EPI == EPI_PLAIN && a.ssq_in)) {
             if (EPI == EPI_LM && a.ssq_exact) {
+#pragma unroll 1
                 for (int t = threadIdx.x >> 3; t < TB; t += 16) {        // eight lanes per row (TB is a multiple of 16)
                     const float ss = ssq_total(t0 + t < a.M ? a.ssq_exact[(size_t)(t0 + t) * SSQ_WORDS + (threadIdx.x & 7)] : 0ull);
                     if ((threadIdx.x & 7) == 0) s_inv[t] = 1.0f / sqrtf(ss * a.inv_d + a.eps);
@@ -409,34 +411,20 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
         const uint32_t lane_base = tmem_base + ((uint32_t)(warp * 32) << 16);
         const int fl = warp * 32 + lane;                        // this thread's feature (TMEM lane) within the tile
         // accumulator columns of layout tile lt: [lt * 2 TBL, +TBL) from the hi rows, the next TBL from the lo rows
+#pragma unroll 1
         for (int lt = 0; lt * TBL < TB; ++lt) {
             const uint32_t col0 = (uint32_t)(lt * 2 * TBL);
-            for (int c = 0; c < TBL; c += 32) {
-                const bool wide = c + 32 <= TBL;                // TBL is a multiple of 16
-                uint32_t r[32];
+#pragma unroll 1
+            for (int c = 0; c < TBL; c += 16) {                 // TBL is a multiple of 16
+                uint32_t r[16], r2[16];
                 if (have) {
-                    if (wide) {
-                        uint32_t r2[32];
-                        tmem_ld32(lane_base + col0 + (uint32_t)c, r);
-                        tmem_ld32(lane_base + col0 + (uint32_t)(TBL + c), r2);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(r2[j]));
-                    } else {
-                        uint32_t q[16], q2[16];
-                        tmem_ld16(lane_base + col0 + (uint32_t)c, q);
-                        tmem_ld16(lane_base + col0 + (uint32_t)(TBL + c), q2);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(__uint_as_float(q[j]) + __uint_as_float(q2[j]));
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) r[j] = 0u;
+                    tmem_ld16(lane_base + col0 + (uint32_t)c, r);
+                    tmem_ld16(lane_base + col0 + (uint32_t)(TBL + c), r2);
+                    tmem_ld_wait();
                 }
 #pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (j < 16 || wide) xch[(lt * TBL + c + j) * BM + fl] = __uint_as_float(r[j]);
+                for (int j = 0; j < 16; ++j)
+                    xch[(lt * TBL + c + j) * BM + fl] = have ? __uint_as_float(r[j]) + __uint_as_float(r2[j]) : 0.f;
             }
         }
     }
@@ -461,6 +449,7 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
             uint32_t peer[8];
 #pragma unroll
             for (int s = 0; s < 8; ++s) peer[s] = cluster_map(xch_addr, (uint32_t)(s < S ? s : 0));
+#pragma unroll 1
             for (int tl = warp; tl < count; tl += 2 * EW) {       // two columns per round: 2 S reads in flight
                 const bool two = tl + EW < count;
                 const uint32_t toff0 = (uint32_t)(rank * per + tl) * (BM * 4), toff1 = toff0 + (uint32_t)EW * (BM * 4);
@@ -489,15 +478,18 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
     // this CTA has finished reading its peers' shared memory; they may leave while it runs the epilogue
     cluster_arrive();
     if (EPI != EPI_LM) {
-#pragma unroll
-        for (int i = 0; i < NPF; ++i)
-            if (warp + EW * i < count) finish(warp + EW * i, pf[i]);
-        for (int tl = warp + EW * NPF; tl < count; tl += EW) finish(tl, prefetch(tl));
+#pragma unroll 1
+        for (int tl = warp; tl < count; tl += EW) {
+            finish(tl, pf[0]);
+            pf[0] = pf[1];
+            pf[1] = pf[2];
+            if (tl + EW * NPF < count) pf[2] = prefetch(tl + EW * NPF);
+        }
     } else {
         // LM head: per token row the largest logit of this 128-feature tile (smallest id on ties), merged
         // across tiles by an atomic max on the packed (value, id) word; the logits themselves are not stored
         // (two token rows per round: their reductions are independent and overlap)
-        const int f = f0 + 4 * lane;
+#pragma unroll 1
         for (int tb = warp; tb < valid; tb += 2 * EW) {
             float4 acc[2];
             uint32_t bk[2], bi[2];
@@ -547,6 +539,7 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
     cluster_wait();
     if (s_fail && warp == 4 && lane == 0) {
         // after a timeout: give this CTA's own tile loads that may still be in flight a bounded time to land
+#pragma unroll 1
         for (int i = 0; i < n_kb; ++i) {
             const int s = i % stages;
             if (i + stages >= n_kb) (void)mbar_wait(bar_full + 8u * s, (uint32_t)(i / stages) & 1u, 2000000ll);
@@ -716,7 +709,7 @@ FusedPlan plan_fused(int M, int N, int K, int epi, int few_tiles, int hd, double
         st = std::min(st, std::max(2, kb_per));
         p.stages = st;
         p.data_bytes = std::max(st * stage_bytes, p.TB * BM * 4) + xch_bytes;
-        int smem = 1024 + p.data_bytes + (2 * st + 2) * 8 + 128 * 4;
+        int smem = 1024 + p.data_bytes + (2 * st + 2) * 8 + 128 * 4 + 128 * 8;
         // TMEM columns held by co-resident CTAs must never exceed 512, or CTAs of different clusters can
         // block each other's allocation while waiting at a cluster barrier: shared memory limits residency.
         // (The LM head has no cluster barrier to wait at; two of its CTAs with 256 columns each share an SM.)
