@@ -24,12 +24,14 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <type_traits>
 
 namespace tasc {
 
 namespace {
 
 constexpr int TKEYS = 64;
+constexpr int MAX_STAGED_PAGES = 1024;
 
 struct AttnArgs {
     const float* q;                    // [M][n_q * hd], RoPE applied
@@ -45,7 +47,8 @@ struct AttnArgs {
     int R, n_q, n_kv, splits, stages;  // R: rows per sequence in this pass
     int Rs, n_sub;                     // a CTA takes Rs of them (sub-block blockIdx.z % n_sub); R = Rs * n_sub
     int hs, n_hsplit;                  // a CTA takes hs of the g query heads of its KV head (blockIdx.y % n_hsplit); g = hs * n_hsplit
-    int use_tma;                       // K/V tiles by TMA box loads (16-token pages); otherwise by cp.async
+    int n_slabs;                       // 16-row slabs of the CTA's hs * Rs query rows
+    SmallDiv by_R, by_TB, by_splits, by_sub, by_hsplit;
     int* status;
     float scale_log2e;
 };
@@ -81,15 +84,6 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int sr
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// two floats -> packed bf16 pair (hi) and the packed pair of the residuals (lo)
-__device__ __forceinline__ void pack_hilo(float x, float y, uint32_t& hi, uint32_t& lo) {
-    __nv_bfloat16 hx, lx, hy, ly;
-    split_bf16(x, hx, lx);
-    split_bf16(y, hy, ly);
-    hi = (uint32_t)__bfloat16_as_ushort(hx) | ((uint32_t)__bfloat16_as_ushort(hy) << 16);
-    lo = (uint32_t)__bfloat16_as_ushort(lx) | ((uint32_t)__bfloat16_as_ushort(ly) << 16);
-}
-
 // Largest ring depth of the K/V tile pipeline (the host picks 2..max per launch).  A CTA streams its key range
 // alone, so the bytes it keeps in flight (ring depth x 8-32 KB per tile) over the memory latency are its
 // bandwidth; a shallower ring lets two CTAs share an SM when many (sequence, KV head) pairs are in flight.
@@ -124,8 +118,13 @@ __device__ __forceinline__ void cp_async_wait_dyn(int n) {      // wait until at
     }
 }
 
-// NS = number of 16-row slabs the padded query tile has (4 or 8); the CTA always has eight warps.
-template <int HD, int NS>
+// NS = number of 16-row slabs the padded query tile has (4 or 8); the CTA always has eight warps.  TMA: K/V tiles by box loads (pages of 16
+// tokens, at most MAX_STAGED_PAGES of them); otherwise by cp.async.
+// What bounds a verify step of a few hundred keys is how fast the SM fetches instructions that it executes once or twice, so the
+// code is kept short: one instance per way of loading, no integer divisions, no copies by loop unrolling, and only the query rows that
+// exist are staged.  Heads of 64: 72 -> 41 KB; a step of the 135M at 96 rows 928 -> 853 us, of the 0.5B at 28 rows 756 -> 705, 255
+// prompt tokens of the 135M 958 -> 873.
+template <int HD, int NS, bool TMA>
 __global__ void __launch_bounds__(256)
 attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const AttnArgs a) {
     constexpr int NW = 8;                        // warps
@@ -140,12 +139,11 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     uint8_t* Ql = Qh + GP * HD * 2;
     uint8_t* Kt = Ql + GP * HD * 2;              // [STAGES][TKEYS][HD]
     uint8_t* Vt = Kt + STAGES * TILE_BYTES;      // [STAGES][TKEYS][HD]
-    constexpr int MAX_STAGED_PAGES = 1024;
     __shared__ int s_pages[MAX_STAGED_PAGES];
     __shared__ uint64_t s_full[8];               // one per ring stage: bytes of its K and V tile have landed (TMA path)
 
-    const int sp = blockIdx.x, kh = blockIdx.y / a.n_hsplit, b = blockIdx.z / a.n_sub, rb = (blockIdx.z % a.n_sub) * a.Rs;
-    const int h0 = kh * (a.n_q / a.n_kv) + (int)(blockIdx.y % a.n_hsplit) * a.hs;      // first query head of this CTA
+    const int sp = blockIdx.x, kh = a.by_hsplit.div(blockIdx.y), b = a.by_sub.div(blockIdx.z), rb = ((int)blockIdx.z - b * a.n_sub) * a.Rs;
+    const int h0 = (int)blockIdx.y * a.hs;                     // first query head of this CTA
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 #ifdef TASC_TIMELINE
     struct LogAtExit { unsigned long long t0, ta, tb, tc, td, te, tf; __device__ ~LogAtExit() { if (threadIdx.x == 0) ctalog_put(t0, ta, tb, 10, tc, td, te, tf); } } log_at_exit{global_ns(), 0, 0, 0, 0, 0, 0};
@@ -153,6 +151,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     const int g = a.hs, R = a.Rs;                              // g: query heads of this CTA; R: rows of its sub-block, the first is rb
     const int G = g * R;
     const int qd = a.n_q * HD;
+    auto out_row = [&](int m) { return (size_t)(a.by_TB.div(m) * a.TB + m); };      // its hi row; the lo row is TB further
 
     // The row plan, the block table and the K/V of committed positions were written before the
     // preceding grid started, so they may be read ahead of griddepcontrol.wait.
@@ -167,11 +166,11 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         griddep_launch_dependents();
         // sequence not in this step: its rows of the output are zero
         if (sp == 0) {
+#pragma unroll 1
             for (int i = tid; i < G * (HD / 4); i += THREADS) {
-                const int rho = i / (HD / 4), d4 = (i % (HD / 4)) * 4;
-                const int m = b * a.R + rb + rho % R;
-                const size_t row = (size_t)(m / a.TB) * (2 * a.TB) + (m % a.TB);
-                const size_t col = (size_t)(h0 + rho / R) * HD + d4;
+                const int rho = i / (HD / 4), d4 = (i % (HD / 4)) * 4, hl = a.by_R.div(rho);
+                const size_t row = out_row(b * a.R + rb + rho - hl * R);
+                const size_t col = (size_t)(h0 + hl) * HD + d4;
                 *reinterpret_cast<uint2*>(a.out + row * qd + col) = make_uint2(0u, 0u);
                 *reinterpret_cast<uint2*>(a.out + (row + a.TB) * qd + col) = make_uint2(0u, 0u);
             }
@@ -181,31 +180,37 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     const int total = pos0 + rows;               // keys visible to the last row
     // the range's 64-key tiles are dealt out evenly: every split gets floor or ceil of tiles / splits of them
     const int tiles_all = (total + TKEYS - 1) / TKEYS;
-    const int t_base = tiles_all / a.splits, t_rem = tiles_all % a.splits;
+    const int t_base = a.by_splits.div(tiles_all), t_rem = tiles_all - t_base * a.splits;
     const int n_tiles = t_base + (sp < t_rem ? 1 : 0);
     const int k_begin = (sp * t_base + min(sp, t_rem)) * TKEYS;
     const int k_end = min(total, k_begin + n_tiles * TKEYS);
-    const int n_slabs = (G + 15) / 16;
+    const int n_slabs = a.n_slabs;
     // A warp owns one 16-row slab of one key tile.  With fewer slabs than warps the warps form ng = 2 or 4 groups
     // of n_slabs warps; group `grp` handles tiles grp, grp + ng, ...; the groups' results are merged in shared memory.
     const int ng = warp_groups(n_slabs, STAGES, n_tiles);
-    const int slab = warp % n_slabs, grp = warp / n_slabs;
+    int slab = warp, grp = 0;
+#pragma unroll 1
+    while (slab >= n_slabs) { slab -= n_slabs; ++grp; }
     const bool computes = grp < ng;
-    const int n_super = (n_tiles + ng - 1) / ng;                 // iterations of ng tiles
-    const int super_stages = STAGES / ng;
+    const int lg = ng >> 1;                                      // log2 (ng is 1, 2 or 4)
+    const int n_super = (n_tiles + ng - 1) >> lg;                // iterations of ng tiles
+    const int super_stages = STAGES >> lg;
 
     // Page ids of this CTA's key range, staged once: the tile loads then need no dependent global read.
-    const int pg_lo = k_begin / a.page_size;
-    const int n_pg = n_tiles > 0 ? (k_end - 1) / a.page_size - pg_lo + 1 : 0;
-    const bool pages_staged = n_pg <= MAX_STAGED_PAGES;
-    const bool use_tma = a.use_tma && pages_staged;
-    if (tid == 0 && use_tma) {
-        for (int i = 0; i < STAGES; ++i) mbar_init(smem_u32(&s_full[i]), 1);
+    const int page_size = TMA ? 16 : a.page_size;
+    const int pg_lo = k_begin / page_size;
+    const int n_pg = n_tiles > 0 ? (k_end - 1) / page_size - pg_lo + 1 : 0;
+    const bool pages_staged = TMA || n_pg <= MAX_STAGED_PAGES;
+    if (TMA && warp == 7) {
+        if (lane < STAGES) mbar_init(smem_u32(&s_full[lane]), 1);
         fence_barrier_init();
-        tma_prefetch_desc(&tmK);
-        tma_prefetch_desc(&tmV);
+        if (lane == 0) {
+            tma_prefetch_desc(&tmK);
+            tma_prefetch_desc(&tmV);
+        }
     }
     if (pages_staged) {
+#pragma unroll 1
         for (int i = tid; i < n_pg; i += THREADS) {
             const int pslot = pg_lo + i;
             int page = -1;
@@ -221,12 +226,13 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // the boxes of up to four tiles are requested in the time one thread needs for two.
     constexpr int HB = HD == 128 ? 2 : 1;                      // 64-column boxes per row
     constexpr int BOXES = (TKEYS / 16) * HB * 2;               // boxes of one tile: pages x halves x (K, V)
-    auto load_tiles_tma = [&](int sup) {
+    auto load_tiles_tma = [&](int sup, int slot) {               // the tiles of iteration `sup` into the ring's slot
+#pragma unroll 1
         for (int idx = lane; idx < ng * BOXES; idx += 32) {
             const int j = idx / BOXES, r = idx % BOXES;
-            const int tile = sup * ng + j;
+            const int tile = (sup << lg) + j;
             if (tile >= n_tiles) continue;
-            const int stage = (sup % super_stages) * ng + j;
+            const int stage = (slot << lg) + j;
             const int pg = r / (HB * 2), h = (r >> 1) % HB, is_v = r & 1;
             const uint32_t bar = smem_u32(&s_full[stage]);
             // the expected bytes may be posted after some of them have arrived: the phase cannot end before
@@ -251,7 +257,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         size_t off = 0;
         int bytes = 0;
         if (key < k_end) {
-            const int pslot = key / a.page_size;
+            const int pslot = key / page_size;
             int page = -1;
             if (pages_staged) page = s_pages[pslot - pg_lo];
             else if (pslot < a.max_pages) {
@@ -259,7 +265,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 if (page >= a.n_pages) page = -1;
             }
             if (page >= 0) {
-                off = (((size_t)page * a.n_kv + kh) * a.page_size + key % a.page_size) * HD;
+                off = (((size_t)page * a.n_kv + kh) * page_size + (key - pslot * page_size)) * HD;
                 bytes = 16;
             }
         }
@@ -270,60 +276,72 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             cp_async16(vdst + so, a.vp + off + (c0 + j) * 8, bytes);
         }
     };
-    auto load_super = [&](int sup) {                             // the ng tiles of iteration `sup`
-        if (use_tma) {
-            if (warp == 0) load_tiles_tma(sup);
+    auto load_super = [&](int sup, int slot) {                   // the ng tiles of iteration `sup`
+        if (TMA) {
+            if (warp == 0) load_tiles_tma(sup, slot);
         } else {
+#pragma unroll 1
             for (int j = 0; j < ng; ++j)
-                if (sup * ng + j < n_tiles) load_tile(sup * ng + j, (sup % super_stages) * ng + j);
+                if ((sup << lg) + j < n_tiles) load_tile((sup << lg) + j, (slot << lg) + j);
             cp_async_commit();                                   // one group per iteration, empty past the end
         }
     };
-    // prologue of the ring (all super_stages slots): iterations that lie wholly inside the committed prefix are
-    // requested before the wait, those holding this step's new rows (written by the preceding grid) after it
-    int issued = 0;
-    while (issued < super_stages && issued < n_super && k_begin + (issued + 1) * ng * TKEYS <= seq_pos0) {
-        load_super(issued);
-        ++issued;
-    }
-    griddep_wait();
-#ifdef TASC_TIMELINE
-    log_at_exit.ta = global_ns();
-#endif
-    griddep_launch_dependents();
-
-    // Q rows of this KV head's group, scaled, as (hi, lo) bf16 in swizzled shared memory.  All global reads
-    // are issued before the first conversion so that their latencies overlap.
-    constexpr int NQ = GP * (HD / 4) / THREADS;
+    // Prologue of the ring (all super_stages slots): iterations that lie wholly inside the committed prefix are
+    // requested before the wait, those holding this step's new rows (written by the preceding grid) after it, while the Q
+    // rows are on their way (past the end: nothing, or for cp.async an empty group).
+    // Q rows of this KV head's group, scaled, as (hi, lo) bf16 in swizzled shared memory.  The global reads of four rows of
+    // a thread are issued before the first conversion so that their latencies overlap.
+    constexpr int RPI = THREADS / (HD / 4);                      // rows of one reading of all threads
+    constexpr int NQ = GP / RPI < 4 ? GP / RPI : 4;
+    const int d4 = (tid % (HD / 4)) * 4;
     float4 qv[NQ];
+    auto q_rows = [&](int rho0) {
 #pragma unroll
-    for (int j = 0; j < NQ; ++j) {
-        const int i = tid + j * THREADS;
-        const int rho = i / (HD / 4), d4 = (i % (HD / 4)) * 4;
-        const int hl = rho / R, rr = rho % R;
-        qv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (rho < G && rr < rows)
-            qv[j] = *reinterpret_cast<const float4*>(a.q + (size_t)(b * a.R + rb + rr) * qd + (size_t)(h0 + hl) * HD + d4);
+        for (int j = 0; j < NQ; ++j) {
+            const int rho = rho0 + j * RPI, hl = a.by_R.div(rho), rr = rho - hl * R;
+            qv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (rho < G && rr < rows)
+                qv[j] = *reinterpret_cast<const float4*>(a.q + (size_t)(b * a.R + rb + rr) * qd + (size_t)(h0 + hl) * HD + d4);
+        }
+    };
+    int issued = 0;
+#pragma unroll 1
+    for (int behind = 0; behind < 2; ++behind) {
+        if (behind) {
+            griddep_wait();
+#ifdef TASC_TIMELINE
+            log_at_exit.ta = global_ns();
+#endif
+            griddep_launch_dependents();
+            q_rows(tid / (HD / 4));
+        }
+#pragma unroll 1
+        for (; issued < super_stages && (behind || (issued < n_super && k_begin + ((issued + 1) << lg) * TKEYS <= seq_pos0)); ++issued)
+            load_super(issued, issued);
     }
-    // the rest of the ring's prologue (tiles holding this step's new rows), requested while the Q rows are on their way
-    for (; issued < super_stages; ++issued) load_super(issued);       // past the end: nothing (cp.async: an empty group)
+#pragma unroll 1
+    for (int rho0 = tid / (HD / 4);;) {
 #pragma unroll
-    for (int j = 0; j < NQ; ++j) {
-        const int i = tid + j * THREADS;
-        const int rho = i / (HD / 4), d4 = (i % (HD / 4)) * 4;
-        const float4 v = make_float4(qv[j].x * a.scale_log2e, qv[j].y * a.scale_log2e, qv[j].z * a.scale_log2e, qv[j].w * a.scale_log2e);
-        uint2 h, l;
-        pack_hilo(v.x, v.y, h.x, l.x);
-        pack_hilo(v.z, v.w, h.y, l.y);
-        const uint32_t so = swz<HD, GP>(rho, d4 >> 3) + (uint32_t)((d4 & 7) * 2);
-        *reinterpret_cast<uint2*>(Qh + so) = h;
-        *reinterpret_cast<uint2*>(Ql + so) = l;
+        for (int j = 0; j < NQ; ++j) {
+            const int rho = rho0 + j * RPI;
+            if (rho >= n_slabs * 16) break;                      // (slabs that no warp works on)
+            uint2 h, l;
+            split_bf16x2(qv[j].x * a.scale_log2e, qv[j].y * a.scale_log2e, h.x, l.x);
+            split_bf16x2(qv[j].z * a.scale_log2e, qv[j].w * a.scale_log2e, h.y, l.y);
+            const uint32_t so = swz<HD, GP>(rho, d4 >> 3) + (uint32_t)((d4 & 7) * 2);
+            *reinterpret_cast<uint2*>(Qh + so) = h;
+            *reinterpret_cast<uint2*>(Ql + so) = l;
+        }
+        rho0 += NQ * RPI;
+        if (rho0 >= n_slabs * 16) break;
+        q_rows(rho0);
     }
 
     // per-thread rows of the slab: r0 = lane / 4 and r0 + 8
     const int rho0 = slab * 16 + (lane >> 2), rho1 = rho0 + 8;
-    const int lim0 = (rho0 < G && rho0 % R < rows) ? min(pos0 + rho0 % R, k_end - 1) : -1;   // last visible key
-    const int lim1 = (rho1 < G && rho1 % R < rows) ? min(pos0 + rho1 % R, k_end - 1) : -1;
+    const int rr0 = rho0 - a.by_R.div(rho0) * R, rr1 = rho1 - a.by_R.div(rho1) * R;
+    const int lim0 = (rho0 < G && rr0 < rows) ? min(pos0 + rr0, k_end - 1) : -1;   // last visible key
+    const int lim1 = (rho1 < G && rr1 < rows) ? min(pos0 + rr1, k_end - 1) : -1;
     float o[HD / 8][4];
 #pragma unroll
     for (int i = 0; i < HD / 8; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
@@ -333,11 +351,14 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     log_at_exit.tc = global_ns();
 #endif
 
+    int slot = 0;                                                  // of iteration `sup` in the ring, and its parity
+    uint32_t parity = 0;
+#pragma unroll 1
     for (int sup = 0; sup < n_super; ++sup) {
-        if (use_tma) {                                             // iteration `sup` has landed (bounded wait)
+        if (TMA) {                                                 // iteration `sup` has landed (bounded wait)
+#pragma unroll 1
             for (int j = 0; j < ng; ++j)
-                if (sup * ng + j < n_tiles &&
-                    !mbar_wait(smem_u32(&s_full[(sup % super_stages) * ng + j]), (uint32_t)(sup / super_stages) & 1u))
+                if ((sup << lg) + j < n_tiles && !mbar_wait(smem_u32(&s_full[(slot << lg) + j]), parity))
                     set_status(a.status, TASC_ETIMEOUT);
         } else {
             cp_async_wait_dyn(super_stages - 1);
@@ -348,9 +369,9 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         if (sup == 1) log_at_exit.te = global_ns();
         if (sup == 2) log_at_exit.tf = global_ns();
 #endif
-        const int tile = sup * ng + grp;
+        const int tile = (sup << lg) + grp;
         if (computes && tile < n_tiles) {
-            const int stage = (sup % super_stages) * ng + grp;
+            const int stage = (slot << lg) + grp;
             const int k0 = k_begin + tile * TKEYS;
             const uint32_t kbase = smem_u32(Kt + stage * TILE_BYTES), vbase = smem_u32(Vt + stage * TILE_BYTES);
             float s[8][4];
@@ -418,10 +439,10 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
             for (int kb = 0; kb < 4; ++kb) {
                 uint32_t ph[4], pl[4];
-                pack_hilo(s[2 * kb][0], s[2 * kb][1], ph[0], pl[0]);
-                pack_hilo(s[2 * kb][2], s[2 * kb][3], ph[1], pl[1]);
-                pack_hilo(s[2 * kb + 1][0], s[2 * kb + 1][1], ph[2], pl[2]);
-                pack_hilo(s[2 * kb + 1][2], s[2 * kb + 1][3], ph[3], pl[3]);
+                split_bf16x2(s[2 * kb][0], s[2 * kb][1], ph[0], pl[0]);
+                split_bf16x2(s[2 * kb][2], s[2 * kb][3], ph[1], pl[1]);
+                split_bf16x2(s[2 * kb + 1][0], s[2 * kb + 1][1], ph[2], pl[2]);
+                split_bf16x2(s[2 * kb + 1][2], s[2 * kb + 1][3], ph[3], pl[3]);
 #pragma unroll
                 for (int dp = 0; dp < HD / 16; dp += 2) {          // four independent accumulators per pass
                     uint32_t vb0[4], vb1[4];
@@ -440,8 +461,9 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         }
         __syncthreads();
         // the slot of this iteration is free again: refill it with the iteration super_stages ahead
-        if (sup + super_stages < n_super) load_super(sup + super_stages);
-        else if (!use_tma) cp_async_commit();
+        if (sup + super_stages < n_super) load_super(sup + super_stages, slot);
+        else if (!TMA) cp_async_commit();
+        if (++slot == super_stages) { slot = 0; parity ^= 1u; }
     }
 #ifdef TASC_TIMELINE
     log_at_exit.tb = global_ns();
@@ -464,6 +486,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         }
         __syncthreads();
         if (grp == 0) {
+#pragma unroll 1
             for (int og = 1; og < ng; ++og) {
                 const float* xg = xg0 + ((size_t)((og - 1) * n_slabs + slab) * 32 + lane) * XG;
                 const float om0 = xg[HD / 2], om1 = xg[HD / 2 + 1], ol0 = xg[HD / 2 + 2], ol1 = xg[HD / 2 + 3];
@@ -490,15 +513,14 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             for (int half = 0; half < 2; ++half) {
                 const int rho = half ? rho1 : rho0;
                 if (rho >= G) continue;
-                const int hl = rho / R, rr = rho % R;
+                const int hl = a.by_R.div(rho), rr = rho - hl * R;
                 const float inv = (rr < rows) ? (half ? inv1 : inv0) : 0.f;
-                const int m = b * a.R + rb + rr;
-                const size_t row = (size_t)(m / a.TB) * (2 * a.TB) + (m % a.TB);
+                const size_t row = out_row(b * a.R + rb + rr);
                 const size_t col = (size_t)(h0 + hl) * HD + 2 * (lane & 3);
 #pragma unroll
                 for (int nt = 0; nt < HD / 8; ++nt) {
                     uint32_t h, l;
-                    pack_hilo(o[nt][2 * half] * inv, o[nt][2 * half + 1] * inv, h, l);
+                    split_bf16x2(o[nt][2 * half] * inv, o[nt][2 * half + 1] * inv, h, l);
                     *reinterpret_cast<uint32_t*>(a.out + row * qd + col + nt * 8) = h;
                     *reinterpret_cast<uint32_t*>(a.out + (row + a.TB) * qd + col + nt * 8) = l;
                 }
@@ -533,10 +555,9 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     uint32_t peer[8];
 #pragma unroll
     for (int sidx = 0; sidx < 8; ++sidx) peer[sidx] = cluster_map(xo_addr, (uint32_t)(sidx < S ? sidx : 0));
-    const int my_rows = rank < G ? (G - rank + S - 1) / S : 0;
-    for (int i = tid; i < my_rows * (HD / 4); i += THREADS) {
-        const int rho = rank + (i / (HD / 4)) * S, d4 = (i % (HD / 4)) * 4;
-        const int hl = rho / R, rr = rho % R;
+#pragma unroll 1
+    for (int rho = rank + tid / (HD / 4) * S; rho < G; rho += RPI * S) {
+        const int hl = a.by_R.div(rho), rr = rho - hl * R;
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         if (rr < rows) {
             float2 ml[8];
@@ -563,12 +584,11 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             const float inv = den > 0.f ? 1.0f / den : 0.f;
             acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
         }
-        const int m = b * a.R + rb + rr;
-        const size_t row = (size_t)(m / a.TB) * (2 * a.TB) + (m % a.TB);
+        const size_t row = out_row(b * a.R + rb + rr);
         const size_t col = (size_t)(h0 + hl) * HD + d4;
         uint2 h, l;
-        pack_hilo(acc.x, acc.y, h.x, l.x);
-        pack_hilo(acc.z, acc.w, h.y, l.y);
+        split_bf16x2(acc.x, acc.y, h.x, l.x);
+        split_bf16x2(acc.z, acc.w, h.y, l.y);
         *reinterpret_cast<uint2*>(a.out + row * qd + col) = h;
         *reinterpret_cast<uint2*>(a.out + (row + a.TB) * qd + col) = l;
     }
@@ -581,14 +601,14 @@ inline size_t attn_smem_bytes(int hd, int gp, int stages) {
     return 1024 + (size_t)2 * gp * hd * 2 + (size_t)2 * stages * TKEYS * hd * 2;      // 1024: alignment slack
 }
 
-template <int HD, int NS>
+template <int HD, int NS, bool TMA>
 tasc_status prepare_inst() {
     static bool done[64] = {false};
     int dev = 0;
     TASC_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return TASC_EINVAL;
     if (!done[dev]) {
-        TASC_CUDA_TRY(cudaFuncSetAttribute(attn_mma_kernel<HD, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+        TASC_CUDA_TRY(cudaFuncSetAttribute(attn_mma_kernel<HD, NS, TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
         done[dev] = true;
     }
     return TASC_OK;
@@ -597,7 +617,7 @@ tasc_status prepare_inst() {
 // Clusters of `splits` CTAs (ring depth `stages`) the device holds at once; 0 if the query fails.
 template <int HD, int NS>
 int fit_inst(int splits, int stages) {
-    if (prepare_inst<HD, NS>() != TASC_OK) return 0;
+    if (prepare_inst<HD, NS, true>() != TASC_OK) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)splits, 1, 1);
     cfg.blockDim = dim3(256, 1, 1);
@@ -610,7 +630,7 @@ int fit_inst(int splits, int stages) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, attn_mma_kernel<HD, NS>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
+    if (cudaOccupancyMaxActiveClusters(&n, attn_mma_kernel<HD, NS, true>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
     return n;
 }
 
@@ -630,12 +650,12 @@ int fit_any(int hd, int nw, int splits, int stages) {
     return n;
 }
 
-template <int HD, int NS>
+template <int HD, int NS, bool TMA>
 tasc_status launch_inst(const AttnArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int B, cudaStream_t stream) {
     constexpr int GP = NS * 16;
     if (a.stages < 2 || a.stages > Ring<HD, NS>::MAX_STAGES) return TASC_EINVAL;
     const size_t smem = attn_smem_bytes(HD, GP, a.stages);
-    tasc_status pst = prepare_inst<HD, NS>();
+    tasc_status pst = prepare_inst<HD, NS, TMA>();
     if (pst != TASC_OK) return pst;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)a.splits, (unsigned)(a.n_kv * a.n_hsplit), (unsigned)B);
@@ -656,7 +676,7 @@ tasc_status launch_inst(const AttnArgs& a, const CUtensorMap& tmK, const CUtenso
     cfg.attrs = at;
     cfg.numAttrs = n_at;
     ProfScope ps(K_ATT_SPLIT, stream);
-    TASC_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_mma_kernel<HD, NS>, tmK, tmV, a));
+    TASC_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_mma_kernel<HD, NS, TMA>, tmK, tmV, a));
     return TASC_OK;
 }
 
@@ -743,26 +763,29 @@ tasc_status launch_attention_mma(const float* qbuf, const __nv_bfloat16* k_pages
     a.R = R; a.Rs = Rs; a.n_sub = n_sub; a.n_q = n_q; a.n_kv = n_kv; a.splits = n_splits; a.stages = plan.stages;
     a.scale_log2e = 1.4426950408889634f / sqrtf((float)hd);
     a.status = status;
-    // 16-token pages arrive as TMA boxes; any other page size takes the cp.async path of the same kernel
-    a.use_tma = page_size == 16 ? 1 : 0;
+    a.n_slabs = (G + 15) / 16;
+    a.by_R = SmallDiv(Rs); a.by_TB = SmallDiv(TB); a.by_splits = SmallDiv(n_splits); a.by_sub = SmallDiv(n_sub); a.by_hsplit = SmallDiv(g / hs);
+    // 16-token pages arrive as TMA boxes; any other page size, and caches of more pages than a CTA keeps the ids of, take the
+    // kernel with cp.async
+    const bool tma = page_size == 16 && (plan.tc || max_pages <= MAX_STAGED_PAGES);
     CUtensorMap tmK, tmV;
     memset(&tmK, 0, sizeof(tmK));
     memset(&tmV, 0, sizeof(tmV));
-    if (a.use_tma) {
+    if (tma) {
         const uint64_t rows = (uint64_t)n_pages * n_kv * 16;
         tasc_status st;
         if ((st = encode_tmap_kv(&tmK, k_pages, rows, hd)) != TASC_OK) return st;
         if ((st = encode_tmap_kv(&tmV, v_pages, rows, hd)) != TASC_OK) return st;
     }
     if (plan.tc) return launch_attention_tc(qbuf, tmK, tmV, block_table, max_pages, n_pages, rp, out, TB, B, R, n_q, n_kv, hd, plan, status, stream);
-    if (GP == 64) {
-        if (hd == 32) return launch_inst<32, 4>(a, tmK, tmV, B * n_sub, stream);
-        if (hd == 64) return launch_inst<64, 4>(a, tmK, tmV, B * n_sub, stream);
-        return launch_inst<128, 4>(a, tmK, tmV, B * n_sub, stream);
-    }
-    if (hd == 32) return launch_inst<32, 8>(a, tmK, tmV, B * n_sub, stream);
-    if (hd == 64) return launch_inst<64, 8>(a, tmK, tmV, B * n_sub, stream);
-    return launch_inst<128, 8>(a, tmK, tmV, B * n_sub, stream);
+    auto launch = [&](auto with_tma) {
+        constexpr bool T = decltype(with_tma)::value;
+        if (GP == 64) return hd == 32 ? launch_inst<32, 4, T>(a, tmK, tmV, B * n_sub, stream) : hd == 64 ? launch_inst<64, 4, T>(a, tmK, tmV, B * n_sub, stream)
+                                                                                                 : launch_inst<128, 4, T>(a, tmK, tmV, B * n_sub, stream);
+        return hd == 32 ? launch_inst<32, 8, T>(a, tmK, tmV, B * n_sub, stream) : hd == 64 ? launch_inst<64, 8, T>(a, tmK, tmV, B * n_sub, stream)
+                                                                                : launch_inst<128, 8, T>(a, tmK, tmV, B * n_sub, stream);
+    };
+    return tma ? launch(std::true_type{}) : launch(std::false_type{});
 }
 
 }  // namespace tasc

@@ -165,6 +165,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long budget = 1000000000ll) {
     if (mbar_try_wait(bar, parity)) return true;
     long long t0 = clock64();
+#pragma unroll 1
     while (!mbar_try_wait(bar, parity)) {
         if (clock64() - t0 > budget) return false;
     }
@@ -225,6 +226,21 @@ __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16& hi, __nv_bflo
     hi = __float2bfloat16_rn(v);
     lo = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
+
+// Two floats -> the packed bf16 pair (hi) and the packed pair of the residuals (lo); the same values as split_bf16 of each.
+__device__ __forceinline__ void split_bf16x2(float x, float y, uint32_t& hi, uint32_t& lo) {
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(y), "f"(x));
+    const float lx = x - __uint_as_float(hi << 16), ly = y - __uint_as_float(hi & 0xFFFF0000u);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(ly), "f"(lx));
+}
+
+// n / d by a multiplication, for n * d < 2^32 (the magic number is at most d / 2^32 too large: n times that stays below 1 / d).
+struct SmallDiv {
+    uint32_t d, magic;
+    __host__ __device__ SmallDiv() : d(1u), magic(0u) {}
+    __host__ explicit SmallDiv(int by) : d((uint32_t)by), magic((uint32_t)(((1ull << 32) + by - 1) / by)) {}
+    __device__ __forceinline__ int div(int n) const { return d == 1u ? n : (int)__umulhi((uint32_t)n, magic); }
+};
 
 // ---------------------------------------------------------------- TMA (tiled bulk tensor load into this CTA only)
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* m) {
