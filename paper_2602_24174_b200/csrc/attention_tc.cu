@@ -18,6 +18,10 @@
 // half of O 0.3, P 0.4, waits 0.4); 0.5B + 8,192 tokens at 32 x 9 rows, 640 keys 15.5 -> 13.4; prefill of 16 x 1,024 tokens
 // on the 1.5B 72 -> 47 us per pass of 2,048 rows.
 //
+// A CTA with a few tiles waits for code that it executes as often, so there is one copy of everything (the first tile's scores, the last
+// tile's O, both halves of a tile's load), ring slots are counted and rows divided by multiplication: 76 - 102 -> 47 - 66 KB.  A step
+// of the 0.5B + 8,192 tokens at 288 rows 1476 -> 1448 us, a generation of the 0.5B with 8 sequences 57.5 -> 56.2 ms.
+//
 // Every wait is bounded; after one that ran out the loops run on without waiting, so that all barriers are still met.
 #include "kernels.h"
 
@@ -45,16 +49,12 @@ struct TcArgs {
     __nv_bfloat16* out;
     int TB;
     int R, Rs, n_sub, n_q, n_kv, splits, stages;
+    int g;                                                       // query heads of a KV head
+    SmallDiv by_R, by_TB, by_splits, by_sub;
     int* status;
     float scale_log2e;
 };
 
-// two floats -> packed bf16 pair (hi) and the packed pair of the residuals (lo)
-__device__ __forceinline__ void pack_hilo(float x, float y, uint32_t& hi, uint32_t& lo) {
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(y), "f"(x));
-    const float rx = x - __uint_as_float(hi << 16), ry = y - __uint_as_float(hi & 0xFFFF0000u);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(ry), "f"(rx));
-}
 // 2^x; results below 2^-126 are zero here (.ftz)
 __device__ __forceinline__ float ex2(float x) {
     float y;
@@ -103,9 +103,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     __shared__ int s_fail;
     volatile int* failed = &s_fail;
 
-    const int sp = blockIdx.x, kh = blockIdx.y, b = blockIdx.z / a.n_sub, rb = (blockIdx.z % a.n_sub) * a.Rs;
+    const int sp = blockIdx.x, kh = blockIdx.y, b = a.by_sub.div(blockIdx.z), rb = ((int)blockIdx.z - b * a.n_sub) * a.Rs;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int g = a.n_q / a.n_kv, R = a.Rs, G = g * R, h0 = kh * g, qd = a.n_q * HD;
+    const int g = a.g, R = a.Rs, G = g * R, h0 = kh * g, qd = a.n_q * HD;
 #ifdef TASC_TIMELINE
     struct LogAtExit { unsigned long long t0, ta, tb, tc, td; __device__ ~LogAtExit() { if (threadIdx.x == 0) ctalog_put(t0, ta, tb, 11, tc, td); } } log_at_exit{global_ns(), 0, 0, 0, 0};
 #endif
@@ -114,18 +114,21 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     int rows = a.seq_rows[b] - rb;
     rows = rows < 0 ? 0 : (rows > R ? R : rows);
     const int pos0 = seq_pos0 + rb;
+    auto head_of = [&](int rho) { return a.by_R.div(rho); };      // a query row's head, and its row of the sequence
+    auto row_of = [&](int rho) { return rho - a.by_R.div(rho) * R; };
     auto out_row = [&](int rho) {
-        const int m = b * a.R + rb + rho % R;
-        return (size_t)(m / a.TB) * (2 * a.TB) + (m % a.TB);
+        const int m = b * a.R + rb + row_of(rho);
+        return (size_t)(a.by_TB.div(m) * a.TB + m);
     };
     if (rows == 0) {
         griddep_wait();
         griddep_launch_dependents();
         // sequence not in this pass: its rows of the output are zero
         if (sp == 0) {
+#pragma unroll 1
             for (int i = tid; i < G * (HD / 4); i += THREADS) {
                 const int rho = i / (HD / 4), d4 = (i % (HD / 4)) * 4;
-                const size_t row = out_row(rho), col = (size_t)(h0 + rho / R) * HD + d4;
+                const size_t row = out_row(rho), col = (size_t)(h0 + head_of(rho)) * HD + d4;
                 *reinterpret_cast<uint2*>(a.out + row * qd + col) = make_uint2(0u, 0u);
                 *reinterpret_cast<uint2*>(a.out + (row + a.TB) * qd + col) = make_uint2(0u, 0u);
             }
@@ -134,7 +137,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     }
     // this CTA's keys: the tiles are dealt out evenly over the splits
     const int total = pos0 + rows;
-    const int tiles_all = (total + TK - 1) / TK, t_base = tiles_all / a.splits, t_rem = tiles_all % a.splits;
+    const int tiles_all = (total + TK - 1) / TK, t_base = a.by_splits.div(tiles_all), t_rem = tiles_all - t_base * a.splits;
     const int n_tiles = t_base + (sp < t_rem ? 1 : 0);
     const int k_begin = (sp * t_base + min(sp, t_rem)) * TK;
     const int k_end = min(total, k_begin + n_tiles * TK);
@@ -147,26 +150,19 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     const uint32_t bar_s_full = bar_v_empty + 8u * MAX_RING, bar_s_empty = bar_s_full + 16u;
     const uint32_t bar_o_full = bar_s_empty + 16u, bar_o_empty = bar_o_full + 16u;
     const uint32_t bar_p_full = bar_o_empty + 16u, bar_q_full = bar_p_full + 8u;
-    if (tid == 0) {
-        s_fail = 0;
-        for (int i = 0; i < a.stages; ++i) {
-            mbar_init(bar_k_full + 8u * i, 1);
-            mbar_init(bar_v_full + 8u * i, 1);
-            mbar_init(bar_k_empty + 8u * i, 1);
-            mbar_init(bar_v_empty + 8u * i, 1);
+    if (warp == SM_WARPS) {
+        // a barrier per lane, in the order of their addresses: the ring's, S full, S empty, O full, O empty (two each), P, Q
+        constexpr int RING = 4 * MAX_RING;
+        if (lane < RING + 10)
+            mbar_init(bar_k_full + 8u * lane, lane == RING + 9 ? SM_WARPS * 32u : lane == RING + 8 || (lane >= RING && ((lane - RING) & 2)) ? arrivals : 1u);
+        if (lane == 31) {
+            s_fail = 0;
+            tma_prefetch_desc(&tmK);
+            tma_prefetch_desc(&tmV);
         }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(bar_s_full + 8u * i, 1);
-            mbar_init(bar_s_empty + 8u * i, arrivals);
-            mbar_init(bar_o_full + 8u * i, 1);
-            mbar_init(bar_o_empty + 8u * i, arrivals);
-        }
-        mbar_init(bar_p_full, arrivals);
-        mbar_init(bar_q_full, SM_WARPS * 32);
         fence_barrier_init();
-        tma_prefetch_desc(&tmK);
-        tma_prefetch_desc(&tmV);
     }
+#pragma unroll 1
     for (int i = tid; i < n_pg; i += THREADS) {
         const int pslot = pg_lo + i;
         int page = -1;
@@ -184,6 +180,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     auto wait = [&](uint32_t bar, uint32_t parity) {             // after a failure: no more waiting
         if (mbar_try_wait(bar, parity)) return;
         const long long t0 = clock64();
+#pragma unroll 1
         while (!mbar_try_wait(bar, parity)) {
             if (*failed) return;
             if (clock64() - t0 > 1000000000ll) { set_status(a.status, TASC_ETIMEOUT); *failed = 1; return; }
@@ -203,35 +200,35 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         // range re-read its last page, ids outside the pool read page 0: both are masked, and nothing unmapped is touched.
         // K and V have barriers of their own: K of a tile is free one softmax earlier than V.
         constexpr int BOXES = (TK / PAGE) * C::HB;
-        auto load = [&](int t, bool is_v) {
-            const int s = t % a.stages;
-            const uint32_t bar = (is_v ? bar_v_full : bar_k_full) + 8u * s;
-            const uint32_t base = smem_u32(ring + (size_t)s * 2 * C::KV_BYTES) + (is_v ? C::KV_BYTES : 0);
-            if (lane == 0) mbar_expect_tx(bar, C::KV_BYTES);
-            __syncwarp();
-            if (lane < BOXES) {
-                const int pg = lane / C::HB, h = lane % C::HB;
-                int key = k_begin + t * TK + pg * PAGE;
-                key = key < k_end ? key : k_end - 1;
-                int page = s_pages[key / PAGE - pg_lo];
-                page = page < 0 ? 0 : page;
-                tma_load_2d(base + h * (TK * 128) + pg * (PAGE * 128), is_v ? &tmV : &tmK, h * 64, (page * a.n_kv + kh) * PAGE, bar);
+        // Tiles of committed positions are requested before the preceding grid has finished, the others after it.
+        bool waited = false;
+        int s = 0;                                               // ring slot of tile t; its parity is the one of its use before
+        uint32_t used = 1u;
+#pragma unroll 1
+        for (int t = 0; t < n_tiles; ++t) {
+            if (!waited && (t >= a.stages || k_begin + (t + 1) * TK > seq_pos0)) { griddep_wait(); waited = true; }
+#pragma unroll 1
+            for (int is_v = 0; is_v < 2; ++is_v) {
+                if (t >= a.stages) wait((is_v ? bar_v_empty : bar_k_empty) + 8u * s, used);
+                if (warp_failed(failed)) break;
+                const uint32_t bar = (is_v ? bar_v_full : bar_k_full) + 8u * s;
+                const uint32_t base = smem_u32(ring + (size_t)s * 2 * C::KV_BYTES) + (is_v ? C::KV_BYTES : 0);
+                if (lane == 0) mbar_expect_tx(bar, C::KV_BYTES);
+                __syncwarp();
+                if (lane < BOXES) {
+                    const int pg = lane / C::HB, h = lane % C::HB;
+                    int key = k_begin + t * TK + pg * PAGE;
+                    key = key < k_end ? key : k_end - 1;
+                    int page = s_pages[key / PAGE - pg_lo];
+                    page = page < 0 ? 0 : page;
+                    tma_load_2d(base + h * (TK * 128) + pg * (PAGE * 128), is_v ? &tmV : &tmK, h * 64, (page * a.n_kv + kh) * PAGE, bar);
+                }
+                __syncwarp();
             }
-            __syncwarp();
-        };
-        // tiles of committed positions are requested before the preceding grid has finished, the others after it
-        int t = 0;
-        for (; t < a.stages && t < n_tiles && k_begin + (t + 1) * TK <= seq_pos0; ++t) { load(t, false); load(t, true); }
-        griddep_wait();
-        for (; t < n_tiles; ++t) {
-            const uint32_t used = (uint32_t)(t / a.stages - 1) & 1u;
-            if (t >= a.stages) wait(bar_k_empty + 8u * (t % a.stages), used);
             if (warp_failed(failed)) break;
-            load(t, false);
-            if (t >= a.stages) wait(bar_v_empty + 8u * (t % a.stages), used);
-            if (warp_failed(failed)) break;
-            load(t, true);
+            if (++s == a.stages) { s = 0; used ^= 1u; }
         }
+        if (!waited) griddep_wait();
         __syncwarp();
     } else if (warp == SM_WARPS + 1) {
         // ------------------------------------------------------------ MMA
@@ -240,38 +237,46 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
             const uint32_t qa = smem_u32(Qs), pa = smem_u32(Ps), kv = smem_u32(ring);
             constexpr uint32_t idesc_s = umma_idesc_bf16_f32(128, TK);
             constexpr uint32_t idesc_o = umma_idesc_bf16_f32(128, HD) | (1u << 16);      // V: columns along N
-            auto issue_s = [&](int t) {
-                wait(bar_k_full + 8u * (t % a.stages), (uint32_t)(t / a.stages) & 1u);
-                if (t >= 2) wait(bar_s_empty + 8u * (t & 1), (uint32_t)((t >> 1) - 1) & 1u);
-                tc_fence_after();
-                const uint32_t kb = kv + (uint32_t)(t % a.stages) * 2u * C::KV_BYTES, d = tmem + C::S_COL + (uint32_t)(t & 1) * TK;
-#pragma unroll
-                for (int p = 0; p < 2; ++p)                      // hi, lo
-#pragma unroll
-                    for (int ks = 0; ks < HD / 16; ++ks)
-                        umma_bf16_warp(d, umma_desc_k_sw128(qa + p * C::Q_BYTES + (ks >> 2) * (RP * 128) + (ks & 3) * 32),
-                                  umma_desc_k_sw128(kb + (ks >> 2) * (TK * 128) + (ks & 3) * 32), idesc_s, (p | ks) ? 1u : 0u);
-                umma_commit_warp(bar_s_full + 8u * (t & 1));
-                umma_commit_warp(bar_k_empty + 8u * (t % a.stages));
-            };
+            const uint64_t dq = umma_desc_k_sw128(qa), dp = umma_desc_k_sw128(pa);
             wait(bar_q_full, 0u);
-            tc_fence_after();
-            issue_s(0);
-            for (int t = 0; t < n_tiles; ++t) {
-                if (t + 1 < n_tiles) issue_s(t + 1);
-                wait(bar_v_full + 8u * (t % a.stages), (uint32_t)(t / a.stages) & 1u);
+            int sk = 0, sv = 0;                                  // ring slots of the next K and V tiles, and their parities
+            uint32_t pk = 0u, pv = 0u;
+#pragma unroll 1
+            for (int t = -1; t < n_tiles; ++t) {
+                if (t + 1 < n_tiles) {
+                    const int u = t + 1;                         // S of the next tile
+                    wait(bar_k_full + 8u * sk, pk);
+                    if (u >= 2) wait(bar_s_empty + 8u * (u & 1), (uint32_t)((u >> 1) - 1) & 1u);
+                    tc_fence_after();
+                    const uint64_t dk = umma_desc_k_sw128(kv + (uint32_t)sk * 2u * C::KV_BYTES);
+                    const uint32_t d = tmem + C::S_COL + (uint32_t)(u & 1) * TK;
+                    // (addresses in units of 16 bytes)
+#pragma unroll
+                    for (int p = 0; p < 2; ++p)                  // hi, lo
+#pragma unroll
+                        for (int ks = 0; ks < HD / 16; ++ks)
+                            umma_bf16_warp(d, dq + (p * C::Q_BYTES + (ks >> 2) * (RP * 128) + (ks & 3) * 32) / 16,
+                                           dk + ((ks >> 2) * (TK * 128) + (ks & 3) * 32) / 16, idesc_s, (p | ks) ? 1u : 0u);
+                    umma_commit_warp(bar_s_full + 8u * (u & 1));
+                    umma_commit_warp(bar_k_empty + 8u * sk);
+                    if (++sk == a.stages) { sk = 0; pk ^= 1u; }
+                }
+                if (t < 0) continue;
+                wait(bar_v_full + 8u * sv, pv);
                 wait(bar_p_full, (uint32_t)t & 1u);
                 if (t >= 2) wait(bar_o_empty + 8u * (t & 1), (uint32_t)((t >> 1) - 1) & 1u);
                 tc_fence_after();
-                const uint32_t vb = kv + (uint32_t)(t % a.stages) * 2u * C::KV_BYTES + C::KV_BYTES, d = tmem + C::O_COL + (uint32_t)(t & 1) * HD;
+                const uint64_t dv = umma_desc_mn_sw128(kv + (uint32_t)sv * 2u * C::KV_BYTES + C::KV_BYTES, TK * 128);
+                const uint32_t d = tmem + C::O_COL + (uint32_t)(t & 1) * HD;
 #pragma unroll
                 for (int p = 0; p < 2; ++p)
 #pragma unroll
                     for (int kk = 0; kk < TK / 16; ++kk)
-                        umma_bf16_warp(d, umma_desc_k_sw128(pa + p * C::P_BYTES + (kk >> 2) * (RP * 128) + (kk & 3) * 32),
-                                  umma_desc_mn_sw128(vb + kk * (16 * 128), TK * 128), idesc_o, (p | kk) ? 1u : 0u);
+                        umma_bf16_warp(d, dp + (p * C::P_BYTES + (kk >> 2) * (RP * 128) + (kk & 3) * 32) / 16, dv + kk * (16 * 128 / 16), idesc_o,
+                                       (p | kk) ? 1u : 0u);
                 umma_commit_warp(bar_o_full + 8u * (t & 1));          // also: P is free
-                umma_commit_warp(bar_v_empty + 8u * (t % a.stages));
+                umma_commit_warp(bar_v_empty + 8u * sv);
+                if (++sv == a.stages) { sv = 0; pv ^= 1u; }
             }
         }
         __syncwarp();
@@ -284,24 +289,27 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         griddep_launch_dependents();
         // Q rows, scaled, as (hi, lo) in shared memory; zeros where there is no row
         {
-            constexpr int NQ = RP * (HD / 4) / (SM_WARPS * 32);
-            float4 qv[NQ];
+            constexpr int RPI = SM_WARPS * 32 / (HD / 4);        // rows of one reading of all threads; four readings under way together
+            const int d4 = (tid % (HD / 4)) * 4, chunk = (d4 & 63) >> 3;
+#pragma unroll 1
+            for (int r0 = tid / (HD / 4); r0 < RP; r0 += 4 * RPI) {
+                float4 qv[4];
 #pragma unroll
-            for (int j = 0; j < NQ; ++j) {
-                const int i = tid + j * (SM_WARPS * 32), r = i / (HD / 4), d4 = (i % (HD / 4)) * 4;
-                qv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (r < G && r % R < rows) qv[j] = *reinterpret_cast<const float4*>(a.q + (size_t)(b * a.R + rb + r % R) * qd + (size_t)(h0 + r / R) * HD + d4);
-            }
+                for (int j = 0; j < 4; ++j) {
+                    const int r = r0 + j * RPI, hl = head_of(r), rr = r - hl * R;
+                    qv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (r < G && rr < rows) qv[j] = *reinterpret_cast<const float4*>(a.q + (size_t)(b * a.R + rb + rr) * qd + (size_t)(h0 + hl) * HD + d4);
+                }
 #pragma unroll
-            for (int j = 0; j < NQ; ++j) {
-                const int i = tid + j * (SM_WARPS * 32), r = i / (HD / 4), d4 = (i % (HD / 4)) * 4;
-                uint2 h, l;
-                pack_hilo(qv[j].x * a.scale_log2e, qv[j].y * a.scale_log2e, h.x, l.x);
-                pack_hilo(qv[j].z * a.scale_log2e, qv[j].w * a.scale_log2e, h.y, l.y);
-                const int chunk = (d4 & 63) >> 3;
-                const uint32_t off = (uint32_t)((d4 >> 6) * (RP * 128) + r * 128 + ((chunk ^ (r & 7)) << 4) + (d4 & 7) * 2);
-                *reinterpret_cast<uint2*>(Qs + off) = h;
-                *reinterpret_cast<uint2*>(Qs + C::Q_BYTES + off) = l;
+                for (int j = 0; j < 4; ++j) {
+                    const int r = r0 + j * RPI;
+                    uint2 h, l;
+                    split_bf16x2(qv[j].x * a.scale_log2e, qv[j].y * a.scale_log2e, h.x, l.x);
+                    split_bf16x2(qv[j].z * a.scale_log2e, qv[j].w * a.scale_log2e, h.y, l.y);
+                    const uint32_t off = (uint32_t)((d4 >> 6) * (RP * 128) + r * 128 + ((chunk ^ (r & 7)) << 4) + (d4 & 7) * 2);
+                    *reinterpret_cast<uint2*>(Qs + off) = h;
+                    *reinterpret_cast<uint2*>(Qs + C::Q_BYTES + off) = l;
+                }
             }
             fence_proxy_async_smem();
             mbar_arrive(bar_q_full);
@@ -313,9 +321,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         for (int e = 0; e < OC; ++e) acc[e] = 0.f;
         if (active) {
             const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-            const int lim = (rho < G && rho % R < rows) ? min(pos0 + rho % R, k_end - 1) : -1;      // last visible key
+            const int lim = (rho < G && row_of(rho) < rows) ? min(pos0 + row_of(rho), k_end - 1) : -1;      // last visible key
             float al_o = 1.f;                                    // from acc's maximum to the one of the tile that is added next
-            auto add_o = [&](int t) {                            // O = O * al_o + the product of tile t
+            // O = O * al_o + the product of tile t.  (One copy of everything: a CTA with two or three tiles waits for code it executes
+            // as often.)
+            auto add_o = [&](int t) {
                 wait(bar_o_full + 8u * (t & 1), (uint32_t)(t >> 1) & 1u);
                 tc_fence_after();
 #pragma unroll
@@ -330,8 +340,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                 mbar_arrive(bar_o_empty + 8u * (t & 1));
             };
             constexpr int SC = C::SC;
-            for (int t = 0; t < n_tiles; ++t) {
-                float s[SC];
+            float s[SC];
+#pragma unroll 1
+            for (int t = 0; n_tiles > 0 && t <= n_tiles; ++t) {
+                float al = 0.f;
+                if (t < n_tiles) {
                 wait(bar_s_full + 8u * (t & 1), (uint32_t)(t >> 1) & 1u);
 #ifdef TASC_TIMELINE
                 if (t == 0) log_at_exit.td = global_ns();
@@ -359,22 +372,24 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                 s_max[t & 1][half][rho] = mx;
                 asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory");      // the quarter's two warps
                 const float mn = fmaxf(m_run, fmaxf(mx, s_max[t & 1][half ^ 1][rho])), mu = mn == -INFINITY ? 0.f : mn;
-                const float al = ex2(m_run - mu);                // 0 while nothing was visible
+                al = ex2(m_run - mu);                            // 0 while nothing was visible
                 m_run = mn;
                 float p4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                 for (int e = 0; e < SC; ++e) { s[e] = ex2(s[e] - mu); p4[e & 3] += s[e]; }
                 l_run = l_run * al + ((p4[0] + p4[1]) + (p4[2] + p4[3]));
+                }
                 if (t > 0) add_o(t - 1);                         // (P of tile t - 1 has been used: its place is free)
+                if (t == n_tiles) break;
                 al_o = al;
                 // P, half row: 16-byte chunks of eight keys
 #pragma unroll
                 for (int c = 0; c < SC / 8; ++c) {
                     uint4 h, l;
-                    pack_hilo(s[8 * c], s[8 * c + 1], h.x, l.x);
-                    pack_hilo(s[8 * c + 2], s[8 * c + 3], h.y, l.y);
-                    pack_hilo(s[8 * c + 4], s[8 * c + 5], h.z, l.z);
-                    pack_hilo(s[8 * c + 6], s[8 * c + 7], h.w, l.w);
+                    split_bf16x2(s[8 * c], s[8 * c + 1], h.x, l.x);
+                    split_bf16x2(s[8 * c + 2], s[8 * c + 3], h.y, l.y);
+                    split_bf16x2(s[8 * c + 4], s[8 * c + 5], h.z, l.z);
+                    split_bf16x2(s[8 * c + 6], s[8 * c + 7], h.w, l.w);
                     const int kc = half * (SC / 8) + c;          // chunk of the row
                     const uint32_t off = (uint32_t)((kc >> 3) * (RP * 128) + rho * 128 + (((kc & 7) ^ (rho & 7)) << 4));
                     *reinterpret_cast<uint4*>(Ps + off) = h;
@@ -383,7 +398,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                 fence_proxy_async_smem();
                 mbar_arrive(bar_p_full);
             }
-            if (n_tiles > 0) add_o(n_tiles - 1);
             s_sum[half][rho] = l_run;
             asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory");
             l_run += s_sum[half ^ 1][rho];
@@ -407,15 +421,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     const int col0 = half * OC;
     if (a.splits == 1) {
         if (active && rho < G) {
-            const float inv = l_run > 0.f && rho % R < rows ? 1.0f / l_run : 0.f;
-            const size_t row = out_row(rho), col = (size_t)(h0 + rho / R) * HD + col0;
+            const float inv = l_run > 0.f && row_of(rho) < rows ? 1.0f / l_run : 0.f;
+            const size_t row = out_row(rho), col = (size_t)(h0 + head_of(rho)) * HD + col0;
 #pragma unroll
             for (int e = 0; e < OC; e += 8) {
                 uint4 h, l;
-                pack_hilo(acc[e] * inv, acc[e + 1] * inv, h.x, l.x);
-                pack_hilo(acc[e + 2] * inv, acc[e + 3] * inv, h.y, l.y);
-                pack_hilo(acc[e + 4] * inv, acc[e + 5] * inv, h.z, l.z);
-                pack_hilo(acc[e + 6] * inv, acc[e + 7] * inv, h.w, l.w);
+                split_bf16x2(acc[e] * inv, acc[e + 1] * inv, h.x, l.x);
+                split_bf16x2(acc[e + 2] * inv, acc[e + 3] * inv, h.y, l.y);
+                split_bf16x2(acc[e + 4] * inv, acc[e + 5] * inv, h.z, l.z);
+                split_bf16x2(acc[e + 6] * inv, acc[e + 7] * inv, h.w, l.w);
                 *reinterpret_cast<uint4*>(a.out + row * qd + col + e) = h;
                 *reinterpret_cast<uint4*>(a.out + (row + a.TB) * qd + col + e) = l;
             }
@@ -436,11 +450,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     uint32_t peer[8];
 #pragma unroll
     for (int s = 0; s < 8; ++s) peer[s] = cluster_map(smem_u32(xo), (uint32_t)(s < S ? s : 0));
-    const int my_rows = rank < G ? (G - rank + S - 1) / S : 0;
-    for (int i = tid; i < my_rows * (HD / 4); i += THREADS) {
-        const int r = rank + (i / (HD / 4)) * S, d4 = (i % (HD / 4)) * 4;
+#pragma unroll 1
+    for (int r = rank + tid / (HD / 4) * S; r < G; r += THREADS / (HD / 4) * S) {
+        const int d4 = (tid % (HD / 4)) * 4;
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r % R < rows) {
+        if (row_of(r) < rows) {
             float2 ml[8];
             float4 ov[8];
 #pragma unroll
@@ -462,10 +476,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
             const float inv = den > 0.f ? 1.0f / den : 0.f;
             o.x *= inv; o.y *= inv; o.z *= inv; o.w *= inv;
         }
-        const size_t row = out_row(r), col = (size_t)(h0 + r / R) * HD + d4;
+        const size_t row = out_row(r), col = (size_t)(h0 + head_of(r)) * HD + d4;
         uint2 h, l;
-        pack_hilo(o.x, o.y, h.x, l.x);
-        pack_hilo(o.z, o.w, h.y, l.y);
+        split_bf16x2(o.x, o.y, h.x, l.x);
+        split_bf16x2(o.z, o.w, h.y, l.y);
         *reinterpret_cast<uint2*>(a.out + row * qd + col) = h;
         *reinterpret_cast<uint2*>(a.out + (row + a.TB) * qd + col) = l;
     }
@@ -589,6 +603,8 @@ tasc_status launch_attention_tc(const float* qbuf, const CUtensorMap& tmK, const
     a.R = R; a.Rs = Rs; a.n_sub = R / Rs; a.n_q = n_q; a.n_kv = n_kv; a.splits = plan.splits; a.stages = plan.stages;
     a.scale_log2e = 1.4426950408889634f / sqrtf((float)hd);
     a.status = status;
+    a.g = n_q / n_kv;
+    a.by_R = SmallDiv(Rs); a.by_TB = SmallDiv(TB); a.by_splits = SmallDiv(plan.splits); a.by_sub = SmallDiv(a.n_sub);
     const int blocks = B * a.n_sub;
     if (hd == 64) return G <= 64 ? launch_inst<64, 64>(a, tmK, tmV, blocks, stream) : launch_inst<64, 128>(a, tmK, tmV, blocks, stream);
     return G <= 64 ? launch_inst<128, 64>(a, tmK, tmV, blocks, stream) : launch_inst<128, 128>(a, tmK, tmV, blocks, stream);
