@@ -31,15 +31,12 @@ constexpr int KEYS = 8;                          // keys of an attention step: f
 constexpr int MAX_HD = 256;
 constexpr int MAX_SMEM = 220 * 1024;
 
-__device__ __forceinline__ void cluster_sync_all() { cluster_arrive(); cluster_wait(); }
 #ifdef TASC_TIMELINE
 // A stage of a CTA: start, rows staged, work done, behind the barrier.
 #define TL_STAGED() (tl_a = global_ns())
 #define TL_END(tag) do { if (threadIdx.x == 0) ctalog_put(tl_0, tl_a, tl_b, tag); tl_0 = tl_a = global_ns(); } while (0)
-#define TL_SYNC(tag) do { tl_b = global_ns(); cluster_sync_all(); TL_END(tag); } while (0)
 #else
 #define TL_STAGED() do { } while (0)
-#define TL_SYNC(tag) cluster_sync_all()
 #endif
 
 // Sums of eight values over the warp's lanes; lane l gets the sum of value l / 4.
@@ -61,23 +58,28 @@ __device__ __forceinline__ float sum8(float (&v)[ROWS]) {
 }
 __device__ __forceinline__ float4 ldg_fresh(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }   // another CTA's result
 
-// y[r] = dot(w0, x row r), z[r] = dot(w1, x row r) for eight rows.
-__device__ __forceinline__ void dot_pair(const float* __restrict__ w0, const float* __restrict__ w1, const float* x0, int K,
+// y[r] = dot(w0, x row r), z[r] = dot(w1, x row r) for eight rows; a, b: the lane's first weights, there already.
+__device__ __forceinline__ void dot_pair(const float* __restrict__ w0, const float* __restrict__ w1, float4 a, float4 b, const float* x0, int K,
                                          float (&y)[ROWS], float (&z)[ROWS]) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) y[r] = z[r] = 0.f;
-#pragma unroll 2
-    for (int k = 4 * lane; k < K; k += 128) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(w0 + k)), b = __ldg(reinterpret_cast<const float4*>(w1 + k));
+#pragma unroll 1
+    for (int k = 4 * lane; k < K;) {
+        const int next = k + 128;
+        float4 a2 = a, b2 = b;
+        if (next < K) { a2 = __ldg(reinterpret_cast<const float4*>(w0 + next)); b2 = __ldg(reinterpret_cast<const float4*>(w1 + next)); }
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
             const float4 x = *reinterpret_cast<const float4*>(x0 + r * K + k);
             y[r] = fmaf(a.x, x.x, fmaf(a.y, x.y, fmaf(a.z, x.z, fmaf(a.w, x.w, y[r]))));
             z[r] = fmaf(b.x, x.x, fmaf(b.y, x.y, fmaf(b.z, x.z, fmaf(b.w, x.w, z[r]))));
         }
+        k = next; a = a2; b = b2;
     }
 }
+
+enum { ST_QKV, ST_ATTN, ST_O, ST_GATE_UP, ST_DOWN, ST_LM };      // the stages of a layer, and the LM head
 
 // NJ: 32-wide pieces of a head.
 template <int NJ>
@@ -94,10 +96,12 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
 
 #ifdef TASC_TIMELINE
     unsigned long long tl_0 = global_ns(), tl_a = tl_0, tl_b = tl_0;
+    int tl_tag = 0;
 #endif
     // ---- row plan: every CTA for itself, CTA 0 for the kernels behind
+#pragma unroll 1
     for (int m = threadIdx.x; m < M; m += THREADS) {
-        const int b = m / a.R, r = m % a.R, L = a.len[b];
+        const int b = a.by_R.div(m), r = m - b * a.R, L = a.len[b];
         const bool len_ok = L >= 1 && L <= a.stride;
         if (!len_ok) set_status(a.status, TASC_EINVAL);
         int tok = 0, pos = -1, pos0 = 0, rows = 0;
@@ -128,112 +132,167 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x + cta * THREADS; i < M * (d / 4); i += CTAS * THREADS) {
-        const int m = i / (d / 4), j = (i % (d / 4)) * 4;
-        *reinterpret_cast<float4*>(a.x + (size_t)m * d + j) = __ldg(reinterpret_cast<const float4*>(a.embed + (size_t)s_tok[m] * d + j));
-    }
-    // rows of the residual stream -> RMS norm * gain in shared memory (first: straight from the embedding)
-    auto stage_norm = [&](const float* gain, bool first) {
-        for (int m = warp; m < M; m += WARPS) {
-            const float* src = first ? a.embed + (size_t)s_tok[m] * d : a.x + (size_t)m * d;
-            float ss = 0.f;
-            for (int j = 4 * lane; j < d; j += 128) {
-                const float4 v = ldg_fresh(src + j);
-                *reinterpret_cast<float4*>(xs + (size_t)m * d + j) = v;
-                ss += (v.x * v.x + v.y * v.y) + (v.z * v.z + v.w * v.w);
+#pragma unroll 1
+    for (int m = warp; m < M; m += WARPS)                        // (row m by CTA m % CTAS)
+        if (m % CTAS == cta)
+            for (int j = 4 * lane; j < d; j += 128) *reinterpret_cast<float4*>(a.x + (size_t)m * d + j) = __ldg(reinterpret_cast<const float4*>(a.embed + (size_t)s_tok[m] * d + j));
+    // One copy of a stage's code for all products: a stage is a microsecond or two, of which the instructions of five copies took
+    // most (128 KB of kernel, a third of the instruction-cache requests missed; now 30 KB).  A stage's first weights, which
+    // depend on nothing, are requested before the barrier that precedes it.
+    int stage = ST_QKV, l = 0;
+    LayerWeightsF32 lw = a.layers[0];
+    bool first = true;
+#pragma unroll 1
+    for (;;) {
+        if (stage == ST_LM && !a.lm_head) { if (!first) cluster_wait(); return; }
+        if (stage != ST_ATTN) {
+            const float* W = stage == ST_QKV ? lw.wqkv : stage == ST_O ? lw.wo : stage == ST_GATE_UP ? lw.w_gate_up : stage == ST_DOWN ? lw.w_down : a.lm_head;
+            const int K = stage == ST_O ? qd : stage == ST_DOWN ? a.dff : d;
+            const int n_pairs = stage == ST_QKV ? (a.n_q + 2 * a.n_kv) * half : stage == ST_GATE_UP ? a.dff : stage == ST_LM ? (a.vocab + 1) / 2 : d / 2;
+            // a pair's weight rows: the halves of a rotary pair (value heads: the same pairs, not rotated), a gate row and its up row,
+            // two neighbouring features
+            auto rows_of = [&](int p, const float*& w0, const float*& w1) {
+                int r0 = 2 * p, r1 = 2 * p + 1;
+                if (stage == ST_QKV) { const int head = a.by_half.div(p); r0 = p + head * half; r1 = r0 + half; }
+                else if (stage == ST_GATE_UP) { r0 = p; r1 = a.dff + p; }
+                else if (stage == ST_LM) r1 = min(r1, a.vocab - 1);
+                w0 = W + (size_t)r0 * K;
+                w1 = W + (size_t)r1 * K;
+            };
+            const float *w0 = W, *w1 = W;
+            float4 wa = make_float4(0.f, 0.f, 0.f, 0.f), wb = wa;
+            if (gw < n_pairs) {
+                rows_of(gw, w0, w1);
+                if (4 * lane < K) { wa = __ldg(reinterpret_cast<const float4*>(w0 + 4 * lane)); wb = __ldg(reinterpret_cast<const float4*>(w1 + 4 * lane)); }
             }
-            const float inv = 1.0f / sqrtf(warp_sum(ss) / (float)d + a.eps);
-            for (int j = 4 * lane; j < d; j += 128) {            // (a lane's own values)
-                float4 v = *reinterpret_cast<float4*>(xs + (size_t)m * d + j);
-                const float4 g = __ldg(reinterpret_cast<const float4*>(gain + j));
-                v.x *= inv * g.x; v.y *= inv * g.y; v.z *= inv * g.z; v.w *= inv * g.w;
-                *reinterpret_cast<float4*>(xs + (size_t)m * d + j) = v;
+            if (!first) cluster_wait();
+#ifdef TASC_TIMELINE
+            if (!first) TL_END(tl_tag);
+#endif
+            if (stage == ST_O || stage == ST_DOWN) {
+                const float* src = stage == ST_O ? a.o : a.act;
+#pragma unroll 1
+                for (int i = threadIdx.x; i < M * (K / 4); i += THREADS) *reinterpret_cast<float4*>(xs + 4 * (size_t)i) = ldg_fresh(src + 4 * (size_t)i);
+            } else {
+                // rows of the residual stream -> RMS norm * gain in shared memory (first: straight from the embedding)
+                const float* gain = stage == ST_QKV ? lw.attn_norm : stage == ST_GATE_UP ? lw.mlp_norm : a.final_norm;
+#pragma unroll 1
+                for (int m = warp; m < M; m += WARPS) {
+                    const float* src = first ? a.embed + (size_t)s_tok[m] * d : a.x + (size_t)m * d;
+                    float ss = 0.f;
+#pragma unroll 1
+                    for (int j = 4 * lane; j < d; j += 128) {
+                        const float4 v = ldg_fresh(src + j);
+                        *reinterpret_cast<float4*>(xs + (size_t)m * d + j) = v;
+                        ss += (v.x * v.x + v.y * v.y) + (v.z * v.z + v.w * v.w);
+                    }
+                    const float inv = 1.0f / sqrtf(warp_sum(ss) / (float)d + a.eps);
+#pragma unroll 1
+                    for (int j = 4 * lane; j < d; j += 128) {    // (a lane's own values)
+                        float4 v = *reinterpret_cast<float4*>(xs + (size_t)m * d + j);
+                        const float4 g = __ldg(reinterpret_cast<const float4*>(gain + j));
+                        v.x *= inv * g.x; v.y *= inv * g.y; v.z *= inv * g.z; v.w *= inv * g.w;
+                        *reinterpret_cast<float4*>(xs + (size_t)m * d + j) = v;
+                    }
+                }
             }
-        }
-        __syncthreads();
-        TL_STAGED();
-    };
-    auto stage_rows = [&](const float* src, int K) {
-        for (int i = threadIdx.x; i < M * (K / 4); i += THREADS) *reinterpret_cast<float4*>(xs + 4 * (size_t)i) = ldg_fresh(src + 4 * (size_t)i);
-        __syncthreads();
-        TL_STAGED();
-    };
-    // n_pairs pairs of weight rows; emit(pair, token row, dot with the first, dot with the second), one lane per value
-    auto product = [&](int n_pairs, int K, auto row0, auto row1, auto emit) {
-        for (int p = gw; p < n_pairs; p += CTAS * WARPS) {
-            const float *w0 = row0(p), *w1 = row1(p);
-            for (int m0 = 0; m0 < M; m0 += ROWS) {
-                float y[ROWS], z[ROWS];
-                dot_pair(w0, w1, xs + (size_t)m0 * K, K, y, z);
-                const float v0 = sum8(y), v1 = sum8(z);
-                const int m = m0 + (lane >> 2);
-                if ((lane & 3) == 0 && m < M) emit(p, m, v0, v1);
+            first = false;
+            __syncthreads();
+            TL_STAGED();
+            float* kp = a.kv_pool + (size_t)l * 2 * a.kv_half;
+#pragma unroll 1
+            for (int p = gw; p < n_pairs;) {
+#pragma unroll 1
+                for (int m0 = 0; m0 < M; m0 += ROWS) {
+                    float y[ROWS], z[ROWS];
+                    dot_pair(w0, w1, wa, wb, xs + (size_t)m0 * K, K, y, z);
+                    float v0 = sum8(y), v1 = sum8(z);
+                    const int m = m0 + (lane >> 2);
+                    if ((lane & 3) != 0 || m >= M) continue;
+                    if (stage == ST_O || stage == ST_DOWN) {
+                        float2* x = reinterpret_cast<float2*>(a.x + (size_t)m * d + 2 * p);
+                        float2 t = __ldcg(x);
+                        t.x += v0; t.y += v1;
+                        *x = t;
+                    } else if (stage == ST_GATE_UP) {
+                        a.act[(size_t)m * a.dff + p] = v0 / (1.0f + expf(-v0)) * v1;
+                    } else if (stage == ST_LM) {
+                        unsigned long long best = pack_argmax(v0, (uint32_t)(2 * p));
+                        if (2 * p + 1 < a.vocab) best = max(best, pack_argmax(v1, (uint32_t)(2 * p + 1)));
+                        atomicMax(&s_best[m], best);
+                        if (a.logits) {
+                            a.logits[(size_t)m * a.vocab + 2 * p] = v0;
+                            if (2 * p + 1 < a.vocab) a.logits[(size_t)m * a.vocab + 2 * p + 1] = v1;
+                        }
+                    } else {
+                        const int head = a.by_half.div(p), i = p - head * half, pos = s_pos[m];
+                        float* out = a.q + (size_t)m * qd + head * hd;
+                        if (pos < 0) {
+                            if (head >= a.n_q) continue;
+                            v0 = v1 = 0.f;
+                        } else if (pos >= a.max_positions) {
+                            set_status(a.status, TASC_EINVAL);
+                            continue;
+                        } else if (head < a.n_q + a.n_kv) {
+                            const float2 c = a.rope[(size_t)pos * half + i];
+                            const float r0 = v0 * c.x - v1 * c.y, r1 = v1 * c.x + v0 * c.y;
+                            v0 = r0; v1 = r1;
+                        }
+                        if (head >= a.n_q) {
+                            const int pslot = (int)((unsigned)pos / (unsigned)a.page_size);
+                            int page = -1;
+                            if (pslot < a.max_pages) page = a.block_table[(size_t)a.by_R.div(m) * a.max_pages + pslot];
+                            if (page < 0 || page >= a.n_pages) { set_status(a.status, TASC_ENOKV); continue; }
+                            const bool is_k = head < a.n_q + a.n_kv;
+                            out = kp + (is_k ? 0 : a.kv_half) + (((size_t)page * a.n_kv + (head - a.n_q - (is_k ? 0 : a.n_kv))) * a.page_size + pos - pslot * a.page_size) * hd;
+                        }
+                        out[i] = v0;
+                        out[i + half] = v1;
+                    }
+                }
+                p += CTAS * WARPS;
+                if (p < n_pairs) {
+                    rows_of(p, w0, w1);
+                    if (4 * lane < K) { wa = __ldg(reinterpret_cast<const float4*>(w0 + 4 * lane)); wb = __ldg(reinterpret_cast<const float4*>(w1 + 4 * lane)); }
+                }
             }
-        }
-    };
-    // a product whose output is added to the residual stream
-    auto residual = [&](const float* W, int K) {
-        product(d / 2, K, [&](int p) { return W + (size_t)(2 * p) * K; }, [&](int p) { return W + (size_t)(2 * p + 1) * K; },
-                [&](int p, int m, float v0, float v1) {
-                    float2* x = reinterpret_cast<float2*>(a.x + (size_t)m * d + 2 * p);
-                    float2 t = __ldcg(x);
-                    t.x += v0; t.y += v1;
-                    *x = t;
-                });
-    };
-
-    for (int l = 0; l < a.n_layers; ++l) {
-        const LayerWeightsF32 lw = a.layers[l];
+            if (stage == ST_LM) {
+                __syncthreads();
+#ifdef TASC_TIMELINE
+                tl_b = global_ns();
+#endif
+                for (int m = threadIdx.x; m < M; m += THREADS) atomicMax(&a.argmax[m], s_best[m]);
+#ifdef TASC_TIMELINE
+                TL_END(45);
+#endif
+                return;
+            }
+        } else {
+        cluster_wait();
+#ifdef TASC_TIMELINE
+        TL_END(tl_tag);
+#endif
         float* kp = a.kv_pool + (size_t)l * 2 * a.kv_half;
         float* vp = kp + a.kv_half;
-        // ---- QKV: rotary pairs (value heads: the same pairs, not rotated)
-        stage_norm(lw.attn_norm, l == 0);
-        auto feat = [&](int p) { return (p / half) * hd + p % half; };
-        product((a.n_q + 2 * a.n_kv) * half, d, [&](int p) { return lw.wqkv + (size_t)feat(p) * d; },
-                [&](int p) { return lw.wqkv + (size_t)(feat(p) + half) * d; },
-                [&](int p, int m, float v0, float v1) {
-                    const int head = p / half, i = p % half, pos = s_pos[m];
-                    if (pos < 0) {
-                        if (head < a.n_q) { a.q[(size_t)m * qd + head * hd + i] = 0.f; a.q[(size_t)m * qd + head * hd + i + half] = 0.f; }
-                        return;
-                    }
-                    if (pos >= a.max_positions) { set_status(a.status, TASC_EINVAL); return; }
-                    if (head < a.n_q + a.n_kv) {
-                        const float2 c = a.rope[(size_t)pos * half + i];
-                        const float r0 = v0 * c.x - v1 * c.y, r1 = v1 * c.x + v0 * c.y;
-                        v0 = r0; v1 = r1;
-                    }
-                    if (head < a.n_q) {
-                        a.q[(size_t)m * qd + head * hd + i] = v0;
-                        a.q[(size_t)m * qd + head * hd + i + half] = v1;
-                        return;
-                    }
-                    const int pslot = pos / a.page_size;
-                    int page = -1;
-                    if (pslot < a.max_pages) page = a.block_table[(size_t)(m / a.R) * a.max_pages + pslot];
-                    if (page < 0 || page >= a.n_pages) { set_status(a.status, TASC_ENOKV); return; }
-                    const bool is_k = head < a.n_q + a.n_kv;
-                    float* dst = (is_k ? kp : vp) + (((size_t)page * a.n_kv + (head - a.n_q - (is_k ? 0 : a.n_kv))) * a.page_size + pos % a.page_size) * hd;
-                    dst[i] = v0;
-                    dst[i + half] = v1;
-                });
-        TL_SYNC(40);
         // ---- attention: unit = (token row, query head)
         const int n_units = M * a.n_q, g = a.n_q / a.n_kv, sub = warp / UNIT_WARPS, sw = warp % UNIT_WARPS;
+#pragma unroll 1
         for (int u0 = cta; u0 < n_units; u0 += CTAS * (WARPS / UNIT_WARPS)) {
             const int u = u0 + sub * CTAS;
-            const int m = u < n_units ? u / a.n_q : 0, h = u < n_units ? u % a.n_q : 0, b = m / a.R;
+            const int m = u < n_units ? a.by_nq.div(u) : 0, h = u < n_units ? u - m * a.n_q : 0, b = a.by_R.div(m), kvh = h / g;
             const int n_keys = u < n_units ? s_pos[m] + 1 : 0;   // none for a row that is not in use
             const float* q = a.q + (size_t)m * qd + h * hd;
             float acc[NJ], mx = -INFINITY, den = 0.f;
 #pragma unroll
             for (int j = 0; j < NJ; ++j) acc[j] = 0.f;
+#pragma unroll 1
             for (int k0 = sw * KEYS; k0 < n_keys; k0 += UNIT_WARPS * KEYS) {
                 const int key = k0 + (lane >> 2);
+                const int pslot = (int)((unsigned)key / (unsigned)a.page_size);
                 int page = -1;
-                if (key < n_keys && key / a.page_size < a.max_pages) page = __ldg(a.block_table + (size_t)b * a.max_pages + key / a.page_size);
+                if (key < n_keys && pslot < a.max_pages) page = __ldg(a.block_table + (size_t)b * a.max_pages + pslot);
                 const bool there = page >= 0 && page < a.n_pages;          // ids outside the pool read as zeros, never as memory
-                const uint32_t row = there ? (uint32_t)((page * a.n_kv + h / g) * a.page_size + key % a.page_size) : 0u;
+                const uint32_t row = there ? (uint32_t)((page * a.n_kv + kvh) * a.page_size + key - pslot * a.page_size) : 0u;
                 // the values are on their way while the scores are worked out
                 float v[KEYS][NJ];
 #pragma unroll
@@ -273,11 +332,15 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
             if (sw == 0 && u < n_units) {
                 const float* p0 = part + (size_t)warp * (hd + 4);
                 float top = -INFINITY, sum = 0.f;
+#pragma unroll 1
                 for (int w = 0; w < UNIT_WARPS; ++w) top = fmaxf(top, p0[w * (hd + 4) + hd]);
+#pragma unroll 1
                 for (int w = 0; w < UNIT_WARPS; ++w)
                     if (p0[w * (hd + 4) + hd] != -INFINITY) sum += expf(p0[w * (hd + 4) + hd] - top) * p0[w * (hd + 4) + hd + 1];
+#pragma unroll 1
                 for (int j = lane; j < hd; j += 32) {
                     float o = 0.f;
+#pragma unroll 1
                     for (int w = 0; w < UNIT_WARPS; ++w)
                         if (p0[w * (hd + 4) + hd] != -INFINITY) o += expf(p0[w * (hd + 4) + hd] - top) * p0[w * (hd + 4) + j];
                     a.o[(size_t)m * qd + h * hd + j] = n_keys > 0 ? o / sum : 0.f;
@@ -285,42 +348,17 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
             }
             __syncthreads();
         }
-        TL_SYNC(41);
-        // ---- O
-        stage_rows(a.o, qd);
-        residual(lw.wo, qd);
-        TL_SYNC(42);
-        // ---- gate / up
-        stage_norm(lw.mlp_norm, false);
-        product(a.dff, d, [&](int p) { return lw.w_gate_up + (size_t)p * d; }, [&](int p) { return lw.w_gate_up + (size_t)(a.dff + p) * d; },
-                [&](int p, int m, float g0, float u) { a.act[(size_t)m * a.dff + p] = g0 / (1.0f + expf(-g0)) * u; });
-        TL_SYNC(43);
-        // ---- down
-        stage_rows(a.act, a.dff);
-        residual(lw.w_down, a.dff);
-        TL_SYNC(44);
+        }
+#ifdef TASC_TIMELINE
+        tl_b = global_ns();
+        tl_tag = 40 + stage;
+#endif
+        cluster_arrive();
+        if (stage == ST_DOWN) {
+            if (++l == a.n_layers) stage = ST_LM;
+            else { stage = ST_QKV; lw = a.layers[l]; }
+        } else ++stage;
     }
-    if (!a.lm_head) return;
-    stage_norm(a.final_norm, false);
-    product((a.vocab + 1) / 2, d, [&](int p) { return a.lm_head + (size_t)(2 * p) * d; },
-            [&](int p) { return a.lm_head + (size_t)min(2 * p + 1, a.vocab - 1) * d; },
-            [&](int p, int m, float v0, float v1) {
-                unsigned long long best = pack_argmax(v0, (uint32_t)(2 * p));
-                if (2 * p + 1 < a.vocab) best = max(best, pack_argmax(v1, (uint32_t)(2 * p + 1)));
-                atomicMax(&s_best[m], best);
-                if (a.logits) {
-                    a.logits[(size_t)m * a.vocab + 2 * p] = v0;
-                    if (2 * p + 1 < a.vocab) a.logits[(size_t)m * a.vocab + 2 * p + 1] = v1;
-                }
-            });
-    __syncthreads();
-#ifdef TASC_TIMELINE
-    tl_b = global_ns();
-#endif
-    for (int m = threadIdx.x; m < M; m += THREADS) atomicMax(&a.argmax[m], s_best[m]);
-#ifdef TASC_TIMELINE
-    TL_END(45);
-#endif
 }
 
 size_t smem_bytes(int M, int width, int hd) {
@@ -384,6 +422,7 @@ bool plan_forward_f32(int M, int d, int n_q, int n_kv, int hd, int dff, int max_
 tasc_status launch_forward_f32(ForwardF32Args a, cudaStream_t stream) {
     a.width = std::max({a.d, a.n_q * a.hd, a.dff});
     a.scale = 1.0f / sqrtf((float)a.hd);
+    a.by_R = SmallDiv(a.R); a.by_half = SmallDiv(a.hd / 2); a.by_nq = SmallDiv(a.n_q);
     return a.hd <= 32 ? launch_inst<1>(a, stream) : a.hd <= 64 ? launch_inst<2>(a, stream) : a.hd <= 128 ? launch_inst<4>(a, stream) : launch_inst<8>(a, stream);
 }
 

@@ -69,16 +69,11 @@ __device__ __forceinline__ float4 shfl_xor4(float4 v, int d) {
 
 // Four consecutive values -> (hi, lo) bf16 quadruples, 8 bytes each.
 __device__ __forceinline__ void store_hilo4(__nv_bfloat16* hi_ptr, __nv_bfloat16* lo_ptr, const float v[4]) {
-    __nv_bfloat16 h[4], l[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) split_bf16(v[e], h[e], l[e]);
-    uint2 ph, pl;
-    ph.x = (uint32_t)__bfloat16_as_ushort(h[0]) | ((uint32_t)__bfloat16_as_ushort(h[1]) << 16);
-    ph.y = (uint32_t)__bfloat16_as_ushort(h[2]) | ((uint32_t)__bfloat16_as_ushort(h[3]) << 16);
-    pl.x = (uint32_t)__bfloat16_as_ushort(l[0]) | ((uint32_t)__bfloat16_as_ushort(l[1]) << 16);
-    pl.y = (uint32_t)__bfloat16_as_ushort(l[2]) | ((uint32_t)__bfloat16_as_ushort(l[3]) << 16);
-    *reinterpret_cast<uint2*>(hi_ptr) = ph;
-    *reinterpret_cast<uint2*>(lo_ptr) = pl;
+    uint2 h, l;
+    split_bf16x2(v[0], v[1], h.x, l.x);
+    split_bf16x2(v[2], v[3], h.y, l.y);
+    *reinterpret_cast<uint2*>(hi_ptr) = h;
+    *reinterpret_cast<uint2*>(lo_ptr) = l;
 }
 __device__ __forceinline__ void store_bf16x4(__nv_bfloat16* p, const float v[4]) {
     uint2 u;
@@ -270,14 +265,11 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
                 const float g0 = (low ? g4.x : g4.z) * sc, g1 = (low ? g4.y : g4.w) * sc;
                 const float u0 = (low ? u4.x : u4.z) * sc, u1 = (low ? u4.y : u4.w) * sc;
                 const float v0 = g0 / (1.0f + expf(-g0)) * u0, v1 = g1 / (1.0f + expf(-g1)) * u1;
-                __nv_bfloat16 h0, l0, h1, l1;
-                split_bf16(v0, h0, l0);
-                split_bf16(v1, h1, l1);
+                uint32_t hi, lo;
+                split_bf16x2(v0, v1, hi, lo);
                 const size_t row = (size_t)m0 + t;
-                *reinterpret_cast<uint32_t*>(a.a_out + row * a.N + j) =
-                    (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-                *reinterpret_cast<uint32_t*>(a.a_out + (row + TBL) * a.N + j) =
-                    (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+                *reinterpret_cast<uint32_t*>(a.a_out + row * a.N + j) = hi;
+                *reinterpret_cast<uint32_t*>(a.a_out + (row + TBL) * a.N + j) = lo;
             }
         }
     };
@@ -440,6 +432,10 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
 #ifdef TASC_TIMELINE
     if (threadIdx.x == 0) g_td = global_ns();
 #endif
+    if (warp == 5) {                                               // (the accumulator has been read)
+        tc_fence_after();
+        tmem_dealloc(tmem_base, ncols);
+    }
 
     if (EPI != EPI_LM) {
         // ------------------------------------------------------------ epilogue, part 2: sum the S partial copies of this CTA's columns
@@ -544,11 +540,6 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
             const int s = i % stages;
             if (i + stages >= n_kb) (void)mbar_wait(bar_full + 8u * s, (uint32_t)(i / stages) & 1u, 2000000ll);
         }
-    }
-    __syncthreads();
-    if (warp == 5) {
-        tc_fence_after();
-        tmem_dealloc(tmem_base, ncols);
     }
     if (threadIdx.x == 0) TL(10);
 #ifdef TASC_TIMELINE

@@ -291,8 +291,9 @@ struct ForwardF32Args {
     unsigned long long* argmax;
     float* logits;
     int* status;
-    int width;                                     // (set by the launch)
+    int width;                                     // (set by the launch, like the rest)
     float scale;
+    SmallDiv by_R, by_half, by_nq;
 };
 // What one cluster runs: four-layer models, a step in us as one launch per stage / in the cluster: 1 MB per layer 323 / 100 at
 // 5 rows and 426 / 376 at 72, 13 MB 653 / 192 at 5 and 900 / 521 at 24, 47 MB 1056 / 470 at 5; the rows are also limited by
