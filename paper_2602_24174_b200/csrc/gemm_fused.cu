@@ -664,11 +664,13 @@ FusedPlan plan_fused(int M, int N, int K, int epi, int few_tiles, int hd, double
         S = std::min(S, 8);
         S = std::min(S, p.num_kb);
         // Fewer splits than fit can be faster.  Per kernel, in microseconds: a CTA's epilogue takes about 0.5 per round of six token
-        // columns (one per warp) of the columns it finishes; a grid that takes more than about two thirds of the SMs keeps the next
-        // kernel's CTAs from starting (and from fetching their weights) while this one runs, about 0.035 per CTA beyond 96; and a
-        // k-block of a CTA's chain counts 0.46.  That is more than its MMAs take (160 to 250 cycles, 0.13): with 0.13 in its place some
-        // passes gain and others lose (135M 128 rows 1031 -> 1010 us a step, 0.5B 128 rows 1255 -> 1236, 144 rows 1301 -> 1294, 96 rows
-        // 1114 -> 1118, 0.5B + 8,192 tokens 288 rows 1562 -> 1568).  Ties go to the larger cluster.
+        // columns (one per warp) of the columns it finishes; every CTA costs 0.026, because it keeps a CTA of the next kernel from
+        // starting (and from fetching its weights) while this kernel runs; a k-block of a CTA's chain costs 0.15, about what its MMAs
+        // take, where the weights were there before the activations (QKV and O), 0.46 in gate/up and 0.6 in down, which follows the
+        // kernel with the largest grid and fetches its weights late.  (0.46 for all, and 0.035 per CTA from the 97th on, before /
+        // now: 135M, step at 96 rows 846 -> 833 us, 100 rows 847 -> 827, 128 rows 823 -> 794, 288 rows 967 -> 966; 0.5B 96 rows
+        // 946 -> 909, 120 rows 1126 -> 1099, 192 rows 1196 -> 1196, 100 prompt tokens 903 -> 872.  With 0.024 per CTA 135M at 128 rows
+        // 815, with 0.028 at 288 rows 972.)  Ties go to the larger cluster.
         // (With a single token tile the chain's kernels are narrow and the largest cluster stays the best.)
         const int cols = std::min(p.TB, M);
         int best = S;
@@ -676,8 +678,8 @@ FusedPlan plan_fused(int M, int N, int K, int epi, int few_tiles, int hd, double
         for (int s = 1; s <= S && p.m_tiles >= 2; ++s) {
             const int ctas = tiles * s;
             const int rounds = ((cols + s - 1) / s + 5) / 6;
-            const float cost = 0.46f * (float)((p.num_kb + s - 1) / s) + 0.5f * (float)rounds +
-                               0.035f * (float)std::max(0, ctas - 96) - 0.01f * (float)s;
+            const float per_kb = epi == EPI_SWIGLU ? 0.46f : K > N ? 0.6f : 0.15f;
+            const float cost = per_kb * (float)((p.num_kb + s - 1) / s) + 0.5f * (float)rounds + 0.026f * (float)ctas;
             if (cost < best_cost) { best_cost = cost; best = s; }
         }
         S = best;
