@@ -685,20 +685,22 @@ tasc_status launch_inst(const AttnArgs& a, const CUtensorMap& tmK, const CUtenso
 int attention_mma_row_pad(int G) { return G <= 64 ? 64 : 128; }
 
 // Query heads per CTA, key-range splits per (sequence, head group) (1..8, the CTAs of a cluster) and ring depth, from a
-// small cost model in microseconds: a CTA needs about 2.5 us to start (Q staging, first tiles) plus one tile time per
+// small cost model in microseconds: a CTA needs about 1.7 us to start (Q staging, first tiles) plus one tile time per
 // iteration (its warp groups take `ng` tiles per iteration; a shallow ring adds memory stalls), the clusters run in as
 // many waves as the device's cluster occupancy dictates (one straggling cluster costs a whole wave), and splitting
 // adds the cluster exchange and merge.  With few sequences the g query heads that share a KV head are dealt out to
 // several CTAs (each re-reads that head's K/V from L2, which is cheap next to leaving most SMs idle): fewer query rows
 // per CTA mean fewer slabs, so more warp groups work on different key tiles at once.
 AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ctx) {
-    // The launch shape is fixed before the lengths are known (and stays fixed in a captured graph): it is chosen
-    // for three quarters of the context the cache can hold; shorter ranges leave the last splits idle.
-    const int n_tiles = std::max(1, ((max_ctx * 3) / 4 + TKEYS - 1) / TKEYS);
+    // The launch shape is fixed before the lengths are known (and stays fixed in a captured graph): it is chosen for three quarters of
+    // the context the cache can hold and for all of it, half each; shorter ranges leave the last splits idle.  (For three quarters
+    // alone, and 2.5 us to start, a step of the 0.5B with 8 sequences x 6 rows behind 300 keys took 823 us instead of 793, with 4 x 6
+    // behind 600 keys 725 instead of 694.)
+    const int n_tiles = std::max(1, ((max_ctx * 3) / 4 + TKEYS - 1) / TKEYS), n_all = std::max(1, (max_ctx + TKEYS - 1) / TKEYS);
     // Measured (microseconds): one iteration of a warp group over a 64-key tile, and the time the SM's mma.sync
     // pipes need per tile and 16-row slab when all warps have work (the lower bound once several groups run).
-    const float t_tile = hd >= 128 ? 2.0f : (hd >= 64 ? 1.3f : 0.8f);
-    const float t_pipe = hd >= 128 ? 0.6f : (hd >= 64 ? 0.3f : 0.15f);
+    const float t_tile = hd >= 128 ? 1.2f : (hd >= 64 ? 1.3f : 0.8f);
+    const float t_pipe = hd >= 128 ? 0.65f : (hd >= 64 ? 0.3f : 0.15f);
     AttnPlan best = {1, 2, g, 0, 1e30f};
     float best_cost = 1e30f;
     // Candidates: all g heads of a KV head in one CTA; and, for few sequences with 128-wide heads (where one warp needs
@@ -723,16 +725,19 @@ AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ct
                 if (fit <= 0) fit = std::max(1, 148 / s);               // no device to ask: assume one CTA per SM
                 const int waves = (groups + fit - 1) / fit;
                 const int tiles_cta = (n_tiles + s - 1) / s;
-                const int ng = warp_groups(n_slabs, stages, tiles_cta);
-                const int iters = (tiles_cta + ng - 1) / ng;
                 const float stall = di == 0 ? 0.f : 0.25f * t_tile;      // a shallow ring hides less latency
-                const float loop = std::max(iters * (t_tile + stall), tiles_cta * n_slabs * t_pipe);
+                auto loop_of = [&](int n) {
+                    const int t = (n + s - 1) / s, ng = warp_groups(n_slabs, stages, t), iters = (t + ng - 1) / ng;
+                    return std::max(iters * (t_tile + stall), t * n_slabs * t_pipe);
+                };
+                const float loop = 0.5f * (loop_of(n_tiles) + loop_of(n_all));
                 const float merge = s > 1 ? 0.5f + 0.25f * s : 0.f;      // cluster barrier + one round of remote reads
                 // a grid that takes (nearly) every SM keeps the next kernel's CTAs from starting early
-                const float crowd = groups * s > 128 ? 3.0f : 0.f;
+                // (1.0: 20 x 4 rows of the 0.5B 907 us instead of 902; 3.0: 24 x 5 rows 1113 instead of 1068)
+                const float crowd = groups * s > 128 ? 1.5f : 0.f;
                 // every head group re-reads its KV head's keys: L2 traffic, about 0.1 us per extra pass over a tile
                 const float reread = 0.1f * tiles_cta * (float)(g / hs - 1) / (float)std::max(1, g / hs);
-                const float cost = waves * (2.5f + loop) + merge + crowd + reread;
+                const float cost = waves * (1.7f + loop) + merge + crowd + reread;
                 if (cost < best_cost - 1e-6f) { best_cost = cost; best = AttnPlan{s, stages, hs, 0, cost}; }
             }
         }

@@ -560,15 +560,16 @@ template <int HD, int RP> int ring_stages() {
 // Splits by a cost in microseconds like plan_attention_mma's: T0 to start, `per_tile` for a tile of TK keys (taken for three
 // quarters of the context and for all of it, half each: the tiles are large), as many waves as the occupancy of the launch
 // dictates (one CTA per SM), the merge of split ranges.  The other kernel's cost is p.cost, and no less than what all its slabs
-// take of the SMs' mma.sync pipes.  Measured, steps and prefills of the 135M, 0.5B and 1.5B shapes: it pays from about 64
-// (sequence, KV head) pairs on, from 8 on with long contexts and four or more slabs of query rows, hardly ever at the 135M's
-// 18 to 27 rows.
+// take of the SMs' mma.sync pipes.  T0 as measured against the other kernel, which starts faster since its code was cut: a step
+// of the 1.5B, 3 x 7 rows behind 400 keys, 1169 us here, 1121 there; 10 x 8 rows of the 0.5B 893 / 877; 1.5B 40 x 5 rows 2512 / 2549,
+// 0.5B + 8,192 tokens 32 x 9 rows behind 640 keys 1441 / 1440.  It pays for many (sequence, KV head) pairs with long contexts and three
+// or more slabs of query rows, hardly ever at the 135M's 18 to 27 rows.
 bool plan_attention_tc(int B, int n_kv, int hd, int g, int rows, int max_ctx, int page_size, AttnPlan& p) {
     const int G = g * rows;
     if ((hd != 64 && hd != 128) || page_size != PAGE || G > 128 || max_ctx / PAGE > MAX_PAGES) return false;
     const bool small = G <= 64;
     const int tk = small ? 128 : 64;
-    const float T0 = 2.4f, per_tile = hd == 128 ? (small ? 1.8f : 1.4f) : (small ? 1.4f : 1.1f);
+    const float T0 = hd == 128 ? 3.9f : 2.8f, per_tile = hd == 128 ? (small ? 1.8f : 1.4f) : (small ? 1.4f : 1.1f);
     const int groups = B * n_kv, tiles_all = std::max(1, (max_ctx + tk - 1) / tk), tiles_34 = std::max(1, (max_ctx * 3 / 4 + tk - 1) / tk);
     const float pipes = (hd == 128 ? 0.6f : 0.3f) * (float)groups * (float)((G + 15) / 16) * (float)((max_ctx * 3 / 4 + 63) / 64) / 148.f;
     int best = 0;

@@ -670,7 +670,7 @@ FusedPlan plan_fused(int M, int N, int K, int epi, int few_tiles, int hd, double
         // kernel with the largest grid and fetches its weights late.  (0.46 for all, and 0.035 per CTA from the 97th on, before /
         // now: 135M, step at 96 rows 846 -> 833 us, 100 rows 847 -> 827, 128 rows 823 -> 794, 288 rows 967 -> 966; 0.5B 96 rows
         // 946 -> 909, 120 rows 1126 -> 1099, 192 rows 1196 -> 1196, 100 prompt tokens 903 -> 872.  With 0.024 per CTA 135M at 128 rows
-        // 815, with 0.028 at 288 rows 972.)  Ties go to the larger cluster.
+        // 815, with 0.028 at 288 rows 972.)
         // (With a single token tile the chain's kernels are narrow and the largest cluster stays the best.)
         const int cols = std::min(p.TB, M);
         int best = S;
