@@ -33,6 +33,10 @@
 // attention 6.9, 2.5 of it the merge of the key ranges.  At 1.5B the weights: gate/up 12.0 (products 8.2), down 7.9 (5.3), QKV 6.5 (CTAs
 // start it 1.4 us apart), O 3.6, attention 9.8 (merge 4.1).
 //
+// Code is kept short, because a layer runs through more of it than the instruction cache holds: one copy of `decode` behind the
+// products instead of two, two chunks in flight instead of four where they do not pay, loops of the attention not unrolled at one
+// token tile, pairs split in two instructions: 64 -> 58 KB with heads of 64; 135M at 6 rows 577 -> 568 us, 0.5B 635 -> 628, 1.5B 1139 -> 1133.
+//
 // Every wait is bounded: a barrier that is not reached in about half a second records TASC_ETIMEOUT and the CTA
 // leaves.  The limit holds for the first barrier too: a cooperative grid starts when all its CTAs can be resident, not one by
 // one (measured: with another stream's kernel on one SM for 1.27 s the pass began behind it, without a time-out).
@@ -121,14 +125,6 @@ __device__ __forceinline__ void sts_f(uint32_t addr, float v) { asm volatile("st
 __device__ __forceinline__ uint32_t pack2(__nv_bfloat16 a, __nv_bfloat16 b) {
     return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
 }
-__device__ __forceinline__ void pack_hilo(float x, float y, uint32_t& hi, uint32_t& lo) {
-    __nv_bfloat16 hx, lx, hy, ly;
-    split_bf16(x, hx, lx);
-    split_bf16(y, hy, ly);
-    hi = pack2(hx, hy);
-    lo = pack2(lx, ly);
-}
-
 // Hides where a value comes from: what is derived from it is computed in this phase, not kept in registers over the
 // whole layer loop (the compiler would otherwise hoist every phase's addresses out of it and spill them).
 __device__ __forceinline__ int fresh(int v) {
@@ -275,7 +271,8 @@ template <int HD, int T>
 struct Cta {
     static constexpr int NW = WARPS, NT = NW * 32;
     static constexpr int LT = T == 4 ? 2 : T - 1;       // log2 T
-    static constexpr int D = T == 1 ? 4 : (T == 2 ? 3 : 2);            // chunks in flight per warp
+    // chunks in flight per warp (64-wide heads: models whose rows are two or three chunks of a warp; four more of them are only code)
+    static constexpr int D = T == 1 ? (HD == 64 ? 2 : 4) : (T == 2 ? 3 : 2);
     const PersistArgs& a;
     int epoch;                 // of the barrier that comes next
 
@@ -477,12 +474,14 @@ struct Cta {
             __syncthreads();
             TL_STAMP(2);
             const int n_items = items_of(tile1 - tile0) << lp;
-            if (tile0 > 0) it = decode(ph, tid, lp, tile0, red, stride, u0, u1, m0);
+            bool decoded = tile0 == 0;
 #pragma unroll 1
-            for (int idx = tid; idx < n_items;) {
+            for (int idx = tid; idx < n_items; idx += NT) {
+                if (!decoded) it = decode(ph, idx, lp, tile0, red, stride, u0, u1, m0);
+                decoded = false;
                 float v0 = 0.f, v1 = 0.f;
                 uint32_t p = it.p;
-#pragma unroll 2
+#pragma unroll (T == 1 ? 1 : 2)
                 for (int k = KG >> lp; k > 0; --k, p += stride << lp) {
                     v0 += lds_f(p);
                     if (kind != PH_RESID) v1 += lds_f(p + 32);
@@ -495,10 +494,10 @@ struct Cta {
                         const float x = lds_f(it.xs) + v0;
                         sts_f(it.xs, x);
                         ss = x * x;
-                        __nv_bfloat16 h, l;
-                        split_bf16(x * it.cs.x, h, l);
-                        *reinterpret_cast<__nv_bfloat16*>(it.out0) = h;
-                        *reinterpret_cast<__nv_bfloat16*>(it.out1) = l;
+                        uint32_t h, l;
+                        split_bf16x2(x * it.cs.x, 0.f, h, l);
+                        *reinterpret_cast<unsigned short*>(it.out0) = (unsigned short)h;
+                        *reinterpret_cast<unsigned short*>(it.out1) = (unsigned short)l;
                     }
                     ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 1);
                     ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 2);
@@ -521,8 +520,6 @@ struct Cta {
                         else { *reinterpret_cast<__nv_bfloat16*>(it.out0) = __float2bfloat16_rn(r0); *reinterpret_cast<__nv_bfloat16*>(it.out1) = __float2bfloat16_rn(r1); }
                     }
                 }
-                idx += NT;
-                if (idx < n_items) it = decode(ph, idx, lp, tile0, red, stride, u0, u1, m0);
             }
             if (tile1 < n_tiles) __syncthreads();       // the parked tiles are overwritten by the next group
         }
@@ -651,8 +648,8 @@ struct Cta {
             for (int e = 0; e < NQ; ++e) {
                 const int i = tid + e * NT, r = i / (HD / 4), d4 = (i % (HD / 4)) * 4;
                 uint2 h, l;
-                pack_hilo(qv[e].x * a.scale_log2e, qv[e].y * a.scale_log2e, h.x, l.x);
-                pack_hilo(qv[e].z * a.scale_log2e, qv[e].w * a.scale_log2e, h.y, l.y);
+                split_bf16x2(qv[e].x * a.scale_log2e, qv[e].y * a.scale_log2e, h.x, l.x);
+                split_bf16x2(qv[e].z * a.scale_log2e, qv[e].w * a.scale_log2e, h.y, l.y);
                 *reinterpret_cast<uint2*>(Qh + r * QS + d4) = h;
                 *reinterpret_cast<uint2*>(Qh + (16 + r) * QS + d4) = l;
             }
@@ -673,7 +670,7 @@ struct Cta {
 #pragma unroll
                     for (int e = 0; e < 4; ++e) { s[nt][e] = 0.f; sl[nt][e] = 0.f; }
                 if (kb + warp * 16 < q.k1) {
-#pragma unroll 4
+#pragma unroll (T == 1 ? 2 : 4)
                     for (int j = 0; j < HD / 16; ++j) {
                         uint32_t ah[4], al[4], kf[4];
                         ldsm_x4(qa + j * 32, ah);
@@ -723,7 +720,7 @@ struct Cta {
                         const float e0 = exp2f(s[nt][2 * hf] - mu), e1 = exp2f(s[nt][2 * hf + 1] - mu);
                         sum += e0 + e1;
                         uint32_t h, l;
-                        pack_hilo(e0, e1, h, l);
+                        split_bf16x2(e0, e1, h, l);
                         const int col = warp * 16 + nt * 8 + 2 * t;
                         *reinterpret_cast<uint32_t*>(Ph + row * PS + col) = h;
                         *reinterpret_cast<uint32_t*>(Ph + (16 + row) * PS + col) = l;
@@ -738,7 +735,7 @@ struct Cta {
                 cp_async_wait<1>();                               // this tile's V (the next K may be on its way)
                 __syncthreads();
                 const int kend = min(KT, q.k1 - kb);
-#pragma unroll 2
+#pragma unroll (T == 1 ? 1 : 2)
                 for (int k32 = 0; k32 < kend; k32 += 32) {
                     uint32_t ah[2][4], al[2][4];
 #pragma unroll
@@ -791,7 +788,7 @@ struct Cta {
 #pragma unroll
                     for (int i = 0; i < NTW; ++i) {
                         uint32_t h, l;
-                        pack_hilo(oh[i][2 * hf] * inv, oh[i][2 * hf + 1] * inv, h, l);
+                        split_bf16x2(oh[i][2 * hf] * inv, oh[i][2 * hf + 1] * inv, h, l);
                         if (rho < G) {
                             __nv_bfloat16* p = a.o + out_at(a, q, rho, gq, (cg + i) * 8 + 2 * t);
                             *reinterpret_cast<uint32_t*>(p) = h;
@@ -868,8 +865,8 @@ struct Cta {
             if (rho >= G) continue;
             const float inv = den > 0.f ? 1.0f / den : 0.f;
             uint2 h, l;
-            pack_hilo(acc.x * inv, acc.y * inv, h.x, l.x);
-            pack_hilo(acc.z * inv, acc.w * inv, h.y, l.y);
+            split_bf16x2(acc.x * inv, acc.y * inv, h.x, l.x);
+            split_bf16x2(acc.z * inv, acc.w * inv, h.y, l.y);
             __nv_bfloat16* dst = a.o + out_at(a, q, rho, gq, d4);
             *reinterpret_cast<uint2*>(dst) = h;
             *reinterpret_cast<uint2*>(dst + 512) = l;
