@@ -9,7 +9,8 @@
 //   128-bit compare-and-swap per new n-gram.  The table is counted in full once and then kept up to date: a merge changes
 //   the windows that overlap a replaced occurrence and no others, so only those are taken out and put back.  The argmax
 //   is unique: largest reward, then the longer n-gram, then the one that occurs first; first occurrences are looked up
-//   only in rounds where the first two tie.  The documents stay at their original offsets and only get shorter.
+//   only in rounds where the first two tie.  Most rounds take it from a short list of the n-grams within a quarter of
+//   the best, which every CTA reads for itself.  The documents stay at their original offsets and only get shorter.
 //   All rounds run in one cooperative kernel without a host round trip.
 // tasc_tok_init_rows -- Section 4.2: the embedding / LM-head row of an added token is the mean of its constituents'
 //   rows (a constituent may itself be an added token).  A thread per column walks the merges in order, so a row is
@@ -34,11 +35,12 @@ constexpr int LEN_BITS = 3;
 // What the merge loop shares across the grid.  Words that a later round uses again exist twice: one CTA prepares the one
 // while all others still read the other.
 struct TokState {
-    int n_merges, status;
-    int rebuild;                                 // the round before which the table has to be counted again (0: the first)
-    unsigned int bar;                            // arrivals at the grid barrier
-    unsigned int first[2];                       // first position of the n-grams that tie
     unsigned long long used[2];                  // slots claimed
+    unsigned int n_cand[2];                      // entries of the candidates' list
+    int rebuild;                                 // the round before which the table has to be counted again (0: the first)
+    int n_merges, status;
+    unsigned int first[2];                       // first position of the n-grams that tie
+    unsigned int bar;                            // arrivals at the grid barrier
 };
 // The best n-gram of a part of the table: its rank (reward and length), one slot that has it, and how many have it.
 struct __align__(16) Best { unsigned long long rank; unsigned int slot, ties; };
@@ -53,6 +55,8 @@ __device__ __forceinline__ unsigned long long tok_rank(uint32_t w) {
 
 constexpr int TOK_THREADS = 1024, TOK_WARPS = TOK_THREADS / 32;
 constexpr int CHUNK_BITS = 7;                    // slots whose best n-gram is kept: 512 bytes of words, one load of a warp
+constexpr unsigned int CAND_MAX = TOK_THREADS;   // candidates: one per thread
+constexpr int TIED_MAX = 8;                      // n-grams that tie and are looked for by their tokens
 constexpr long long TOK_BARRIER_CYCLES = 20000000000ll;           // (a document of millions of tokens is one warp's work)
 
 struct TokArgs {
@@ -67,6 +71,7 @@ struct TokArgs {
     uint32_t* words;
     uint8_t* dirty;                              // per chunk of slots: its best has to be looked up again
     Best *chunk_best, *cta_best;
+    uint32_t* cand;                              // two lists of CAND_MAX slots
     uint64_t cap;
     TokState* st;
     int32_t* merges;
@@ -93,9 +98,21 @@ __device__ __forceinline__ KeyPair tok_pair(const TokArgs& a, uint64_t pair) {
     asm volatile("ld.global.cg.v2.u64 {%0, %1}, [%2];" : "=l"(v.k[1].x), "=l"(v.k[1].y) : "l"(a.keys + 4 * pair + 2) : "memory");
     return v;
 }
+// The list of candidates: every slot whose rank is `floor` or more.  Filled when the whole table has been looked through; a slot
+// whose rank rises past the floor later is added by whoever raised it (one that falls and rises again is in it twice: a tie with
+// itself).  floor 0: there is none.
+struct Candidates {
+    uint32_t* slots;
+    unsigned int* n;
+    unsigned long long floor;
+    __device__ __forceinline__ void add(uint64_t slot) const {
+        const unsigned int at = atomicAdd(n, 1u);
+        if (at < CAND_MAX) slots[at] = (uint32_t)slot;
+    }
+};
 // Adds an occurrence of a window, or takes one out that was counted before this round.  1 if that claimed a slot.  (One loop
 // for both: the lanes of a warp make their trips to the table together.)
-__device__ __forceinline__ int tok_change(const TokArgs& a, const Key& key, int n, bool add, int round) {
+__device__ __forceinline__ int tok_change(const TokArgs& a, const Key& key, int n, bool add, int round, const Candidates& cand) {
     Probe p(a, key);
     for (uint64_t probe = 0; probe <= p.mask; ++probe, p.next()) {
         const KeyPair v = tok_pair(a, p.pair);
@@ -113,8 +130,11 @@ __device__ __forceinline__ int tok_change(const TokArgs& a, const Key& key, int 
         }
         if (at0 || (k1.lo == key.lo && k1.hi == key.hi)) {
             const uint64_t slot = 2 * p.pair + (at0 ? 0 : 1);
-            atomicAdd(&a.words[slot], !add ? 0xFFFFFFFFu : claimed ? ((uint32_t)n << CNT_BITS) + 1u : 1u);
+            const uint32_t old = atomicAdd(&a.words[slot], !add ? 0xFFFFFFFFu : claimed ? ((uint32_t)n << CNT_BITS) + 1u : 1u) & CNT_MASK;
             a.dirty[slot >> CHUNK_BITS] = 1;
+            // (the length from here: whoever claimed the slot may not have written it yet)
+            const uint32_t len = (uint32_t)n << CNT_BITS;
+            if (add && cand.floor && tok_rank(len | (old + 1u)) >= cand.floor && tok_rank(len | old) < cand.floor) cand.add(slot);
             return claimed;
         }
         if (!add && k1.lo == 0 && k1.hi == 0) break;
@@ -167,17 +187,23 @@ struct TokShared {
     Best red[TOK_WARPS];
     int n, tok[MAX_N];                           // this round's n-gram
     int stop;
-    int n_hits, next_hit;
-    int hits[HIT_MAX];
+    int n_tied;                                  // candidates of the best rank
+    uint32_t tied_slot[TIED_MAX];
+    Key tied_key[TIED_MAX];
+    int n_hits, next_hit, more_hits;
+    int hits[HIT_MAX], hit_len[HIT_MAX];         // documents, their lengths
+    int64_t hit_at[HIT_MAX];                     // and where they start
     TokWarp warp[TOK_WARPS];
 };
 
-// Grid barrier; false when the wait ran out (a cooperative launch: all CTAs are resident).
-__device__ __forceinline__ bool tok_barrier(TokState* st, unsigned int& epoch, TokShared& sh) {
+// Grid barrier in two halves; the wait is false when it ran out (a cooperative launch: all CTAs are resident).
+__device__ __forceinline__ void tok_arrive(TokState* st, unsigned int& epoch) {
     ++epoch;
     __syncthreads();
+    if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&st->bar) : "memory");
+}
+__device__ __noinline__ bool tok_wait(TokState* st, unsigned int epoch, TokShared& sh) {
     if (threadIdx.x == 0) {
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&st->bar) : "memory");
         const unsigned int target = epoch * gridDim.x;
         const long long t0 = clock64();
         for (;;) {
@@ -189,6 +215,10 @@ __device__ __forceinline__ bool tok_barrier(TokState* st, unsigned int& epoch, T
     }
     __syncthreads();
     return sh.stop == 0;
+}
+__device__ __forceinline__ bool tok_barrier(TokState* st, unsigned int& epoch, TokShared& sh) {
+    tok_arrive(st, epoch);
+    return tok_wait(st, epoch, sh);
 }
 
 // A warp's list of windows: all lanes call everything.
@@ -219,7 +249,7 @@ struct TokList {
     }
     __device__ __forceinline__ bool full() const { return total + 32 * (MAX_N - 1) > LIST_MAX; }
     // looks the windows up; returns the slots this lane has claimed
-    __device__ __forceinline__ int flush(const TokArgs& a, int round) {
+    __device__ __forceinline__ int flush(const TokArgs& a, int round, const Candidates& cand) {
         int claimed = 0;
         __syncwarp();
         for (int p = threadIdx.x & 31; p < total; p += 32) {
@@ -229,7 +259,7 @@ struct TokList {
             Key key = key_make(m);
 #pragma unroll
             for (int j = 0; j < MAX_N; ++j) if (j < m) key_put(key, j, (uint32_t)tok[j]);
-            claimed += tok_change(a, key, m, add, round);
+            claimed += tok_change(a, key, m, add, round, cand);
         }
         __syncwarp();
         total = 0;
@@ -237,65 +267,119 @@ struct TokList {
     }
 };
 
-// Replaces the occurrences of the round's n-gram in one document, in place: left to right, non-overlapping.  A document of
-// at most DOC_SMEM tokens is worked on in shared memory, so that all its windows, old and new, are looked up together (a
-// look-up is a trip to L2 or to memory behind it); a longer one where it is, its windows chunk by chunk.
-template <bool SMALL>
-__device__ __noinline__ int tok_rewrite(const TokArgs& a, TokShared& sh, int d, int64_t s0, int L, int new_id, int round) {
-    const int lane = threadIdx.x & 31, n = sh.n;
+// The occurrences of the round's n-gram among the 32 positions from c on: first tokens and the others of occurrences, as bits.
+// skip: first position that is not part of the last occurrence.  (Left to right, non-overlapping.)
+__device__ __forceinline__ void tok_occurrences(const TokShared& sh, const int32_t* tok, int L, int c, int& skip, uint32_t& starts, uint32_t& inside) {
+    const int i = c + (threadIdx.x & 31), n = sh.n;
+    bool hit = i + n <= L;
+    for (int j = 0; hit && j < n; ++j) hit = tok[i + j] == sh.tok[j];
+    uint32_t hits = __ballot_sync(0xFFFFFFFFu, hit);
+    starts = inside = 0u;
+    if (skip > c) inside = skip - c >= 32 ? 0xFFFFFFFFu : (1u << (skip - c)) - 1u;
+    while (hits) {
+        const int p = c + __ffs(hits) - 1;
+        hits &= hits - 1u;
+        if (p < skip) continue;
+        starts |= 1u << (p - c);
+        skip = p + n;
+        for (int q = p + 1; q < skip && q < c + 32; ++q) inside |= 1u << (q - c);
+    }
+}
+
+// Replaces the occurrences of the round's n-gram in a document of at most DOC_SMEM tokens, in two steps.  First the document: it is worked
+// on in shared memory and leaves its old and new tokens and marks there.  (Only this CTA reads it, so that does not wait for the
+// others.)  Returns its new length and the chunks of 32 positions with a mark, old and new.
+struct Rewritten { int len; uint32_t old_chunks, new_chunks; };
+__device__ __noinline__ Rewritten tok_rewrite_short(const TokArgs& a, TokShared& sh, int d, int64_t s0, int L, int new_id) {
+    const int lane = threadIdx.x & 31;
     TokWarp& w = sh.warp[threadIdx.x >> 5];
     int32_t* doc = a.cur + s0;
-    const int32_t* old_tok = SMALL ? w.old_tok : doc;
-    uint8_t* old_mark = SMALL ? w.old_mark : a.mark + s0;
-    int32_t* new_tok = SMALL ? w.new_tok : doc;
-    uint8_t* new_mark = SMALL ? w.new_mark : a.mark + s0;
-    if (SMALL) {
-        int x[DOC_SMEM / 32];
+    int x[DOC_SMEM / 32];
 #pragma unroll
-        for (int u = 0; u < DOC_SMEM / 32; ++u) x[u] = u * 32 + lane < L ? doc[u * 32 + lane] : -1;
+    for (int u = 0; u < DOC_SMEM / 32; ++u) x[u] = u * 32 + lane < L ? doc[u * 32 + lane] : -1;
 #pragma unroll
-        for (int u = 0; u < DOC_SMEM / 32; ++u) w.old_tok[u * 32 + lane] = x[u];
-        __syncwarp();
-    }
-    int skip = 0;                                              // first position that is not part of the last occurrence
+    for (int u = 0; u < DOC_SMEM / 32; ++u) if (u * 32 < L) w.old_tok[u * 32 + lane] = x[u];
+    __syncwarp();
+    // marks (1 = first of an occurrence, 2 = the others), and the document as it will be
+    int skip = 0, wr = 0;
+    uint32_t old_chunks = 0u, new_chunks = 0u;                 // chunks with a mark
+#pragma unroll 1
     for (int c = 0; c < L; c += 32) {
-        const int i = c + lane;
-        bool hit = i + n <= L;
-        for (int j = 0; hit && j < n; ++j) hit = old_tok[i + j] == sh.tok[j];
-        uint32_t hits = __ballot_sync(0xFFFFFFFFu, hit), starts = 0u, inside = 0u;
-        if (skip > c) inside = skip - c >= 32 ? 0xFFFFFFFFu : (1u << (skip - c)) - 1u;
-        while (hits) {
-            const int p = c + __ffs(hits) - 1;
-            hits &= hits - 1u;
-            if (p < skip) continue;
-            starts |= 1u << (p - c);
-            skip = p + n;
-            for (int q = p + 1; q < skip && q < c + 32; ++q) inside |= 1u << (q - c);
+        uint32_t starts, inside;
+        tok_occurrences(sh, w.old_tok, L, c, skip, starts, inside);
+        const int i = c + lane, f = (starts >> lane) & 1u ? 1 : ((inside >> lane) & 1u ? 2 : 0);
+        if (starts | inside) old_chunks |= 1u << (c >> 5);
+        const bool kept = i < L && f != 2;
+        const uint32_t keep = __ballot_sync(0xFFFFFFFFu, kept);
+        const int at = wr + __popc(keep & ((1u << lane) - 1u));
+        if (i < L) w.old_mark[i] = (uint8_t)f;
+        if (kept) {
+            const int t = f == 1 ? new_id : w.old_tok[i];
+            w.new_tok[at] = t;
+            w.new_mark[at] = (uint8_t)f;
+            doc[at] = t;
         }
-        // 1 = first of an occurrence, 2 = the others
-        if (i < L) old_mark[i] = (starts >> lane) & 1u ? 1 : ((inside >> lane) & 1u ? 2 : 0);
+        new_chunks |= __reduce_or_sync(0xFFFFFFFFu, kept && f == 1 ? 1u << (at >> 5) : 0u);
+        wr += __popc(keep);
+    }
+    for (int i = lane; i < L; i += 32) {
+        if (i < wr) a.rem[s0 + i] = (uint8_t)min(wr - 1 - i, 255);
+        else doc[i] = -1;
+    }
+    if (lane == 0) a.doc_len[d] = wr;
+    __syncwarp();
+    return Rewritten{wr, old_chunks, new_chunks};
+}
+// Then the windows that change, old and new: put on the warp's list, which is looked up as a whole (a look-up is a trip to L2 or to
+// memory behind it).  Chunks without a changed token near are passed over.
+__device__ __noinline__ int tok_recount_short(const TokArgs& a, TokShared& sh, int L, Rewritten r, int round, const Candidates& cand) {
+    TokWarp& w = sh.warp[threadIdx.x >> 5];
+    TokList list = {w, w.old_tok, w.new_tok, 0};
+    int claimed = 0;
+#pragma unroll 1
+    for (int c = 0; c < 2 * DOC_SMEM; c += 32) {
+        const bool add = c >= DOC_SMEM;
+        const int at = c & (DOC_SMEM - 1), len = add ? r.len : L;
+        // (a window that holds a mark of the next chunk starts in this one)
+        if (at < len && (((add ? r.new_chunks : r.old_chunks) >> (at >> 5)) & 3u)) {
+            list.collect(a, add ? w.new_mark : w.old_mark, len, at, 0, add);
+            if (list.full()) claimed += list.flush(a, round, cand);
+        }
+    }
+    return claimed + list.flush(a, round, cand);
+}
+
+// The same for a longer document, in place, its windows chunk by chunk.
+__device__ __noinline__ int tok_rewrite_long(const TokArgs& a, TokShared& sh, int d, int64_t s0, int L, int new_id, int round, const Candidates& cand) {
+    const int lane = threadIdx.x & 31;
+    TokWarp& w = sh.warp[threadIdx.x >> 5];
+    int32_t* doc = a.cur + s0;
+    uint8_t* mark = a.mark + s0;
+    int skip = 0;
+    for (int c = 0; c < L; c += 32) {
+        uint32_t starts, inside;
+        tok_occurrences(sh, doc, L, c, skip, starts, inside);
+        if (c + lane < L) mark[c + lane] = (starts >> lane) & 1u ? 1 : ((inside >> lane) & 1u ? 2 : 0);
     }
     __syncwarp();
-    TokList list = {w, old_tok, new_tok, 0};
+    TokList list = {w, doc, doc, 0};
     int claimed = 0;
     for (int c = 0; c < L; c += 32) {
-        if (!SMALL) list.old_tok = doc + c;
-        list.collect(a, old_mark, L, c, SMALL ? 0 : c, false);
-        if (!SMALL || list.full()) claimed += list.flush(a, round);
+        list.old_tok = doc + c;
+        list.collect(a, mark, L, c, c, false);
+        claimed += list.flush(a, round, cand);
     }
     // a chunk's tokens are in registers before any of them is overwritten, and what is written lies before it
     int wr = 0;
     for (int c = 0; c < L; c += 32) {
         const int i = c + lane;
-        const int tok = i < L ? old_tok[i] : 0, f = i < L ? old_mark[i] : 2;
+        const int tok = i < L ? doc[i] : 0, f = i < L ? mark[i] : 2;
         const uint32_t keep = __ballot_sync(0xFFFFFFFFu, f != 2);
         const int at = wr + __popc(keep & ((1u << lane) - 1u));
         __syncwarp();
         if (f != 2) {
-            const int t = f == 1 ? new_id : tok;
-            new_tok[at] = t;
-            new_mark[at] = (uint8_t)f;
-            if (SMALL) doc[at] = t;
+            doc[at] = f == 1 ? new_id : tok;
+            mark[at] = (uint8_t)f;
         }
         wr += __popc(keep);
         __syncwarp();
@@ -307,24 +391,29 @@ __device__ __noinline__ int tok_rewrite(const TokArgs& a, TokShared& sh, int d, 
     if (lane == 0) a.doc_len[d] = wr;
     __syncwarp();
     for (int c = 0; c < wr; c += 32) {
-        if (!SMALL) list.new_tok = doc + c;
-        list.collect(a, new_mark, wr, c, SMALL ? 0 : c, true);
-        if (!SMALL || list.full()) claimed += list.flush(a, round);
+        list.new_tok = doc + c;
+        list.collect(a, mark, wr, c, c, true);
+        claimed += list.flush(a, round, cand);
     }
-    return claimed + list.flush(a, round);
+    return claimed;
 }
 
-// All rounds of Algorithm 1.  A warp looks for the n-gram in the documents that start in its share of the positions; the
-// documents found are handed out to the warps of the CTA.  A round is a chain of short steps: the best n-gram of the slots
-// that have changed, a grid barrier, the documents that hold it, a barrier.
+// All rounds of Algorithm 1.  A round is a chain of short steps: the best n-gram, the documents that hold it (a warp looks
+// through those that start in its share of the positions), a grid barrier, their rewriting (handed out to the warps of the CTA), a barrier.
+//   The best n-gram comes from the list of candidates while the best of them is above its floor; every CTA finds it for
+// itself.  Otherwise the table is looked through (the chunks that have changed; a barrier) and the list is made anew: the n-grams of three
+// quarters of the best reward and more.  Where those are more than the list holds, the next round looks through the table again, and
+// the list after it takes in half the distance from the best.
 //   Measured on 20,000 documents (1.4 M tokens, 4.1 M windows, n_max 4), per round: 525 us when every round cleared and
-//   recounted the table, 31 us now, of which about 11 are the re-tokenising of one document (a warp, hundreds of instructions in a chain).
+// recounted the table, 33 when every round looked through the table's changed chunks (8 us, 4 more for the barrier and the best of
+// all CTAs; a tie 30 us, because every window of the corpus was looked up to find the first), 27 now.  A round of 100 to 400 documents:
+// 9 until they are listed, 11 to rewrite them (half of it the look-ups); rounds of thousands, which come first, 20 to 90.
 __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid_constant__ TokArgs a) {
     extern __shared__ __align__(16) uint8_t dyn[];
     TokShared& sh = *reinterpret_cast<TokShared*>(dyn);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t nw = (int64_t)gridDim.x * TOK_WARPS, wid = (int64_t)warp * gridDim.x + blockIdx.x;
-    if (threadIdx.x == 0) { sh.stop = 0; sh.n_hits = 0; sh.next_hit = 0; }
+    if (threadIdx.x == 0) { sh.stop = 0; sh.n_hits = 0; sh.next_hit = 0; sh.more_hits = 0; }
     // this warp's documents
     auto doc_at = [&](int64_t pos) {
         int64_t lo = 0, hi = a.n_docs;
@@ -339,16 +428,21 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
     const int64_t s = a.offsets[doc_at(own * a.T / nw)], e = own + 1 == nw ? a.T : a.offsets[doc_at((own + 1) * a.T / nw)];
     const uint64_t n_chunks = a.cap >> CHUNK_BITS;
     unsigned int epoch = 0;
-    int n_merges = 0, n_ties = 0, n_rebuilds = 0;
+    int n_merges = 0, n_ties = 0, n_rebuilds = 0, n_lists = 0, part = 2;
+    Candidates cand = {a.cand, &a.st->n_cand[0], 0ull};
     __syncthreads();
     auto publish_claims = [&](int claimed) {
         claimed = __reduce_add_sync(0xFFFFFFFFu, claimed);
         if (lane == 0 && claimed) atomicAdd(&a.st->used[n_rebuilds & 1], (unsigned long long)claimed);
     };
     for (int round = 0;; ++round) {
-        // ---- the table, if it has to be counted (again): n-grams that no longer occur keep their slots until then
+        // ---- the table, if it has to be counted (again): n-grams that no longer occur keep their slots until then.  (One trip for all
+        // that a round looks at first.)
         const unsigned long long used = *(volatile unsigned long long*)&a.st->used[n_rebuilds & 1];
-        if (*(volatile int*)&a.st->rebuild == round || used * 4 > a.cap * 3) {
+        const int rebuild = *(volatile int*)&a.st->rebuild;
+        unsigned int n_cand = *(volatile unsigned int*)cand.n;
+        const uint32_t cand_slot = __ldcg(cand.slots + threadIdx.x);
+        if (rebuild == round || used * 4 > a.cap * 3) {
             const uint64_t gt = (uint64_t)blockIdx.x * TOK_THREADS + threadIdx.x, gn = (uint64_t)gridDim.x * TOK_THREADS;
             for (uint64_t i = gt; i < a.cap; i += gn) {
                 reinterpret_cast<ulonglong2*>(a.keys)[i] = make_ulonglong2(0ull, 0ull);
@@ -356,6 +450,7 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
             }
             for (uint64_t i = gt; i < n_chunks; i += gn) a.dirty[i] = 1;
             ++n_rebuilds;
+            cand.floor = 0ull;
             if (gt == 0) a.st->used[n_rebuilds & 1] = 0ull;
             if (!tok_barrier(a.st, epoch, sh)) return;
             int claimed = 0;
@@ -365,82 +460,184 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
                 for (int n = 2; n <= lim; ++n) {
                     Key key = key_make(n);
                     for (int j = 0; j < n; ++j) key_put(key, j, (uint32_t)a.cur[i + j]);
-                    claimed += tok_change(a, key, n, true, round);
+                    claimed += tok_change(a, key, n, true, round, cand);
                 }
             }
             __syncwarp();
             publish_claims(claimed);
             if (!tok_barrier(a.st, epoch, sh)) return;
         }
-        // ---- the best of this warp's chunks of the table
-        Best v = {0ull, 0u, 0u};
-        for (uint64_t c0 = 0; c0 * nw < n_chunks; c0 += 32) {
-            const uint64_t c = (c0 + lane) * nw + wid;
-            const bool mine = c < n_chunks, stale = mine && __ldcg(a.dirty + c);
-            Best b = {0ull, 0u, 0u};
-            if (mine) b = a.chunk_best[c];
-            uint32_t todo = __ballot_sync(0xFFFFFFFFu, stale);
-            while (todo) {
-                int src[4];                                    // four chunks at a time
-                uint4 w[4];
+        // ---- the best of the candidates.  (Nothing changes the table before every CTA has passed the next barrier.)
+        Best best = {0ull, 0u, 0u};
+        bool listed = false;
+        int n_tied = 0;                                        // candidates of the best rank, in sh.tied as far as they fit
+        if (cand.floor == 0ull) n_cand = 0u;
+        if (n_cand > CAND_MAX) part = min(part + 1, 31);       // (did not fit: fewer the next time)
+        else if (cand.floor) {
+            uint32_t reward = 0u, len = 0u;
+            Key key = {0ull, 0ull};
+            if (threadIdx.x < n_cand) {
+                const ulonglong2 k = __ldcg(reinterpret_cast<const ulonglong2*>(a.keys) + cand_slot);
+                const unsigned long long rank = tok_rank(__ldcg(a.words + cand_slot));
+                key = Key{k.x, k.y};
+                reward = (uint32_t)(rank >> LEN_BITS);
+                len = (uint32_t)rank & ((1u << LEN_BITS) - 1u);
+            }
+            if (threadIdx.x == 0) sh.n_tied = 0;
+            uint32_t top = __reduce_max_sync(0xFFFFFFFFu, reward);
+            uint32_t top_len = __reduce_max_sync(0xFFFFFFFFu, reward == top ? len : 0u);
+            if (lane == 0) sh.red[warp].rank = ((unsigned long long)top << LEN_BITS) | top_len;
+            __syncthreads();
+            const unsigned long long r = sh.red[lane].rank;
+            top = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(r >> LEN_BITS));
+            top_len = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(r >> LEN_BITS) == top ? (uint32_t)r & ((1u << LEN_BITS) - 1u) : 0u);
+            best.rank = ((unsigned long long)top << LEN_BITS) | top_len;
+            listed = best.rank >= cand.floor;
+            if (listed && reward == top && len == top_len) {
+                const int at = atomicAdd(&sh.n_tied, 1);
+                if (at < TIED_MAX) { sh.tied_slot[at] = cand_slot; sh.tied_key[at] = key; }
+            }
+            __syncthreads();
+            n_tied = listed ? sh.n_tied : 0;
+        }
+        if (!listed) {
+            // ---- the best of this warp's chunks of the table
+            Best v = {0ull, 0u, 0u};
+            for (uint64_t c0 = 0; c0 * nw < n_chunks; c0 += 32) {
+                const uint64_t c = (c0 + lane) * nw + wid;
+                const bool mine = c < n_chunks, stale = mine && __ldcg(a.dirty + c);
+                Best b = {0ull, 0u, 0u};
+                if (mine) b = a.chunk_best[c];
+                uint32_t todo = __ballot_sync(0xFFFFFFFFu, stale);
+                while (todo) {
+                    int src[4];                                    // four chunks at a time
+                    uint4 w[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    src[u] = __ffs(todo) - 1;
-                    todo &= todo - 1u;
-                    w[u] = make_uint4(0u, 0u, 0u, 0u);
-                    if (src[u] >= 0) w[u] = __ldcg(reinterpret_cast<const uint4*>(a.words + (((c0 + src[u]) * nw + wid) << CHUNK_BITS)) + lane);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (src[u] < 0) break;
-                    const uint32_t y[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
-                    // the chunk's largest reward, then the lengths that have it (a reward is below 2^31)
-                    uint32_t top = 0u;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) top = max(top, (y[q] & CNT_MASK) * ((y[q] >> CNT_BITS) - 1u));
-                    top = __reduce_max_sync(0xFFFFFFFFu, top);
-                    Best x = {0ull, 0u, 0u};
-                    if (top) {
-                        uint32_t len = 0u;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) if ((uint32_t)(tok_rank(y[q]) >> LEN_BITS) == top) len = max(len, y[q] >> CNT_BITS);
-                        len = __reduce_max_sync(0xFFFFFFFFu, len);
-                        x.rank = ((unsigned long long)top << LEN_BITS) | len;
-                        uint32_t n_top = 0u, at = 0xFFFFFFFFu;
-#pragma unroll
-                        for (int q = 3; q >= 0; --q) if (tok_rank(y[q]) == x.rank) { ++n_top; at = lane * 4 + q; }
-                        x.ties = __reduce_add_sync(0xFFFFFFFFu, n_top);
-                        x.slot = (unsigned int)((((c0 + src[u]) * nw + wid) << CHUNK_BITS) + __reduce_min_sync(0xFFFFFFFFu, at));
+                    for (int u = 0; u < 4; ++u) {
+                        src[u] = __ffs(todo) - 1;
+                        todo &= todo - 1u;
+                        w[u] = make_uint4(0u, 0u, 0u, 0u);
+                        if (src[u] >= 0) w[u] = __ldcg(reinterpret_cast<const uint4*>(a.words + (((c0 + src[u]) * nw + wid) << CHUNK_BITS)) + lane);
                     }
-                    if (lane == src[u]) { b = x; a.chunk_best[c] = x; a.dirty[c] = 0; }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if (src[u] < 0) break;
+                        const uint32_t y[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+                        // the chunk's largest reward, then the lengths that have it (a reward is below 2^31)
+                        uint32_t top = 0u;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) top = max(top, (y[q] & CNT_MASK) * ((y[q] >> CNT_BITS) - 1u));
+                        top = __reduce_max_sync(0xFFFFFFFFu, top);
+                        Best x = {0ull, 0u, 0u};
+                        if (top) {
+                            uint32_t len = 0u;
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) if ((uint32_t)(tok_rank(y[q]) >> LEN_BITS) == top) len = max(len, y[q] >> CNT_BITS);
+                            len = __reduce_max_sync(0xFFFFFFFFu, len);
+                            x.rank = ((unsigned long long)top << LEN_BITS) | len;
+                            uint32_t n_top = 0u, at = 0xFFFFFFFFu;
+#pragma unroll
+                            for (int q = 3; q >= 0; --q) if (tok_rank(y[q]) == x.rank) { ++n_top; at = lane * 4 + q; }
+                            x.ties = __reduce_add_sync(0xFFFFFFFFu, n_top);
+                            x.slot = (unsigned int)((((c0 + src[u]) * nw + wid) << CHUNK_BITS) + __reduce_min_sync(0xFFFFFFFFu, at));
+                        }
+                        if (lane == src[u]) { b = x; a.chunk_best[c] = x; a.dirty[c] = 0; }
+                    }
+                }
+                best_merge(v, b);
+            }
+            auto block_best = [&](Best x) {
+                x = best_warp(x);
+                if (lane == 0) sh.red[warp] = x;
+                __syncthreads();
+                x = best_warp(sh.red[lane]);
+                __syncthreads();
+                return x;
+            };
+            v = block_best(v);
+            if (threadIdx.x == 0) {
+                a.cta_best[blockIdx.x] = v;
+                if (blockIdx.x == 0) a.st->n_cand[(n_lists + 1) & 1] = 0u;
+            }
+            if (!tok_barrier(a.st, epoch, sh)) return;
+            // ---- the best of all, found by every CTA for itself
+            v = Best{0ull, 0u, 0u};
+            if (warp == 0)
+                for (int i = lane; i < (int)gridDim.x; i += 32) best_merge(v, best_load(a.cta_best + i));
+            best = block_best(v);
+            // ---- the candidates
+            ++n_lists;
+            const unsigned long long reward = best.rank >> LEN_BITS;
+            cand = Candidates{a.cand + (n_lists & 1) * CAND_MAX, &a.st->n_cand[n_lists & 1], reward ? (reward - (reward >> part)) << LEN_BITS : 0ull};
+            for (uint64_t c0 = 0; reward && c0 * nw < n_chunks; c0 += 32) {
+                const uint64_t c = (c0 + lane) * nw + wid;
+                uint32_t todo = __ballot_sync(0xFFFFFFFFu, c < n_chunks && a.chunk_best[c].rank >= cand.floor);
+                for (; todo; todo &= todo - 1u) {
+                    const uint64_t first = ((c0 + __ffs(todo) - 1) * nw + wid) << CHUNK_BITS;
+                    // (a word that has been raised past the floor meanwhile is in the list twice, one that has fallen below is not missed)
+                    const uint4 w = __ldcg(reinterpret_cast<const uint4*>(a.words + first) + lane);
+                    const uint32_t y[4] = {w.x, w.y, w.z, w.w};
+                    uint32_t full = 0u;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const bool in = tok_rank(y[q]) >= cand.floor;
+                        const uint32_t who = __ballot_sync(0xFFFFFFFFu, in);
+                        uint32_t at = 0u;
+                        if (lane == 0 && who) at = atomicAdd(cand.n, (unsigned int)__popc(who));
+                        at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(who & ((1u << lane) - 1u));
+                        if (in && at < CAND_MAX) cand.slots[at] = (uint32_t)(first + lane * 4 + q);
+                        full |= at >= CAND_MAX;
+                    }
+                    if (__any_sync(0xFFFFFFFFu, full)) { c0 = n_chunks; break; }
                 }
             }
-            best_merge(v, b);
         }
-        v = best_warp(v);
-        if (lane == 0) sh.red[warp] = v;
-        __syncthreads();
-        if (warp == 0) {
-            v = best_warp(sh.red[lane]);
-            if (lane == 0) a.cta_best[blockIdx.x] = v;
+        if (best.rank == 0ull || n_merges >= a.budget) break;
+        const int n = (int)(best.rank & ((1u << LEN_BITS) - 1u));
+        bool tie = listed ? n_tied > 1 : best.ties > 1;
+        if (n_tied > TIED_MAX) n_tied = 0;
+        else if (tie && listed) {                              // several slots, or one several times?
+            tie = false;
+#pragma unroll 1
+            for (int i = 1; i < n_tied; ++i) tie = tie || sh.tied_slot[i] != sh.tied_slot[0];
         }
-        if (!tok_barrier(a.st, epoch, sh)) return;
-        // ---- the best of all, found by every CTA for itself
-        if (warp == 0) {
-            v = Best{0ull, 0u, 0u};
-            for (int i = lane; i < (int)gridDim.x; i += 32) best_merge(v, best_load(a.cta_best + i));
-            v = best_warp(v);
-            if (lane == 0) sh.red[0] = v;
-        }
-        __syncthreads();
-        const unsigned long long best = sh.red[0].rank;
-        if (best == 0ull || n_merges >= a.budget) break;
-        const int n = (int)(best & ((1u << LEN_BITS) - 1u));
-        const bool tie = sh.red[0].ties > 1;
         if (tie) {
             // ---- several: the one with the first position
             unsigned int* first = &a.st->first[n_ties & 1];
             if (blockIdx.x == 0 && threadIdx.x == 0) a.st->first[~n_ties & 1] = 0xFFFFFFFFu;
+            if (n_tied) {
+                // by their tokens, 512 positions at a time
+                for (int64_t p = s & ~3ll; p < e; p += 512) {
+                    if ((int64_t)__shfl_sync(0xFFFFFFFFu, *(volatile unsigned int*)first, 0) <= p) break;
+                    int4 x[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int64_t q = p + u * 128 + 4 * lane;
+                        x[u] = q < e ? *reinterpret_cast<const int4*>(a.cur + q) : make_int4(-1, -1, -1, -1);
+                    }
+                    unsigned int at = 0xFFFFFFFFu;
+                    for (int i = 0; i < n_tied; ++i) {
+                        const int f = (int)key_get(sh.tied_key[i], 0);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int y[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const int64_t q = p + u * 128 + 4 * lane + j;
+                                if (y[j] != f || q < s || q >= e || q >= (int64_t)at || (int)a.rem[q] < n - 1) continue;
+                                bool hit = true;
+                                for (int k = 1; hit && k < n; ++k) hit = a.cur[q + k] == (int)key_get(sh.tied_key[i], k);
+                                if (hit) at = (unsigned int)q;
+                            }
+                        }
+                    }
+                    at = __reduce_min_sync(0xFFFFFFFFu, at);
+                    if (at != 0xFFFFFFFFu) {
+                        if (lane == 0) atomicMin(first, at);
+                        break;
+                    }
+                }
+            } else
             for (int64_t c = s; c < e; c += 32) {
                 // (one lane's reading decides for all: the value changes meanwhile)
                 if ((int64_t)__shfl_sync(0xFFFFFFFFu, *(volatile unsigned int*)first, 0) <= c) break;
@@ -449,7 +646,7 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
                 if (i < e && a.cur[i] >= 0 && (int)a.rem[i] >= n - 1) {
                     Key key = key_make(n);
                     for (int j = 0; j < n; ++j) key_put(key, j, (uint32_t)a.cur[i + j]);
-                    hit = tok_rank_of(a, key) == best;
+                    hit = tok_rank_of(a, key) == best.rank;
                 }
                 const uint32_t hits = __ballot_sync(0xFFFFFFFFu, hit);
                 if (hits) {
@@ -460,80 +657,90 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
             ++n_ties;
             if (!tok_barrier(a.st, epoch, sh)) return;
         }
-        if (threadIdx.x == 0) {
+        if (threadIdx.x < MAX_N) {
+            const int j = threadIdx.x;
             Key k = {0ull, 0ull};
             int64_t at = 0;
             if (tie) at = *(volatile unsigned int*)&a.st->first[~n_ties & 1];
-            else { const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(a.keys) + sh.red[0].slot); k = Key{v.x, v.y}; }
+            else if (listed) k = sh.tied_key[0];
+            else { const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(a.keys) + best.slot); k = Key{v.x, v.y}; }
+            const int t = j >= n ? -1 : tie ? __ldcg(a.cur + at + j) : (int)key_get(k, j);
             sh.n = n;
-            for (int j = 0; j < MAX_N; ++j) {
-                const int t = j >= n ? -1 : tie ? __ldcg(a.cur + at + j) : (int)key_get(k, j);
-                sh.tok[j] = t;
-                if (blockIdx.x == 0) a.merges[(size_t)n_merges * MAX_N + j] = t;
-            }
+            sh.tok[j] = t;
+            if (blockIdx.x == 0) a.merges[(size_t)n_merges * MAX_N + j] = t;
         }
         const int new_id = a.base_vocab + n_merges++;
         __syncthreads();
-        // ---- its documents
+        // ---- its documents: listed, and rewritten once every CTA has its n-gram; those that the list has no room for in another turn
         const int t0 = sh.tok[0];
         int claimed = 0;
-        auto rewrite = [&](int d) {
-            const int L = a.doc_len[d];
-            const int64_t s0 = a.offsets[d];
-            claimed += L <= DOC_SMEM ? tok_rewrite<true>(a, sh, d, s0, L, new_id, round) : tok_rewrite<false>(a, sh, d, s0, L, new_id, round);
-        };
-        for (int64_t p = s & ~3ll; p < e; p += 512) {
-            int4 x[4];
+        // (A tie's n-gram is read from a document, which has to stay as it is until every CTA has read it; behind a look through the table
+        // all CTAs are past what they read of it.)
+        for (bool passed = !listed && !tie, more = true; more;) {
+            for (int64_t p = s & ~3ll; p < e; p += 512) {
+                int4 x[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t q = p + u * 128 + 4 * lane;
-                x[u] = q < e ? *reinterpret_cast<const int4*>(a.cur + q) : make_int4(-1, -1, -1, -1);
-            }
-            uint32_t mine = 0u;                                // positions with the first token
+                for (int u = 0; u < 4; ++u) {
+                    const int64_t q = p + u * 128 + 4 * lane;
+                    x[u] = q < e ? *reinterpret_cast<const int4*>(a.cur + q) : make_int4(-1, -1, -1, -1);
+                }
+                uint32_t mine = 0u;                            // positions with the first token
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int y[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+                for (int u = 0; u < 4; ++u) {
+                    const int y[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) mine |= y[j] == t0 ? 1u << (u * 4 + j) : 0u;
-            }
-            while (__any_sync(0xFFFFFFFFu, mine != 0u)) {
-                int d = -1;
-                if (mine) {
+                    for (int j = 0; j < 4; ++j) mine |= y[j] == t0 ? 1u << (u * 4 + j) : 0u;
+                }
+                for (; mine; mine &= mine - 1u) {
                     const int b = __ffs(mine) - 1;
-                    mine &= mine - 1u;
                     const int64_t q = p + (b >> 2) * 128 + 4 * lane + (b & 3);
                     // (an occurrence across the end of a document is found not to be one when the document is rewritten)
-                    bool hit = q >= s && q + n <= a.T;
-                    for (int i = 1; hit && i < n; ++i) hit = a.cur[q + i] == sh.tok[i];
+                    if (q < s || q >= e || q + n > a.T) continue;
+                    const int d = a.doc_of[q];
+                    bool hit = true;                           // (all tokens in one trip)
+#pragma unroll
+                    for (int i = 1; i < MAX_N; ++i) if (i < n) hit = (a.cur[q + i] == sh.tok[i]) & hit;
                     // the first hit of a document in this round puts it on the list
-                    if (hit && q < e) {
-                        d = a.doc_of[q];
-                        if (atomicExch(&a.doc_round[d], round + 1) == round + 1) d = -1;
-                    }
-                }
-                uint32_t docs = __ballot_sync(0xFFFFFFFFu, d >= 0);
-                if (docs) {
-                    int slot = 0;
-                    if (lane == 0) slot = atomicAdd(&sh.n_hits, __popc(docs));
-                    slot = __shfl_sync(0xFFFFFFFFu, slot, 0) + __popc(docs & ((1u << lane) - 1u));
-                    if (d >= 0 && slot < HIT_MAX) sh.hits[slot] = d;
-                    for (docs = __ballot_sync(0xFFFFFFFFu, d >= 0 && slot >= HIT_MAX); docs; docs &= docs - 1u)
-                        rewrite(__shfl_sync(0xFFFFFFFFu, d, __ffs(docs) - 1));
+                    if (!hit) continue;
+                    if (atomicExch(&a.doc_round[d], round + 1) == round + 1) continue;
+                    const int L = a.doc_len[d];
+                    const int64_t s0 = a.offsets[d];
+                    const int slot = atomicAdd(&sh.n_hits, 1);
+                    if (slot < HIT_MAX) { sh.hits[slot] = d; sh.hit_len[slot] = L; sh.hit_at[slot] = s0; }
+                    else { atomicExch(&a.doc_round[d], round); sh.more_hits = 1; }
                 }
             }
-        }
-        __syncthreads();
-        const int n_hits = min(sh.n_hits, HIT_MAX);
-        for (;;) {
-            int slot = 0;
-            if (lane == 0) slot = atomicAdd(&sh.next_hit, 1);
-            slot = __shfl_sync(0xFFFFFFFFu, slot, 0);
-            if (slot >= n_hits) break;
-            rewrite(sh.hits[slot]);
+            __syncthreads();
+            more = sh.more_hits != 0;
+            const int n_hits = min(sh.n_hits, HIT_MAX);
+            // while the barrier is on its way the warps work on their first documents
+            if (!passed) tok_arrive(a.st, epoch);
+            if (tie && !passed) {
+                if (!tok_wait(a.st, epoch, sh)) return;
+                passed = true;
+            }
+            for (;;) {
+                int slot = 0;
+                if (lane == 0) slot = atomicAdd(&sh.next_hit, 1);
+                slot = __shfl_sync(0xFFFFFFFFu, slot, 0);
+                const bool work = slot < n_hits;
+                const int d = work ? sh.hits[slot] : 0, L = work ? sh.hit_len[slot] : 0;
+                const int64_t s0 = work ? sh.hit_at[slot] : 0;
+                Rewritten r = {0, 0u, 0u};
+                if (work && L <= DOC_SMEM) r = tok_rewrite_short(a, sh, d, s0, L, new_id);
+                if (!passed) {
+                    if (!tok_wait(a.st, epoch, sh)) return;
+                    passed = true;
+                }
+                if (!work) break;
+                claimed += L <= DOC_SMEM ? tok_recount_short(a, sh, L, r, round, cand) : tok_rewrite_long(a, sh, d, s0, L, new_id, round, cand);
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) { sh.n_hits = 0; sh.next_hit = 0; sh.more_hits = 0; }
+            if (more) __syncthreads();
         }
         publish_claims(claimed);
         if (!tok_barrier(a.st, epoch, sh)) return;
-        if (threadIdx.x == 0) { sh.n_hits = 0; sh.next_hit = 0; }          // (two barriers before their next use)
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) a.st->n_merges = n_merges;
 }
@@ -778,14 +985,14 @@ extern "C" tasc_status tasc_tok_enrich(const int32_t* corpus_tokens, const int64
     const uint64_t cap = std::max<uint64_t>(pow2_at_least(2 * hc.windows), 1ull << CHUNK_BITS), chunks = cap >> CHUNK_BITS;
     const size_t t = (size_t)T + 4, nd = (size_t)n_docs;
     const size_t o_keys = slab.add(cap * 16), o_words = slab.add(cap * 4), o_dirty = slab.add(chunks), o_chunk = slab.add(chunks * sizeof(Best)),
-                 o_cta = slab.add(grid * sizeof(Best)), o_st = slab.add(sizeof(TokState)), o_cur = slab.add(t * 4), o_of = slab.add(t * 4),
+                 o_cta = slab.add(grid * sizeof(Best)), o_cand = slab.add(2 * CAND_MAX * 4), o_st = slab.add(sizeof(TokState)), o_cur = slab.add(t * 4), o_of = slab.add(t * 4),
                  o_rem = slab.add(t), o_mark = slab.add(t), o_len = slab.add(nd * 4), o_round = slab.add(nd * 4), o_tot = slab.add(scan_blocks(n_docs) * 8);
     if (!slab.allocate(stream)) return TASC_ENOMEM;
     TokArgs a = {};
     a.cur = slab.at<int32_t>(o_cur); a.rem = slab.at<uint8_t>(o_rem); a.mark = slab.at<uint8_t>(o_mark); a.doc_of = slab.at<int32_t>(o_of);
     a.offsets = doc_offsets; a.doc_len = slab.at<int32_t>(o_len); a.doc_round = slab.at<int32_t>(o_round); a.n_docs = n_docs; a.T = T;
     a.keys = slab.at<uint64_t>(o_keys); a.words = slab.at<uint32_t>(o_words); a.dirty = slab.at<uint8_t>(o_dirty);
-    a.chunk_best = slab.at<Best>(o_chunk); a.cta_best = slab.at<Best>(o_cta); a.cap = cap; a.st = slab.at<TokState>(o_st);
+    a.chunk_best = slab.at<Best>(o_chunk); a.cta_best = slab.at<Best>(o_cta); a.cand = slab.at<uint32_t>(o_cand); a.cap = cap; a.st = slab.at<TokState>(o_st);
     a.merges = merges; a.base_vocab = base_vocab; a.budget = budget; a.n_max = n_max;
     TokState hs = {};
     TASC_CUDA_TRY(cudaMemsetAsync(a.st, 0, sizeof(TokState), stream));
