@@ -685,6 +685,8 @@ draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t 
 
     const int b = blockIdx.x;
     const int tid = threadIdx.x, warp = tid >> 5;
+    griddep_wait();
+    griddep_launch_dependents();
     int L = len[b];
     L = L < 0 ? 0 : (L > stride ? (int)stride : L);
     const int n_max = dt.n_max;
@@ -1170,8 +1172,7 @@ extern "C" tasc_status tasc_draft(const tasc_drafter* d, const int32_t* tokens, 
         }
     }
     ProfScope ps(K_DRAFT, static_cast<cudaStream_t>(stream));
-    draft_kernel<<<B, DRAFT_THREADS, smem, static_cast<cudaStream_t>(stream)>>>(
-        d->dt, tokens, stride, len, k, (uint32_t)lambda_num, (uint32_t)lambda_den, drafts, (int)(hs - 1));
-    TASC_CUDA_TRY(cudaGetLastError());
+    TASC_CUDA_TRY(launch_ahead(draft_kernel, dim3(B), dim3(DRAFT_THREADS), smem, static_cast<cudaStream_t>(stream),
+                               d->dt, tokens, stride, len, k, (uint32_t)lambda_num, (uint32_t)lambda_den, drafts, (int)(hs - 1)));
     return TASC_OK;
 }

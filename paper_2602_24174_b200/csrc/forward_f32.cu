@@ -12,8 +12,8 @@
 // keys in blocks of eight (four lanes to a key for the scores, lanes = dimensions for P V) and merge their softmax states.
 // (Blocks of 32 keys left most of the eight warps idle at 100 keys: 11 us per layer against 5.)
 //
-// Measured, draft + verify step of that configuration at one sequence: 174 us as a chain, 60 us so
-// (41 in this kernel, 10 in the draft).
+// Measured, draft + verify step of that configuration at one sequence: 174 us as a chain, 60 us so, 54 since it is set up while the
+// draft runs and its stages are one copy of code (9 in the draft; replayed from a graph 52).
 #include "kernels.h"
 
 #include <algorithm>
@@ -98,6 +98,8 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
     unsigned long long tl_0 = global_ns(), tl_a = tl_0, tl_b = tl_0;
     int tl_tag = 0;
 #endif
+    griddep_wait();
+    griddep_launch_dependents();
     // ---- row plan: every CTA for itself, CTA 0 for the kernels behind
 #pragma unroll 1
     for (int m = threadIdx.x; m < M; m += THREADS) {
@@ -136,9 +138,9 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
     for (int m = warp; m < M; m += WARPS)                        // (row m by CTA m % CTAS)
         if (m % CTAS == cta)
             for (int j = 4 * lane; j < d; j += 128) *reinterpret_cast<float4*>(a.x + (size_t)m * d + j) = __ldg(reinterpret_cast<const float4*>(a.embed + (size_t)s_tok[m] * d + j));
-    // One copy of a stage's code for all products: a stage is a microsecond or two, of which the instructions of five copies took
-    // most (128 KB of kernel, a third of the instruction-cache requests missed; now 30 KB).  A stage's first weights, which
-    // depend on nothing, are requested before the barrier that precedes it.
+    // One copy of a stage's code for all products (five copies: 114 - 128 KB of kernel, a third of the instruction-cache requests
+    // missed and the kernel took 61 us under ncu; now 49 - 62 KB, 7 % and 50 us).  A stage's first weights, which depend on
+    // nothing, are requested before the barrier that precedes it.
     int stage = ST_QKV, l = 0;
     LayerWeightsF32 lw = a.layers[0];
     bool first = true;
@@ -365,15 +367,17 @@ size_t smem_bytes(int M, int width, int hd) {
     return ((size_t)((M + ROWS - 1) / ROWS * ROWS) * width + (size_t)WARPS * (hd + 4)) * 4 + (size_t)M * 16 + 16;
 }
 
-void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, size_t smem) {
+void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[2], size_t smem) {
     cfg.gridDim = dim3(CTAS, 1, 1);
     cfg.blockDim = dim3(THREADS, 1, 1);
     cfg.dynamicSmemBytes = smem;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = CTAS;
-    at.val.clusterDim.y = 1;
-    at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CTAS;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // (set up while the draft runs)
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
     cfg.numAttrs = 1;
 }
 // The kernel's attributes are set and the device takes its cluster.
@@ -390,7 +394,7 @@ bool cluster_available() {
                   cudaFuncSetAttribute(forward_f32_kernel<NJ>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
         if (ok) {
             cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute at;
+            cudaLaunchAttribute at[2];
             cluster_config(cfg, at, MAX_SMEM);
             ok = cudaOccupancyMaxActiveClusters(&n, forward_f32_kernel<NJ>, &cfg) == cudaSuccess && n > 0;
         }
@@ -402,8 +406,9 @@ bool cluster_available() {
 template <int NJ>
 tasc_status launch_inst(const ForwardF32Args& a, cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at;
+    cudaLaunchAttribute at[2];
     cluster_config(cfg, at, smem_bytes(a.M, a.width, a.hd));
+    cfg.numAttrs = 2;
     cfg.stream = stream;
     ProfScope ps(K_LAYERS, stream);
     TASC_CUDA_TRY(cudaLaunchKernelEx(&cfg, forward_f32_kernel<NJ>, a));

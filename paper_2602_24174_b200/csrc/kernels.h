@@ -204,6 +204,22 @@ tasc_status launch_persist(PersistArgs a, const PersistPlan& p, cudaStream_t str
 void launch_gemm_f32(const float* X, const float* W, float* partials, int M, int N, int K,
                      unsigned long long* argmax, float* logits, cudaStream_t stream);
 
+// Launches a kernel that may be set up while the kernel before it in the stream still runs.  The kernel begins with griddep_wait().
+template <typename... P, typename... A>
+inline cudaError_t launch_ahead(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ------------------------------------------------------------------ layer kernels (layers.cu)
 struct RowPlan {              // per-step row bookkeeping, all device pointers into the workspace
     int* row_tok;             // [M] token id of each row

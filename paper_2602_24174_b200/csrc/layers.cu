@@ -95,6 +95,8 @@ rows_embed_kernel(RowPlan rp, const int32_t* __restrict__ tokens, int64_t stride
     __shared__ float red[4];
     __shared__ int s_tok;
     const int m = blockIdx.x;
+    griddep_wait();
+    griddep_launch_dependents();
     for (int i = m * blockDim.x + threadIdx.x; i < n_zero; i += gridDim.x * blockDim.x) zero[i] = 0u;
     if (threadIdx.x == 0) {
         const int b = m / R, r = m % R;
@@ -258,28 +260,30 @@ __global__ void fill_u64_kernel(unsigned long long* p, unsigned long long v, int
 }
 
 __global__ void accept_kernel(const unsigned long long* __restrict__ argmax, RowPlan rp, const int32_t* __restrict__ drafts,
-                              const int32_t* __restrict__ forced, int32_t* tokens, int64_t stride, int32_t* len, int B, int R,
+                              const int32_t* __restrict__ forced, int32_t* tokens, int64_t stride, int32_t* len, int R,
                               int32_t* n_accepted, int32_t* next_token, int32_t* target_tokens, long long* hist) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const int k = R - 1;
-    if (target_tokens)
-        for (int i = 0; i < R; ++i) target_tokens[b * R + i] = (int32_t)packed_id(argmax[b * R + i]);
-    if (rp.seq_rows[b] == 0) {
-        n_accepted[b] = 0;
-        next_token[b] = -1;
+    griddep_wait();
+    // a warp per sequence, a lane per row: everything is requested together
+    static_assert(TASC_MAX_ROWS <= 32, "a lane per row");
+    const int b = blockIdx.x, i = threadIdx.x, k = R - 1;
+    const int32_t y = i < R ? (int32_t)packed_id(argmax[b * R + i]) : 0, t = forced && i < R ? forced[b * R + i] : y;
+    const int32_t draft = i < k ? drafts[b * k + i] : 0;
+    const int rows = rp.seq_rows[b], L = len[b];
+    if (target_tokens && i < R) target_tokens[b * R + i] = y;
+    // the longest prefix of drafts that are the tokens of their rows
+    const int a = __ffs(~__ballot_sync(0xFFFFFFFFu, i < k && draft == t)) - 1;
+    const int nxt = __shfl_sync(0xFFFFFFFFu, t, a);
+    if (rows == 0) {
+        if (i == 0) {
+            n_accepted[b] = 0;
+            next_token[b] = -1;
+        }
         return;
     }
-    auto target = [&](int i) { return forced ? forced[b * R + i] : (int32_t)packed_id(argmax[b * R + i]); };
-    int a = 0;
-    while (a < k && drafts[b * k + a] == target(a)) ++a;
-    const int nxt = target(a);
-    const int L = len[b];
     int32_t* row = tokens + (int64_t)b * stride;
-    int w = 0;
-    for (; w < a && L + w < stride; ++w) row[L + w] = drafts[b * k + w];
-    if (L + a < stride) { row[L + a] = nxt; w = a + 1; }
-    len[b] = L + w;            // w = a + 1 unless the token buffer is full
+    if (i <= a && L + i < stride) row[L + i] = i < a ? draft : nxt;
+    if (i) return;
+    len[b] = (int)min((int64_t)L + a + 1, stride);       // (less than a + 1 more where the token buffer is full)
     n_accepted[b] = a;
     next_token[b] = nxt;
     if (hist) atomicAdd(reinterpret_cast<unsigned long long*>(hist + a), 1ull);
@@ -381,8 +385,8 @@ void launch_rows_embed(const RowPlan& rp, const int32_t* tokens, int64_t stride,
                        const float* gain, float* x, __nv_bfloat16* a_out, float* ssq, int ssq_slots, unsigned long long* argmax,
                        int d, int TB, unsigned long long* ssq_p, int n_stage, unsigned* zero, int n_zero, cudaStream_t stream) {
     ProfScope ps(K_EMBED, stream);
-    rows_embed_kernel<<<B * R, 128, 0, stream>>>(rp, tokens, stride, len, stop_len, drafts, R, chunk, vocab, status, embed, gain,
-                                                 x, a_out, ssq, ssq_slots, argmax, d, TB, ssq_p, n_stage, zero, n_zero);
+    if (launch_ahead(rows_embed_kernel, dim3(B * R), dim3(128), 0, stream, rp, tokens, stride, len, stop_len, drafts, R, chunk, vocab, status, embed, gain,
+                     x, a_out, ssq, ssq_slots, argmax, d, TB, ssq_p, n_stage, zero, n_zero) != cudaSuccess) return;      // (found by the caller's cudaGetLastError)
 }
 template <typename T>
 void launch_residual_norm(const float* partials, int splits, float* x, const float* gain, float eps, T* h, int M, int d,
@@ -423,8 +427,8 @@ void launch_accept(const unsigned long long* argmax, const RowPlan& rp, const in
                    int32_t* n_accepted, int32_t* next_token, int32_t* target_tokens, long long* hist,
                    cudaStream_t stream) {
     ProfScope ps(K_ACCEPT, stream);
-    accept_kernel<<<(B + 63) / 64, 64, 0, stream>>>(argmax, rp, drafts, forced_targets, tokens, stride, len, B, R,
-                                                    n_accepted, next_token, target_tokens, hist);
+    if (launch_ahead(accept_kernel, dim3(B), dim3(32), 0, stream, argmax, rp, drafts, forced_targets, tokens, stride, len, R,
+                     n_accepted, next_token, target_tokens, hist) != cudaSuccess) return;
 }
 void launch_wait_selftest(long long budget_cycles, int* status, cudaStream_t stream) {
     ProfScope ps(K_OTHER, stream);
