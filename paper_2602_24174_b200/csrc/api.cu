@@ -257,16 +257,21 @@ tasc_status forward_f32(const tasc_model* m, const tasc_kv* kv, const Workspace&
 //      18    816 / 709      758 / 749
 //      24    801 / 731      758 / 748
 //      32    822 / 744      769 / 761         795 / 729      955 / 948 (28)
-//      33    883 / 802      795 / 787
-//      48    936 / 869      849 / 838         905 / 850      1197 / 1187
-//      64    889 / 818      830 / 819
+//      48                                     905 / 850      1197 / 1187
 //      96    965 / 898      1052 / 1042
 // (270 - 380, 560 and 1,071 keys).  The one kernel's time hardly changes between 17 and 32 rows and between 33 and 64 (blocks of
 // 32); a generation replays, so 17 to 32 rows are not its (plan_persist).
+// 33 to 64 rows of the 135M, enqueued, since the five kernels have shorter code and token tiles of 16 rows:
+//     48 rows    150 keys 723, 782    300 keys 748, 789    500 keys 759, 836          35 rows, 300 keys 721, 780
+//     64 rows    150 keys 686, 787    480 keys 751, 835    prefill of 40 / 60 tokens 651 / 632, 684 / 694
+// so there it keeps the verify steps of caches of up to PERSIST_BLOCKS_CTX tokens only, where the difference is smallest and which the
+// tests of the one-kernel layers are about.
+constexpr int PERSIST_BLOCKS_CTX = 352;
 // Its attention has at most one unit per SM and 12 key ranges, so the bytes of a unit's keys are bounded too, by 512 keys of 64:
 //     1.5B, 7 rows    1,500 keys 1235 / 1155, 1160 / 1150   3,000 (250 per unit) 1357 / 1273, 1296 / 1288   3,600 1340 / 1266, 1357 / 1348
 //     135M, 48 rows   1,500 (500 per unit) 1100 / 1010, 1070 / 1061                                         4,000 1385 / 1290, 1676 / 1666
-bool persist_pays(const tasc_model* m, int M, int max_ctx, const PersistPlan& pp) {
+bool persist_pays(const tasc_model* m, int M, int R, int max_ctx, const PersistPlan& pp) {
+    if (M > 32 && (R > TASC_MAX_ROWS || max_ctx > PERSIST_BLOCKS_CTX)) return false;
     if (max_ctx / pp.splits * m->desc.head_dim > 512 * 64) return false;
     return M <= 8 || m->layer_mb <= 12.0;
 }
@@ -300,7 +305,7 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
             sp.persist = !wide_pass && m->aligned32 &&
                          plan_persist(d.n_layers, M, B, R, d.d_model, m->q_dim, d.n_q_heads, d.n_kv_heads, d.head_dim, d.d_ff, max_ctx,
                                       d.page_size, sp.pp) &&
-                         persist_pays(m, M, max_ctx, sp.pp);
+                         persist_pays(m, M, R, max_ctx, sp.pp);
             sp.TB = gemm_token_tile(M, true, m->few_tiles, wide_min_mb >= 0.0);
             sp.rows = (uint64_t)((M + sp.TB - 1) / sp.TB) * 2 * sp.TB;
             if ((st = encode_tmap_bf16(&sp.tm_h, w.h, sp.rows, d.d_model, 2 * sp.TB)) != TASC_OK) return st;

@@ -717,8 +717,9 @@ FusedPlan plan_fused(int M, int N, int K, int epi, int few_tiles, int hd, double
     // token columns a CTA reduces and finishes after the cluster exchange
     const int cols_cta = (std::min(p.TB, M) + p.S - 1) / p.S;
     // (only for grids of one wave: with two CTAs per SM the schedulers have warps enough, and twelve warps of 100 to 126
-    // registers would not leave room for the second CTA)
-    p.threads = (epi != EPI_LM && epi != EPI_PLAIN && cols_cta >= FINISHERS_MIN_COLS && tiles * p.S <= 148) ? MAX_THREADS : THREADS;
+    // registers would not leave room for the second CTA.  The LM head's 56 registers do: a step of the 135M at 96 rows 827.8 -> 824.6 us,
+    // of the 0.5B at 28 rows 697.7 -> 693.7.)
+    p.threads = epi != EPI_PLAIN && cols_cta >= FINISHERS_MIN_COLS && (epi == EPI_LM || tiles * p.S <= 148) ? MAX_THREADS : THREADS;
     return p;
 }
 

@@ -222,7 +222,12 @@ int gemm_token_tile(int M, bool pair, int few_tiles, bool many_rows) {
     // The few-row kernel's time per tile grows with its token columns (the MMA's 40 to 63 cycles per 16 of k, the split-K
     // exchange, the accumulator read-out, the epilogue), but every token tile streams the weight tile again, from L2, and
     // occupies more SMs.  Which wins depends on the layer's weights (few_tiles).  A step in us, by rows of a tile:
-    //     7 MB per layer    128 rows  32: 1039  48: 1079  64: 1131      256 rows  32: 1248  48: 1219  64: 1267  96: 1322
+    //     7 MB per layer    35 rows   16: 721  32: 736  48: 771         48 rows   16: 748  32: 761  48: 834
+    //                       64 rows   16: 686  32: 718  64: 799         72 rows   16: 744  32: 771  48: 807
+    //                       96 rows   16: 808  32: 819  48: 867         100 rows  16: 841  32: 821  48: 843
+    //                       20 rows   16: 714  32: 680                  288 rows  32: 1057  48: 963  64: 1013
+    //     (and with longer kernels, before their code was cut)
+    //                       128 rows  32: 1039  48: 1079  64: 1131      256 rows  32: 1248  48: 1219  64: 1267  96: 1322
     //                       192 rows  32: 1152  48: 1186  64: 1217      prefill of 512  32: 1565  48: 1385  64: 1400  128: 1584
     //     30 MB             48 rows  16: 904  48: 920     45 rows  16: 917  48: 912     96 rows  32: 1112  48: 1144  96: 1183
     //                       128 rows  32: 1355  48: 1236  64: 1267      192 rows  48: 1572  64: 1440  96: 1733
@@ -231,7 +236,7 @@ int gemm_token_tile(int M, bool pair, int few_tiles, bool many_rows) {
     // few tiles of at most 128 rows as hold them.
     if (pair && !many_rows) {
         auto tiles_of = [&](int rows) { return std::max(3, (M + rows - 1) / rows); };
-        if (few_tiles >= 3 && M > 48) m_tiles = std::max(m_tiles, tiles_of(M <= 192 ? 32 : 48));
+        if (few_tiles >= 3 && M > 32) m_tiles = std::max(m_tiles, tiles_of(M <= 96 ? 16 : M <= 192 ? 32 : 48));
         else if (few_tiles == 2 && M > 45) m_tiles = std::max(m_tiles, tiles_of(64));
         else if (M > 128) m_tiles = std::max(m_tiles, 3);
     }
