@@ -75,14 +75,8 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 // four consecutive values -> bf16; -> (hi, lo) bf16
 __device__ __forceinline__ uint2 bf16x4(const float4& v) { return make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w)); }
 __device__ __forceinline__ void hilo4(const float4& v, uint2& hi, uint2& lo) {
-    __nv_bfloat16 h[4], l[4];
-    split_bf16(v.x, h[0], l[0]);
-    split_bf16(v.y, h[1], l[1]);
-    split_bf16(v.z, h[2], l[2]);
-    split_bf16(v.w, h[3], l[3]);
-    auto two = [](const __nv_bfloat16* p) { return (uint32_t)__bfloat16_as_ushort(p[0]) | ((uint32_t)__bfloat16_as_ushort(p[1]) << 16); };
-    hi = make_uint2(two(h), two(h + 2));
-    lo = make_uint2(two(l), two(l + 2));
+    split_bf16x2(v.x, v.y, hi.x, lo.x);
+    split_bf16x2(v.z, v.w, hi.y, lo.y);
 }
 __device__ __forceinline__ void store_f32x32(float* p, const float (&v)[32]) {
 #pragma unroll
@@ -97,7 +91,11 @@ __device__ __forceinline__ void acc32(uint32_t taddr, float (&v)[32]) {
     for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(r[e]);
 }
 
-template <int EPI, bool PAIR>
+// SPLIT: split-K clusters, one tile each, in place of persistent CTAs (or pairs).  Instances of their own: with the choice at run time
+// every kernel carried both epilogues, 42 - 118 KB of code where it is 32 - 73 now, and the TMA lane worked out ring slots, tiles and rows by
+// division at every k-block.  Step of the 0.5B + 8,192 tokens, 288 rows 1430 -> 1388 us; 1.5B, 448 rows 4242 -> 4181; prefill of 16 prompts of
+// up to 1,024 tokens 77.5 -> 75.7 ms.
+template <int EPI, bool PAIR, bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const FusedArgs a) {
     extern __shared__ uint8_t smem_raw[];
@@ -124,9 +122,9 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     // tokens a quarter of all tiles.  1.5B: 85 ms with them, 79 without.)
     __shared__ int s_tt[MAX_TT];
     __shared__ int s_n_tt;
-    const int S = PAIR ? 1 : (int)cluster_nctarank();
-    const int kb0 = PAIR ? 0 : (int)(((long long)num_kb * rank) / S);
-    const int nkb = PAIR ? num_kb : (int)(((long long)num_kb * (rank + 1)) / S) - kb0;      // k-blocks of this CTA (all of them when S = 1)
+    const int S = SPLIT ? (int)cluster_nctarank() : 1;
+    const int kb0 = SPLIT ? (int)((unsigned)(num_kb * rank) / (unsigned)S) : 0;
+    const int nkb = SPLIT ? (int)((unsigned)(num_kb * (rank + 1)) / (unsigned)S) - kb0 : num_kb;      // k-blocks of this CTA (all of them when S = 1)
     constexpr int XPAD = 4;                                                 // floats: rows of the parked tile fall on distinct banks
     float* xch = reinterpret_cast<float*>(smem);                            // [128][BNW + XPAD], split-K only
     constexpr int FLD = 4 * 32 + XPAD;                                      // a CTA finishes at most four 32-column chunks of a split tile
@@ -176,8 +174,8 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     const int n_tt = PAIR ? (live_tt + 1) / 2 : live_tt;        // token tiles, or pairs of them
     const int n_tiles = a.n_ft * n_tt;
     // S = 1: persistent, tiles blockIdx.x, + gridDim.x, ...   S > 1: the grid is S * n_tiles CTAs, one tile per cluster
-    const int tile0 = PAIR ? (int)blockIdx.x / 2 : S > 1 ? (int)blockIdx.x / S : (int)blockIdx.x;
-    const int tstep = PAIR ? (int)gridDim.x / 2 : S > 1 ? n_tiles : (int)gridDim.x;
+    const int tile0 = PAIR ? (int)blockIdx.x / 2 : SPLIT ? (int)blockIdx.x / S : (int)blockIdx.x;
+    const int tstep = PAIR ? (int)gridDim.x / 2 : SPLIT ? n_tiles : (int)gridDim.x;
     const int my_tiles = tile0 < n_tiles ? (n_tiles - tile0 + tstep - 1) / tstep : 0;
 
     if (warp == EPI_WARPS) {
@@ -191,11 +189,20 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 if (!PAIR) mbar_expect_tx(bar_full + 8u * s, stage_bytes);
                 else if (rank == 0) mbar_expect_tx(bar_full + 8u * s, 2u * stage_bytes);
             };
-            auto load_w = [&](int i) {
-                const int tile = tile0 + (i / nkb) * tstep;
-                const int f0 = (tile / n_tt) * FT, kc = (kb0 + i % nkb) * BK;
-                const int s = i % stages;
-                const uint32_t dst = smem_u32(smem + (size_t)s * stage_bytes) + a_bytes, bar = full0 + 8u * s;
+            // where the loads are: ring slot, k-block, tile (its first feature and first row of the activation buffer)
+            struct At { int s, kb, tile, f0, row; };
+            auto place = [&](At& c) {
+                const int t = (int)((unsigned)c.tile / (unsigned)n_tt), i = c.tile - t * n_tt;
+                c.f0 = t * FT;
+                c.row = token_tile(PAIR ? 2 * i + rank : i) * 2 * TBL;
+            };
+            auto advance = [&](At& c) {
+                if (++c.s == stages) c.s = 0;
+                if (++c.kb == nkb) { c.kb = 0; c.tile += tstep; place(c); }
+            };
+            auto load_w = [&](const At& c) {
+                const int f0 = c.f0, kc = (kb0 + c.kb) * BK;
+                const uint32_t dst = smem_u32(smem + (size_t)c.s * stage_bytes) + a_bytes, bar = full0 + 8u * c.s;
                 if (PAIR) {                                // 128 of the 256 weight rows: the gate rows or the up rows; the lower or the upper half
                     if (EPI == EPI_SWIGLU)
                         for (int r = 0; r < FT; r += 64) tma_load_2d_pair(dst + (uint32_t)r * 128u, &tmW, kc, rank * a.N + f0 + r, bar, pol_w);
@@ -209,28 +216,33 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     for (int r = 0; r < BNW; r += 128) tma_load_2d_hint(dst + (uint32_t)r * 128u, &tmW, kc, f0 + r, bar, pol_w);
                 }
             };
-            auto load_x = [&](int i) {
-                const int tile = tile0 + (i / nkb) * tstep;
-                const int s = i % stages;
-                const uint32_t dst = smem_u32(smem + (size_t)s * stage_bytes);
-                if (PAIR) tma_load_2d_pair(dst, &tmX, (i % nkb) * BK, token_tile(2 * (tile % n_tt) + rank) * 2 * TBL, full0 + 8u * s, pol_x);
-                else tma_load_2d_hint(dst, &tmX, (kb0 + i % nkb) * BK, token_tile(tile % n_tt) * 2 * TBL, bar_full + 8u * s, pol_x);
+            auto load_x = [&](const At& c) {
+                const uint32_t dst = smem_u32(smem + (size_t)c.s * stage_bytes);
+                if (PAIR) tma_load_2d_pair(dst, &tmX, c.kb * BK, c.row, full0 + 8u * c.s, pol_x);
+                else tma_load_2d_hint(dst, &tmX, (kb0 + c.kb) * BK, c.row, bar_full + 8u * c.s, pol_x);
             };
             // The weights of the first stages depend on no earlier kernel: they are requested before the
             // preceding grid has finished, the token rows after it.
             const int pre = total < stages ? total : stages;
-            for (int i = 0; i < pre; ++i) {
-                expect(i % stages);
-                load_w(i);
+            At w = {0, 0, tile0, 0, 0};
+            if (total > 0) place(w);
+            At x = w;
+#pragma unroll 1
+            for (int i = 0; i < pre; ++i, advance(w)) {
+                expect(w.s);
+                load_w(w);
             }
             griddep_wait();
-            for (int i = 0; i < pre; ++i) load_x(i);
-            for (int i = pre; i < total; ++i) {
-                const int s = i % stages;
-                if (!wait_or_fail<PAIR>(bar_empty + 8u * s, (((uint32_t)(i / stages)) & 1u) ^ 1u, failed)) { fail(); break; }
-                expect(s);
-                load_w(i);
-                load_x(i);
+#pragma unroll 1
+            for (int i = 0; i < pre; ++i, advance(x)) load_x(x);
+            uint32_t parity = 0u;                          // of the stage's previous use
+#pragma unroll 1
+            for (int i = pre; i < total; ++i, advance(w)) {
+                if (!wait_or_fail<PAIR>(bar_empty + 8u * w.s, parity, failed)) { fail(); break; }
+                if (w.s == stages - 1) parity ^= 1u;
+                expect(w.s);
+                load_w(w);
+                load_x(w);
             }
             griddep_launch_dependents();
         }
@@ -249,12 +261,14 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             int s = 0;
             uint32_t round = 0;
             bool ok = true;
+#pragma unroll 1
             for (int j = 0; j < my_tiles && ok; ++j) {
                 const int b = j & 1;
                 ok = __all_sync(0xFFFFFFFFu, wait_or_fail<PAIR>(bar_acc_empty + 8u * b, (((uint32_t)(j >> 1)) & 1u) ^ 1u, failed));
                 if (!ok) { fail(); break; }
                 tc_fence_after();
                 const uint32_t d = tmem_base + (uint32_t)(b * BNW);
+#pragma unroll 1
                 for (int kb = 0; kb < nkb; ++kb) {
                     ok = __all_sync(0xFFFFFFFFu, wait_or_fail<PAIR>(bar_full + 8u * s, round & 1u, failed));
                     if (!ok) { fail(); break; }
@@ -280,7 +294,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     const int rowl = quarter * 32 + lane;                             // row within the token tile = TMEM lane
     const int XLD = BNW + XPAD;
     uint32_t peer[8];
-    {
+    if (SPLIT) {
 #pragma unroll
         for (int s = 0; s < 8; ++s) peer[s] = cluster_map(smem_u32(xch), (uint32_t)(s < S ? s : 0));
     }
@@ -292,7 +306,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         const int m = tt * TBL + rowl;
         const bool rowok = rowl < TBL && m < a.M;
         auto get32 = [&](int col, float (&v)[32]) {
-            if (S == 1) {
+            if (!SPLIT) {
                 acc32(acc + (uint32_t)col, v);
             } else {
                 // the reduced columns of this CTA's units, packed in the order of their 32-column chunks
@@ -309,7 +323,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         // swizzled 4 KB, or with split-K the reduced chunk they came from), and come back as emit(row within the quarter, column,
         // four values) with eight lanes to a row: 4 lines per access, where a thread per row touched 32.
         auto staged = [&](int col, int r, int c4) {
-            return S == 1 ? reinterpret_cast<float4*>(stage + r * 32 + ((c4 ^ (r & 7)) << 2))
+            return !SPLIT ? reinterpret_cast<float4*>(stage + r * 32 + ((c4 ^ (r & 7)) << 2))
                           : reinterpret_cast<float4*>(fin + (size_t)(quarter * 32 + r) * FLD + __popc(own_mask & ((1u << (col >> 5)) - 1u)) * 32 + 4 * c4);
         };
         auto rows_out = [&](int col, const float (&v)[32], auto&& emit) {
@@ -332,18 +346,20 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         int unit = 0;                                                 // running index of the tile's work units
         int owned = 0;                                                // ... of those of this CTA (every S-th)
         auto mine = [&]() {                                           // the quarter's two warps alternate over the CTA's units
-            const bool own = PAIR || (unit++ % S) == rank;
+            const bool own = !SPLIT || (unit++ % S) == rank;
             return own && (owned++ & 1) == wq;
         };
         float sc = 1.0f;
         if (a.ssq_in && rowok) {
             float ss = 0.f;
             const float4* sp = reinterpret_cast<const float4*>(a.ssq_in + (size_t)m * a.ssq_slots);
+#pragma unroll 4
             for (int q = 0; q < a.ssq_slots / 4; ++q) { const float4 t = sp[q]; ss += (t.x + t.y) + (t.z + t.w); }
             sc = 1.0f / sqrtf(ss * a.inv_d + a.eps);
         }
 
         if (EPI == EPI_SWIGLU) {
+#pragma unroll 1
             for (int c = 0; c < FT && f0 + c < a.N; c += 32) {
                 if (!mine()) continue;
                 float g[32], u[32];
@@ -358,6 +374,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             }
         } else if (EPI == EPI_RESID) {
             // ssq_out has one slot per 32 features here (a.ssq_out_slots of them, a multiple of four per 128 features)
+#pragma unroll 1
             for (int c = 0; c < BNW && f0 + c < a.N; c += 32) {
                 if (!mine()) continue;
                 const int f = f0 + c;
@@ -385,7 +402,8 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     if ((lane & 7) == 0) {
                         a.ssq_out[(size_t)(m0 + r) * a.ssq_out_slots + f / 32] = ss;
                         if (f + 32 >= a.N)                            // the slots past the last 32 features
-                            for (int q = f / 32 + 1; q < a.ssq_out_slots; ++q) a.ssq_out[(size_t)(m0 + r) * a.ssq_out_slots + q] = 0.f;
+    #pragma unroll 1
+                        for (int q = f / 32 + 1; q < a.ssq_out_slots; ++q) a.ssq_out[(size_t)(m0 + r) * a.ssq_out_slots + q] = 0.f;
                     }
                 });
             }
@@ -402,6 +420,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     if (page < 0 || page >= a.n_pages) { set_status(a.status, TASC_ENOKV); page = -1; }
                 }
             }
+#pragma unroll 1
             for (int hc = 0; hc < BNW && f0 + hc < a.N; hc += hd) {
                 const int fh = f0 + hc;                               // first feature of this head
                 if (fh < qd + kvd) {
@@ -409,6 +428,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     const bool is_q = fh < qd;
                     const long long kdst = !is_q && pos >= 0 && page >= 0
                         ? (long long)((((size_t)page * a.n_kv + (fh - qd) / hd) * a.page_size + pos % a.page_size) * hd) : -1ll;
+#pragma unroll 1
                     for (int jj = 0; jj < half; jj += 32) {
                         if (!mine()) continue;
                         float lo[32], hi[32];
@@ -442,6 +462,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     // a value head
                     const long long vdst = pos >= 0 && page >= 0
                         ? (long long)((((size_t)page * a.n_kv + (fh - qd - kvd) / hd) * a.page_size + pos % a.page_size) * hd) : -1ll;
+#pragma unroll 1
                     for (int c = 0; c < hd; c += 32) {
                         if (!mine()) continue;
                         float v[32];
@@ -459,6 +480,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             // the row's largest logit in this tile (smallest id on ties), merged across tiles by an atomic max on
             // the packed (value, id) word
             uint32_t bk = 0u, bi = 0xFFFFFFFFu;
+#pragma unroll 1
             for (int c = 0; c < BNW && f0 + c < a.N; c += 32) {
                 if (!mine()) continue;
                 float v[32];
@@ -486,7 +508,8 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 #endif
         const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
         const uint32_t acc_empty0 = PAIR ? cluster_map(bar_acc_empty, 0u) : bar_acc_empty;      // the MMAs are issued by the even CTA
-        if (S == 1) {
+        if (!SPLIT) {
+#pragma unroll 1
             for (int j = 0; j < my_tiles; ++j) {
                 const int b = j & 1;
                 bool ok = wait_or_fail<PAIR>(bar_acc_full + 8u * b, ((uint32_t)(j >> 1)) & 1u, failed);
@@ -511,6 +534,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             g_tb = global_ns();
 #endif
             tc_fence_after();
+#pragma unroll 1
             for (int c = 32 * wq; c < BNW; c += 64) {
                 float v[32];
                 if (ok) {
@@ -524,7 +548,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             tc_fence_before();
         }
     }
-    if (S > 1) {
+    if (SPLIT) {
         // every CTA's partial tile is in its shared memory (release / acquire at cluster scope)
 #ifdef TASC_TIMELINE
         g_tc = global_ns();
@@ -556,12 +580,13 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 }
             }
             const int n_own = __popc(own_mask);
+#pragma unroll 1
             for (int idx = warp; idx < n_own * 4; idx += EPI_WARPS) {
                 const int jc = idx >> 2, q = idx & 3;
                 const int chunk = __fns(own_mask, 0, jc + 1);         // the jc-th chunk of the mask
                 const uint32_t off = (uint32_t)((q * 32 + (lane >> 3)) * XLD + chunk * 32 + 4 * (lane & 7)) * 4u;
                 float* dst = fin + (size_t)(q * 32 + (lane >> 3)) * FLD + jc * 32 + 4 * (lane & 7);
-#pragma unroll
+#pragma unroll 1
                 for (int ib = 0; ib < 8; ib += 2) {                   // rows lane / 8 + 4 i, two i at a time: 2 S reads in flight
                     float4 u[8][2];
 #pragma unroll
@@ -611,7 +636,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 #endif
 }
 
-template <int EPI, bool PAIR>
+template <int EPI, bool PAIR, bool SPLIT>
 tasc_status prepare_wide() {
     static std::mutex mu;
     static bool attr_done[64] = {false};
@@ -620,16 +645,16 @@ tasc_status prepare_wide() {
     if (dev < 0 || dev >= 64) return TASC_EINVAL;
     std::lock_guard<std::mutex> lk(mu);
     if (!attr_done[dev]) {
-        TASC_CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel<EPI, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
+        TASC_CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel<EPI, PAIR, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
         attr_done[dev] = true;
     }
     return TASC_OK;
 }
 
-template <int EPI, bool PAIR>
+template <int EPI, bool PAIR, bool SPLIT>
 tasc_status launch_wide(const CUtensorMap* tmW, const CUtensorMap* tmX, const FusedArgs& a, const FusedPlan& p, int kind,
                         cudaStream_t stream) {
-    tasc_status pst = prepare_wide<EPI, PAIR>();
+    tasc_status pst = prepare_wide<EPI, PAIR, SPLIT>();
     if (pst != TASC_OK) return pst;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)p.grid, 1, 1);
@@ -641,7 +666,7 @@ tasc_status launch_wide(const CUtensorMap* tmW, const CUtensorMap* tmX, const Fu
     at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[n].val.programmaticStreamSerializationAllowed = 1;
     ++n;
-    if (PAIR || p.S > 1) {
+    if (PAIR || SPLIT) {
         at[n].id = cudaLaunchAttributeClusterDimension;
         at[n].val.clusterDim.x = PAIR ? 2u : (unsigned)p.S;
         at[n].val.clusterDim.y = 1;
@@ -651,14 +676,14 @@ tasc_status launch_wide(const CUtensorMap* tmW, const CUtensorMap* tmX, const Fu
     cfg.attrs = at;
     cfg.numAttrs = n;
     ProfScope ps(kind, stream);
-    TASC_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_wide_kernel<EPI, PAIR>, *tmW, *tmX, a));
+    TASC_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_wide_kernel<EPI, PAIR, SPLIT>, *tmW, *tmX, a));
     return TASC_OK;
 }
 
 // Clusters of S CTAs with `smem` bytes each that the device can hold at once (0 if the query fails).
 template <int EPI>
 int wide_clusters(int S, int smem) {
-    if (prepare_wide<EPI, false>() != TASC_OK) return 0;
+    if (prepare_wide<EPI, false, true>() != TASC_OK) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)S, 1, 1);
     cfg.blockDim = dim3(THREADS, 1, 1);
@@ -671,7 +696,7 @@ int wide_clusters(int S, int smem) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_wide_kernel<EPI, false>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_wide_kernel<EPI, false, true>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
     return n;
 }
 
@@ -775,11 +800,17 @@ tasc_status launch_gemm_wide(int epi, const CUtensorMap* tmW, const CUtensorMap*
     a.num_kb = p.num_kb; a.BN = p.BN; a.TB = p.TB; a.TBL = p.TBL; a.stages = p.stages; a.pair = 1; a.data_bytes = p.data_bytes;
     a.BNW = p.BNW; a.n_ft = p.out_tiles; a.n_tt = p.m_tiles;
     if (a.n_tt > MAX_TT) a.seq_rows = nullptr;
-    switch (epi) {
-        case EPI_QKV:    return p.cta_pair ? launch_wide<EPI_QKV, true>(tmW, tmX, a, p, K_GEMM, stream) : launch_wide<EPI_QKV, false>(tmW, tmX, a, p, K_GEMM, stream);
-        case EPI_RESID:  return p.cta_pair ? launch_wide<EPI_RESID, true>(tmW, tmX, a, p, K_GEMM, stream) : launch_wide<EPI_RESID, false>(tmW, tmX, a, p, K_GEMM, stream);
-        case EPI_SWIGLU: return p.cta_pair ? launch_wide<EPI_SWIGLU, true>(tmW, tmX, a, p, K_GEMM, stream) : launch_wide<EPI_SWIGLU, false>(tmW, tmX, a, p, K_GEMM, stream);
-        case EPI_LM:     return p.cta_pair ? launch_wide<EPI_LM, true>(tmW, tmX, a, p, K_GEMM_LM, stream) : launch_wide<EPI_LM, false>(tmW, tmX, a, p, K_GEMM_LM, stream);
+    switch (epi) {                                                 // (gate/up and the LM head are never split: plan_wide)
+        case EPI_QKV:    return p.cta_pair ? launch_wide<EPI_QKV, true, false>(tmW, tmX, a, p, K_GEMM, stream)
+                              : p.S > 1    ? launch_wide<EPI_QKV, false, true>(tmW, tmX, a, p, K_GEMM, stream)
+                                           : launch_wide<EPI_QKV, false, false>(tmW, tmX, a, p, K_GEMM, stream);
+        case EPI_RESID:  return p.cta_pair ? launch_wide<EPI_RESID, true, false>(tmW, tmX, a, p, K_GEMM, stream)
+                              : p.S > 1    ? launch_wide<EPI_RESID, false, true>(tmW, tmX, a, p, K_GEMM, stream)
+                                           : launch_wide<EPI_RESID, false, false>(tmW, tmX, a, p, K_GEMM, stream);
+        case EPI_SWIGLU: return p.cta_pair ? launch_wide<EPI_SWIGLU, true, false>(tmW, tmX, a, p, K_GEMM, stream)
+                                           : launch_wide<EPI_SWIGLU, false, false>(tmW, tmX, a, p, K_GEMM, stream);
+        case EPI_LM:     return p.cta_pair ? launch_wide<EPI_LM, true, false>(tmW, tmX, a, p, K_GEMM_LM, stream)
+                                           : launch_wide<EPI_LM, false, false>(tmW, tmX, a, p, K_GEMM_LM, stream);
         default: return TASC_EINVAL;
     }
 }
