@@ -43,9 +43,9 @@ UNIT = "tokens/s"
 # layers and the LM head, per launch), keyed by (configuration, batch, k).  A figure is valid for the kernel sources whose
 # digest is stored with it; after any change of them `traffic` reads null.
 NCU_TRAFFIC = {
-    # configuration 4, B = 1, k = 6: the model cut to 2 and 4 layers (--layers), 208.5 and 416.8 MB in the layers' launch, so 2,916 MB
-    # at 28, and 467.2 MB in the LM head's (algorithmic: 1,557 MB per launch)
-    (4, 1, 6): {"bytes_per_launch": (208545152 + 26 * 104150016 + 467210240) / 2, "kernel_sha256_16": "641d0621fcad257a"},
+    # configuration 4, B = 1, k = 6: the model cut to 2 and 4 layers (--layers), 204.2 and 417.2 MB in the layers' launch, so 2,973 MB
+    # at 28, and 467.1 MB in the LM head's (algorithmic: 1,557 MB per launch)
+    (4, 1, 6): {"bytes_per_launch": (204227456 + 26 * 106471616 + 467145152) / 2, "kernel_sha256_16": "b3446930f10e99ba"},
 }
 
 
