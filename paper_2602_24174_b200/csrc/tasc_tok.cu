@@ -586,7 +586,7 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
                         if (lane == 0 && who) at = atomicAdd(cand.n, (unsigned int)__popc(who));
                         at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(who & ((1u << lane) - 1u));
                         if (in && at < CAND_MAX) cand.slots[at] = (uint32_t)(first + lane * 4 + q);
-                        full |= at >= CAND_MAX;
+                        full |= in && at >= CAND_MAX;              // (the counter has passed CAND_MAX: the next round sees the list as cut short)
                     }
                     if (__any_sync(0xFFFFFFFFu, full)) { c0 = n_chunks; break; }
                 }

@@ -3,9 +3,10 @@ candidates holds, ties of more n-grams than are looked for by their tokens, more
 documents too long for shared memory.  Bit-exact against the oracle, like tests/test_gpu_tasc_tok.py."""
 import numpy as np
 import pytest
+import torch
 
 from tests.gpu_harness import need_gpu
-from tests.test_gpu_tasc_tok import check_enrich, flat
+from tests.test_gpu_tasc_tok import check_enrich, flat, merges_as_tuples, to_dev
 
 
 @pytest.mark.gpu
@@ -41,3 +42,49 @@ def test_candidates_come_and_go(n_max):
     phrases = [r.integers(0, 30, r.integers(2, 7)).tolist() for _ in range(60)]
     docs = [sum((phrases[min(59, int(r.zipf(1.3)))] for _ in range(r.integers(1, 12))), []) for _ in range(1500)]
     check_enrich(b, *flat(docs), 30, 80, n_max)
+
+
+# (the hash of csrc/ngram_table.cuh: key_make(2), key_put, key_hash)
+def first_pair(x, y, cap):
+    """First pair of slots that the table of `cap` slots looks at for the bigrams (x[i], y[i])."""
+    x, y = x.astype(np.uint64), y.astype(np.uint64)
+    u = np.uint64
+    with np.errstate(over="ignore"):
+        h = (x | y << u(20)) * u(0x9E3779B97F4A7C15) ^ u(((1 << 63 | 2 << 56) + 0xD6E8FEB86659FD93) % (1 << 64))
+        h = (h ^ h >> u(32)) * u(0xD6E8FEB86659FD93)
+        h = (h ^ h >> u(29)) * u(0x9E3779B97F4A7C15)
+    return (h ^ h >> u(32)) & u(cap // 2 - 1)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("early", [1022, 1023, 1024, 1025])
+def test_a_list_that_is_just_full(early):
+    """The list of candidates holds 1,024.  All candidates lie in chunks of the table that one warp looks through in turn: `early` with
+    the same count, the last of them alone in its chunk, then the next-best n-gram, then the best.  Where the early ones are exactly
+    1,024, the two behind them have to be seen to be missing."""
+    b = need_gpu()
+    r = np.random.default_rng(17)
+    vocab, cap, chunk, warp = 2 ** 20 - 8, 2 ** 24, 128, 777
+    warps = 32 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert cap // chunk > 26 * warps + warp
+    # over four million windows of other n-grams, so that the table has 2^24 slots
+    filler = r.integers(0, vocab, (66, 1000), dtype=np.int64)
+    x, y = r.integers(0, vocab, (2, 16_000_000), dtype=np.int64)
+    pair = first_pair(x, y, cap)
+    turn, whose = np.divmod(pair // np.uint64(chunk // 2), np.uint64(warps))     # a chunk's place among its warp's, and the warp
+    # n-grams by chunk, one to a pair of slots that no other n-gram looks at first: all lie there
+    used = set(first_pair(filler[:, :-1].ravel(), filler[:, 1:].ravel(), cap).tolist())
+    chunks = [[] for _ in range(27)]
+    for i in np.flatnonzero((whose == warp) & (turn < 27)):
+        if int(pair[i]) not in used:
+            used.add(int(pair[i]))
+            chunks[int(turn[i])].append((int(x[i]), int(y[i])))
+    chosen = sum(chunks[:24], [])[:early - 1] + chunks[24][:1]
+    assert len(chosen) == early
+    next_best, best = chunks[25][0], chunks[26][0]
+    counts = [(best, 200), (next_best, 180)] + [(g, 160) for g in chosen]
+    docs = np.concatenate([np.tile(np.array(g, np.int32), n) for g, n in counts] + [np.tile(filler.astype(np.int32).ravel(), 67)])
+    lens = np.concatenate([np.full(sum(n for _, n in counts), 2), np.full(66 * 67, 1000)])
+    assert cap // 4 < (lens - 1).sum() <= cap // 2
+    merges, _, _ = b.tasc_tok_enrich(*to_dev(docs, np.concatenate([[0], np.cumsum(lens)])), vocab, 4, 2)
+    assert merges_as_tuples(merges) == [best, next_best, chosen[0], chosen[1]]
