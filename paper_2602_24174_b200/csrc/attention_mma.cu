@@ -199,8 +199,10 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // Page ids of this CTA's key range, staged once: the tile loads then need no dependent global read.
     const int page_size = TMA ? 16 : a.page_size;
     const int pg_lo = k_begin / page_size;
-    const int n_pg = n_tiles > 0 ? (k_end - 1) / page_size - pg_lo + 1 : 0;
+    int n_pg = n_tiles > 0 ? (k_end - 1) / page_size - pg_lo + 1 : 0;
     const bool pages_staged = TMA || n_pg <= MAX_STAGED_PAGES;
+    // (a sequence that is longer than its cache: no pages behind the staged ones either; the append reports it)
+    n_pg = min(n_pg, MAX_STAGED_PAGES);
     if (TMA && warp == 7) {
         if (lane < STAGES) mbar_init(smem_u32(&s_full[lane]), 1);
         fence_barrier_init();
@@ -240,7 +242,8 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             if (r == 0) mbar_expect_tx(bar, 2u * TILE_BYTES);
             int key = k_begin + tile * TKEYS + pg * 16;
             key = key < k_end ? key : k_end - 1;
-            int page = s_pages[key / 16 - pg_lo];
+            int page = key / 16 - pg_lo;
+            page = page < n_pg ? s_pages[page] : -1;
             page = page < 0 ? 0 : page;
             const int y = (page * a.n_kv + kh) * 16;
             constexpr int BOXB = (HD >= 64 ? 128 : 64) * 16;       // bytes of one box: 16 rows of at most 128 bytes

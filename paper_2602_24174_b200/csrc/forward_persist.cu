@@ -561,7 +561,8 @@ struct Cta {
         }
         __syncthreads();
         const Unit& q = sh().unit;
-        const int p0 = q.k0 >> a.page_shift, np = q.k1 > q.k0 ? ((q.k1 - 1) >> a.page_shift) - p0 + 1 : 0;
+        // (at most MAX_PAGES: a sequence that is longer than its cache has no pages behind them either; the append reports it)
+        const int p0 = q.k0 >> a.page_shift, np = q.k1 > q.k0 ? min(((q.k1 - 1) >> a.page_shift) - p0 + 1, MAX_PAGES) : 0;
         for (int i = threadIdx.x; i < np; i += NT) {
             int page = -1;
             if (p0 + i < a.max_pages) page = a.block_table[(size_t)q.b * a.max_pages + p0 + i];
@@ -579,7 +580,8 @@ struct Cta {
         const int p0 = q.k0 >> a.page_shift, c = threadIdx.x % CPR;
 #pragma unroll 1
         for (int key = lo + (int)threadIdx.x / CPR; key < hi; key += NT / CPR) {
-            int row = key < q.k1 ? sh().pg[(key >> a.page_shift) - p0] : -1;
+            const int pg = (key >> a.page_shift) - p0;
+            int row = key < q.k1 && pg < MAX_PAGES ? sh().pg[pg] : -1;
             const int bytes = row >= 0 ? 16 : 0;
             row = row >= 0 ? row + (key & (a.page_size - 1)) : 0;
             const int kr = key - kb;
