@@ -689,7 +689,7 @@ __device__ __forceinline__ bool warp_lookup(const OrderTable& t, Key key, CtxVal
 }
 
 __global__ void __launch_bounds__(DRAFT_THREADS)
-draft_kernel(const DeviceTables dt, const int32_t* __restrict__ tokens, int64_t stride, const int32_t* __restrict__ len,
+draft_kernel(const DeviceTables dt, const int32_t* tokens, int64_t stride, const int32_t* len,
              int k, uint32_t lam_num, uint32_t lam_den, int32_t* __restrict__ drafts, int hs_mask) {
     extern __shared__ int32_t dsm[];
     int32_t* h_tok = dsm;                                          // [hs] token or -1

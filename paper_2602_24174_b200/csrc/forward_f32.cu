@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
                 const int key = k0 + (lane >> 2);
                 const int pslot = (int)((unsigned)key / (unsigned)a.page_size);
                 int page = -1;
-                if (key < n_keys && pslot < a.max_pages) page = __ldg(a.block_table + (size_t)b * a.max_pages + pslot);
+                if (key < n_keys && pslot < a.max_pages) page = a.block_table[(size_t)b * a.max_pages + pslot];
                 const bool there = page >= 0 && page < a.n_pages;          // ids outside the pool read as zeros, never as memory
                 const uint32_t row = there ? (uint32_t)((page * a.n_kv + kvh) * a.page_size + key - pslot * a.page_size) : 0u;
                 // the values are on their way while the scores are worked out

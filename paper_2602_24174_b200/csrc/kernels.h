@@ -204,7 +204,9 @@ tasc_status launch_persist(PersistArgs a, const PersistPlan& p, cudaStream_t str
 void launch_gemm_f32(const float* X, const float* W, float* partials, int M, int N, int K,
                      unsigned long long* argmax, float* logits, cudaStream_t stream);
 
-// Launches a kernel that may be set up while the kernel before it in the stream still runs.  The kernel begins with griddep_wait().
+// Launches a kernel that may be set up while the kernel before it in the stream still runs.  The kernel begins with griddep_wait(), and
+// what a call is given (tokens, lengths, drafts, results of the kernel before) is read through pointers that are neither __restrict__
+// nor __ldg'ed: loads by the non-coherent path are for memory that nothing writes while the grid is there, and they may be moved up over the wait.
 template <typename... P, typename... A>
 inline cudaError_t launch_ahead(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
     cudaLaunchConfig_t cfg = {};

@@ -87,8 +87,8 @@ embed_norm_kernel(const T* __restrict__ embed, const int* __restrict__ row_tok, 
 // chunk*R .. limited to positions <= len-2), and the embedding of every row.  The RMS factor is applied by the
 // consumer GEMM, so the row leaves here as x * gain (hi, lo) plus its sum of squares.
 __global__ void __launch_bounds__(128)
-rows_embed_kernel(RowPlan rp, const int32_t* __restrict__ tokens, int64_t stride, const int32_t* __restrict__ len,
-                  const int32_t* __restrict__ stop_len, const int32_t* __restrict__ drafts, int R, int chunk, int vocab,
+rows_embed_kernel(RowPlan rp, const int32_t* tokens, int64_t stride, const int32_t* len,
+                  const int32_t* stop_len, const int32_t* drafts, int R, int chunk, int vocab,
                   int* status, const __nv_bfloat16* __restrict__ embed, const float* __restrict__ gain, float* __restrict__ x,
                   __nv_bfloat16* __restrict__ a_out, float* __restrict__ ssq, int ssq_slots, unsigned long long* argmax, int d,
                   int TB, unsigned long long* __restrict__ ssq_p, int n_stage, unsigned* __restrict__ zero, int n_zero) {
@@ -259,8 +259,8 @@ __global__ void fill_u64_kernel(unsigned long long* p, unsigned long long v, int
     if (i < n) p[i] = v;
 }
 
-__global__ void accept_kernel(const unsigned long long* __restrict__ argmax, RowPlan rp, const int32_t* __restrict__ drafts,
-                              const int32_t* __restrict__ forced, int32_t* tokens, int64_t stride, int32_t* len, int R,
+__global__ void accept_kernel(const unsigned long long* argmax, RowPlan rp, const int32_t* drafts,
+                              const int32_t* forced, int32_t* tokens, int64_t stride, int32_t* len, int R,
                               int32_t* n_accepted, int32_t* next_token, int32_t* target_tokens, long long* hist) {
     griddep_wait();
     // a warp per sequence, a lane per row: everything is requested together
