@@ -617,7 +617,8 @@ tasc_status prepare_inst() {
     return TASC_OK;
 }
 
-// Clusters of `splits` CTAs (ring depth `stages`) the device holds at once; 0 if the query fails.
+// Clusters of `splits` CTAs (ring depth `stages`) the device holds at once; 0 if the query fails.  (Both ways of loading: two CTAs per SM
+// by their registers with heads of 32 and 64, one with heads of 128.)
 template <int HD, int NS>
 int fit_inst(int splits, int stages) {
     if (prepare_inst<HD, NS, true>() != TASC_OK) return 0;
@@ -773,9 +774,12 @@ tasc_status launch_attention_mma(const float* qbuf, const __nv_bfloat16* k_pages
     a.status = status;
     a.n_slabs = (G + 15) / 16;
     a.by_R = SmallDiv(Rs); a.by_TB = SmallDiv(TB); a.by_splits = SmallDiv(n_splits); a.by_sub = SmallDiv(n_sub); a.by_hsplit = SmallDiv(g / hs);
-    // 16-token pages arrive as TMA boxes; any other page size, and caches of more pages than a CTA keeps the ids of, take the
-    // kernel with cp.async
-    const bool tma = page_size == 16 && (plan.tc || max_pages <= MAX_STAGED_PAGES);
+    // 16-token pages arrive as TMA boxes; any other page size, and key ranges of more pages than a CTA keeps the ids of, take the
+    // kernel with cp.async.  (By the cache's pages instead of the range's, caches of 17,000 tokens lost the boxes: a step of the
+    // 0.5B with 16 sequences behind 15,000 tokens 2977 -> 3062 us, of the 1.5B with 8 behind 16,000 3632 -> 3720, of the 135M with 5
+    // behind 300 698 -> 705.)
+    const int range_tiles = ((int)(((long long)max_pages * page_size + TKEYS - 1) / TKEYS) + n_splits - 1) / n_splits;      // of the longest sequence
+    const bool tma = page_size == 16 && (plan.tc || range_tiles <= MAX_STAGED_PAGES * 16 / TKEYS);
     CUtensorMap tmK, tmV;
     memset(&tmK, 0, sizeof(tmK));
     memset(&tmV, 0, sizeof(tmV));

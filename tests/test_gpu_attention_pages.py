@@ -40,3 +40,33 @@ def test_logits_do_not_depend_on_how_keys_are_loaded(hd):
     for page_size, pages in ((16, 1024), (16, 1025), (8, None), (32, None), (64, 3)):
         got = logits_of(hd, page_size, pages)
         assert np.abs(got - want).max() <= 5e-3, (page_size, pages)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("capacity", [17000, 8 * 1024 * 16, 8 * 1024 * 16 + 64])
+def test_long_caches_read_by_range(capacity):
+    """Caches of more pages than a CTA keeps the ids of: TMA boxes while each of eight key ranges has no more than 1,024 pages, cp.async
+    beyond; against pages of 32 tokens, which are never boxes.  (The same ranges and sums: the bound is for the second layer's keys.)"""
+    b = need_gpu()
+    k = 5
+    cfg = configs.shrunk(configs.get(1), n_layers=2, vocab=4096, n_docs=200)
+    gen = torch.Generator(device="cuda")
+    m = cfg.model
+    got = []
+    for page_size in (16, 32):
+        s = make_setup(replace(cfg, page_size=page_size, prompt_len=capacity), build_drafter=False, oracle_ngrams=False)
+        gen.manual_seed(3)
+        T = capacity // 32 * 32 + 32                                 # tokens of both caches
+        kv_tokens = torch.empty((2, 2, 2, T, m.n_kv_heads, m.head_dim), dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.5, generator=gen)
+        pool, bt, kv = s.model.new_kv(2, capacity)
+        pages = bt.shape[1]
+        for i in range(2):
+            x = kv_tokens[:, :, i, :pages * page_size].reshape(2, 2, pages, page_size, m.n_kv_heads, m.head_dim)
+            pool[:, :, bt[i].long()] = x.transpose(3, 4)
+        tokens = torch.randint(0, 4096, (2, capacity), generator=gen, device="cuda", dtype=torch.int32)
+        drafts = torch.randint(0, 4096, (2, k), generator=gen, device="cuda", dtype=torch.int32)
+        length = torch.tensor([capacity - k - 1, capacity // 2], dtype=torch.int32, device="cuda")
+        ws = s.model.new_workspace(2, k)
+        got.append(b.tasc_verify_step(s.model, kv, b.make_seqs(tokens, length), drafts, ws, want_logits=True)[3].cpu().numpy())
+        b.tasc_poll_status(ws)
+    assert np.abs(got[0] - got[1]).max() <= 5e-3
