@@ -727,6 +727,12 @@ AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ct
             for (int s = 1; s <= 8 && s <= n_tiles; ++s) {
                 int fit = fit_any(hd, nw, s, stages);
                 if (fit <= 0) fit = std::max(1, 148 / s);               // no device to ask: assume one CTA per SM
+                // Two CTAs to an SM: of clusters that just fit an empty chip, up to four find no room beside the CTAs that the kernel before
+                // still has there, and run behind the others.  A layer of the 0.5B and the 135M, us, by clusters (that fit), against the
+                // next best plan: 15,000 tokens 32 (33) 104.7, 81.6; 36 (37) 105.4, 73.7; 42 (45) 92.2, 83.4; 30 (33) 72.5, 66.8;
+                // 4,000 tokens 54 (56) 60.9, 47.3.  With more to spare they start together: 28 (33), 40 (45), 64 (71) and 48 (56) are the
+                // best plans there are.
+                if (s > 1 && fit * s > 148) fit = std::max(1, fit - 4);
                 const int waves = (groups + fit - 1) / fit;
                 const int tiles_cta = (n_tiles + s - 1) / s;
                 const float stall = di == 0 ? 0.f : 0.25f * t_tile;      // a shallow ring hides less latency
