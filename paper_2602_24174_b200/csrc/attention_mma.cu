@@ -21,6 +21,7 @@
 #include "kernels.h"
 
 #include <algorithm>
+#include <climits>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -181,7 +182,9 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // the range's 64-key tiles are dealt out evenly: every split gets floor or ceil of tiles / splits of them
     const int tiles_all = (total + TKEYS - 1) / TKEYS;
     const int t_base = a.by_splits.div(tiles_all), t_rem = tiles_all - t_base * a.splits;
-    const int n_tiles = t_base + (sp < t_rem ? 1 : 0);
+    // (No more keys than the staged pages hold where they are TMA boxes: the host sees to that for all that the cache can hold; a
+    // sequence that is longer than its cache is reported by the append.)
+    const int n_tiles = min(t_base + (sp < t_rem ? 1 : 0), TMA ? MAX_STAGED_PAGES * 16 / TKEYS : INT_MAX);
     const int k_begin = (sp * t_base + min(sp, t_rem)) * TKEYS;
     const int k_end = min(total, k_begin + n_tiles * TKEYS);
     const int n_slabs = a.n_slabs;
@@ -199,10 +202,8 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // Page ids of this CTA's key range, staged once: the tile loads then need no dependent global read.
     const int page_size = TMA ? 16 : a.page_size;
     const int pg_lo = k_begin / page_size;
-    int n_pg = n_tiles > 0 ? (k_end - 1) / page_size - pg_lo + 1 : 0;
+    const int n_pg = n_tiles > 0 ? (k_end - 1) / page_size - pg_lo + 1 : 0;
     const bool pages_staged = TMA || n_pg <= MAX_STAGED_PAGES;
-    // (a sequence that is longer than its cache: no pages behind the staged ones either; the append reports it)
-    n_pg = min(n_pg, MAX_STAGED_PAGES);
     if (TMA && warp == 7) {
         if (lane < STAGES) mbar_init(smem_u32(&s_full[lane]), 1);
         fence_barrier_init();
@@ -242,8 +243,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             if (r == 0) mbar_expect_tx(bar, 2u * TILE_BYTES);
             int key = k_begin + tile * TKEYS + pg * 16;
             key = key < k_end ? key : k_end - 1;
-            int page = key / 16 - pg_lo;
-            page = page < n_pg ? s_pages[page] : -1;
+            int page = s_pages[key / 16 - pg_lo];
             page = page < 0 ? 0 : page;
             const int y = (page * a.n_kv + kh) * 16;
             constexpr int BOXB = (HD >= 64 ? 128 : 64) * 16;       // bytes of one box: 16 rows of at most 128 bytes

@@ -138,11 +138,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     // this CTA's keys: the tiles are dealt out evenly over the splits
     const int total = pos0 + rows;
     const int tiles_all = (total + TK - 1) / TK, t_base = a.by_splits.div(tiles_all), t_rem = tiles_all - t_base * a.splits;
-    const int n_tiles = t_base + (sp < t_rem ? 1 : 0);
+    // (no more keys than the staged pages hold: a sequence that is longer than its cache is reported by the append)
+    const int n_tiles = min(t_base + (sp < t_rem ? 1 : 0), MAX_PAGES * PAGE / TK);
     const int k_begin = (sp * t_base + min(sp, t_rem)) * TK;
     const int k_end = min(total, k_begin + n_tiles * TK);
-    // (at most MAX_PAGES: a sequence that is longer than its cache has no pages behind them either; the append reports it)
-    const int pg_lo = k_begin / PAGE, n_pg = n_tiles > 0 ? min((k_end - 1) / PAGE - pg_lo + 1, MAX_PAGES) : 0;
+    const int pg_lo = k_begin / PAGE, n_pg = n_tiles > 0 ? (k_end - 1) / PAGE - pg_lo + 1 : 0;
     const int quarters = (G + 31) / 32;                          // TMEM lane quarters with rows: 2 softmax warps each
     const uint32_t arrivals = (uint32_t)quarters * 64u;
 
@@ -220,8 +220,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                     const int pg = lane / C::HB, h = lane % C::HB;
                     int key = k_begin + t * TK + pg * PAGE;
                     key = key < k_end ? key : k_end - 1;
-                    int page = key / PAGE - pg_lo;
-                    page = page < n_pg ? s_pages[page] : -1;
+                    int page = s_pages[key / PAGE - pg_lo];
                     page = page < 0 ? 0 : page;
                     tma_load_2d(base + h * (TK * 128) + pg * (PAGE * 128), is_v ? &tmV : &tmK, h * 64, (page * a.n_kv + kh) * PAGE, bar);
                 }

@@ -556,13 +556,13 @@ struct Cta {
             if (inside && first >= r.rows) total = 0;
             const int per = ((total + a.splits - 1) / a.splits + 15) / 16 * 16;
             r.k0 = min(total, r.sp * per);
-            r.k1 = min(total, r.k0 + per);
+            // (no more keys than MAX_PAGES pages hold: a sequence that is longer than its cache is reported by the append)
+            r.k1 = (int)min((long long)min(total, r.k0 + per), (long long)((r.k0 >> a.page_shift) + MAX_PAGES) << a.page_shift);
             sh().unit = r;
         }
         __syncthreads();
         const Unit& q = sh().unit;
-        // (at most MAX_PAGES: a sequence that is longer than its cache has no pages behind them either; the append reports it)
-        const int p0 = q.k0 >> a.page_shift, np = q.k1 > q.k0 ? min(((q.k1 - 1) >> a.page_shift) - p0 + 1, MAX_PAGES) : 0;
+        const int p0 = q.k0 >> a.page_shift, np = q.k1 > q.k0 ? ((q.k1 - 1) >> a.page_shift) - p0 + 1 : 0;
         for (int i = threadIdx.x; i < np; i += NT) {
             int page = -1;
             if (p0 + i < a.max_pages) page = a.block_table[(size_t)q.b * a.max_pages + p0 + i];
@@ -580,8 +580,7 @@ struct Cta {
         const int p0 = q.k0 >> a.page_shift, c = threadIdx.x % CPR;
 #pragma unroll 1
         for (int key = lo + (int)threadIdx.x / CPR; key < hi; key += NT / CPR) {
-            const int pg = (key >> a.page_shift) - p0;
-            int row = key < q.k1 && pg < MAX_PAGES ? sh().pg[pg] : -1;
+            int row = key < q.k1 ? sh().pg[(key >> a.page_shift) - p0] : -1;
             const int bytes = row >= 0 ? 16 : 0;
             row = row >= 0 ? row + (key & (a.page_size - 1)) : 0;
             const int kr = key - kb;
