@@ -781,11 +781,13 @@ tasc_status launch_attention_mma(const float* qbuf, const __nv_bfloat16* k_pages
     a.n_slabs = (G + 15) / 16;
     a.by_R = SmallDiv(Rs); a.by_TB = SmallDiv(TB); a.by_splits = SmallDiv(n_splits); a.by_sub = SmallDiv(n_sub); a.by_hsplit = SmallDiv(g / hs);
     // 16-token pages arrive as TMA boxes; any other page size, and key ranges of more pages than a CTA keeps the ids of, take the
-    // kernel with cp.async.  (By the cache's pages instead of the range's, caches of 17,000 tokens lost the boxes: a step of the
-    // 0.5B with 16 sequences behind 15,000 tokens 2977 -> 3062 us, of the 1.5B with 8 behind 16,000 3632 -> 3720, of the 135M with 5
-    // behind 300 698 -> 705.)
+    // kernel with cp.async.  So do 64-wide heads with one CTA per SM (the deep ring) in caches of more than 1,024 pages, which are
+    // there for long sequences.  Boxes / cp.async, us, such a step behind 20,000 tokens: 135M, 1 sequence 1508 / 1464, 7 2060 / 2016;
+    // 0.5B, 7 of 4 rows 1448 / 1412 (behind 560 of at most 17,000: 708 / 716).  Two CTAs per SM: 0.5B, 16 of 6 rows behind 15,000
+    // of 17,000 2977 / 3062.  128-wide heads: 1.5B, 1 sequence behind 20,000 2144 / 2182, 7 3529 / 3616.
     const int range_tiles = ((int)(((long long)max_pages * page_size + TKEYS - 1) / TKEYS) + n_splits - 1) / n_splits;      // of the longest sequence
-    const bool tma = page_size == 16 && (plan.tc || range_tiles <= MAX_STAGED_PAGES * 16 / TKEYS);
+    const bool tma = page_size == 16 && (plan.tc || max_pages <= MAX_STAGED_PAGES ||
+                                         ((hd == 128 || plan.stages <= 4) && range_tiles <= MAX_STAGED_PAGES * 16 / TKEYS));
     CUtensorMap tmK, tmV;
     memset(&tmK, 0, sizeof(tmK));
     memset(&tmV, 0, sizeof(tmV));

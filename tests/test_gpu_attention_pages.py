@@ -43,13 +43,14 @@ def test_logits_do_not_depend_on_how_keys_are_loaded(hd):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("capacity", [17000, 8 * 1024 * 16, 8 * 1024 * 16 + 64])
-def test_long_caches_read_by_range(capacity):
-    """Caches of more pages than a CTA keeps the ids of: TMA boxes while each of eight key ranges has no more than 1,024 pages, cp.async
-    beyond; against pages of 32 tokens, which are never boxes.  (The same ranges and sums: the bound is for the second layer's keys.)"""
+@pytest.mark.parametrize("index,capacity", [(1, 17000), (4, 17000), (4, 8 * 1024 * 16), (4, 8 * 1024 * 16 + 64)])
+def test_long_caches_read_by_range(index, capacity):
+    """Caches of more pages than a CTA keeps the ids of.  With heads of 128 TMA boxes while each of eight key ranges has no more than 1,024
+    pages, cp.async beyond; against pages of 32 tokens, which are never boxes.  (The same ranges and sums: the bound is for the second
+    layer's keys.)"""
     b = need_gpu()
     k = 5
-    cfg = configs.shrunk(configs.get(1), n_layers=2, vocab=4096, n_docs=200)
+    cfg = configs.shrunk(configs.get(index), n_layers=2, vocab=4096, n_docs=200)
     gen = torch.Generator(device="cuda")
     m = cfg.model
     got = []
