@@ -36,10 +36,10 @@ constexpr int LEN_BITS = 3;
 // while all others still read the other.
 struct TokState {
     unsigned long long used[2];                  // slots claimed
+    unsigned long long first[2];                 // first position of the n-grams that tie, and the slot of the one that is there
     unsigned int n_cand[2];                      // entries of the candidates' list
     int rebuild;                                 // the round before which the table has to be counted again (0: the first)
     int n_merges, status;
-    unsigned int first[2];                       // first position of the n-grams that tie
     unsigned int bar;                            // arrivals at the grid barrier
 };
 // The best n-gram of a part of the table: its rank (reward and length), one slot that has it, and how many have it.
@@ -142,14 +142,17 @@ __device__ __forceinline__ int tok_change(const TokArgs& a, const Key& key, int 
     a.st->rebuild = round + 1;                   // the table is full: all is counted again before the next round
     return 0;
 }
-// Rank of a window's n-gram while no window is being added or taken out.
-__device__ __forceinline__ unsigned long long tok_rank_of(const TokArgs& a, const Key& key) {
+// Rank and slot of a window's n-gram while no window is being added or taken out.
+__device__ __forceinline__ unsigned long long tok_rank_of(const TokArgs& a, const Key& key, uint32_t& slot) {
     Probe p(a, key);
     for (uint64_t probe = 0; probe <= p.mask; ++probe, p.next()) {
         const KeyPair v = tok_pair(a, p.pair);
 #pragma unroll
         for (int i = 0; i < 2; ++i)
-            if (v.k[i].x == key.lo && v.k[i].y == key.hi) return tok_rank(__ldcg(a.words + 2 * p.pair + i));
+            if (v.k[i].x == key.lo && v.k[i].y == key.hi) {
+                slot = (uint32_t)(2 * p.pair + i);
+                return tok_rank(__ldcg(a.words + slot));
+            }
         if (v.k[1].x == 0 && v.k[1].y == 0) break;
     }
     return 0ull;
@@ -423,7 +426,7 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
         }
         return lo;
     };
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.st->first[0] = a.st->first[1] = 0xFFFFFFFFu;
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.st->first[0] = a.st->first[1] = ~0ull;
     const int64_t own = (int64_t)blockIdx.x * TOK_WARPS + warp;           // (neighbouring documents: one CTA's)
     const int64_t s = a.offsets[doc_at(own * a.T / nw)], e = own + 1 == nw ? a.T : a.offsets[doc_at((own + 1) * a.T / nw)];
     const uint64_t n_chunks = a.cap >> CHUNK_BITS;
@@ -603,19 +606,21 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
         }
         if (tie) {
             // ---- several: the one with the first position
-            unsigned int* first = &a.st->first[n_ties & 1];
-            if (blockIdx.x == 0 && threadIdx.x == 0) a.st->first[~n_ties & 1] = 0xFFFFFFFFu;
+            // (its slot comes along, so that its tokens are read from the table and the documents may change behind the next barrier)
+            unsigned long long* first = &a.st->first[n_ties & 1];
+            auto found_before = [&](int64_t p) { return (int64_t)__shfl_sync(0xFFFFFFFFu, (unsigned int)(*(volatile unsigned long long*)first >> 32), 0) <= p; };
+            if (blockIdx.x == 0 && threadIdx.x == 0) a.st->first[~n_ties & 1] = ~0ull;
             if (n_tied) {
                 // by their tokens, 512 positions at a time
                 for (int64_t p = s & ~3ll; p < e; p += 512) {
-                    if ((int64_t)__shfl_sync(0xFFFFFFFFu, *(volatile unsigned int*)first, 0) <= p) break;
+                    if (found_before(p)) break;
                     int4 x[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int64_t q = p + u * 128 + 4 * lane;
                         x[u] = q < e ? *reinterpret_cast<const int4*>(a.cur + q) : make_int4(-1, -1, -1, -1);
                     }
-                    unsigned int at = 0xFFFFFFFFu;
+                    unsigned int at = 0xFFFFFFFFu, slot = 0u;
                     for (int i = 0; i < n_tied; ++i) {
                         const int f = (int)key_get(sh.tied_key[i], 0);
 #pragma unroll
@@ -627,30 +632,31 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
                                 if (y[j] != f || q < s || q >= e || q >= (int64_t)at || (int)a.rem[q] < n - 1) continue;
                                 bool hit = true;
                                 for (int k = 1; hit && k < n; ++k) hit = a.cur[q + k] == (int)key_get(sh.tied_key[i], k);
-                                if (hit) at = (unsigned int)q;
+                                if (hit) { at = (unsigned int)q; slot = sh.tied_slot[i]; }
                             }
                         }
                     }
-                    at = __reduce_min_sync(0xFFFFFFFFu, at);
-                    if (at != 0xFFFFFFFFu) {
-                        if (lane == 0) atomicMin(first, at);
+                    const unsigned int best_at = __reduce_min_sync(0xFFFFFFFFu, at);
+                    if (best_at != 0xFFFFFFFFu) {
+                        if (at == best_at) atomicMin(first, ((unsigned long long)at << 32) | slot);
                         break;
                     }
                 }
             } else
             for (int64_t c = s; c < e; c += 32) {
                 // (one lane's reading decides for all: the value changes meanwhile)
-                if ((int64_t)__shfl_sync(0xFFFFFFFFu, *(volatile unsigned int*)first, 0) <= c) break;
+                if (found_before(c)) break;
                 const int64_t i = c + lane;
                 bool hit = false;
+                uint32_t slot = 0u;
                 if (i < e && a.cur[i] >= 0 && (int)a.rem[i] >= n - 1) {
                     Key key = key_make(n);
                     for (int j = 0; j < n; ++j) key_put(key, j, (uint32_t)a.cur[i + j]);
-                    hit = tok_rank_of(a, key) == best.rank;
+                    hit = tok_rank_of(a, key, slot) == best.rank;
                 }
                 const uint32_t hits = __ballot_sync(0xFFFFFFFFu, hit);
                 if (hits) {
-                    if (lane == 0) atomicMin(first, (unsigned int)(c + __ffs(hits) - 1));
+                    if (lane == __ffs(hits) - 1) atomicMin(first, ((unsigned long long)i << 32) | slot);
                     break;
                 }
             }
@@ -659,12 +665,13 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
         }
         if (threadIdx.x < MAX_N) {
             const int j = threadIdx.x;
-            Key k = {0ull, 0ull};
-            int64_t at = 0;
-            if (tie) at = *(volatile unsigned int*)&a.st->first[~n_ties & 1];
-            else if (listed) k = sh.tied_key[0];
-            else { const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(a.keys) + best.slot); k = Key{v.x, v.y}; }
-            const int t = j >= n ? -1 : tie ? __ldcg(a.cur + at + j) : (int)key_get(k, j);
+            Key k = sh.tied_key[0];
+            if (tie || !listed) {
+                const uint32_t slot = tie ? (uint32_t)*(volatile unsigned long long*)&a.st->first[~n_ties & 1] : best.slot;
+                const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(a.keys) + slot);
+                k = Key{v.x, v.y};
+            }
+            const int t = j < n ? (int)key_get(k, j) : -1;
             sh.n = n;
             sh.tok[j] = t;
             if (blockIdx.x == 0) a.merges[(size_t)n_merges * MAX_N + j] = t;
@@ -674,9 +681,8 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
         // ---- its documents: listed, and rewritten once every CTA has its n-gram; those that the list has no room for in another turn
         const int t0 = sh.tok[0];
         int claimed = 0;
-        // (A tie's n-gram is read from a document, which has to stay as it is until every CTA has read it; behind a look through the table
-        // all CTAs are past what they read of it.)
-        for (bool passed = !listed && !tie, more = true; more;) {
+        // (Behind a look through the table, and behind a tie, all CTAs are past what they read of it and of the documents.)
+        for (bool passed = !listed || tie, more = true; more;) {
             for (int64_t p = s & ~3ll; p < e; p += 512) {
                 int4 x[4];
 #pragma unroll
@@ -715,10 +721,6 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
             const int n_hits = min(sh.n_hits, HIT_MAX);
             // while the barrier is on its way the warps work on their first documents
             if (!passed) tok_arrive(a.st, epoch);
-            if (tie && !passed) {
-                if (!tok_wait(a.st, epoch, sh)) return;
-                passed = true;
-            }
             for (;;) {
                 int slot = 0;
                 if (lane == 0) slot = atomicAdd(&sh.next_hit, 1);
