@@ -747,7 +747,10 @@ AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ct
                 const float crowd = groups * s > 128 ? 1.5f : 0.f;
                 // every head group re-reads its KV head's keys: L2 traffic, about 0.1 us per extra pass over a tile
                 const float reread = 0.1f * tiles_cta * (float)(g / hs - 1) / (float)std::max(1, g / hs);
-                const float cost = waves * (1.7f + loop) + merge + crowd + reread;
+                // Every wave merges, and one that does not begin beside the kernel before takes a microsecond more to start.  (With one merge
+                // for all and 1.7 us for each, 56 to 128 sequences were split into several waves: a layer of the 135M, 64 x 6 rows,
+                // 1,024 tokens of cache, 58.2 us in 4 splits against 50.8 whole, and behind 170 of them 49.6 against 36.2.)
+                const float cost = waves * (1.7f + loop + merge) + (waves - 1) * 1.0f + crowd + reread;
                 if (cost < best_cost - 1e-6f) { best_cost = cost; best = AttnPlan{s, stages, hs, 0, cost}; }
             }
         }

@@ -580,7 +580,9 @@ bool plan_attention_tc(int B, int n_kv, int hd, int g, int rows, int max_ctx, in
         if (fit <= 0) continue;
         const int waves = (groups + fit - 1) / fit;
         const float tiles = 0.5f * (float)((tiles_all + s - 1) / s + (tiles_34 + s - 1) / s);
-        const float cost = waves * (T0 + tiles * per_tile) + (s > 1 ? 0.5f + 0.25f * s : 0.f) + (groups * s > 128 ? 3.0f : 0.f);
+        // (merges and later waves as in the other kernel's plan: a layer of the 1.5B, 80 x 5 rows, 1,024 tokens of cache, 148.9 us whole
+        // and 153.4 in 2 splits, 121.7 and 132.1 behind 170 of them; 48 x 3 rows, 4,096 tokens 137.8 whole, 137.9 in 4, 82.6 and 98.3 behind 680)
+        const float cost = waves * (T0 + tiles * per_tile + (s > 1 ? 0.5f + 0.25f * s : 0.f)) + (waves - 1) * 1.0f + (groups * s > 128 ? 3.0f : 0.f);
         if (cost < best_cost - 1e-6f) { best_cost = cost; best = s; }
     }
     if (!best) return false;
