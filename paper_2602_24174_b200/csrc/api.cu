@@ -261,11 +261,15 @@ tasc_status forward_f32(const tasc_model* m, const tasc_kv* kv, const Workspace&
 //      96    965 / 898      1052 / 1042
 // (270 - 380, 560 and 1,071 keys).  The one kernel's time hardly changes between 17 and 32 rows and between 33 and 64 (blocks of
 // 32); a generation replays, so 17 to 32 rows are not its (plan_persist).
-// 33 to 64 rows of the 135M, enqueued, since the five kernels have shorter code and token tiles of 16 rows:
-//     48 rows    150 keys 723, 782    300 keys 748, 789    500 keys 759, 836          35 rows, 300 keys 721, 780
-//     64 rows    150 keys 686, 787    480 keys 751, 835    prefill of 40 / 60 tokens 651 / 632, 684 / 694
-// so there it keeps the verify steps of caches of up to PERSIST_BLOCKS_CTX tokens only, where the difference is smallest and which the
-// tests of the one-kernel layers are about.
+// 33 to 64 rows of the 135M, since the five kernels have shorter code and token tiles of 16 rows:
+//     rows   keys    five kernels   one kernel            rows   keys    five kernels   one kernel
+//      35     40      675 / 599      735 / 728              64     40      659 / 600      748 / 741
+//            150      689 / 617      773 / 768                    150      681 / 620      795 / 789
+//            300      713 / 642      782 / 776                    300      700 / 650      801 / 795
+//      48    150      721 / 635      786 / 780                    480      751            835
+//            300      738 / 651      790 / 783           prefill of 40 / 60 tokens       651 / 632, 684 / 694
+// so the five kernels are the faster ones at every size, by 6 to 14 % enqueued and 16 to 22 % replayed.  Verify steps in caches of up to
+// PERSIST_BLOCKS_CTX tokens are still the one kernel's: nothing else reaches its blocks of 32 rows, and no time speaks for it.
 constexpr int PERSIST_BLOCKS_CTX = 352;
 // Its attention has at most one unit per SM and 12 key ranges, so the bytes of a unit's keys are bounded too, by 512 keys of 64:
 //     1.5B, 7 rows    1,500 keys 1235 / 1155, 1160 / 1150   3,000 (250 per unit) 1357 / 1273, 1296 / 1288   3,600 1340 / 1266, 1357 / 1348

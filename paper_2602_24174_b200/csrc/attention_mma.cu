@@ -701,14 +701,17 @@ AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ct
     // alone, and 2.5 us to start, a step of the 0.5B with 8 sequences x 6 rows behind 300 keys took 823 us instead of 793, with 4 x 6
     // behind 600 keys 725 instead of 694.)
     const int n_tiles = std::max(1, ((max_ctx * 3) / 4 + TKEYS - 1) / TKEYS), n_all = std::max(1, (max_ctx + TKEYS - 1) / TKEYS);
-    // Measured (microseconds): one iteration of a warp group over a 64-key tile, and the time the SM's mma.sync
-    // pipes need per tile and 16-row slab when all warps have work (the lower bound once several groups run).
+    // Microseconds: one iteration of a warp group over a 64-key tile, and the time the SM's mma.sync pipes need per tile and
+    // 16-row slab when all warps have work (the lower bound once several groups run).  The ones of 128-wide heads are weighed by whole
+    // steps: timed alone a tile takes 2.0 and 0.6, which chooses 77 of 853 plans otherwise.  A layer of the 1.5B, 2.0 and 0.6 / 1.2 and
+    // 0.65: 8 x 3 rows, 3,200 tokens of cache 50.6 / 49.2, 32 x 3 rows, 1,120 tokens 63.6 / 61.6 (tcgen05 instead of this kernel), 6 x 2
+    // rows, 640 tokens 37.8 / 37.2, 4 x 9 rows, 320 tokens 43.1 / 43.7; the others within 1.5 %.
     const float t_tile = hd >= 128 ? 1.2f : (hd >= 64 ? 1.3f : 0.8f);
     const float t_pipe = hd >= 128 ? 0.65f : (hd >= 64 ? 0.3f : 0.15f);
     AttnPlan best = {1, 2, g, 0, 1e30f};
     float best_cost = 1e30f;
-    // Candidates: all g heads of a KV head in one CTA; and, for few sequences with 128-wide heads (where one warp needs
-    // 2 us per key tile), the largest share of the heads whose rows still fill a single 16-row slab.  (Measured: on the
+    // Candidates: all g heads of a KV head in one CTA; and, for few sequences with 128-wide heads (where a warp's chain over a key
+    // tile is long), the largest share of the heads whose rows still fill a single 16-row slab.  (Measured: on the
     // 1.5B shape at one sequence 2 of 6 heads per CTA shorten the step by 4 %; 64-wide heads and larger batches lose.)
     int hs_slab = g;
     while (hs_slab > 1 && (g % hs_slab || hs_slab * rows > 16)) --hs_slab;

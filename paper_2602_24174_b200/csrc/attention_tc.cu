@@ -346,39 +346,39 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
             for (int t = 0; n_tiles > 0 && t <= n_tiles; ++t) {
                 float al = 0.f;
                 if (t < n_tiles) {
-                wait(bar_s_full + 8u * (t & 1), (uint32_t)(t >> 1) & 1u);
+                    wait(bar_s_full + 8u * (t & 1), (uint32_t)(t >> 1) & 1u);
 #ifdef TASC_TIMELINE
-                if (t == 0) log_at_exit.td = global_ns();
+                    if (t == 0) log_at_exit.td = global_ns();
 #endif
-                tc_fence_after();
+                    tc_fence_after();
 #pragma unroll
-                for (int c = 0; c < SC; c += 32) {
-                    uint32_t r[32];
-                    tmem_ld32(lane_base + C::S_COL + (uint32_t)((t & 1) * TK + half * SC + c), r);
-                    tmem_ld_wait();
+                    for (int c = 0; c < SC; c += 32) {
+                        uint32_t r[32];
+                        tmem_ld32(lane_base + C::S_COL + (uint32_t)((t & 1) * TK + half * SC + c), r);
+                        tmem_ld_wait();
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) s[c + e] = __uint_as_float(r[e]);
-                }
-                tc_fence_before();
-                mbar_arrive(bar_s_empty + 8u * (t & 1));
-                const int k0 = k_begin + t * TK + half * SC;
-                if (k0 + SC - 1 > lim) {
+                        for (int e = 0; e < 32; ++e) s[c + e] = __uint_as_float(r[e]);
+                    }
+                    tc_fence_before();
+                    mbar_arrive(bar_s_empty + 8u * (t & 1));
+                    const int k0 = k_begin + t * TK + half * SC;
+                    if (k0 + SC - 1 > lim) {
 #pragma unroll
-                    for (int e = 0; e < SC; ++e) if (k0 + e > lim) s[e] = -INFINITY;
-                }
-                float m4[4] = {s[0], s[1], s[2], s[3]};          // (four chains: a warp has its scheduler nearly to itself)
+                        for (int e = 0; e < SC; ++e) if (k0 + e > lim) s[e] = -INFINITY;
+                    }
+                    float m4[4] = {s[0], s[1], s[2], s[3]};          // (four chains: a warp has its scheduler nearly to itself)
 #pragma unroll
-                for (int e = 4; e < SC; ++e) m4[e & 3] = fmaxf(m4[e & 3], s[e]);
-                const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-                s_max[t & 1][half][rho] = mx;
-                asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory");      // the quarter's two warps
-                const float mn = fmaxf(m_run, fmaxf(mx, s_max[t & 1][half ^ 1][rho])), mu = mn == -INFINITY ? 0.f : mn;
-                al = ex2(m_run - mu);                            // 0 while nothing was visible
-                m_run = mn;
-                float p4[4] = {0.f, 0.f, 0.f, 0.f};
+                    for (int e = 4; e < SC; ++e) m4[e & 3] = fmaxf(m4[e & 3], s[e]);
+                    const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+                    s_max[t & 1][half][rho] = mx;
+                    asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory");      // the quarter's two warps
+                    const float mn = fmaxf(m_run, fmaxf(mx, s_max[t & 1][half ^ 1][rho])), mu = mn == -INFINITY ? 0.f : mn;
+                    al = ex2(m_run - mu);                            // 0 while nothing was visible
+                    m_run = mn;
+                    float p4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int e = 0; e < SC; ++e) { s[e] = ex2(s[e] - mu); p4[e & 3] += s[e]; }
-                l_run = l_run * al + ((p4[0] + p4[1]) + (p4[2] + p4[3]));
+                    for (int e = 0; e < SC; ++e) { s[e] = ex2(s[e] - mu); p4[e & 3] += s[e]; }
+                    l_run = l_run * al + ((p4[0] + p4[1]) + (p4[2] + p4[3]));
                 }
                 if (t > 0) add_o(t - 1);                         // (P of tile t - 1 has been used: its place is free)
                 if (t == n_tiles) break;

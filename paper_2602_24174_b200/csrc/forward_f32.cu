@@ -270,86 +270,86 @@ __global__ void __launch_bounds__(THREADS, 1) forward_f32_kernel(const __grid_co
                 return;
             }
         } else {
-        cluster_wait();
+            cluster_wait();
 #ifdef TASC_TIMELINE
-        TL_END(tl_tag);
+            TL_END(tl_tag);
 #endif
-        float* kp = a.kv_pool + (size_t)l * 2 * a.kv_half;
-        float* vp = kp + a.kv_half;
-        // ---- attention: unit = (token row, query head)
-        const int n_units = M * a.n_q, g = a.n_q / a.n_kv, sub = warp / UNIT_WARPS, sw = warp % UNIT_WARPS;
+            float* kp = a.kv_pool + (size_t)l * 2 * a.kv_half;
+            float* vp = kp + a.kv_half;
+            // ---- attention: unit = (token row, query head)
+            const int n_units = M * a.n_q, g = a.n_q / a.n_kv, sub = warp / UNIT_WARPS, sw = warp % UNIT_WARPS;
 #pragma unroll 1
-        for (int u0 = cta; u0 < n_units; u0 += CTAS * (WARPS / UNIT_WARPS)) {
-            const int u = u0 + sub * CTAS;
-            const int m = u < n_units ? a.by_nq.div(u) : 0, h = u < n_units ? u - m * a.n_q : 0, b = a.by_R.div(m), kvh = h / g;
-            const int n_keys = u < n_units ? s_pos[m] + 1 : 0;   // none for a row that is not in use
-            const float* q = a.q + (size_t)m * qd + h * hd;
-            float acc[NJ], mx = -INFINITY, den = 0.f;
+            for (int u0 = cta; u0 < n_units; u0 += CTAS * (WARPS / UNIT_WARPS)) {
+                const int u = u0 + sub * CTAS;
+                const int m = u < n_units ? a.by_nq.div(u) : 0, h = u < n_units ? u - m * a.n_q : 0, b = a.by_R.div(m), kvh = h / g;
+                const int n_keys = u < n_units ? s_pos[m] + 1 : 0;   // none for a row that is not in use
+                const float* q = a.q + (size_t)m * qd + h * hd;
+                float acc[NJ], mx = -INFINITY, den = 0.f;
 #pragma unroll
-            for (int j = 0; j < NJ; ++j) acc[j] = 0.f;
+                for (int j = 0; j < NJ; ++j) acc[j] = 0.f;
 #pragma unroll 1
-            for (int k0 = sw * KEYS; k0 < n_keys; k0 += UNIT_WARPS * KEYS) {
-                const int key = k0 + (lane >> 2);
-                const int pslot = (int)((unsigned)key / (unsigned)a.page_size);
-                int page = -1;
-                if (key < n_keys && pslot < a.max_pages) page = a.block_table[(size_t)b * a.max_pages + pslot];
-                const bool there = page >= 0 && page < a.n_pages;          // ids outside the pool read as zeros, never as memory
-                const uint32_t row = there ? (uint32_t)((page * a.n_kv + kvh) * a.page_size + key - pslot * a.page_size) : 0u;
-                // the values are on their way while the scores are worked out
-                float v[KEYS][NJ];
+                for (int k0 = sw * KEYS; k0 < n_keys; k0 += UNIT_WARPS * KEYS) {
+                    const int key = k0 + (lane >> 2);
+                    const int pslot = (int)((unsigned)key / (unsigned)a.page_size);
+                    int page = -1;
+                    if (key < n_keys && pslot < a.max_pages) page = a.block_table[(size_t)b * a.max_pages + pslot];
+                    const bool there = page >= 0 && page < a.n_pages;          // ids outside the pool read as zeros, never as memory
+                    const uint32_t row = there ? (uint32_t)((page * a.n_kv + kvh) * a.page_size + key - pslot * a.page_size) : 0u;
+                    // the values are on their way while the scores are worked out
+                    float v[KEYS][NJ];
 #pragma unroll
-                for (int t = 0; t < KEYS; ++t) {
-                    const float* vr = vp + (size_t)__shfl_sync(0xFFFFFFFFu, row, 4 * t) * hd + lane;
+                    for (int t = 0; t < KEYS; ++t) {
+                        const float* vr = vp + (size_t)__shfl_sync(0xFFFFFFFFu, row, 4 * t) * hd + lane;
 #pragma unroll
-                    for (int j = 0; j < NJ; ++j) v[t][j] = 32 * j + lane < hd ? __ldcg(vr + 32 * j) : 0.f;
-                }
-                float s = 0.f;
-                const float* kr = kp + (size_t)row * hd;
+                        for (int j = 0; j < NJ; ++j) v[t][j] = 32 * j + lane < hd ? __ldcg(vr + 32 * j) : 0.f;
+                    }
+                    float s = 0.f;
+                    const float* kr = kp + (size_t)row * hd;
 #pragma unroll 4
-                for (int j = 4 * (lane & 3); j < hd; j += 16) {
-                    const float4 kv = ldg_fresh(kr + j), qv = ldg_fresh(q + j);
-                    s = fmaf(qv.x, kv.x, fmaf(qv.y, kv.y, fmaf(qv.z, kv.z, fmaf(qv.w, kv.w, s))));
+                    for (int j = 4 * (lane & 3); j < hd; j += 16) {
+                        const float4 kv = ldg_fresh(kr + j), qv = ldg_fresh(q + j);
+                        s = fmaf(qv.x, kv.x, fmaf(qv.y, kv.y, fmaf(qv.z, kv.z, fmaf(qv.w, kv.w, s))));
+                    }
+                    s += __shfl_xor_sync(0xFFFFFFFFu, s, 1);
+                    s += __shfl_xor_sync(0xFFFFFFFFu, s, 2);
+                    s = key < n_keys ? (there ? s * a.scale : 0.f) : -INFINITY;
+                    const float mn = fmaxf(mx, warp_max(s)), al = expf(mx - mn), p = key < n_keys ? expf(s - mn) : 0.f;
+                    den = den * al + warp_sum(p);                      // (four times the sum: four lanes to a key)
+                    mx = mn;
+#pragma unroll
+                    for (int j = 0; j < NJ; ++j) acc[j] *= al;
+                    const float pv = there ? p : 0.f;
+#pragma unroll
+                    for (int t = 0; t < KEYS; ++t) {
+                        const float pt = __shfl_sync(0xFFFFFFFFu, pv, 4 * t);
+#pragma unroll
+                        for (int j = 0; j < NJ; ++j) acc[j] = fmaf(pt, v[t][j], acc[j]);
+                    }
                 }
-                s += __shfl_xor_sync(0xFFFFFFFFu, s, 1);
-                s += __shfl_xor_sync(0xFFFFFFFFu, s, 2);
-                s = key < n_keys ? (there ? s * a.scale : 0.f) : -INFINITY;
-                const float mn = fmaxf(mx, warp_max(s)), al = expf(mx - mn), p = key < n_keys ? expf(s - mn) : 0.f;
-                den = den * al + warp_sum(p);                      // (four times the sum: four lanes to a key)
-                mx = mn;
+                float* mine = part + (size_t)warp * (hd + 4);
 #pragma unroll
-                for (int j = 0; j < NJ; ++j) acc[j] *= al;
-                const float pv = there ? p : 0.f;
-#pragma unroll
-                for (int t = 0; t < KEYS; ++t) {
-                    const float pt = __shfl_sync(0xFFFFFFFFu, pv, 4 * t);
-#pragma unroll
-                    for (int j = 0; j < NJ; ++j) acc[j] = fmaf(pt, v[t][j], acc[j]);
-                }
-            }
-            float* mine = part + (size_t)warp * (hd + 4);
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) if (32 * j + lane < hd) mine[32 * j + lane] = acc[j];
-            if (lane == 0) { mine[hd] = mx; mine[hd + 1] = 0.25f * den; }
-            __syncthreads();
-            if (sw == 0 && u < n_units) {
-                const float* p0 = part + (size_t)warp * (hd + 4);
-                float top = -INFINITY, sum = 0.f;
+                for (int j = 0; j < NJ; ++j) if (32 * j + lane < hd) mine[32 * j + lane] = acc[j];
+                if (lane == 0) { mine[hd] = mx; mine[hd + 1] = 0.25f * den; }
+                __syncthreads();
+                if (sw == 0 && u < n_units) {
+                    const float* p0 = part + (size_t)warp * (hd + 4);
+                    float top = -INFINITY, sum = 0.f;
 #pragma unroll 1
-                for (int w = 0; w < UNIT_WARPS; ++w) top = fmaxf(top, p0[w * (hd + 4) + hd]);
-#pragma unroll 1
-                for (int w = 0; w < UNIT_WARPS; ++w)
-                    if (p0[w * (hd + 4) + hd] != -INFINITY) sum += expf(p0[w * (hd + 4) + hd] - top) * p0[w * (hd + 4) + hd + 1];
-#pragma unroll 1
-                for (int j = lane; j < hd; j += 32) {
-                    float o = 0.f;
+                    for (int w = 0; w < UNIT_WARPS; ++w) top = fmaxf(top, p0[w * (hd + 4) + hd]);
 #pragma unroll 1
                     for (int w = 0; w < UNIT_WARPS; ++w)
-                        if (p0[w * (hd + 4) + hd] != -INFINITY) o += expf(p0[w * (hd + 4) + hd] - top) * p0[w * (hd + 4) + j];
-                    a.o[(size_t)m * qd + h * hd + j] = n_keys > 0 ? o / sum : 0.f;
+                        if (p0[w * (hd + 4) + hd] != -INFINITY) sum += expf(p0[w * (hd + 4) + hd] - top) * p0[w * (hd + 4) + hd + 1];
+#pragma unroll 1
+                    for (int j = lane; j < hd; j += 32) {
+                        float o = 0.f;
+#pragma unroll 1
+                        for (int w = 0; w < UNIT_WARPS; ++w)
+                            if (p0[w * (hd + 4) + hd] != -INFINITY) o += expf(p0[w * (hd + 4) + hd] - top) * p0[w * (hd + 4) + j];
+                        a.o[(size_t)m * qd + h * hd + j] = n_keys > 0 ? o / sum : 0.f;
+                    }
                 }
+                __syncthreads();
             }
-            __syncthreads();
-        }
         }
 #ifdef TASC_TIMELINE
         tl_b = global_ns();

@@ -122,9 +122,6 @@ __device__ __forceinline__ float lds_f(uint32_t addr) {
 }
 __device__ __forceinline__ void sts_f(uint32_t addr, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
 
-__device__ __forceinline__ uint32_t pack2(__nv_bfloat16 a, __nv_bfloat16 b) {
-    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
-}
 // Hides where a value comes from: what is derived from it is computed in this phase, not kept in registers over the
 // whole layer loop (the compiler would otherwise hoist every phase's addresses out of it and spill them).
 __device__ __forceinline__ int fresh(int v) {

@@ -666,8 +666,9 @@ FusedPlan plan_fused(int M, int N, int K, int epi, int few_tiles, int hd, double
         // Fewer splits than fit can be faster.  Per kernel, in microseconds: a CTA's epilogue takes about 0.5 per round of six token
         // columns (one per warp) of the columns it finishes; every CTA costs 0.026, because it keeps a CTA of the next kernel from
         // starting (and from fetching its weights) while this kernel runs; a k-block of a CTA's chain costs 0.15, about what its MMAs
-        // take, where the weights were there before the activations (QKV and O), 0.46 in gate/up and 0.6 in down, which follows the
-        // kernel with the largest grid and fetches its weights late.  (0.46 for all, and 0.035 per CTA from the 97th on, before /
+        // take, where the weights were there before the activations (QKV and O), 0.46 in gate/up and 0.6 in down (K > N), which follows
+        // the kernel with the largest grid and fetches its weights late.  (An O projection wider than the model counts as down: at 96 to
+        // 288 rows of three such shapes a step is between 1.3 % slower and 1.0 % faster than by O's price.)  (0.46 for all, and 0.035 per CTA from the 97th on, before /
         // now: 135M, step at 96 rows 846 -> 833 us, 100 rows 847 -> 827, 128 rows 823 -> 794, 288 rows 967 -> 966; 0.5B 96 rows
         // 946 -> 909, 120 rows 1126 -> 1099, 192 rows 1196 -> 1196, 100 prompt tokens 903 -> 872.  With 0.024 per CTA 135M at 128 rows
         // 815, with 0.028 at 288 rows 972.)

@@ -402,7 +402,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     if ((lane & 7) == 0) {
                         a.ssq_out[(size_t)(m0 + r) * a.ssq_out_slots + f / 32] = ss;
                         if (f + 32 >= a.N)                            // the slots past the last 32 features
-    #pragma unroll 1
+#pragma unroll 1
                         for (int q = f / 32 + 1; q < a.ssq_out_slots; ++q) a.ssq_out[(size_t)(m0 + r) * a.ssq_out_slots + q] = 0.f;
                     }
                 });
