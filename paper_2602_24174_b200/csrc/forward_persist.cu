@@ -28,10 +28,10 @@
 // the barrier.  Key ranges of one group are merged by the CTA that finishes last, in range order.
 //
 // Measured (one verify step, five kernels per layer / this kernel): 135M at 6 rows 747 / 594 us, 0.5B at 6 rows 746 / 650, 1.5B
-// at 7 rows 1213 / 1144; more of it at persist_pays.  What is left, by stamps (which add about 0.3 us a phase): at 135M 3.1 - 3.3 us per
+// at 7 rows 1213 / 1144; more of it at persist_pays.  What is left, by stamps (which add about 0.3 us a phase): at 135M 3.0 - 3.5 us per
 // projection, 0.8 - 1.0 of it the barrier, 0.7 - 1.0 the products behind their first fresh read, 1.5 the epilogue and the arrival;
-// attention 6.9, 2.5 of it the merge of the key ranges.  At 1.5B the weights: gate/up 12.0 (products 8.2), down 7.9 (5.3), QKV 6.5 (CTAs
-// start it 1.4 us apart), O 3.6, attention 9.8 (merge 4.1).
+// attention 6.6, 2.6 of it the merge of the key ranges.  At 1.5B the weights: gate/up 11.9 (products 8.2), down 7.9 (5.4), QKV 6.4 (CTAs
+// start it 1.4 us apart), O 3.5, attention 9.5 (merge 3.9).
 //
 // Code is kept short, because a layer runs through more of it than the instruction cache holds: one copy of `decode` behind the
 // products instead of two, two chunks in flight instead of four where they do not pay, loops of the attention not unrolled at one
