@@ -15,9 +15,9 @@
 // in the attention is the KV cache's own.  Softmax statistics and O are float32.
 //
 // Merge (only when the key range is split): the splits of one (sequence, KV head) are the CTAs of a
-// thread-block cluster.  Each parks its unnormalised O and (max, sum) in its shared memory; after a cluster
-// barrier CTA r merges every S-th row from the S copies (distributed shared memory reads, rank order) and
-// writes it as (hi, lo) bf16 in the layout the O-projection GEMM loads.  Nothing goes through global memory.
+// thread-block cluster.  CTA r merges every S-th row, in rank order, and writes it as (hi, lo) bf16 in the layout the
+// O-projection GEMM loads.  Every CTA stores its unnormalised O and (max, sum) straight into the shared memory of the rows'
+// mergers (distributed shared memory), and a cluster barrier later they are there.  Nothing goes through global memory.
 #include "kernels.h"
 
 #include <algorithm>
@@ -46,6 +46,7 @@ struct AttnArgs {
     __nv_bfloat16* out;                // (hi, lo) activation buffer, row length n_q * hd
     int TB;
     int R, n_q, n_kv, splits, stages;  // R: rows per sequence in this pass
+    int push_rows;                     // split key ranges: query rows per CTA of the cluster, whose shares are stored into its shared memory; 0: fetched
     int Rs, n_sub;                     // a CTA takes Rs of them (sub-block blockIdx.z % n_sub); R = Rs * n_sub
     int hs, n_hsplit;                  // a CTA takes hs of the g query heads of its KV head (blockIdx.y % n_hsplit); g = hs * n_hsplit
     int n_slabs;                       // 16-row slabs of the CTA's hs * Rs query rows
@@ -178,6 +179,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         }
         return;
     }
+    if (a.push_rows) cluster_arrive();           // (nothing is stored to a CTA that has not started)
     const int total = pos0 + rows;               // keys visible to the last row
     // the range's 64-key tiles are dealt out evenly: every split gets floor or ceil of tiles / splits of them
     const int tiles_all = (total + TKEYS - 1) / TKEYS;
@@ -532,43 +534,47 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         return;
     }
 
-    // The key range was split over the S CTAs of this cluster: every CTA parks its unnormalised rows
-    // (O, running maximum, running sum) in its own shared memory (the K/V ring is idle); after a cluster
-    // barrier CTA r merges the rows rho = r, r + S, ... from all S copies, in rank order, and writes them.
-    constexpr int XS = HD + 4;                                 // floats per parked row: O[HD], max, sum, pad
-    float* xo = reinterpret_cast<float*>(Kt);
-    __syncthreads();                                           // the warp groups' exchange area is inside the ring too
+    // The key range was split over the S CTAs of this cluster: CTA r merges the rows rho = r, r + S, ... from the unnormalised rows
+    // (O, running maximum, running sum) of all S, in rank order, and writes them.  Where there is memory for it every CTA stores its
+    // rows straight into their mergers' shared memory, behind the ring, and one cluster barrier is all that is waited for; otherwise it
+    // parks them in its own (the K/V ring is idle), they are fetched behind the barrier, and nobody leaves before all are.  Fetched / stored,
+    // by stamps from the last key tile until the CTA has left: 135M, 96 rows 3.6 / 2.8 us, 0.5B, 42 rows 3.2 / 2.5; a step of the 135M at 96
+    // rows 808 -> 785 us, of the 0.5B at 28 rows 690 -> 666, 255 prompt tokens of the 135M 855 -> 848.
+    constexpr int XS = HD + 4;                                 // floats per row: O[HD], max, sum, pad
+    const int S = a.splits, rank = (int)cluster_ctarank(), push = a.push_rows;
+    const uint32_t ring = smem_u32(Kt), given = smem_u32(Vt + STAGES * TILE_BYTES);      // [S][push_rows][XS]
+    if (push) cluster_wait();
+    else __syncthreads();                                      // the warp groups' exchange area is inside the ring too
     if (writer) {
-        float* r0p = xo + (size_t)rho0 * XS + 2 * (lane & 3);
-        float* r1p = xo + (size_t)rho1 * XS + 2 * (lane & 3);
 #pragma unroll
-        for (int nt = 0; nt < HD / 8; ++nt) {
-            *reinterpret_cast<float2*>(r0p + nt * 8) = make_float2(o[nt][0], o[nt][1]);
-            *reinterpret_cast<float2*>(r1p + nt * 8) = make_float2(o[nt][2], o[nt][3]);
-        }
-        if ((lane & 3) == 0) {
-            *reinterpret_cast<float2*>(xo + (size_t)rho0 * XS + HD) = make_float2(m_run[0], l_run[0]);
-            *reinterpret_cast<float2*>(xo + (size_t)rho1 * XS + HD) = make_float2(m_run[1], l_run[1]);
+        for (int half = 0; half < 2; ++half) {
+            const int rho = half ? rho1 : rho0;
+            if (rho >= G) continue;
+            const int at = a.by_splits.div(rho);
+            const uint32_t dst = push ? cluster_map(given + (uint32_t)((rank * push + at) * XS) * 4u, (uint32_t)(rho - at * S))
+                                      : cluster_map(ring + (uint32_t)(rho * XS) * 4u, (uint32_t)rank);
+#pragma unroll
+            for (int nt = 0; nt < HD / 8; ++nt) st_cluster_f2(dst + (uint32_t)(nt * 8 + 2 * (lane & 3)) * 4u, o[nt][2 * half], o[nt][2 * half + 1]);
+            if ((lane & 3) == 0) st_cluster_f2(dst + HD * 4u, m_run[half], l_run[half]);
         }
     }
     cluster_arrive();
     cluster_wait();
-    const int S = a.splits, rank = (int)cluster_ctarank();
-    const uint32_t xo_addr = smem_u32(xo);
     uint32_t peer[8];
 #pragma unroll
-    for (int sidx = 0; sidx < 8; ++sidx) peer[sidx] = cluster_map(xo_addr, (uint32_t)(sidx < S ? sidx : 0));
+    for (int sidx = 0; sidx < 8; ++sidx)
+        peer[sidx] = push ? cluster_map(given + (uint32_t)((sidx < S ? sidx : 0) * push * XS) * 4u, (uint32_t)rank) : cluster_map(ring, (uint32_t)(sidx < S ? sidx : 0));
 #pragma unroll 1
-    for (int rho = rank + tid / (HD / 4) * S; rho < G; rho += RPI * S) {
-        const int hl = a.by_R.div(rho), rr = rho - hl * R;
+    for (int i = tid / (HD / 4); rank + i * S < G; i += RPI) {
+        const int rho = rank + i * S, hl = a.by_R.div(rho), rr = rho - hl * R;
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         if (rr < rows) {
             float2 ml[8];
             float4 ov[8];
 #pragma unroll
             for (int sidx = 0; sidx < 8; ++sidx)
-                if (sidx < S) {                                 // all remote reads are issued before the first is used
-                    const uint32_t rowa = peer[sidx] + (uint32_t)(rho * XS) * 4u;
+                if (sidx < S) {                                 // all reads are issued before the first is used
+                    const uint32_t rowa = peer[sidx] + (uint32_t)((push ? i : rho) * XS) * 4u;
                     ml[sidx] = ld_cluster_f2(rowa + HD * 4u);
                     ov[sidx] = ld_cluster_f4(rowa + (uint32_t)d4 * 4u);
                 }
@@ -595,6 +601,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         *reinterpret_cast<uint2*>(a.out + row * qd + col) = h;
         *reinterpret_cast<uint2*>(a.out + (row + a.TB) * qd + col) = l;
     }
+    if (push) return;
     // peers may still be reading this CTA's parked rows
     cluster_arrive();
     cluster_wait();
@@ -658,7 +665,7 @@ template <int HD, int NS, bool TMA>
 tasc_status launch_inst(const AttnArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int B, cudaStream_t stream) {
     constexpr int GP = NS * 16;
     if (a.stages < 2 || a.stages > Ring<HD, NS>::MAX_STAGES) return TASC_EINVAL;
-    const size_t smem = attn_smem_bytes(HD, GP, a.stages);
+    const size_t smem = attn_smem_bytes(HD, GP, a.stages) + (size_t)a.push_rows * a.splits * (HD + 4) * 4;
     tasc_status pst = prepare_inst<HD, NS, TMA>();
     if (pst != TASC_OK) return pst;
     cudaLaunchConfig_t cfg = {};
@@ -785,6 +792,9 @@ tasc_status launch_attention_mma(const float* qbuf, const __nv_bfloat16* k_pages
     a.scale_log2e = 1.4426950408889634f / sqrtf((float)hd);
     a.status = status;
     a.n_slabs = (G + 15) / 16;
+    // Rows go straight to their mergers where the memory for that leaves as many CTAs to an SM.
+    const size_t base = attn_smem_bytes(hd, GP, plan.stages), extra = (size_t)((G + n_splits - 1) / n_splits) * n_splits * (hd + 4) * 4, sm = 228 * 1024;
+    a.push_rows = n_splits > 1 && base + extra <= 220 * 1024 && sm / (base + 1024) == sm / (base + extra + 1024) ? (G + n_splits - 1) / n_splits : 0;
     a.by_R = SmallDiv(Rs); a.by_TB = SmallDiv(TB); a.by_splits = SmallDiv(n_splits); a.by_sub = SmallDiv(n_sub); a.by_hsplit = SmallDiv(g / hs);
     // 16-token pages arrive as TMA boxes; any other page size, and key ranges of more pages than a CTA keeps the ids of, take the
     // kernel with cp.async.  So do 64-wide heads with one CTA per SM (the deep ring) in caches of more than 1,024 pages, which are
