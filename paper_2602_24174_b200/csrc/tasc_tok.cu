@@ -193,7 +193,11 @@ struct TokShared {
     int n_tied;                                  // candidates of the best rank
     uint32_t tied_slot[TIED_MAX];
     Key tied_key[TIED_MAX];
-    int n_hits, next_hit, more_hits;
+    unsigned long long used;                     // of the round's state, read by one thread for all
+    int rebuild;
+    unsigned int n_cand;
+    int windows[TOK_WARPS];                      // on the warps' lists
+    int n_hits, more_hits;
     int hits[HIT_MAX], hit_len[HIT_MAX];         // documents, their lengths
     int64_t hit_at[HIT_MAX];                     // and where they start
     TokWarp warp[TOK_WARPS];
@@ -333,8 +337,9 @@ __device__ __noinline__ Rewritten tok_rewrite_short(const TokArgs& a, TokShared&
     __syncwarp();
     return Rewritten{wr, old_chunks, new_chunks};
 }
-// Then the windows that change, old and new: put on the warp's list, which is looked up as a whole (a look-up is a trip to L2 or to
-// memory behind it).  Chunks without a changed token near are passed over.
+// Then the windows that change, old and new, are put on the warp's list.  Chunks without a changed token near are passed over.
+// FLUSH: looks them up, and returns the slots that this lane has claimed.  Otherwise their number, -1 if they are more than the list holds.
+template <bool FLUSH>
 __device__ __noinline__ int tok_recount_short(const TokArgs& a, TokShared& sh, int L, Rewritten r, int round, const Candidates& cand) {
     TokWarp& w = sh.warp[threadIdx.x >> 5];
     TokList list = {w, w.old_tok, w.new_tok, 0};
@@ -345,11 +350,46 @@ __device__ __noinline__ int tok_recount_short(const TokArgs& a, TokShared& sh, i
         const int at = c & (DOC_SMEM - 1), len = add ? r.len : L;
         // (a window that holds a mark of the next chunk starts in this one)
         if (at < len && (((add ? r.new_chunks : r.old_chunks) >> (at >> 5)) & 3u)) {
+            if (list.full()) {
+                if (!FLUSH) return -1;
+                claimed += list.flush(a, round, cand);
+            }
             list.collect(a, add ? w.new_mark : w.old_mark, len, at, 0, add);
-            if (list.full()) claimed += list.flush(a, round, cand);
         }
     }
-    return claimed + list.flush(a, round, cand);
+    return FLUSH ? claimed + list.flush(a, round, cand) : list.total;
+}
+// Looks up the windows of all warps' lists, dealt out to all threads of the CTA; returns the slots that this one has claimed.  (A look-up is
+// two or three trips to L2 or to memory behind it, one after the other.  A round has a handful of documents per CTA: with every warp's
+// windows looked up by itself, the warps with documents took 7 us of them and the others none.)
+__device__ __noinline__ int tok_look_up(const TokArgs& a, TokShared& sh, int round, const Candidates& cand) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, mine = sh.windows[lane];
+    int end = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, end, o);
+        if (lane >= o) end += y;
+    }
+    const int total = __shfl_sync(0xFFFFFFFFu, end, 31);
+    int claimed = 0;
+#pragma unroll 1
+    for (int p0 = 0; p0 < total; p0 += TOK_THREADS) {
+        const int p = p0 + lane * TOK_WARPS + warp;
+        int of = 0;                                            // the list that has window p
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) if (__shfl_sync(0xFFFFFFFFu, end, of + o - 1) <= p) of += o;
+        const int first = __shfl_sync(0xFFFFFFFFu, end - mine, of);
+        if (p >= total) continue;
+        const TokWarp& w = sh.warp[of];
+        const int e = w.list[p - first], m = ((e >> 8) & 7) + 2;
+        const bool add = (e >> 11) & 1;
+        const int32_t* tok = (add ? w.new_tok : w.old_tok) + (e & 255);
+        Key key = key_make(m);
+#pragma unroll
+        for (int j = 0; j < MAX_N; ++j) if (j < m) key_put(key, j, (uint32_t)tok[j]);
+        claimed += tok_change(a, key, m, add, round, cand);
+    }
+    return claimed;
 }
 
 // The same for a longer document, in place, its windows chunk by chunk.
@@ -409,14 +449,16 @@ __device__ __noinline__ int tok_rewrite_long(const TokArgs& a, TokShared& sh, in
 // the list after it takes in half the distance from the best.
 //   Measured on 20,000 documents (1.4 M tokens, 4.1 M windows, n_max 4), per round: 525 us when every round cleared and
 // recounted the table, 33 when every round looked through the table's changed chunks (8 us, 4 more for the barrier and the best of
-// all CTAs; a tie 30 us, because every window of the corpus was looked up to find the first), 27 now.  A round of 100 to 400 documents:
-// 9 until they are listed, 11 to rewrite them (half of it the look-ups); rounds of thousands, which come first, 20 to 90.
+// all CTAs; a tie 30 us, because every window of the corpus was looked up to find the first), 27 when every warp read the round's state and looked
+// up the windows of its own documents (256 rounds and the first count 6.7 ms), 22 now (5.6 ms).  By stamps, a round of 100 to 400 documents
+// takes 18: 6 until they are listed, 3 to 5 to rewrite them, 1 the barrier, 4 to 5 the look-ups, 3 the barrier at its end; rounds of thousands, which
+// come first, 20 to 90.
 __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid_constant__ TokArgs a) {
     extern __shared__ __align__(16) uint8_t dyn[];
     TokShared& sh = *reinterpret_cast<TokShared*>(dyn);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t nw = (int64_t)gridDim.x * TOK_WARPS, wid = (int64_t)warp * gridDim.x + blockIdx.x;
-    if (threadIdx.x == 0) { sh.stop = 0; sh.n_hits = 0; sh.next_hit = 0; sh.more_hits = 0; }
+    if (threadIdx.x == 0) { sh.stop = 0; sh.n_hits = 0; sh.more_hits = 0; }
     // this warp's documents
     auto doc_at = [&](int64_t pos) {
         int64_t lo = 0, hi = a.n_docs;
@@ -441,10 +483,20 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
     for (int round = 0;; ++round) {
         // ---- the table, if it has to be counted (again): n-grams that no longer occur keep their slots until then.  (One trip for all
         // that a round looks at first.)
-        const unsigned long long used = *(volatile unsigned long long*)&a.st->used[n_rebuilds & 1];
-        const int rebuild = *(volatile int*)&a.st->rebuild;
-        unsigned int n_cand = *(volatile unsigned int*)cand.n;
-        const uint32_t cand_slot = __ldcg(cand.slots + threadIdx.x);
+        // (By one thread: read by all of them, 4,736 warps asked for the same three words, which took 2 us more.  A candidate's key and
+        // count are on their way before it is known how many there are: a place that is not one is a slot of the table all the same.)
+        if (threadIdx.x == 0) {
+            sh.used = *(volatile unsigned long long*)&a.st->used[n_rebuilds & 1];
+            sh.rebuild = *(volatile int*)&a.st->rebuild;
+            sh.n_cand = *(volatile unsigned int*)cand.n;
+        }
+        const uint32_t cand_slot = __ldcg(cand.slots + threadIdx.x) & (uint32_t)(a.cap - 1);
+        const ulonglong2 cand_key = __ldcg(reinterpret_cast<const ulonglong2*>(a.keys) + cand_slot);
+        const uint32_t cand_word = __ldcg(a.words + cand_slot);
+        __syncthreads();
+        const unsigned long long used = sh.used;
+        const int rebuild = sh.rebuild;
+        unsigned int n_cand = sh.n_cand;
         if (rebuild == round || used * 4 > a.cap * 3) {
             const uint64_t gt = (uint64_t)blockIdx.x * TOK_THREADS + threadIdx.x, gn = (uint64_t)gridDim.x * TOK_THREADS;
             for (uint64_t i = gt; i < a.cap; i += gn) {
@@ -480,9 +532,8 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
             uint32_t reward = 0u, len = 0u;
             Key key = {0ull, 0ull};
             if (threadIdx.x < n_cand) {
-                const ulonglong2 k = __ldcg(reinterpret_cast<const ulonglong2*>(a.keys) + cand_slot);
-                const unsigned long long rank = tok_rank(__ldcg(a.words + cand_slot));
-                key = Key{k.x, k.y};
+                const unsigned long long rank = tok_rank(cand_word);
+                key = Key{cand_key.x, cand_key.y};
                 reward = (uint32_t)(rank >> LEN_BITS);
                 len = (uint32_t)rank & ((1u << LEN_BITS) - 1u);
             }
@@ -721,24 +772,29 @@ __global__ void __launch_bounds__(TOK_THREADS, 1) tok_rounds_kernel(const __grid
             const int n_hits = min(sh.n_hits, HIT_MAX);
             // while the barrier is on its way the warps work on their first documents
             if (!passed) tok_arrive(a.st, epoch);
-            for (;;) {
-                int slot = 0;
-                if (lane == 0) slot = atomicAdd(&sh.next_hit, 1);
-                slot = __shfl_sync(0xFFFFFFFFu, slot, 0);
+#pragma unroll 1
+            for (int base = 0; base < n_hits || !passed; base += TOK_WARPS) {
+                const int slot = base + warp;
                 const bool work = slot < n_hits;
                 const int d = work ? sh.hits[slot] : 0, L = work ? sh.hit_len[slot] : 0;
                 const int64_t s0 = work ? sh.hit_at[slot] : 0;
                 Rewritten r = {0, 0u, 0u};
-                if (work && L <= DOC_SMEM) r = tok_rewrite_short(a, sh, d, s0, L, new_id);
-                if (!passed) {
-                    if (!tok_wait(a.st, epoch, sh)) return;
-                    passed = true;
+                int windows = 0;
+                if (work && L <= DOC_SMEM) {
+                    r = tok_rewrite_short(a, sh, d, s0, L, new_id);
+                    windows = tok_recount_short<false>(a, sh, L, r, round, cand);
                 }
-                if (!work) break;
-                claimed += L <= DOC_SMEM ? tok_recount_short(a, sh, L, r, round, cand) : tok_rewrite_long(a, sh, d, s0, L, new_id, round, cand);
+                if (lane == 0) sh.windows[warp] = max(windows, 0);
+                if (passed) __syncthreads();
+                else if (!tok_wait(a.st, epoch, sh)) return;
+                passed = true;
+                claimed += tok_look_up(a, sh, round, cand);
+                __syncthreads();                               // the lists are used again
+                if (windows < 0) claimed += tok_recount_short<true>(a, sh, L, r, round, cand);
+                if (work && L > DOC_SMEM) claimed += tok_rewrite_long(a, sh, d, s0, L, new_id, round, cand);
             }
             __syncthreads();
-            if (threadIdx.x == 0) { sh.n_hits = 0; sh.next_hit = 0; sh.more_hits = 0; }
+            if (threadIdx.x == 0) { sh.n_hits = 0; sh.more_hits = 0; }
             if (more) __syncthreads();
         }
         publish_claims(claimed);
