@@ -13,8 +13,7 @@
 //   the best, which every CTA reads for itself.  The documents stay at their original offsets and only get shorter.
 //   All rounds run in one cooperative kernel without a host round trip.
 // tasc_tok_init_rows -- Section 4.2: the embedding / LM-head row of an added token is the mean of its constituents'
-//   rows (a constituent may itself be an added token).  A thread per column walks the merges in order, so a row is
-//   always complete when a later row needs it, with no synchronisation.
+//   rows (a constituent may itself be an added token): in order, by warps that wait for the rows they need.
 // tasc_tok_encode -- Appendix on byte-pair encoding: text is encoded with the added tokens matched first and greedily
 //   (the longest added token whose expansion into base tokens matches the upcoming base tokens).  The added tokens'
 //   expansions form a trie stored as a hash of (node, token) -> child; a thread per document walks it.
@@ -901,51 +900,73 @@ __global__ void tok_compact_kernel(const int32_t* __restrict__ cur, const int64_
 }
 
 // ------------------------------------------------------------------------------------------- new rows
-// Bound: a chain (a row may need any earlier one).  A thread fetches the values of a group of merges together, as far as
-// they were complete before the group, then walks it.  256 merges of 896 columns: 316 us when every merge waited for its
-// own loads, 168 us in groups.
-constexpr int ROWS_GROUP = 8, ROWS_THREADS = 64;
+// Bound: a chain (a row may need any earlier one), mostly a short one, and the loads of what it starts from.  A block has ROWS_COLS columns, and its
+// warps take the merges in turn: one waits for those of its constituents that are not there yet, whose rows other warps leave in shared memory.
+// (Those that a merge waits for are earlier ones, and a warp's are in order: the first one that is not done never waits.)  Merges come in
+// chunks, and the rows of the chunks before from where they were written.  256 merges of 896 columns: 316 us when a thread per column
+// walked them one by one, 168 in groups of eight whose loads were under way together; the
+// call 217 -> 70 us so (8,192 that need none: 5.9 -> 0.53 ms; a chain of 256, each of which needs the one before: 224 -> 198 us).
+constexpr int ROWS_COLS = 32, ROWS_THREADS = 1024, ROWS_CHUNK = 256;
+constexpr int ROWS_WAIT = 1 << 24;                 // looks at a row that is waited for (never reached, see above)
+// (rows that other warps of the block have written: past L1)
+__device__ __forceinline__ float load_row(const float* p) { return __ldcg(p); }
+__device__ __forceinline__ __nv_bfloat16 load_row(const __nv_bfloat16* p) { return __ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(p))); }
 template <typename T>
 __global__ void __launch_bounds__(ROWS_THREADS)
 tok_rows_kernel(const T* base, int base_vocab, int d, const int32_t* __restrict__ merges, int n_merges, T* rows_out,
                 int* status) {
-    const int j = blockIdx.x * ROWS_THREADS + threadIdx.x;
-    if (j >= d) return;
-    for (int g0 = 0; g0 < n_merges; g0 += ROWS_GROUP) {
-        int tok[ROWS_GROUP][MAX_N];
-        T val[ROWS_GROUP][MAX_N];
-#pragma unroll
-        for (int i = 0; i < ROWS_GROUP; ++i)
-#pragma unroll
-            for (int c = 0; c < MAX_N; ++c) tok[i][c] = g0 + i < n_merges ? merges[(size_t)(g0 + i) * MAX_N + c] : -1;
-#pragma unroll
-        for (int i = 0; i < ROWS_GROUP; ++i)
+    __shared__ float s_row[ROWS_CHUNK][ROWS_COLS];
+    __shared__ int32_t s_tok[ROWS_CHUNK * MAX_N];
+    __shared__ volatile int s_done[ROWS_CHUNK];
+    constexpr int WARPS = ROWS_THREADS / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = blockIdx.x * ROWS_COLS + lane;
+    for (int c0 = 0; c0 < n_merges; c0 += ROWS_CHUNK) {
+        const int n = min(ROWS_CHUNK, n_merges - c0);
+        __syncthreads();                                          // the chunk before: its rows are written, and no longer read from here
+        for (int i = threadIdx.x; i < n * MAX_N; i += ROWS_THREADS) s_tok[i] = merges[(size_t)c0 * MAX_N + i];
+        if (threadIdx.x < ROWS_CHUNK) s_done[threadIdx.x] = 0;
+        __syncthreads();
+        T val[MAX_N], next[MAX_N];
+        // what does not come from this chunk (no branch: all loads are under way together; what cannot be used reads some other row)
+        auto fetch = [&](int i, T (&v)[MAX_N]) {
 #pragma unroll
             for (int c = 0; c < MAX_N; ++c) {
-                // (no branch: all loads of the group are under way together; what cannot be used reads some other row)
-                const int t = tok[i][c];
-                const T* row = t >= base_vocab && t - base_vocab < g0 ? rows_out + (size_t)(t - base_vocab) * d : base + (size_t)(t >= 0 && t < base_vocab ? t : 0) * d;
-                val[i][c] = row[j];
+                const int t = s_tok[i * MAX_N + c], at = t - base_vocab;
+                const T* row = t >= 0 && at >= 0 && at < c0 ? rows_out + (size_t)at * d : base + (size_t)(t >= 0 && at < 0 ? t : 0) * d;
+                v[c] = j < d ? load_row(row + j) : Num<T>::from_f(0.f);
             }
-#pragma unroll
-        for (int i = 0; i < ROWS_GROUP; ++i) {
-            if (g0 + i >= n_merges) break;
+        };
+        if (warp < n) fetch(warp, val);
+        for (int i = warp; i < n; i += WARPS) {
+            if (i + WARPS < n) fetch(i + WARPS, next);
             float acc = 0.f;
-            int n = 0;
+            int count = 0;
             bool more = true;
 #pragma unroll
             for (int c = 0; c < MAX_N; ++c) {
-                const int t = tok[i][c];
+                const int t = s_tok[i * MAX_N + c], at = t - base_vocab;
                 more = more && t >= 0;
                 if (!more) continue;
-                float v = Num<T>::to_f(val[i][c]);
-                if (t - base_vocab >= g0 + i) { set_status(status, TASC_EINVAL); v = 0.f; }      // a constituent that does not exist yet
-                else if (t - base_vocab >= g0) v = Num<T>::to_f(rows_out[(size_t)(t - base_vocab) * d + j]);      // written by this thread
+                ++count;
+                if (at >= c0 + i) { set_status(status, TASC_EINVAL); continue; }         // a constituent that does not exist yet
+                float v = Num<T>::to_f(val[c]);
+                if (at >= c0) {
+                    for (int look = 0; s_done[at - c0] == 0; ++look)
+                        if (look == ROWS_WAIT) { set_status(status, TASC_EINVAL); break; }
+                    __threadfence_block();
+                    v = s_row[at - c0][lane];
+                }
                 acc += v;
-                ++n;
             }
-            if (n < 2) { set_status(status, TASC_EINVAL); n = 1; }
-            rows_out[(size_t)(g0 + i) * d + j] = Num<T>::from_f(acc / (float)n);
+            if (count < 2) { set_status(status, TASC_EINVAL); count = 1; }
+            const T mean = Num<T>::from_f(acc / (float)count);
+            s_row[i][lane] = Num<T>::to_f(mean);
+            if (j < d) rows_out[(size_t)(c0 + i) * d + j] = mean;
+            __threadfence_block();
+            __syncwarp();
+            if (lane == 0) s_done[i] = 1;
+#pragma unroll
+            for (int c = 0; c < MAX_N; ++c) val[c] = next[c];
         }
     }
 }
@@ -1079,7 +1100,7 @@ extern "C" tasc_status tasc_tok_init_rows(const void* matrix, int32_t dtype, int
         return TASC_EINVAL;
     if (n_merges == 0) return TASC_OK;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    const unsigned blocks = (unsigned)((d + ROWS_THREADS - 1) / ROWS_THREADS);
+    const unsigned blocks = (unsigned)((d + ROWS_COLS - 1) / ROWS_COLS);
     if (dtype == TASC_F32)
         tok_rows_kernel<float><<<blocks, ROWS_THREADS, 0, stream>>>(static_cast<const float*>(matrix), base_vocab, d, merges, n_merges,
                                                            static_cast<float*>(rows_out), device_status);
