@@ -8,15 +8,19 @@
 // one warp, S and O in TMEM, K and V staged by TMA, so that the softmax is what is left: a thread owns half of the keys
 // of one row, registers hold its half of the row's O.  Per tile of TK keys
 //   MMA warp       S(t + 1) while the softmax works on S(t); then P(t) V(t) into an O tile of its own
-//   softmax warps  S(t) -> maximum (exchanged between the two threads of a row) -> P(t) as hi, lo in shared memory;
+//   softmax warps  S(t) -> maximum (exchanged between the two threads of a row) -> P(t) as hi, lo, in TMEM in the place of S(t);
 //                  then O += O tile (t - 1), rescaled: O is accumulated in registers, so a new maximum costs no pass over TMEM
 //   TMA warp       K and V tiles, a ring of two or more
-// Query tiles of up to 64 rows take 128 keys per tile, up to 128 rows 64 keys (P is TK x rows x 4 bytes of shared memory).
+// P as the MMA's A operand in TMEM takes no pass through shared memory, does not wait for P(t - 1) to be used, and leaves the ring its
+// memory, so that 128 keys make a tile for up to 128 rows too (64 before).  With up to 64 rows four of the eight softmax warps have any;
+// two of the others are the TMA and the MMA warp then.
 // Key ranges split over a cluster are merged as in attention_mma.cu.
 //
 // Measured, per layer: 1.5B at 64 sequences x 7 rows and up to 1,530 keys 61 -> 33 us (2.0 us per 128 keys: softmax 0.9, its
 // half of O 0.3, P 0.4, waits 0.4); 0.5B + 8,192 tokens at 32 x 9 rows, 640 keys 15.5 -> 13.4; prefill of 16 x 1,024 tokens
-// on the 1.5B 72 -> 47 us per pass of 2,048 rows.
+// on the 1.5B 72 -> 47 us per pass of 2,048 rows.  With P in TMEM, whole steps: 1.5B, 64 x 7 rows behind 1,500 keys 4,204 -> 4,190 us, and with
+// the warps' places 4,094; 40 x 5 rows behind 1,400 2,859 -> 2,821, 2,736; 0.5B + 8,192 tokens 1,392 -> 1,370, 1,371; a prefill of
+// 4 x 1,000 tokens of the 1.5B (96 rows) 19.68 -> 19.45 ms with tiles of 64 keys, 19.90 -> 19.47 with tiles of 128.
 //
 // A CTA with a few tiles waits for code that it executes as often, so there is one copy of everything (the first tile's scores, the last
 // tile's O, both halves of a tile's load), ring slots are counted and rows divided by multiplication: 76 - 102 -> 47 - 66 KB.  A step
@@ -33,7 +37,6 @@ namespace tasc {
 namespace {
 
 constexpr int SM_WARPS = 8;                      // softmax: two per TMEM lane quarter, which share its rows
-constexpr int THREADS = (SM_WARPS + 2) * 32;     // + TMA warp, MMA warp
 constexpr int PAGE = 16;
 constexpr int MAX_PAGES = 1024;
 constexpr int MAX_SMEM = 216 * 1024;
@@ -74,12 +77,15 @@ __device__ __forceinline__ uint64_t umma_desc_mn_sw128(uint32_t smem_addr, uint3
 }
 
 template <int HD, int RP> struct Tc {
-    static constexpr int TK = RP == 64 ? 128 : 64;               // keys of a tile
+    static constexpr int TK = 128;                               // keys of a tile
     static constexpr int HB = HD / 64;                           // blocks of 64 columns of a head
+    // Query tiles of 64 rows have rows in the first two lane quarters: two warps of the others feed the tensor cores.  (Theirs are the other two
+    // schedulers, and eight warps have more registers each than ten.)
+    static constexpr int TMA_WARP = RP == 64 ? 2 : SM_WARPS, MMA_WARP = TMA_WARP + 1;
+    static constexpr int WARPS = RP == 64 ? SM_WARPS : SM_WARPS + 2, THREADS = WARPS * 32, LOADERS = THREADS - 64;
     static constexpr int Q_BYTES = RP * HD * 2;                  // hi or lo
-    static constexpr int P_BYTES = RP * TK * 2;
     static constexpr int KV_BYTES = TK * HD * 2;                 // K or V tile
-    static constexpr int FIXED = 2 * Q_BYTES + 2 * P_BYTES;
+    static constexpr int FIXED = 2 * Q_BYTES;
     static constexpr int S_COL = 0, O_COL = 2 * TK;              // TMEM columns: two S tiles, two O tiles
     static constexpr int COLS = 2 * TK + 2 * HD <= 256 ? 256 : 512;
     static constexpr int SC = TK / 2, OC = HD / 2;               // a thread's share of a row of S, of O
@@ -87,18 +93,17 @@ template <int HD, int RP> struct Tc {
 };
 
 template <int HD, int RP>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(Tc<HD, RP>::THREADS, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const TcArgs a) {
     using C = Tc<HD, RP>;
-    constexpr int TK = C::TK;
+    constexpr int TK = C::TK, THREADS = C::THREADS, TMA_WARP = C::TMA_WARP, MMA_WARP = C::MMA_WARP;
     extern __shared__ uint8_t sm_raw[];
     uint8_t* sm = sm_raw + ((1024u - (smem_u32(sm_raw) & 1023u)) & 1023u);
     uint8_t* Qs = sm;                                            // hi, then lo: [HB][RP][128 bytes]
-    uint8_t* Ps = Qs + 2 * C::Q_BYTES;                           // hi, then lo: [TK / 64][RP][128 bytes]
-    uint8_t* ring = Ps + 2 * C::P_BYTES;                         // [stages] K [HB][TK][128 bytes], V the same
+    uint8_t* ring = Qs + 2 * C::Q_BYTES;                         // [stages] K [HB][TK][128 bytes], V the same
     __shared__ int s_pages[MAX_PAGES];
     __shared__ float s_max[2][2][RP], s_sum[2][RP];
-    __shared__ uint64_t s_bars[4 * MAX_RING + 10];
+    __shared__ uint64_t s_bars[4 * MAX_RING + 9];
     __shared__ uint32_t s_tmem;
     __shared__ int s_fail;
     volatile int* failed = &s_fail;
@@ -148,14 +153,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
 
     const uint32_t bar_k_full = smem_u32(s_bars), bar_v_full = bar_k_full + 8u * MAX_RING;
     const uint32_t bar_k_empty = bar_v_full + 8u * MAX_RING, bar_v_empty = bar_k_empty + 8u * MAX_RING;
-    const uint32_t bar_s_full = bar_v_empty + 8u * MAX_RING, bar_s_empty = bar_s_full + 16u;
-    const uint32_t bar_o_full = bar_s_empty + 16u, bar_o_empty = bar_o_full + 16u;
-    const uint32_t bar_p_full = bar_o_empty + 16u, bar_q_full = bar_p_full + 8u;
-    if (warp == SM_WARPS) {
-        // a barrier per lane, in the order of their addresses: the ring's, S full, S empty, O full, O empty (two each), P, Q
+    const uint32_t bar_s_full = bar_v_empty + 8u * MAX_RING, bar_p_full = bar_s_full + 16u;
+    const uint32_t bar_o_full = bar_p_full + 16u, bar_o_empty = bar_o_full + 16u, bar_q_full = bar_o_empty + 16u;
+    if (warp == TMA_WARP) {
+        // a barrier per lane, in the order of their addresses: the ring's, S full, P full, O full, O empty (two each), Q
         constexpr int RING = 4 * MAX_RING;
-        if (lane < RING + 10)
-            mbar_init(bar_k_full + 8u * lane, lane == RING + 9 ? SM_WARPS * 32u : lane == RING + 8 || (lane >= RING && ((lane - RING) & 2)) ? arrivals : 1u);
+        if (lane < RING + 9)
+            mbar_init(bar_k_full + 8u * lane, lane == RING + 8 ? (uint32_t)C::LOADERS : lane >= RING && ((lane - RING) & 2) ? arrivals : 1u);
         if (lane == 31) {
             s_fail = 0;
             tma_prefetch_desc(&tmK);
@@ -170,7 +174,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         if (pslot < a.max_pages) page = a.block_table[(size_t)b * a.max_pages + pslot];
         s_pages[i] = (page >= 0 && page < a.n_pages) ? page : -1;      // ids outside the pool are never used as addresses
     }
-    if (warp == SM_WARPS + 1) {
+    if (warp == MMA_WARP) {
         tmem_alloc(smem_u32(&s_tmem), (uint32_t)C::COLS);
         tmem_relinquish();
     }
@@ -193,9 +197,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     float m_run = -INFINITY, l_run = 0.f;
     const int quarter = warp & 3, half = (warp >> 2) & 1;
     const int rho = quarter * 32 + lane;                         // row of the query tile = TMEM lane
-    const bool active = warp < SM_WARPS && quarter < quarters;
+    const bool active = warp < SM_WARPS && warp != TMA_WARP && warp != MMA_WARP && quarter < quarters;
 
-    if (warp == SM_WARPS) {
+    if (warp == TMA_WARP) {
         // ------------------------------------------------------------ TMA
         // A tile is TK / 16 pages; a page of this KV head is one box (two for 128-wide heads) of K and one of V.  Rows past the
         // range re-read its last page, ids outside the pool read page 0: both are masked, and nothing unmapped is touched.
@@ -231,14 +235,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         }
         if (!waited) griddep_wait();
         __syncwarp();
-    } else if (warp == SM_WARPS + 1) {
+    } else if (warp == MMA_WARP) {
         // ------------------------------------------------------------ MMA
         // (the whole warp, see umma_bf16_warp)
         if (n_tiles > 0) {
-            const uint32_t qa = smem_u32(Qs), pa = smem_u32(Ps), kv = smem_u32(ring);
+            const uint32_t qa = smem_u32(Qs), kv = smem_u32(ring);
             constexpr uint32_t idesc_s = umma_idesc_bf16_f32(128, TK);
             constexpr uint32_t idesc_o = umma_idesc_bf16_f32(128, HD) | (1u << 16);      // V: columns along N
-            const uint64_t dq = umma_desc_k_sw128(qa), dp = umma_desc_k_sw128(pa);
+            const uint64_t dq = umma_desc_k_sw128(qa);
             wait(bar_q_full, 0u);
             int sk = 0, sv = 0;                                  // ring slots of the next K and V tiles, and their parities
             uint32_t pk = 0u, pv = 0u;
@@ -247,7 +251,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                 if (t + 1 < n_tiles) {
                     const int u = t + 1;                         // S of the next tile
                     wait(bar_k_full + 8u * sk, pk);
-                    if (u >= 2) wait(bar_s_empty + 8u * (u & 1), (uint32_t)((u >> 1) - 1) & 1u);
+                    // (S and P of tile u - 2 were there: P V of that tile was issued, and MMAs run in order)
                     tc_fence_after();
                     const uint64_t dk = umma_desc_k_sw128(kv + (uint32_t)sk * 2u * C::KV_BYTES);
                     const uint32_t d = tmem + C::S_COL + (uint32_t)(u & 1) * TK;
@@ -264,7 +268,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                 }
                 if (t < 0) continue;
                 wait(bar_v_full + 8u * sv, pv);
-                wait(bar_p_full, (uint32_t)t & 1u);
+                wait(bar_p_full + 8u * (t & 1), (uint32_t)(t >> 1) & 1u);
                 if (t >= 2) wait(bar_o_empty + 8u * (t & 1), (uint32_t)((t >> 1) - 1) & 1u);
                 tc_fence_after();
                 const uint64_t dv = umma_desc_mn_sw128(kv + (uint32_t)sv * 2u * C::KV_BYTES + C::KV_BYTES, TK * 128);
@@ -273,9 +277,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                 for (int p = 0; p < 2; ++p)
 #pragma unroll
                     for (int kk = 0; kk < TK / 16; ++kk)
-                        umma_bf16_warp(d, dp + (p * C::P_BYTES + (kk >> 2) * (RP * 128) + (kk & 3) * 32) / 16, dv + kk * (16 * 128 / 16), idesc_o,
-                                       (p | kk) ? 1u : 0u);
-                umma_commit_warp(bar_o_full + 8u * (t & 1));          // also: P is free
+                        umma_bf16_ts_warp(d, tmem + C::S_COL + (uint32_t)((t & 1) * TK + p * (TK / 2) + kk * 8), dv + kk * (16 * 128 / 16), idesc_o,
+                                          (p | kk) ? 1u : 0u);
+                umma_commit_warp(bar_o_full + 8u * (t & 1));
                 umma_commit_warp(bar_v_empty + 8u * sv);
                 if (++sv == a.stages) { sv = 0; pv ^= 1u; }
             }
@@ -290,20 +294,21 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         griddep_launch_dependents();
         // Q rows, scaled, as (hi, lo) in shared memory; zeros where there is no row
         {
-            constexpr int RPI = SM_WARPS * 32 / (HD / 4);        // rows of one reading of all threads; four readings under way together
-            const int d4 = (tid % (HD / 4)) * 4, chunk = (d4 & 63) >> 3;
+            constexpr int RPI = C::LOADERS / (HD / 4);           // rows of one reading of all threads; four readings under way together
+            const int li = warp > MMA_WARP ? tid - 64 : tid, d4 = (li % (HD / 4)) * 4, chunk = (d4 & 63) >> 3;
 #pragma unroll 1
-            for (int r0 = tid / (HD / 4); r0 < RP; r0 += 4 * RPI) {
+            for (int r0 = li / (HD / 4); r0 < RP; r0 += 4 * RPI) {
                 float4 qv[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int r = r0 + j * RPI, hl = head_of(r), rr = r - hl * R;
+                    const int r = r0 + j * RPI, hl = head_of(r), rr = r - hl * R;      // (rows past the tile: not stored)
                     qv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (r < G && rr < rows) qv[j] = *reinterpret_cast<const float4*>(a.q + (size_t)(b * a.R + rb + rr) * qd + (size_t)(h0 + hl) * HD + d4);
                 }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int r = r0 + j * RPI;
+                    if (RP % (4 * RPI) && r >= RP) break;
                     uint2 h, l;
                     split_bf16x2(qv[j].x * a.scale_log2e, qv[j].y * a.scale_log2e, h.x, l.x);
                     split_bf16x2(qv[j].z * a.scale_log2e, qv[j].w * a.scale_log2e, h.y, l.y);
@@ -360,7 +365,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                         for (int e = 0; e < 32; ++e) s[c + e] = __uint_as_float(r[e]);
                     }
                     tc_fence_before();
-                    mbar_arrive(bar_s_empty + 8u * (t & 1));
                     const int k0 = k_begin + t * TK + half * SC;
                     if (k0 + SC - 1 > lim) {
 #pragma unroll
@@ -379,25 +383,22 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
 #pragma unroll
                     for (int e = 0; e < SC; ++e) { s[e] = ex2(s[e] - mu); p4[e & 3] += s[e]; }
                     l_run = l_run * al + ((p4[0] + p4[1]) + (p4[2] + p4[3]));
-                }
-                if (t > 0) add_o(t - 1);                         // (P of tile t - 1 has been used: its place is free)
-                if (t == n_tiles) break;
-                al_o = al;
-                // P, half row: 16-byte chunks of eight keys
+                    // P, half row, in the place of S (which both threads of the row have read: the barrier above): hi, then lo
 #pragma unroll
-                for (int c = 0; c < SC / 8; ++c) {
-                    uint4 h, l;
-                    split_bf16x2(s[8 * c], s[8 * c + 1], h.x, l.x);
-                    split_bf16x2(s[8 * c + 2], s[8 * c + 3], h.y, l.y);
-                    split_bf16x2(s[8 * c + 4], s[8 * c + 5], h.z, l.z);
-                    split_bf16x2(s[8 * c + 6], s[8 * c + 7], h.w, l.w);
-                    const int kc = half * (SC / 8) + c;          // chunk of the row
-                    const uint32_t off = (uint32_t)((kc >> 3) * (RP * 128) + rho * 128 + (((kc & 7) ^ (rho & 7)) << 4));
-                    *reinterpret_cast<uint4*>(Ps + off) = h;
-                    *reinterpret_cast<uint4*>(Ps + C::P_BYTES + off) = l;
+                    for (int c = 0; c < SC; c += 16) {
+                        uint32_t h[8], l[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) split_bf16x2(s[c + 2 * e], s[c + 2 * e + 1], h[e], l[e]);
+                        const uint32_t to = lane_base + C::S_COL + (uint32_t)((t & 1) * TK + (half * SC + c) / 2);
+                        tmem_st8(to, h);
+                        tmem_st8(to + TK / 2, l);
+                    }
+                    tmem_st_wait();
+                    tc_fence_before();
+                    mbar_arrive(bar_p_full + 8u * (t & 1));
                 }
-                fence_proxy_async_smem();
-                mbar_arrive(bar_p_full);
+                if (t > 0) add_o(t - 1);
+                al_o = al;
             }
             s_sum[half][rho] = l_run;
             asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory");
@@ -415,7 +416,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         while (clock64() - t0 < 2000000ll) { }
     }
     __syncthreads();
-    if (warp == SM_WARPS + 1) {
+    if (warp == MMA_WARP) {
         tc_fence_after();
         tmem_dealloc(tmem, (uint32_t)C::COLS);
     }
@@ -505,7 +506,7 @@ bool prepare() {
 template <int HD, int RP>
 void config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[2], int splits, int n_kv, int B, int stages) {
     cfg.gridDim = dim3((unsigned)splits, (unsigned)n_kv, (unsigned)B);
-    cfg.blockDim = dim3(THREADS, 1, 1);
+    cfg.blockDim = dim3(Tc<HD, RP>::THREADS, 1, 1);
     cfg.dynamicSmemBytes = (size_t)Tc<HD, RP>::smem(stages);
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -563,14 +564,16 @@ template <int HD, int RP> int ring_stages() {
 // dictates (one CTA per SM), the merge of split ranges.  The other kernel's cost is p.cost, and no less than what all its slabs
 // take of the SMs' mma.sync pipes.  T0 as measured against the other kernel, which starts faster since its code was cut: a step
 // of the 1.5B, 3 x 7 rows behind 400 keys, 1169 us here, 1121 there; 10 x 8 rows of the 0.5B 893 / 877; 1.5B 40 x 5 rows 2512 / 2549,
-// 0.5B + 8,192 tokens 32 x 9 rows behind 640 keys 1441 / 1440.  It pays for many (sequence, KV head) pairs with long contexts and three
+// 0.5B + 8,192 tokens 32 x 9 rows behind 640 keys 1441 / 1440.  (T0 was 3.9 and 2.8, a tile 1.8 and 1.4, before P was in TMEM: a step of the
+// 0.5B, 32 x 9 rows behind 1,000 keys, was left with the other kernel then, 1445 us, 1409 here.  With T0 as it was a step of 2 x 7 rows
+// behind 900 keys came here, 699 us instead of 660, and one of 7 x 4 rows behind 560, 680 instead of 666.)  It pays for many (sequence, KV head) pairs with long contexts and three
 // or more slabs of query rows, hardly ever at the 135M's 18 to 27 rows.
 bool plan_attention_tc(int B, int n_kv, int hd, int g, int rows, int max_ctx, int page_size, AttnPlan& p) {
     const int G = g * rows;
     if ((hd != 64 && hd != 128) || page_size != PAGE || G > 128 || max_ctx / PAGE > MAX_PAGES) return false;
     const bool small = G <= 64;
-    const int tk = small ? 128 : 64;
-    const float T0 = hd == 128 ? 3.9f : 2.8f, per_tile = hd == 128 ? (small ? 1.8f : 1.4f) : (small ? 1.4f : 1.1f);
+    constexpr int tk = 128;
+    const float T0 = hd == 128 ? 4.3f : 3.2f, per_tile = hd == 128 ? (small ? 1.6f : 1.8f) : (small ? 1.2f : 1.4f);
     const int groups = B * n_kv, tiles_all = std::max(1, (max_ctx + tk - 1) / tk), tiles_34 = std::max(1, (max_ctx * 3 / 4 + tk - 1) / tk);
     const float pipes = (hd == 128 ? 0.6f : 0.3f) * (float)groups * (float)((G + 15) / 16) * (float)((max_ctx * 3 / 4 + 63) / 64) / 148.f;
     int best = 0;

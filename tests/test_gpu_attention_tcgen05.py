@@ -1,0 +1,31 @@
+"""The tcgen05 attention: query tiles of up to 64 and up to 128 rows, 64- and 128-wide heads, contexts that end just before, at and just behind
+a tile of 128 keys, one key range and several, ranges of one, two and more tiles (the two places of S and P, and of O, are used in
+turn), a ragged batch; the oracle runs the first and the last sequence."""
+from dataclasses import replace
+
+import pytest
+
+from tests.gpu_harness import lockstep, make_setup
+from tests.test_gpu_verify import BF16_TOL, check
+from workload import configs, corpus
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("hd,n_q,n_kv,B,k,P", [
+    (64, 14, 2, 34, 8, 127),        # 63 rows
+    (64, 14, 2, 34, 7, 128),        # 56 rows
+    (64, 16, 2, 34, 7, 249),        # 64 rows: a full tile
+    (64, 16, 2, 34, 8, 250),        # 72 rows: the wider one
+    (64, 16, 2, 20, 15, 385),        # 128 rows
+    (128, 12, 2, 40, 4, 126),       # 30 rows
+    (128, 12, 2, 66, 6, 260),       # 42 rows
+    (128, 12, 2, 30, 8, 700),       # 54 rows, split
+    (128, 16, 2, 34, 8, 383),       # 72 rows
+    (128, 16, 2, 24, 15, 640),       # 128 rows
+])
+def test_tiles_and_key_ranges(hd, n_q, n_kv, B, k, P):
+    base = configs.shrunk(configs.get(2), n_layers=2, vocab=4096, n_docs=500, d_ff=1024)
+    cfg = replace(base, model=replace(base.model, d_model=n_q * hd, n_q_heads=n_q, n_kv_heads=n_kv, head_dim=hd), prompt_len=P)
+    s = make_setup(cfg)
+    rep = lockstep(s, corpus.make_prompts(cfg, B, prompt_len=P), k + 3, k, oracle_rows=sorted({0, B - 1}), **BF16_TOL)
+    check(rep, f"tcgen05 attention, heads of {hd}, {n_q} / {n_kv}, B={B} k={k} P={P}")
