@@ -53,6 +53,7 @@ struct TcArgs {
     int TB;
     int R, Rs, n_sub, n_q, n_kv, splits, stages;
     int g;                                                       // query heads of a KV head
+    int push_rows;                                               // split key ranges: query rows per CTA of the cluster, whose shares are stored into its shared memory; 0: fetched
     SmallDiv by_R, by_TB, by_splits, by_sub;
     int* status;
     float scale_log2e;
@@ -140,6 +141,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         }
         return;
     }
+    if (a.push_rows) cluster_arrive();                           // (nothing is stored to a CTA that has not started)
     // this CTA's keys: the tiles are dealt out evenly over the splits
     const int total = pos0 + rows;
     const int tiles_all = (total + TK - 1) / TK, t_base = a.by_splits.div(tiles_all), t_rem = tiles_all - t_base * a.splits;
@@ -438,32 +440,45 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         }
         return;
     }
-    // Every CTA of the cluster parks its unnormalised rows in its shared memory; CTA r merges the rows r, r + S, ...
-    constexpr int XS = HD + 4;                                   // floats per parked row: O, maximum, sum, padding
-    float* xo = reinterpret_cast<float*>(ring);
+    // CTA r of the cluster merges the rows r, r + S, ...: the others' shares of them are stored into its shared memory, behind the ring.  Where there
+    // is no room for that every CTA parks its rows in its own ring, and the mergers fetch them, which takes a barrier more and a trip on the chain: steps
+    // of the 0.5B, 32 x 9 rows behind 1,000 keys, 1,409 -> 1,400 us, of the 1.5B, 24 x 7 rows, 2,411 -> 2,400.
+    constexpr int XS = HD + 4;                                   // floats per row: O, maximum, sum, padding
+    const int S = a.splits, rank = (int)cluster_ctarank(), push = a.push_rows;
+    const uint32_t parked = smem_u32(ring), given = parked + (uint32_t)a.stages * 2u * C::KV_BYTES;      // given: [S][push_rows][XS]
+    __syncwarp();
+    if (push) cluster_wait();
     if (active && rho < G) {
+        if (push) {
+            const int at = a.by_splits.div(rho);
+            const uint32_t to = cluster_map(given + (uint32_t)((rank * push + at) * XS) * 4u, (uint32_t)(rho - at * S));
 #pragma unroll
-        for (int e = 0; e < OC; e += 4) *reinterpret_cast<float4*>(xo + (size_t)rho * XS + col0 + e) = make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
-        if (half == 0) *reinterpret_cast<float2*>(xo + (size_t)rho * XS + HD) = make_float2(m_run, l_run);
+            for (int e = 0; e < OC; e += 4) st_cluster_f4(to + (uint32_t)(col0 + e) * 4u, make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]));
+            if (half == 0) st_cluster_f2(to + HD * 4u, m_run, l_run);
+        } else {
+            float* to = reinterpret_cast<float*>(ring) + (size_t)rho * XS;
+#pragma unroll
+            for (int e = 0; e < OC; e += 4) *reinterpret_cast<float4*>(to + col0 + e) = make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
+            if (half == 0) *reinterpret_cast<float2*>(to + HD) = make_float2(m_run, l_run);
+        }
     }
+    __syncwarp();
     cluster_arrive();
     cluster_wait();
-    const int S = a.splits, rank = (int)cluster_ctarank();
-    uint32_t peer[8];
-#pragma unroll
-    for (int s = 0; s < 8; ++s) peer[s] = cluster_map(smem_u32(xo), (uint32_t)(s < S ? s : 0));
 #pragma unroll 1
-    for (int r = rank + tid / (HD / 4) * S; r < G; r += THREADS / (HD / 4) * S) {
-        const int d4 = (tid % (HD / 4)) * 4;
+    for (int at = tid / (HD / 4); at * S + rank < G; at += THREADS / (HD / 4)) {
+        const int r = at * S + rank, d4 = (tid % (HD / 4)) * 4;
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
         if (row_of(r) < rows) {
             float2 ml[8];
             float4 ov[8];
 #pragma unroll
             for (int s = 0; s < 8; ++s)
-                if (s < S) {                                     // all remote reads are issued before the first is used
-                    ml[s] = ld_cluster_f2(peer[s] + (uint32_t)(r * XS + HD) * 4u);
-                    ov[s] = ld_cluster_f4(peer[s] + (uint32_t)(r * XS + d4) * 4u);
+                if (s < S) {                                     // all reads are issued before the first is used
+                    const uint32_t from = push ? cluster_map(given + (uint32_t)((s * push + at) * XS) * 4u, (uint32_t)rank)
+                                               : cluster_map(parked + (uint32_t)(r * XS) * 4u, (uint32_t)s);
+                    ml[s] = ld_cluster_f2(from + HD * 4u);
+                    ov[s] = ld_cluster_f4(from + (uint32_t)d4 * 4u);
                 }
             float top = -INFINITY, den = 0.f;
 #pragma unroll
@@ -485,6 +500,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         *reinterpret_cast<uint2*>(a.out + row * qd + col) = h;
         *reinterpret_cast<uint2*>(a.out + (row + a.TB) * qd + col) = l;
     }
+    if (push) return;                                            // (its shared memory is its own again)
+    __syncwarp();
     cluster_arrive();                                            // peers may still be reading this CTA's rows
     cluster_wait();
 }
@@ -519,11 +536,14 @@ void config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[2], int splits, i
 }
 
 template <int HD, int RP>
-tasc_status launch_inst(const TcArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int B, cudaStream_t stream) {
+tasc_status launch_inst(TcArgs a, const CUtensorMap& tmK, const CUtensorMap& tmV, int B, cudaStream_t stream) {
     if (!prepare<HD, RP>()) return TASC_ECUDA;
+    const int share = (a.g * a.Rs + a.splits - 1) / a.splits;
+    a.push_rows = a.splits > 1 && Tc<HD, RP>::smem(a.stages) + share * a.splits * (HD + 4) * 4 <= MAX_SMEM ? share : 0;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[2];
     config<HD, RP>(cfg, at, a.splits, a.n_kv, B, a.stages);
+    cfg.dynamicSmemBytes += (size_t)a.push_rows * a.splits * (HD + 4) * 4;
     cfg.stream = stream;
     ProfScope ps(K_ATT_SPLIT, stream);
     TASC_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD, RP>, tmK, tmV, a));
