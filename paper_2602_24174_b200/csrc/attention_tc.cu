@@ -53,7 +53,8 @@ struct TcArgs {
     int TB;
     int R, Rs, n_sub, n_q, n_kv, splits, stages;
     int g;                                                       // query heads of a KV head
-    int push_rows;                                               // split key ranges: query rows per CTA of the cluster, whose shares are stored into its shared memory; 0: fetched
+    // split key ranges: query rows per CTA of the cluster, whose shares are stored into its shared memory; 0: fetched
+    int push_rows;
     SmallDiv by_R, by_TB, by_splits, by_sub;
     int* status;
     float scale_log2e;
@@ -585,9 +586,9 @@ template <int HD, int RP> int ring_stages() {
 // take of the SMs' mma.sync pipes.  T0 as measured against the other kernel, which starts faster since its code was cut: a step
 // of the 1.5B, 3 x 7 rows behind 400 keys, 1169 us here, 1121 there; 10 x 8 rows of the 0.5B 893 / 877; 1.5B 40 x 5 rows 2512 / 2549,
 // 0.5B + 8,192 tokens 32 x 9 rows behind 640 keys 1441 / 1440.  (T0 was 3.9 and 2.8, a tile 1.8 and 1.4, before P was in TMEM: a step of the
-// 0.5B, 32 x 9 rows behind 1,000 keys, was left with the other kernel then, 1445 us, 1409 here.  With T0 as it was a step of 2 x 7 rows
-// behind 900 keys came here, 699 us instead of 660, and one of 7 x 4 rows behind 560, 680 instead of 666.)  It pays for many (sequence, KV head) pairs with long contexts and three
-// or more slabs of query rows, hardly ever at the 135M's 18 to 27 rows.
+// 0.5B, 32 x 9 rows behind 1,000 keys, was left with the other kernel then, 1445 us, 1409 here.  With shorter tiles and T0 as it was a step of
+// 2 x 7 rows behind 900 keys came here, 699 us, 648 there.)  It pays for many (sequence, KV head) pairs with long contexts and three or
+// more slabs of query rows, hardly ever at the 135M's 18 to 27 rows.
 bool plan_attention_tc(int B, int n_kv, int hd, int g, int rows, int max_ctx, int page_size, AttnPlan& p) {
     const int G = g * rows;
     if ((hd != 64 && hd != 128) || page_size != PAGE || G > 128 || max_ctx / PAGE > MAX_PAGES) return false;
