@@ -558,8 +558,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             if ((lane & 3) == 0) st_cluster_f2(dst + HD * 4u, m_run[half], l_run[half]);
         }
     }
-    cluster_arrive();
-    cluster_wait();
+    cluster_sync();
     uint32_t peer[8];
 #pragma unroll
     for (int sidx = 0; sidx < 8; ++sidx)
@@ -603,8 +602,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     }
     if (push) return;
     // peers may still be reading this CTA's parked rows
-    cluster_arrive();
-    cluster_wait();
+    cluster_sync();
 }
 
 inline size_t attn_smem_bytes(int hd, int gp, int stages) {

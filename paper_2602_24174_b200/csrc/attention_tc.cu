@@ -179,7 +179,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     }
     if (warp == MMA_WARP) {
         tmem_alloc(smem_u32(&s_tmem), (uint32_t)C::COLS);
-        tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
@@ -447,7 +446,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     constexpr int XS = HD + 4;                                   // floats per row: O, maximum, sum, padding
     const int S = a.splits, rank = (int)cluster_ctarank(), push = a.push_rows;
     const uint32_t parked = smem_u32(ring), given = parked + (uint32_t)a.stages * 2u * C::KV_BYTES;      // given: [S][push_rows][XS]
-    __syncwarp();
     if (push) cluster_wait();
     if (active && rho < G) {
         if (push) {
@@ -463,9 +461,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
             if (half == 0) *reinterpret_cast<float2*>(to + HD) = make_float2(m_run, l_run);
         }
     }
-    __syncwarp();
-    cluster_arrive();
-    cluster_wait();
+    cluster_sync();
 #pragma unroll 1
     for (int at = tid / (HD / 4); at * S + rank < G; at += THREADS / (HD / 4)) {
         const int r = at * S + rank, d4 = (tid % (HD / 4)) * 4;
@@ -502,9 +498,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         *reinterpret_cast<uint2*>(a.out + (row + a.TB) * qd + col) = l;
     }
     if (push) return;                                            // (its shared memory is its own again)
-    __syncwarp();
-    cluster_arrive();                                            // peers may still be reading this CTA's rows
-    cluster_wait();
+    cluster_sync();                                            // peers may still be reading this CTA's rows
 }
 
 template <int HD, int RP>

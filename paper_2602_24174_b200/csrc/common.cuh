@@ -187,9 +187,20 @@ __device__ __forceinline__ uint32_t cluster_nctarank() {
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
     return r;
 }
-// Every thread of every CTA of the cluster must execute both halves, warp-convergently.
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// Every thread of every CTA of the cluster executes both halves.  (They are .aligned: a warp has to reach them as one, and behind a branch or a
+// loop that its lanes leave one by one it is left to the compiler where they meet again.  So they meet here.)
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The same for warps that are one already: behind a warp-wide barrier, with nothing in between that depends on the lane.  (The few-row GEMM's 90 to
+// 120 launches of a step: 0.5B, prefill of 100 tokens 834 us, 840 where the lanes meet again at each of its barriers; 135M, 256 tokens 848 / 852.)
+__device__ __forceinline__ void cluster_arrive_converged() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync_converged() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 // Address of this CTA's shared-memory location `addr` in the CTA of rank `rank` of the cluster.
 __device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
     uint32_t r;
@@ -280,14 +291,14 @@ __device__ __forceinline__ uint64_t policy_evict_last() {
 }
 
 // ---------------------------------------------------------------- tcgen05 (5th-gen tensor cores, TMEM)
-// Allocate `ncols` (power of two, 32..512) TMEM columns; executed by one full warp.
+// Allocate `ncols` (power of two, 32..512) TMEM columns, and let others; executed by one full warp, as one (.aligned, see cluster_arrive).
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish() {
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    __syncwarp();
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n\ttcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;"
+                 ::"r"(smem_dst), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
+    __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -357,14 +368,14 @@ __device__ __forceinline__ void umma_commit_warp(uint32_t bar) {
 }
 // ---- and on a pair of CTAs (cluster ranks 2 i and 2 i + 1): one MMA of both SMs' tensor cores, issued by the even CTA.  Each
 // CTA supplies its own half of A's rows and of B's rows from its shared memory (same offsets) and holds its half of D's rows.
-// Allocation, release and relinquishing are executed by one warp of either CTA.
+// Allocation and release are executed by one warp of either CTA.
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t smem_dst, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish_pair() {
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    __syncwarp();
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n\ttcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;"
+                 ::"r"(smem_dst), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+    __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void umma_bf16_pair_warp(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {

@@ -296,7 +296,6 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
         __syncwarp();
     } else if (warp == 5) {
         tmem_alloc(smem_u32(tmem_slot), ncols);
-        tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
@@ -425,9 +424,9 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
     if (threadIdx.x == 0) g_tc = global_ns();
 #endif
     tc_fence_before();
-    // every CTA's partial tile is in its shared memory (release / acquire at cluster scope)
-    cluster_arrive();
-    cluster_wait();
+    // every CTA's partial tile is in its shared memory (release / acquire at cluster scope; the lanes of warps 0 to 3 have met at their barrier,
+    // those of 4 and 5 behind their branches)
+    cluster_sync_converged();
     if (threadIdx.x == 0) TL(8);
 #ifdef TASC_TIMELINE
     if (threadIdx.x == 0) g_td = global_ns();
@@ -472,7 +471,7 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
     if (threadIdx.x == 0) g_te = global_ns();
 #endif
     // this CTA has finished reading its peers' shared memory; they may leave while it runs the epilogue
-    cluster_arrive();
+    cluster_arrive_converged();
     if (EPI != EPI_LM) {
 #pragma unroll 1
         for (int tl = warp; tl < count; tl += EW) {

@@ -79,7 +79,6 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     }
     if (warp == 5) {
         tmem_alloc(smem_u32(tmem_slot), ncols);
-        tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();

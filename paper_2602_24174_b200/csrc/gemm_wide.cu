@@ -153,8 +153,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         tma_prefetch_desc(&tmX);
     }
     if (warp == EPI_WARPS + 1) {
-        if (PAIR) { tmem_alloc_pair(smem_u32(&s_tmem), (uint32_t)(2 * BNW)); tmem_relinquish_pair(); }
-        else { tmem_alloc(smem_u32(&s_tmem), (uint32_t)(2 * BNW)); tmem_relinquish(); }
+        if (PAIR) tmem_alloc_pair(smem_u32(&s_tmem), (uint32_t)(2 * BNW)); else tmem_alloc(smem_u32(&s_tmem), (uint32_t)(2 * BNW));
     }
     if (warp == 0 && a.seq_rows) {
         if (!a.rows_early) griddep_wait();
@@ -165,7 +164,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     }
     tc_fence_before();
     __syncthreads();
-    if (PAIR) { cluster_arrive(); cluster_wait(); }              // both CTAs' barriers are set up before either is signalled
+    if (PAIR) cluster_sync();                                    // both CTAs' barriers are set up before either is signalled
     tc_fence_after();
     const uint32_t tmem_base = s_tmem;
     const int live_tt = a.seq_rows ? s_n_tt : a.n_tt;
@@ -553,8 +552,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 #ifdef TASC_TIMELINE
         g_tc = global_ns();
 #endif
-        cluster_arrive();
-        cluster_wait();
+        cluster_sync();
 #ifdef TASC_TIMELINE
         g_td = global_ns();
 #endif
@@ -613,8 +611,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         g_te = global_ns();
 #endif
         // peers may still be reading this CTA's partial tile
-        cluster_arrive();
-        cluster_wait();
+        cluster_sync();
     }
 #ifdef TASC_TIMELINE
     g_tf = global_ns();
@@ -626,7 +623,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         while (clock64() - t0 < 2000000ll) { }
     }
     __syncthreads();
-    if (PAIR) { cluster_arrive(); cluster_wait(); }              // neither CTA leaves while the other may signal or read it
+    if (PAIR) cluster_sync();                                    // neither CTA leaves while the other may signal or read it
     if (warp == EPI_WARPS + 1) {
         tc_fence_after();
         if (PAIR) tmem_dealloc_pair(tmem_base, (uint32_t)(2 * BNW)); else tmem_dealloc(tmem_base, (uint32_t)(2 * BNW));
