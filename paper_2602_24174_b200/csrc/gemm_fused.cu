@@ -408,11 +408,10 @@ gemm_fused_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
 #pragma unroll 1
             for (int c = 0; c < TBL; c += 16) {                 // TBL is a multiple of 16
                 uint32_t r[16], r2[16];
-                if (have) {
-                    tmem_ld16(lane_base + col0 + (uint32_t)c, r);
-                    tmem_ld16(lane_base + col0 + (uint32_t)(TBL + c), r2);
-                    tmem_ld_wait();
-                }
+                // (by the whole warp whatever its lanes' waits said)
+                tmem_ld16(lane_base + col0 + (uint32_t)c, r);
+                tmem_ld16(lane_base + col0 + (uint32_t)(TBL + c), r2);
+                tmem_ld_wait();
 #pragma unroll
                 for (int j = 0; j < 16; ++j)
                     xch[(lt * TBL + c + j) * BM + fl] = have ? __uint_as_float(r[j]) + __uint_as_float(r2[j]) : 0.f;

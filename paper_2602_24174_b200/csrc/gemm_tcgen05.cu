@@ -135,26 +135,23 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         const bool f_ok = f < a.N;
         for (int c = 0; c < TBk / 16; ++c) {
             uint32_t r[16];
-            if (have) {
-                const uint32_t lane_base = tmem_base + ((uint32_t)(warp * 32) << 16);
-                tmem_ld16(lane_base + (uint32_t)(c * 16), r);
-                if (a.pair) {
-                    uint32_t r2[16];
-                    tmem_ld16(lane_base + (uint32_t)(TBk + c * 16), r2);
-                    tmem_ld_wait();
+            const uint32_t lane_base = tmem_base + ((uint32_t)(warp * 32) << 16);
+            // (by the whole warp whatever its lanes' waits said)
+            __syncwarp();
+            tmem_ld16(lane_base + (uint32_t)(c * 16), r);
+            if (a.pair) {
+                uint32_t r2[16];
+                tmem_ld16(lane_base + (uint32_t)(TBk + c * 16), r2);
+                tmem_ld_wait();
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(r2[j]));
-                } else {
-                    tmem_ld_wait();
-                }
+                for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(r2[j]));
             } else {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) r[j] = 0u;
+                tmem_ld_wait();
             }
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 const int m = t0 + c * 16 + j;
-                if (f_ok && m < a.M) a.partials[((size_t)split * a.M + m) * a.N + f] = __uint_as_float(r[j]);
+                if (f_ok && m < a.M) a.partials[((size_t)split * a.M + m) * a.N + f] = have ? __uint_as_float(r[j]) : 0.f;
             }
         }
     }

@@ -27,3 +27,11 @@ def test_the_flag_is_read_by_vote_where_the_whole_warp_loads_tiles():
     assert len(re.findall(r"if \(warp_failed\(failed\)\) break;", text)) == 2
     vote = "".join(code_lines(os.path.join(CSRC, "common.cuh")))
     assert re.search(r"bool warp_failed\([^)]*\)\s*\{\s*return __any_sync\(0xFFFFFFFFu, \*failed != 0\);", vote)
+
+
+@pytest.mark.parametrize("name", ["gemm_fused.cu", "gemm_tcgen05.cu"])
+def test_the_accumulator_is_read_by_the_whole_warp(name):
+    """A lane whose own wait for it ran out would stay away from the warp-wide loads that the others go on to: they depend on no lane's wait."""
+    text = "".join(code_lines(os.path.join(CSRC, name)))
+    assert len(re.findall(r"\bhave\b[^;]*mbar_wait\(bar_acc, 0\)|mbar_wait\(bar_acc, 0\)[^;]*;[^;]*\bhave\b", text)) == 1
+    assert "tmem_ld16(" in text and not re.search(r"if \(have\) \{[^{}]*tmem_ld", text)
