@@ -253,7 +253,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                 if (t + 1 < n_tiles) {
                     const int u = t + 1;                         // S of the next tile
                     wait(bar_k_full + 8u * sk, pk);
-                    // (S and P of tile u - 2 were there: P V of that tile was issued, and MMAs run in order)
+                    // S and P of tile u - 2 were there: until P V of that tile is done.  (MMAs of one accumulator and shape follow one another;
+                    // these have two accumulators, and the one reads what the other writes.)
+                    if (u >= 2) wait(bar_o_full + 8u * (u & 1), (uint32_t)((u >> 1) - 1) & 1u);
                     tc_fence_after();
                     const uint64_t dk = umma_desc_k_sw128(kv + (uint32_t)sk * 2u * C::KV_BYTES);
                     const uint32_t d = tmem + C::S_COL + (uint32_t)(u & 1) * TK;
@@ -335,6 +337,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
             // as often.)
             auto add_o = [&](int t) {
                 wait(bar_o_full + 8u * (t & 1), (uint32_t)(t >> 1) & 1u);
+                __syncwarp();                                    // (a lane waits by itself, TMEM is read by the warp as one)
                 tc_fence_after();
 #pragma unroll
                 for (int c = 0; c < OC; c += 32) {
@@ -357,6 +360,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
 #ifdef TASC_TIMELINE
                     if (t == 0) log_at_exit.td = global_ns();
 #endif
+                    __syncwarp();
                     tc_fence_after();
 #pragma unroll
                     for (int c = 0; c < SC; c += 32) {
@@ -378,6 +382,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                     const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
                     s_max[t & 1][half][rho] = mx;
                     asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory");      // the quarter's two warps
+                    tc_fence_after();                                // (P goes where the other warp has read S)
                     const float mn = fmaxf(m_run, fmaxf(mx, s_max[t & 1][half ^ 1][rho])), mu = mn == -INFINITY ? 0.f : mn;
                     al = ex2(m_run - mu);                            // 0 while nothing was visible
                     m_run = mn;
