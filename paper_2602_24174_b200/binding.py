@@ -132,6 +132,8 @@ lib.tasc_profile_read.argtypes = [C.POINTER(C.c_double), C.POINTER(C.c_int64), C
 lib.tasc_profile_read.restype = C.c_int32
 lib.tasc_launch_counts.argtypes = [C.POINTER(C.c_int64), C.c_int32]
 lib.tasc_launch_counts.restype = C.c_int32
+lib.tasc_attention_plan.argtypes = [C.c_void_p, C.POINTER(Kv), C.c_int32, C.c_int32, C.POINTER(C.c_int32)]
+lib.tasc_attention_plan.restype = C.c_int32
 
 
 def _check(code: int, where: str):
@@ -482,6 +484,13 @@ def tasc_profile_read() -> dict:
     cnt = (C.c_int64 * n)()
     _check(lib.tasc_profile_read(ms, cnt, n), "tasc_profile_read")
     return {k: (ms[i], cnt[i]) for i, k in enumerate(profile_kinds())}
+
+
+def tasc_attention_plan(model: Model, kv: Kv, B: int, rows: int) -> dict:
+    """What the attention of a pass of B sequences of `rows` rows runs as (bf16 models)."""
+    plan = (C.c_int32 * 4)()
+    _check(lib.tasc_attention_plan(model._h, C.byref(kv), B, rows, plan), "tasc_attention_plan")
+    return {"tcgen05": bool(plan[0]), "splits": plan[1], "heads": plan[2], "push_rows": plan[3]}
 
 
 def tasc_launch_counts() -> dict:

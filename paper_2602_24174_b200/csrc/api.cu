@@ -280,6 +280,15 @@ bool persist_pays(const tasc_model* m, int M, int R, int max_ctx, const PersistP
     return M <= 8 || m->layer_mb <= 12.0;
 }
 
+// The attention of a pass of B sequences of R rows.  It works on blocks of at most 16 rows per sequence: one in a verify step, several in a
+// prefill pass.
+AttnPlan plan_attention(const tasc_model_desc& d, int B, int R, int max_ctx) {
+    const int rows = std::min(R, 16), blocks = B * (R / rows), g = d.n_q_heads / d.n_kv_heads;
+    AttnPlan p = plan_attention_mma(blocks, d.n_kv_heads, d.head_dim, g, rows, max_ctx);
+    plan_attention_tc(blocks, d.n_kv_heads, d.head_dim, g, rows, max_ctx, d.page_size, p);
+    return p;
+}
+
 // bf16 models: five launches per layer (QKV+RoPE+KV append, attention, O+residual, gate/up+SiLU*mul, down+residual),
 // each with programmatic stream serialisation (gemm_fused.cu, attention_mma.cu), or one launch for all layers.
 tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace& w, const RowSource& src, int B, int R,
@@ -297,10 +306,7 @@ tasc_status forward_bf16(const tasc_model* m, const tasc_kv* kv, const Workspace
             sp = *it;
         } else {
             sp.B = B; sp.R = R; sp.max_ctx = max_ctx; sp.ws_h = w.h;
-            // attention works on blocks of at most 16 rows per sequence (one block in a verify step, several in a prefill pass)
-            const int att_rows = R <= 16 ? R : 16;
-            sp.att = plan_attention_mma(B * (R / att_rows), d.n_kv_heads, d.head_dim, d.n_q_heads / d.n_kv_heads, att_rows, max_ctx);
-            plan_attention_tc(B * (R / att_rows), d.n_kv_heads, d.head_dim, d.n_q_heads / d.n_kv_heads, att_rows, max_ctx, d.page_size, sp.att);
+            sp.att = plan_attention(d, B, R, max_ctx);
             // passes of many rows: the products with large weight matrices take the many-row kernel
             const double big_mb = 2.0 * 2.0 * (double)d.d_ff * d.d_model / 1e6;      // the largest matrix of a layer (gate/up)
             const double matrix_mb = M > WIDE_1K ? WIDE_MATRIX_MB_1K : WIDE_MATRIX_MB;
@@ -561,6 +567,16 @@ extern "C" tasc_status tasc_model_destroy(tasc_model* m) {
 extern "C" size_t tasc_workspace_bytes(const tasc_model* m, int32_t B_max, int32_t k_max) {
     if (!m || B_max < 1 || k_max < 1 || k_max > TASC_MAX_ROWS - 1) return 0;
     return layout_workspace(m, B_max, nullptr).bytes;
+}
+
+extern "C" tasc_status tasc_attention_plan(const tasc_model* m, const tasc_kv* kv, int32_t B, int32_t rows, int32_t* plan) {
+    if (!m || !kv || !plan || m->desc.dtype != TASC_BF16 || kv->max_pages_per_seq < 1 || B < 1 || rows < 1 || (rows > 16 && rows % 16)) return TASC_EINVAL;
+    const AttnPlan p = plan_attention(m->desc, B, rows, kv->max_pages_per_seq * m->desc.page_size);
+    plan[0] = p.tc;
+    plan[1] = p.splits;
+    plan[2] = p.heads;
+    plan[3] = p.push_rows;
+    return TASC_OK;
 }
 
 extern "C" tasc_status tasc_prefill(const tasc_model* m, const tasc_kv* kv, const tasc_seqs* seqs, int32_t B, int32_t max_len,

@@ -16,8 +16,9 @@
 //
 // Merge (only when the key range is split): the splits of one (sequence, KV head) are the CTAs of a
 // thread-block cluster.  CTA r merges every S-th row, in rank order, and writes it as (hi, lo) bf16 in the layout the
-// O-projection GEMM loads.  Every CTA stores its unnormalised O and (max, sum) straight into the shared memory of the rows'
-// mergers (distributed shared memory), and a cluster barrier later they are there.  Nothing goes through global memory.
+// O-projection GEMM loads.  Where there is room every CTA stores its unnormalised O and (max, sum) straight into the shared memory
+// of the rows' mergers (distributed shared memory), and a cluster barrier later they are there; elsewhere it parks them in
+// its own, and the mergers fetch them.  Nothing goes through global memory.
 #include "kernels.h"
 
 #include <algorithm>
@@ -609,6 +610,10 @@ inline size_t attn_smem_bytes(int hd, int gp, int stages) {
     return 1024 + (size_t)2 * gp * hd * 2 + (size_t)2 * stages * TKEYS * hd * 2;      // 1024: alignment slack
 }
 
+// The rows that the CTAs of a cluster of `splits` store into one another's shared memory
+inline size_t push_bytes(int hd, int splits, int push_rows) { return (size_t)splits * push_rows * (hd + 4) * 4; }
+constexpr size_t MAX_SMEM = 220 * 1024;
+
 template <int HD, int NS, bool TMA>
 tasc_status prepare_inst() {
     static bool done[64] = {false};
@@ -616,21 +621,21 @@ tasc_status prepare_inst() {
     TASC_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return TASC_EINVAL;
     if (!done[dev]) {
-        TASC_CUDA_TRY(cudaFuncSetAttribute(attn_mma_kernel<HD, NS, TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+        TASC_CUDA_TRY(cudaFuncSetAttribute(attn_mma_kernel<HD, NS, TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM));
         done[dev] = true;
     }
     return TASC_OK;
 }
 
-// Clusters of `splits` CTAs (ring depth `stages`) the device holds at once; 0 if the query fails.  (Both ways of loading: two CTAs per SM
+// Clusters of `splits` CTAs (ring depth `stages`, room for `push_rows`) the device holds at once; 0 if the query fails.  (Both ways of loading: two CTAs per SM
 // by their registers with heads of 32 and 64, one with heads of 128.)
 template <int HD, int NS>
-int fit_inst(int splits, int stages) {
+int fit_inst(int splits, int stages, int push_rows) {
     if (prepare_inst<HD, NS, true>() != TASC_OK) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)splits, 1, 1);
     cfg.blockDim = dim3(256, 1, 1);
-    cfg.dynamicSmemBytes = attn_smem_bytes(HD, NS * 16, stages);
+    cfg.dynamicSmemBytes = attn_smem_bytes(HD, NS * 16, stages) + push_bytes(HD, splits, push_rows);
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)splits;
@@ -643,18 +648,21 @@ int fit_inst(int splits, int stages) {
     return n;
 }
 
-int fit_any(int hd, int nw, int splits, int stages) {
+int fit_any(int hd, int nw, int splits, int stages, int push_rows) {
     static std::mutex mu;
     static std::map<long long, int> cache;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
-    const long long key = ((((long long)dev * 256 + hd) * 16 + nw) * 16 + splits) * 16 + stages;
+    const long long key = (((((long long)dev * 256 + hd) * 16 + nw) * 16 + splits) * 16 + stages) * 256 + push_rows;
     std::lock_guard<std::mutex> lk(mu);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     int n = 0;
-    if (nw == 4) n = hd == 32 ? fit_inst<32, 4>(splits, stages) : hd == 64 ? fit_inst<64, 4>(splits, stages) : fit_inst<128, 4>(splits, stages);
-    else n = hd == 32 ? fit_inst<32, 8>(splits, stages) : hd == 64 ? fit_inst<64, 8>(splits, stages) : fit_inst<128, 8>(splits, stages);
+    auto ask = [&](auto slabs) {
+        constexpr int NS = decltype(slabs)::value;
+        return hd == 32 ? fit_inst<32, NS>(splits, stages, push_rows) : hd == 64 ? fit_inst<64, NS>(splits, stages, push_rows) : fit_inst<128, NS>(splits, stages, push_rows);
+    };
+    n = nw == 4 ? ask(std::integral_constant<int, 4>{}) : ask(std::integral_constant<int, 8>{});
     cache[key] = n;
     return n;
 }
@@ -663,7 +671,7 @@ template <int HD, int NS, bool TMA>
 tasc_status launch_inst(const AttnArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int B, cudaStream_t stream) {
     constexpr int GP = NS * 16;
     if (a.stages < 2 || a.stages > Ring<HD, NS>::MAX_STAGES) return TASC_EINVAL;
-    const size_t smem = attn_smem_bytes(HD, GP, a.stages) + (size_t)a.push_rows * a.splits * (HD + 4) * 4;
+    const size_t smem = attn_smem_bytes(HD, GP, a.stages) + push_bytes(HD, a.splits, a.push_rows);
     tasc_status pst = prepare_inst<HD, NS, TMA>();
     if (pst != TASC_OK) return pst;
     cudaLaunchConfig_t cfg = {};
@@ -713,7 +721,7 @@ AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ct
     // rows, 640 tokens 37.8 / 37.2, 4 x 9 rows, 320 tokens 43.1 / 43.7; the others within 1.5 %.
     const float t_tile = hd >= 128 ? 1.2f : (hd >= 64 ? 1.3f : 0.8f);
     const float t_pipe = hd >= 128 ? 0.65f : (hd >= 64 ? 0.3f : 0.15f);
-    AttnPlan best = {1, 2, g, 0, 1e30f};
+    AttnPlan best = {1, 2, g, 0, 0, 1e30f};
     float best_cost = 1e30f;
     // Candidates: all g heads of a KV head in one CTA; and, for few sequences with 128-wide heads (where a warp's chain over a key
     // tile is long), the largest share of the heads whose rows still fill a single 16-row slab.  (Measured: on the
@@ -733,7 +741,7 @@ AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ct
         for (int di = 0; di < 2; ++di) {
             const int stages = depths[di];
             for (int s = 1; s <= 8 && s <= n_tiles; ++s) {
-                int fit = fit_any(hd, nw, s, stages);
+                int fit = fit_any(hd, nw, s, stages, 0);
                 if (fit <= 0) fit = std::max(1, 148 / s);               // no device to ask: assume one CTA per SM
                 // Two CTAs to an SM: of clusters that just fit an empty chip, up to four find no room beside the CTAs that the kernel before
                 // still has there, and run behind the others.  A layer of the 0.5B and the 135M, us, by clusters (that fit), against the
@@ -749,7 +757,7 @@ AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ct
                     return std::max(iters * (t_tile + stall), t * n_slabs * t_pipe);
                 };
                 const float loop = 0.5f * (loop_of(n_tiles) + loop_of(n_all));
-                const float merge = s > 1 ? 0.5f + 0.25f * s : 0.f;      // cluster barrier + one round of remote reads
+                const float merge = s > 1 ? 0.5f + 0.25f * s : 0.f;      // cluster barrier + the rows' way to their mergers
                 // a grid that takes (nearly) every SM keeps the next kernel's CTAs from starting early
                 // (1.0: 20 x 4 rows of the 0.5B 907 us instead of 902; 3.0: 24 x 5 rows 1113 instead of 1068)
                 const float crowd = groups * s > 128 ? 1.5f : 0.f;
@@ -759,10 +767,15 @@ AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ct
                 // for all and 1.7 us for each, 56 to 128 sequences were split into several waves: a layer of the 135M, 64 x 6 rows,
                 // 1,024 tokens of cache, 58.2 us in 4 splits against 50.8 whole, and behind 170 of them 49.6 against 36.2.)
                 const float cost = waves * (1.7f + loop + merge) + (waves - 1) * 1.0f + crowd + reread;
-                if (cost < best_cost - 1e-6f) { best_cost = cost; best = AttnPlan{s, stages, hs, 0, cost}; }
+                if (cost < best_cost - 1e-6f) { best_cost = cost; best = AttnPlan{s, stages, hs, 0, 0, cost}; }
             }
         }
     }
+    // Rows go straight to their mergers where the memory for that leaves room for as many clusters.
+    const int G = best.heads * rows, GP = attention_mma_row_pad(G), share = (G + best.splits - 1) / best.splits;
+    if (best.splits > 1 && attn_smem_bytes(hd, GP, best.stages) + push_bytes(hd, best.splits, share) <= MAX_SMEM &&
+        fit_any(hd, GP / 16, best.splits, best.stages, share) == fit_any(hd, GP / 16, best.splits, best.stages, 0))
+        best.push_rows = share;
     return best;
 }
 
@@ -790,9 +803,7 @@ tasc_status launch_attention_mma(const float* qbuf, const __nv_bfloat16* k_pages
     a.scale_log2e = 1.4426950408889634f / sqrtf((float)hd);
     a.status = status;
     a.n_slabs = (G + 15) / 16;
-    // Rows go straight to their mergers where the memory for that leaves as many CTAs to an SM.
-    const size_t base = attn_smem_bytes(hd, GP, plan.stages), extra = (size_t)((G + n_splits - 1) / n_splits) * n_splits * (hd + 4) * 4, sm = 228 * 1024;
-    a.push_rows = n_splits > 1 && base + extra <= 220 * 1024 && sm / (base + 1024) == sm / (base + extra + 1024) ? (G + n_splits - 1) / n_splits : 0;
+    a.push_rows = plan.push_rows;
     a.by_R = SmallDiv(Rs); a.by_TB = SmallDiv(TB); a.by_splits = SmallDiv(n_splits); a.by_sub = SmallDiv(n_sub); a.by_hsplit = SmallDiv(g / hs);
     // 16-token pages arrive as TMA boxes; any other page size, and key ranges of more pages than a CTA keeps the ids of, take the
     // kernel with cp.async.  So do 64-wide heads with one CTA per SM (the deep ring) in caches of more than 1,024 pages, which are

@@ -536,10 +536,8 @@ void config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[2], int splits, i
 }
 
 template <int HD, int RP>
-tasc_status launch_inst(TcArgs a, const CUtensorMap& tmK, const CUtensorMap& tmV, int B, cudaStream_t stream) {
+tasc_status launch_inst(const TcArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int B, cudaStream_t stream) {
     if (!prepare<HD, RP>()) return TASC_ECUDA;
-    const int share = (a.g * a.Rs + a.splits - 1) / a.splits;
-    a.push_rows = a.splits > 1 && Tc<HD, RP>::smem(a.stages) + share * a.splits * (HD + 4) * 4 <= MAX_SMEM ? share : 0;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[2];
     config<HD, RP>(cfg, at, a.splits, a.n_kv, B, a.stages);
@@ -613,6 +611,9 @@ bool plan_attention_tc(int B, int n_kv, int hd, int g, int rows, int max_ctx, in
     p.heads = g;
     p.splits = best;
     p.stages = hd == 64 ? (small ? ring_stages<64, 64>() : ring_stages<64, 128>()) : (small ? ring_stages<128, 64>() : ring_stages<128, 128>());
+    const int share = (G + best - 1) / best;
+    const int smem = hd == 64 ? (small ? Tc<64, 64>::smem(p.stages) : Tc<64, 128>::smem(p.stages)) : (small ? Tc<128, 64>::smem(p.stages) : Tc<128, 128>::smem(p.stages));
+    p.push_rows = best > 1 && smem + share * best * (hd + 4) * 4 <= MAX_SMEM ? share : 0;      // (one CTA per SM with or without it)
     return true;
 }
 
@@ -631,6 +632,7 @@ tasc_status launch_attention_tc(const float* qbuf, const CUtensorMap& tmK, const
     a.scale_log2e = 1.4426950408889634f / sqrtf((float)hd);
     a.status = status;
     a.g = n_q / n_kv;
+    a.push_rows = plan.push_rows;
     a.by_R = SmallDiv(Rs); a.by_TB = SmallDiv(TB); a.by_splits = SmallDiv(plan.splits); a.by_sub = SmallDiv(a.n_sub);
     const int blocks = B * a.n_sub;
     if (hd == 64) return G <= 64 ? launch_inst<64, 64>(a, tmK, tmV, blocks, stream) : launch_inst<64, 128>(a, tmK, tmV, blocks, stream);

@@ -338,6 +338,8 @@ struct AttnPlan {
     int stages;      // depth of the K/V tile ring
     int heads;       // query heads per CTA: a divisor of n_q / n_kv (the heads sharing a KV head are dealt out to several CTAs)
     int tc;          // 1: attention_tc.cu
+    // splits > 1: query rows per CTA of the cluster, which the others store into its shared memory; 0: it fetches them from theirs
+    int push_rows;
     float cost;      // what the planner expects, us
 };
 // Same contract as launch_attention; the result goes to `out` as (hi, lo) bf16 rows; needs no scratch memory.

@@ -76,6 +76,22 @@ class Guarded:
         assert bool((before == CANARY).all()) and bool((after == CANARY).all()), f"write outside {what}"
 
 
+def attention_of_steps(b, monkeypatch) -> list:
+    """The plan of the attention of every verify step from now on (tasc_attention_plan), which also has to be what the step launches: a kernel
+    per layer."""
+    plans, step = [], b.tasc_verify_step
+
+    def watched(model, kv, seqs, drafts, *args, **kw):
+        plans.append(b.tasc_attention_plan(model, kv, drafts.shape[0], drafts.shape[1] + 1))
+        before = b.tasc_launch_counts()["attention_split"]
+        out = step(model, kv, seqs, drafts, *args, **kw)
+        assert b.tasc_launch_counts()["attention_split"] - before == model.shape.n_layers
+        return out
+
+    monkeypatch.setattr(b, "tasc_verify_step", watched)
+    return plans
+
+
 @dataclass
 class LockstepReport:
     steps: int = 0
@@ -106,26 +122,29 @@ def record_parity(name: str, rep: LockstepReport, **extra):
 
 
 def lockstep(s: Setup, prompts: np.ndarray, max_new: int, k: int, *, logit_atol: float, logit_rtol: float, gap_tol: float,
-             check_logits: bool = True, lam=(3, 4), oracle_kwargs=None, forced_mode=None, oracle_rows=None) -> LockstepReport:
+             check_logits: bool = True, lam=(3, 4), oracle_kwargs=None, forced_mode=None, oracle_rows=None, lengths=None,
+             spare: int = 0) -> LockstepReport:
     """Run the oracle's speculative decoding per sequence, then replay every step on the GPU from the
     oracle's committed state and compare drafts (bit-exact), logits, argmax rows, accepted length and next token.
 
     ``oracle_rows``: the sequences of the batch the oracle runs and the comparison covers (all by default); the
-    other sequences of the batch decode on from whatever the device committed for them."""
+    other sequences of the batch decode on from whatever the device committed for them.
+    ``lengths``: tokens of every prompt (all P by default); ``spare``: tokens that the cache holds beyond what is needed."""
     b = need_gpu()
     B, P = prompts.shape
+    lengths = [P] * B if lengths is None else [int(n) for n in lengths]
     checked = list(range(B)) if oracle_rows is None else list(oracle_rows)
     traces = {}
     for i in checked:
         kw = dict(oracle_kwargs[i]) if oracle_kwargs else {}
-        traces[i] = G.greedy_speculative(s.oracle, s.ngrams, prompts[i], max_new, k, lam[0], lam[1],
+        traces[i] = G.greedy_speculative(s.oracle, s.ngrams, prompts[i][:lengths[i]], max_new, k, lam[0], lam[1],
                                          keep_logits=check_logits, **kw)
     n_steps = min(len(traces[i].steps) for i in checked)
     stride = P + max(max_new, n_steps * (k + 1)) + 2 * k + 2
     tokens = torch.zeros((B, stride), dtype=torch.int32, device="cuda")
     tokens[:, :P] = torch.from_numpy(prompts).cuda()
-    length = torch.full((B,), P, dtype=torch.int32, device="cuda")
-    pool, bt, kv = s.model.new_kv(B, stride + b.MAX_ROWS)
+    length = torch.tensor(lengths, dtype=torch.int32, device="cuda")
+    pool, bt, kv = s.model.new_kv(B, stride + b.MAX_ROWS + spare)
     # workspace and every output of the step sit between canary bands, checked after every call
     g_ws = Guarded((s.model.workspace_bytes(B, k),), torch.uint8)
     g_ws.inner.zero_()
@@ -140,7 +159,7 @@ def lockstep(s: Setup, prompts: np.ndarray, max_new: int, k: int, *, logit_atol:
     b.tasc_prefill(s.model, kv, seqs, B, P, ws)
     g_ws.check("the workspace (prefill)")
     rep = LockstepReport()
-    committed = {i: list(map(int, prompts[i])) for i in checked}
+    committed = {i: list(map(int, prompts[i][:lengths[i]])) for i in checked}
     sel = torch.tensor(checked, dtype=torch.long, device="cuda")
     for step in range(n_steps):
         sts = {i: traces[i].steps[step] for i in checked}

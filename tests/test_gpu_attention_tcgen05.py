@@ -1,31 +1,36 @@
 """The tcgen05 attention: query tiles of up to 64 and up to 128 rows, 64- and 128-wide heads, contexts that end just before, at and just behind
-a tile of 128 keys, one key range and several, ranges of one, two and more tiles (the two places of S and P, and of O, are used in
-turn), a ragged batch; the oracle runs the first and the last sequence."""
+a tile of 128 keys, one key range and several, ranges of one, two and more tiles (the two places of S and P, and of O, are used in turn), prompts
+of one length and of different ones; the oracle runs the first and the last sequence.  That a case takes this kernel is looked at."""
 from dataclasses import replace
 
 import pytest
 
-from tests.gpu_harness import lockstep, make_setup
+from tests.gpu_harness import attention_of_steps, lockstep, make_setup, need_gpu
 from tests.test_gpu_verify import BF16_TOL, check
 from workload import configs, corpus
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("hd,n_q,n_kv,B,k,P", [
-    (64, 14, 2, 34, 8, 127),        # 63 rows
-    (64, 14, 2, 34, 7, 128),        # 56 rows
-    (64, 16, 2, 34, 7, 249),        # 64 rows: a full tile
-    (64, 16, 2, 34, 8, 250),        # 72 rows: the wider one
-    (64, 16, 2, 20, 15, 385),        # 128 rows
-    (128, 12, 2, 40, 4, 126),       # 30 rows
-    (128, 12, 2, 66, 6, 260),       # 42 rows
-    (128, 12, 2, 30, 8, 700),       # 54 rows, split
-    (128, 16, 2, 34, 8, 383),       # 72 rows
-    (128, 16, 2, 24, 15, 640),       # 128 rows
+@pytest.mark.parametrize("hd,n_q,n_kv,B,k,P,split,spare", [
+    (64, 14, 2, 34, 8, 127, False, 150),        # 63 rows
+    (64, 14, 2, 34, 7, 128, False, 150),        # 56 rows
+    (64, 16, 2, 34, 7, 249, False, 0),          # 64 rows: a full tile
+    (64, 16, 2, 34, 8, 250, False, 0),          # 72 rows: the wider one
+    (64, 16, 2, 20, 15, 385, True, 0),          # 128 rows
+    (128, 12, 2, 48, 4, 600, False, 0),         # 30 rows
+    (128, 12, 2, 66, 6, 260, False, 0),         # 42 rows
+    (128, 12, 2, 30, 8, 700, True, 0),          # 54 rows, split
+    (128, 16, 2, 34, 8, 383, False, 0),         # 72 rows
+    (128, 16, 2, 24, 15, 640, True, 0),         # 128 rows
 ])
-def test_tiles_and_key_ranges(hd, n_q, n_kv, B, k, P):
+@pytest.mark.parametrize("ragged", [False, True])
+def test_tiles_and_key_ranges(hd, n_q, n_kv, B, k, P, split, spare, ragged, monkeypatch):
     base = configs.shrunk(configs.get(2), n_layers=2, vocab=4096, n_docs=500, d_ff=1024)
-    cfg = replace(base, model=replace(base.model, d_model=n_q * hd, n_q_heads=n_q, n_kv_heads=n_kv, head_dim=hd), prompt_len=P)
+    cfg = replace(base, model=replace(base.model, d_model=n_q * hd, n_q_heads=n_q, n_kv_heads=n_kv, head_dim=hd), prompt_len=P + spare)
+    plans = attention_of_steps(need_gpu(), monkeypatch)
     s = make_setup(cfg)
-    rep = lockstep(s, corpus.make_prompts(cfg, B, prompt_len=P), k + 3, k, oracle_rows=sorted({0, B - 1}), **BF16_TOL)
+    lengths = [P - i * (P // 2) // B for i in range(B)] if ragged else None
+    rep = lockstep(s, corpus.make_prompts(cfg, B, prompt_len=P), k + 3, k, oracle_rows=sorted({0, B - 1}), lengths=lengths, spare=spare, **BF16_TOL)
     check(rep, f"tcgen05 attention, heads of {hd}, {n_q} / {n_kv}, B={B} k={k} P={P}")
+    for p in plans:
+        assert p["tcgen05"] and (p["splits"] > 1) == split, plans
