@@ -459,9 +459,9 @@ tasc_status tasc_launch_counts(int64_t* launches_by_kind, int32_t n);
 /*
  * What the attention of a pass of a bf16 model runs as, where its layers are not one kernel.  Host only; asks the current device for its occupancy.
  *   B, rows  sequences, and rows of each: k + 1 in a verify step, a multiple of 16 in a prefill pass
- *   plan     host [4]: 1 the tcgen05 kernel, 0 the warp-level one; key ranges of a sequence (the CTAs of a cluster); query heads per CTA;
+ *   plan     host [5]: 1 the tcgen05 kernel, 0 the warp-level one; key ranges of a sequence (the CTAs of a cluster); query heads per CTA;
  *            query rows that a CTA of the cluster merges where the others store them into its shared memory, 0 where it fetches
- *            them or there is one key range
+ *            them or there is one key range; keys per tile
  * Errors: EINVAL.
  */
 tasc_status tasc_attention_plan(const tasc_model* m, const tasc_kv* kv, int32_t B, int32_t rows, int32_t* plan);

@@ -488,9 +488,9 @@ def tasc_profile_read() -> dict:
 
 def tasc_attention_plan(model: Model, kv: Kv, B: int, rows: int) -> dict:
     """What the attention of a pass of B sequences of `rows` rows runs as (bf16 models)."""
-    plan = (C.c_int32 * 4)()
+    plan = (C.c_int32 * 5)()
     _check(lib.tasc_attention_plan(model._h, C.byref(kv), B, rows, plan), "tasc_attention_plan")
-    return {"tcgen05": bool(plan[0]), "splits": plan[1], "heads": plan[2], "push_rows": plan[3]}
+    return {"tcgen05": bool(plan[0]), "splits": plan[1], "heads": plan[2], "push_rows": plan[3], "tile": plan[4]}
 
 
 def tasc_launch_counts() -> dict:

@@ -576,6 +576,7 @@ extern "C" tasc_status tasc_attention_plan(const tasc_model* m, const tasc_kv* k
     plan[1] = p.splits;
     plan[2] = p.heads;
     plan[3] = p.push_rows;
+    plan[4] = p.tile;
     return TASC_OK;
 }
 

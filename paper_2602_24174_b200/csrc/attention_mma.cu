@@ -721,7 +721,7 @@ AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ct
     // rows, 640 tokens 37.8 / 37.2, 4 x 9 rows, 320 tokens 43.1 / 43.7; the others within 1.5 %.
     const float t_tile = hd >= 128 ? 1.2f : (hd >= 64 ? 1.3f : 0.8f);
     const float t_pipe = hd >= 128 ? 0.65f : (hd >= 64 ? 0.3f : 0.15f);
-    AttnPlan best = {1, 2, g, 0, 0, 1e30f};
+    AttnPlan best = {1, 2, g, 0, TKEYS, 0, 1e30f};
     float best_cost = 1e30f;
     // Candidates: all g heads of a KV head in one CTA; and, for few sequences with 128-wide heads (where a warp's chain over a key
     // tile is long), the largest share of the heads whose rows still fill a single 16-row slab.  (Measured: on the
@@ -767,7 +767,7 @@ AttnPlan plan_attention_mma(int B, int n_kv, int hd, int g, int rows, int max_ct
                 // for all and 1.7 us for each, 56 to 128 sequences were split into several waves: a layer of the 135M, 64 x 6 rows,
                 // 1,024 tokens of cache, 58.2 us in 4 splits against 50.8 whole, and behind 170 of them 49.6 against 36.2.)
                 const float cost = waves * (1.7f + loop + merge) + (waves - 1) * 1.0f + crowd + reread;
-                if (cost < best_cost - 1e-6f) { best_cost = cost; best = AttnPlan{s, stages, hs, 0, 0, cost}; }
+                if (cost < best_cost - 1e-6f) { best_cost = cost; best = AttnPlan{s, stages, hs, 0, TKEYS, 0, cost}; }
             }
         }
     }

@@ -12,12 +12,12 @@
 //                  then O += O tile (t - 1), rescaled: O is accumulated in registers, so a new maximum costs no pass over TMEM
 //   TMA warp       K and V tiles, a ring of two or more
 // P as the MMA's A operand in TMEM takes no pass through shared memory, does not wait for P(t - 1) to be used, and leaves the ring its
-// memory, so that 128 keys make a tile for up to 128 rows too (64 before).  With up to 64 rows four of the eight softmax warps have any;
-// two of the others are the TMA and the MMA warp then.
+// memory, so that 128 keys make a tile for up to 128 rows too (64 before, and in short caches, see SHORT_CTX).  With up to 64 rows four of the
+// eight softmax warps have any; two of the others are the TMA and the MMA warp then.
 // Key ranges split over a cluster are merged as in attention_mma.cu.
 //
 // Measured, per layer: 1.5B at 64 sequences x 7 rows and up to 1,530 keys 61 -> 33 us (2.0 us per 128 keys: softmax 0.9, its
-// half of O 0.3, P 0.4, waits 0.4); 0.5B + 8,192 tokens at 32 x 9 rows, 640 keys 15.5 -> 13.4; prefill of 16 x 1,024 tokens
+// half of O 0.3, P 0.4, waits 0.4; with P in TMEM and the warps' places 1.6); 0.5B + 8,192 tokens at 32 x 9 rows, 640 keys 15.5 -> 13.4; prefill of 16 x 1,024 tokens
 // on the 1.5B 72 -> 47 us per pass of 2,048 rows.  With P in TMEM, whole steps: 1.5B, 64 x 7 rows behind 1,500 keys 4,204 -> 4,190 us, and with
 // the warps' places 4,094; 40 x 5 rows behind 1,400 2,859 -> 2,821, 2,736; 0.5B + 8,192 tokens 1,392 -> 1,370, 1,371; a prefill of
 // 4 x 1,000 tokens of the 1.5B (96 rows) 19.68 -> 19.45 ms with tiles of 64 keys, 19.90 -> 19.47 with tiles of 128.
@@ -78,8 +78,9 @@ __device__ __forceinline__ uint64_t umma_desc_mn_sw128(uint32_t smem_addr, uint3
     return d;
 }
 
-template <int HD, int RP> struct Tc {
-    static constexpr int TK = 128;                               // keys of a tile
+// HD: head width, RP: rows of the query tile, TK: keys of a tile
+template <int HD_, int RP_, int TK_> struct Tc {
+    static constexpr int HD = HD_, RP = RP_, TK = TK_;
     static constexpr int HB = HD / 64;                           // blocks of 64 columns of a head
     // Query tiles of 64 rows have rows in the first two lane quarters: two warps of the others feed the tensor cores.  (Theirs are the other two
     // schedulers, and eight warps have more registers each than ten.)
@@ -90,15 +91,16 @@ template <int HD, int RP> struct Tc {
     static constexpr int FIXED = 2 * Q_BYTES;
     static constexpr int S_COL = 0, O_COL = 2 * TK;              // TMEM columns: two S tiles, two O tiles
     static constexpr int COLS = 2 * TK + 2 * HD <= 256 ? 256 : 512;
-    static constexpr int SC = TK / 2, OC = HD / 2;               // a thread's share of a row of S, of O
+    // A thread's share of a row of S, of O.  (128-wide heads and 128 rows: 40 bytes are spilled, ten warps have 168 registers each.  With S loaded 16
+    // columns at a time 12 bytes, and slower: a prefill of 100 tokens of the 1.5B 1,581 -> 1,593 us, of 1,000 5,883 -> 5,899.)
+    static constexpr int SC = TK / 2, OC = HD / 2;
     static int smem(int stages) { return 1024 + FIXED + stages * 2 * KV_BYTES; }
 };
 
-template <int HD, int RP>
-__global__ void __launch_bounds__(Tc<HD, RP>::THREADS, 1)
+template <class C>
+__global__ void __launch_bounds__(C::THREADS, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const TcArgs a) {
-    using C = Tc<HD, RP>;
-    constexpr int TK = C::TK, THREADS = C::THREADS, TMA_WARP = C::TMA_WARP, MMA_WARP = C::MMA_WARP;
+    constexpr int HD = C::HD, RP = C::RP, TK = C::TK, THREADS = C::THREADS, TMA_WARP = C::TMA_WARP, MMA_WARP = C::MMA_WARP;
     extern __shared__ uint8_t sm_raw[];
     uint8_t* sm = sm_raw + ((1024u - (smem_u32(sm_raw) & 1023u)) & 1023u);
     uint8_t* Qs = sm;                                            // hi, then lo: [HB][RP][128 bytes]
@@ -506,7 +508,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     cluster_sync();                                            // peers may still be reading this CTA's rows
 }
 
-template <int HD, int RP>
+template <class C>
 bool prepare() {
     static std::mutex mu;
     static int known[64] = {0};                                  // 1 yes, 2 no
@@ -514,17 +516,17 @@ bool prepare() {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { (void)cudaGetLastError(); return false; }
     std::lock_guard<std::mutex> lk(mu);
     if (!known[dev]) {
-        known[dev] = cudaFuncSetAttribute(attn_tc_kernel<HD, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM) == cudaSuccess ? 1 : 2;
+        known[dev] = cudaFuncSetAttribute(attn_tc_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM) == cudaSuccess ? 1 : 2;
         if (known[dev] == 2) (void)cudaGetLastError();
     }
     return known[dev] == 1;
 }
 
-template <int HD, int RP>
+template <class C>
 void config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[2], int splits, int n_kv, int B, int stages) {
     cfg.gridDim = dim3((unsigned)splits, (unsigned)n_kv, (unsigned)B);
-    cfg.blockDim = dim3(Tc<HD, RP>::THREADS, 1, 1);
-    cfg.dynamicSmemBytes = (size_t)Tc<HD, RP>::smem(stages);
+    cfg.blockDim = dim3(C::THREADS, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)C::smem(stages);
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     at[1].id = cudaLaunchAttributeClusterDimension;
@@ -535,45 +537,59 @@ void config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&at)[2], int splits, i
     cfg.numAttrs = splits > 1 ? 2 : 1;                           // the key-range splits of one (sequence, KV head) form a cluster
 }
 
-template <int HD, int RP>
+template <class C>
 tasc_status launch_inst(const TcArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int B, cudaStream_t stream) {
-    if (!prepare<HD, RP>()) return TASC_ECUDA;
+    if (!prepare<C>()) return TASC_ECUDA;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[2];
-    config<HD, RP>(cfg, at, a.splits, a.n_kv, B, a.stages);
-    cfg.dynamicSmemBytes += (size_t)a.push_rows * a.splits * (HD + 4) * 4;
+    config<C>(cfg, at, a.splits, a.n_kv, B, a.stages);
+    cfg.dynamicSmemBytes += (size_t)a.push_rows * a.splits * (C::HD + 4) * 4;
     cfg.stream = stream;
     ProfScope ps(K_ATT_SPLIT, stream);
-    TASC_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD, RP>, tmK, tmV, a));
+    TASC_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<C>, tmK, tmV, a));
     return TASC_OK;
 }
 
-template <int HD, int RP> int ring_stages();
+template <class C> int ring_stages();
 // Clusters of `splits` CTAs that the device holds at once (0: it cannot be asked).
-template <int HD, int RP>
+template <class C>
 int clusters(int splits) {
     static std::mutex mu;
     static int known[64][9] = {{0}};                             // + 1
     int dev = 0;
-    if (!prepare<HD, RP>() || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { (void)cudaGetLastError(); return 0; }
+    if (!prepare<C>() || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { (void)cudaGetLastError(); return 0; }
     std::lock_guard<std::mutex> lk(mu);
     if (!known[dev][splits]) {
         int n = 0;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[2];
-        config<HD, RP>(cfg, at, splits, 1, 1, ring_stages<HD, RP>());
+        config<C>(cfg, at, splits, 1, 1, ring_stages<C>());
         cfg.attrs = at + 1;
         cfg.numAttrs = 1;
-        if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<HD, RP>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
+        if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<C>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
         known[dev][splits] = n + 1;
     }
     return known[dev][splits] - 1;
 }
-template <int HD, int RP> int ring_stages() {
+template <class C> int ring_stages() {
     int s = MAX_RING;
-    while (s > 2 && Tc<HD, RP>::smem(s) > MAX_SMEM) --s;
+    while (s > 2 && C::smem(s) > MAX_SMEM) --s;
     return s;
 }
+// f(the instance for heads of hd, a query tile of up to 64 rows or more, tiles of `tile` keys)
+template <class F>
+auto with_instance(int hd, bool small, int tile, F f) {
+    if (small) return hd == 64 ? f(Tc<64, 64, 128>{}) : f(Tc<128, 64, 128>{});
+    if (tile == 64) return hd == 64 ? f(Tc<64, 128, 64>{}) : f(Tc<128, 128, 64>{});
+    return hd == 64 ? f(Tc<64, 128, 128>{}) : f(Tc<128, 128, 128>{});
+}
+
+// Caches of up to so many tokens (64 and a step's 16 rows) take tiles of 64 keys for 65 to 128 rows, where most of a tile of 128 would be empty.  A prefill
+// with tiles of 128 / 64 keys, us: 1.5B, 48 tokens 1,179 / 1,157, 60 tokens 1,266 / 1,257, 16 x 48 4,384 / 4,374; 0.5B, 16 x 48 1,686 / 1,669.  Two
+// tiles of 64 for one of 128: 70 tokens 1,369 / 1,394, 0.5B 780 / 802; more of them: 1.5B, 1,000 tokens 5,929 / 6,003, 0.5B, 4 x 100 1,499 / 1,522.
+// (Key ranges dealt out in units of 64, the last tile of a range half a tile, by branches in the kernel: 48 tokens 1,171, 100 tokens 1,598
+// instead of 1,574.)
+constexpr int SHORT_CTX = 80;
 
 }  // namespace
 
@@ -583,21 +599,22 @@ template <int HD, int RP> int ring_stages() {
 // take of the SMs' mma.sync pipes.  T0 as measured against the other kernel, which starts faster since its code was cut: a step
 // of the 1.5B, 3 x 7 rows behind 400 keys, 1169 us here, 1121 there; 10 x 8 rows of the 0.5B 893 / 877; 1.5B 40 x 5 rows 2512 / 2549,
 // 0.5B + 8,192 tokens 32 x 9 rows behind 640 keys 1441 / 1440.  (T0 was 3.9 and 2.8, a tile 1.8 and 1.4, before P was in TMEM: a step of the
-// 0.5B, 32 x 9 rows behind 1,000 keys, was left with the other kernel then, 1445 us, 1409 here.  With shorter tiles and T0 as it was a step of
-// 2 x 7 rows behind 900 keys came here, 699 us, 648 there.)  It pays for many (sequence, KV head) pairs with long contexts and three or
+// 0.5B, 32 x 9 rows behind 1,000 keys, was left with the other kernel then, 1445 us, 1409 here.  With T0 as it was the tiles' shorter times
+// bring steps here that the other kernel is faster at: 0.5B, 2 x 7 rows behind 900 keys 675 us here, 630 there, 4 x 7 rows 740 / 698, 3 x 9
+// behind 600 731 / 690.)  It pays for many (sequence, KV head) pairs with long contexts and three or
 // more slabs of query rows, hardly ever at the 135M's 18 to 27 rows.
 bool plan_attention_tc(int B, int n_kv, int hd, int g, int rows, int max_ctx, int page_size, AttnPlan& p) {
     const int G = g * rows;
     if ((hd != 64 && hd != 128) || page_size != PAGE || G > 128 || max_ctx / PAGE > MAX_PAGES) return false;
     const bool small = G <= 64;
-    constexpr int tk = 128;
-    const float T0 = hd == 128 ? 4.3f : 3.2f, per_tile = hd == 128 ? (small ? 1.6f : 1.8f) : (small ? 1.2f : 1.4f);
-    const int groups = B * n_kv, tiles_all = std::max(1, (max_ctx + tk - 1) / tk), tiles_34 = std::max(1, (max_ctx * 3 / 4 + tk - 1) / tk);
+    const int tile = !small && max_ctx <= SHORT_CTX ? 64 : 128;
+    const float T0 = hd == 128 ? 4.3f : 3.2f, per_tile = hd == 128 ? (small ? 1.6f : tile == 64 ? 1.2f : 1.8f) : (small ? 1.2f : tile == 64 ? 0.95f : 1.4f);
+    const int groups = B * n_kv, tiles_all = std::max(1, (max_ctx + tile - 1) / tile), tiles_34 = std::max(1, (max_ctx * 3 / 4 + tile - 1) / tile);
     const float pipes = (hd == 128 ? 0.6f : 0.3f) * (float)groups * (float)((G + 15) / 16) * (float)((max_ctx * 3 / 4 + 63) / 64) / 148.f;
     int best = 0;
     float best_cost = std::max(p.cost, 2.5f + pipes);
     for (int s = 1; s <= 8 && s <= tiles_all; ++s) {
-        const int fit = hd == 64 ? (small ? clusters<64, 64>(s) : clusters<64, 128>(s)) : (small ? clusters<128, 64>(s) : clusters<128, 128>(s));
+        const int fit = with_instance(hd, small, tile, [&](auto c) { return clusters<decltype(c)>(s); });
         if (fit <= 0) continue;
         const int waves = (groups + fit - 1) / fit;
         const float tiles = 0.5f * (float)((tiles_all + s - 1) / s + (tiles_34 + s - 1) / s);
@@ -610,10 +627,14 @@ bool plan_attention_tc(int B, int n_kv, int hd, int g, int rows, int max_ctx, in
     p.tc = 1;
     p.heads = g;
     p.splits = best;
-    p.stages = hd == 64 ? (small ? ring_stages<64, 64>() : ring_stages<64, 128>()) : (small ? ring_stages<128, 64>() : ring_stages<128, 128>());
+    p.tile = tile;
     const int share = (G + best - 1) / best;
-    const int smem = hd == 64 ? (small ? Tc<64, 64>::smem(p.stages) : Tc<64, 128>::smem(p.stages)) : (small ? Tc<128, 64>::smem(p.stages) : Tc<128, 128>::smem(p.stages));
-    p.push_rows = best > 1 && smem + share * best * (hd + 4) * 4 <= MAX_SMEM ? share : 0;      // (one CTA per SM with or without it)
+    with_instance(hd, small, tile, [&](auto c) {
+        using C = decltype(c);
+        p.stages = ring_stages<C>();
+        p.push_rows = best > 1 && C::smem(p.stages) + share * best * (hd + 4) * 4 <= MAX_SMEM ? share : 0;      // (one CTA per SM with or without it)
+        return 0;
+    });
     return true;
 }
 
@@ -635,8 +656,7 @@ tasc_status launch_attention_tc(const float* qbuf, const CUtensorMap& tmK, const
     a.push_rows = plan.push_rows;
     a.by_R = SmallDiv(Rs); a.by_TB = SmallDiv(TB); a.by_splits = SmallDiv(plan.splits); a.by_sub = SmallDiv(a.n_sub);
     const int blocks = B * a.n_sub;
-    if (hd == 64) return G <= 64 ? launch_inst<64, 64>(a, tmK, tmV, blocks, stream) : launch_inst<64, 128>(a, tmK, tmV, blocks, stream);
-    return G <= 64 ? launch_inst<128, 64>(a, tmK, tmV, blocks, stream) : launch_inst<128, 128>(a, tmK, tmV, blocks, stream);
+    return with_instance(hd, G <= 64, plan.tile, [&](auto c) { return launch_inst<decltype(c)>(a, tmK, tmV, blocks, stream); });
 }
 
 }  // namespace tasc

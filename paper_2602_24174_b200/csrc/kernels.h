@@ -338,6 +338,7 @@ struct AttnPlan {
     int stages;      // depth of the K/V tile ring
     int heads;       // query heads per CTA: a divisor of n_q / n_kv (the heads sharing a KV head are dealt out to several CTAs)
     int tc;          // 1: attention_tc.cu
+    int tile;        // keys per tile
     // splits > 1: query rows per CTA of the cluster, which the others store into its shared memory; 0: it fetches them from theirs
     int push_rows;
     float cost;      // what the planner expects, us

@@ -1,6 +1,6 @@
 """The tcgen05 attention: query tiles of up to 64 and up to 128 rows, 64- and 128-wide heads, contexts that end just before, at and just behind
-a tile of 128 keys, one key range and several, ranges of one, two and more tiles (the two places of S and P, and of O, are used in turn), prompts
-of one length and of different ones; the oracle runs the first and the last sequence.  That a case takes this kernel is looked at."""
+a tile of 128 keys, one key range and several, ranges of one, two and more tiles (the two places of S and P, and of O, are used in turn), tiles of 64
+keys, prompts of one length and of different ones; the oracle runs the first and the last sequence.  That a case takes this kernel is looked at."""
 from dataclasses import replace
 
 import pytest
@@ -34,3 +34,25 @@ def test_tiles_and_key_ranges(hd, n_q, n_kv, B, k, P, split, spare, ragged, monk
     check(rep, f"tcgen05 attention, heads of {hd}, {n_q} / {n_kv}, B={B} k={k} P={P}")
     for p in plans:
         assert p["tcgen05"] and (p["splits"] > 1) == split, plans
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("hd,P,tile", [(128, 49, 64)] + [(hd, P, 64 if P < 68 else 128) for hd in (64, 128) for P in (64, 65, 67, 84, 100, 128, 130, 260)])
+def test_prompts_in_short_and_longer_caches(hd, P, tile, monkeypatch):
+    """Blocks of 16 prompt tokens and 8 query heads are 128 rows: tiles of 64 keys in caches of up to 80 tokens, of 128 in longer ones."""
+    b, k, B = need_gpu(), 2, 3
+    base = configs.shrunk(configs.get(2), n_layers=2, vocab=4096, n_docs=500, d_ff=1024)
+    cfg = replace(base, model=replace(base.model, d_model=16 * hd, n_q_heads=16, n_kv_heads=2, head_dim=hd), prompt_len=P)
+    plans, prefill = [], b.tasc_prefill
+
+    def watched(model, kv, *args):
+        plans.append(b.tasc_attention_plan(model, kv, B, (P + 14) // 16 * 16))
+        before = b.tasc_launch_counts()["attention_split"]
+        prefill(model, kv, *args)
+        assert b.tasc_launch_counts()["attention_split"] - before == model.shape.n_layers
+
+    monkeypatch.setattr(b, "tasc_prefill", watched)
+    s = make_setup(cfg)
+    rep = lockstep(s, corpus.make_prompts(cfg, B, prompt_len=P), 2, k, oracle_rows=[0, B - 1], lengths=[P, P // 2, P - 5], spare=-16, **BF16_TOL)
+    check(rep, f"tcgen05 attention, prompts of {P}, heads of {hd}")
+    assert [(p["tcgen05"], p["tile"]) for p in plans] == [(True, tile)]
