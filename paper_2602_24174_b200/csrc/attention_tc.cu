@@ -12,12 +12,12 @@
 //                  then O += O tile (t - 1), rescaled: O is accumulated in registers, so a new maximum costs no pass over TMEM
 //   TMA warp       K and V tiles, a ring of two or more
 // P as the MMA's A operand in TMEM takes no pass through shared memory, does not wait for P(t - 1) to be used, and leaves the ring its
-// memory, so that 128 keys make a tile for up to 128 rows too (64 before, and in short caches, see SHORT_CTX).  With up to 64 rows four of the
+// memory, so that 128 keys make a tile for up to 128 rows too (64 before, and where the plan has more of them, see plan_attention_tc).  With up to 64 rows four of the
 // eight softmax warps have any; two of the others are the TMA and the MMA warp then.
 // Key ranges split over a cluster are merged as in attention_mma.cu.
 //
-// Measured, per layer: 1.5B at 64 sequences x 7 rows and up to 1,530 keys 61 -> 33 us (2.0 us per 128 keys: softmax 0.9, its
-// half of O 0.3, P 0.4, waits 0.4; with P in TMEM and the warps' places 1.6); 0.5B + 8,192 tokens at 32 x 9 rows, 640 keys 15.5 -> 13.4; prefill of 16 x 1,024 tokens
+// Measured, per layer: 1.5B at 64 sequences x 7 rows and up to 1,530 keys 61 -> 33 us (by stamps 2.2 us per 128 keys, 2.0
+// with P in TMEM and the warps' places; the softmax 0.9 of it); 0.5B + 8,192 tokens at 32 x 9 rows, 640 keys 15.5 -> 13.4; prefill of 16 x 1,024 tokens
 // on the 1.5B 72 -> 47 us per pass of 2,048 rows.  With P in TMEM, whole steps: 1.5B, 64 x 7 rows behind 1,500 keys 4,204 -> 4,190 us, and with
 // the warps' places 4,094; 40 x 5 rows behind 1,400 2,859 -> 2,821, 2,736; 0.5B + 8,192 tokens 1,392 -> 1,370, 1,371; a prefill of
 // 4 x 1,000 tokens of the 1.5B (96 rows) 19.68 -> 19.45 ms with tiles of 64 keys, 19.90 -> 19.47 with tiles of 128.
@@ -584,13 +584,6 @@ auto with_instance(int hd, bool small, int tile, F f) {
     return hd == 64 ? f(Tc<64, 128, 128>{}) : f(Tc<128, 128, 128>{});
 }
 
-// Caches of up to so many tokens (64 and a step's 16 rows) take tiles of 64 keys for 65 to 128 rows, where most of a tile of 128 would be empty.  A prefill
-// with tiles of 128 / 64 keys, us: 1.5B, 48 tokens 1,179 / 1,157, 60 tokens 1,266 / 1,257, 16 x 48 4,384 / 4,374; 0.5B, 16 x 48 1,686 / 1,669.  Two
-// tiles of 64 for one of 128: 70 tokens 1,369 / 1,394, 0.5B 780 / 802; more of them: 1.5B, 1,000 tokens 5,929 / 6,003, 0.5B, 4 x 100 1,499 / 1,522.
-// (Key ranges dealt out in units of 64, the last tile of a range half a tile, by branches in the kernel: 48 tokens 1,171, 100 tokens 1,598
-// instead of 1,574.)
-constexpr int SHORT_CTX = 80;
-
 }  // namespace
 
 // Splits by a cost in microseconds like plan_attention_mma's: T0 to start, `per_tile` for a tile of TK keys (taken for three
@@ -603,25 +596,34 @@ constexpr int SHORT_CTX = 80;
 // bring steps here that the other kernel is faster at: 0.5B, 2 x 7 rows behind 900 keys 675 us here, 630 there, 4 x 7 rows 740 / 698, 3 x 9
 // behind 600 731 / 690.)  It pays for many (sequence, KV head) pairs with long contexts and three or
 // more slabs of query rows, hardly ever at the 135M's 18 to 27 rows.
+//   With 65 to 128 rows (prefill passes) tiles of 64 keys are weighed too: they start sooner and split finer, and two of them take longer
+// than one of 128.  A prefill of one prompt with tiles of 128 / 64 keys and the splits that go with them, us: 1.5B, 48 tokens 1,181 / 1,156, 180
+// 2,155 / 2,126, 256 2,284 / 2,258; but 100 1,571 / 1,598, 600 4,121 / 4,163, 1,000 5,929 / 6,003, 0.5B, 4 x 100 1,499 / 1,522.  A capacity of more than 64
+// keys and a step's 16 rows, up to 144 (128 and 16), hardly ever means more than 128 keys, and one tile of 128 is the better one for them: 115 tokens
+// 1,651 / 1,668, of the 0.5B 833 / 849.
 bool plan_attention_tc(int B, int n_kv, int hd, int g, int rows, int max_ctx, int page_size, AttnPlan& p) {
     const int G = g * rows;
     if ((hd != 64 && hd != 128) || page_size != PAGE || G > 128 || max_ctx / PAGE > MAX_PAGES) return false;
     const bool small = G <= 64;
-    const int tile = !small && max_ctx <= SHORT_CTX ? 64 : 128;
-    const float T0 = hd == 128 ? 4.3f : 3.2f, per_tile = hd == 128 ? (small ? 1.6f : tile == 64 ? 1.2f : 1.8f) : (small ? 1.2f : tile == 64 ? 0.95f : 1.4f);
-    const int groups = B * n_kv, tiles_all = std::max(1, (max_ctx + tile - 1) / tile), tiles_34 = std::max(1, (max_ctx * 3 / 4 + tile - 1) / tile);
+    const int groups = B * n_kv;
     const float pipes = (hd == 128 ? 0.6f : 0.3f) * (float)groups * (float)((G + 15) / 16) * (float)((max_ctx * 3 / 4 + 63) / 64) / 148.f;
-    int best = 0;
+    int best = 0, tile = 128;
     float best_cost = std::max(p.cost, 2.5f + pipes);
-    for (int s = 1; s <= 8 && s <= tiles_all; ++s) {
-        const int fit = with_instance(hd, small, tile, [&](auto c) { return clusters<decltype(c)>(s); });
-        if (fit <= 0) continue;
-        const int waves = (groups + fit - 1) / fit;
-        const float tiles = 0.5f * (float)((tiles_all + s - 1) / s + (tiles_34 + s - 1) / s);
-        // (merges and later waves as in the other kernel's plan: a layer of the 1.5B, 80 x 5 rows, 1,024 tokens of cache, 148.9 us whole
-        // and 153.4 in 2 splits, 121.7 and 132.1 behind 170 of them; 48 x 3 rows, 4,096 tokens 137.8 whole, 137.9 in 4, 82.6 and 98.3 behind 680)
-        const float cost = waves * (T0 + tiles * per_tile + (s > 1 ? 0.5f + 0.25f * s : 0.f)) + (waves - 1) * 1.0f + (groups * s > 128 ? 3.0f : 0.f);
-        if (cost < best_cost - 1e-6f) { best_cost = cost; best = s; }
+    for (int tk = 128; tk >= 64; tk -= 64) {
+        if (tk == 64 && (small || (max_ctx > 64 + 16 && max_ctx <= 128 + 16))) break;
+        const float T0 = hd == 128 ? (tk == 64 ? 3.8f : 4.3f) : (tk == 64 ? 3.1f : 3.2f);
+        const float per_tile = hd == 128 ? (small ? 1.6f : tk == 64 ? 1.3f : 1.8f) : (small ? 1.2f : tk == 64 ? 0.95f : 1.4f);
+        const int tiles_all = std::max(1, (max_ctx + tk - 1) / tk), tiles_34 = std::max(1, (max_ctx * 3 / 4 + tk - 1) / tk);
+        for (int s = 1; s <= 8 && s <= tiles_all; ++s) {
+            const int fit = with_instance(hd, small, tk, [&](auto c) { return clusters<decltype(c)>(s); });
+            if (fit <= 0) continue;
+            const int waves = (groups + fit - 1) / fit;
+            const float tiles = 0.5f * (float)((tiles_all + s - 1) / s + (tiles_34 + s - 1) / s);
+            // (merges and later waves as in the other kernel's plan: a layer of the 1.5B, 80 x 5 rows, 1,024 tokens of cache, 148.9 us whole
+            // and 153.4 in 2 splits, 121.7 and 132.1 behind 170 of them; 48 x 3 rows, 4,096 tokens 137.8 whole, 137.9 in 4, 82.6 and 98.3 behind 680)
+            const float cost = waves * (T0 + tiles * per_tile + (s > 1 ? 0.5f + 0.25f * s : 0.f)) + (waves - 1) * 1.0f + (groups * s > 128 ? 3.0f : 0.f);
+            if (cost < best_cost - 1e-6f) { best_cost = cost; best = s; tile = tk; }
+        }
     }
     if (!best) return false;
     p.tc = 1;

@@ -37,10 +37,11 @@ def test_tiles_and_key_ranges(hd, n_q, n_kv, B, k, P, split, spare, ragged, monk
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("hd,P,tile", [(128, 49, 64)] + [(hd, P, 64 if P < 68 else 128) for hd in (64, 128) for P in (64, 65, 67, 84, 100, 128, 130, 260)])
-def test_prompts_in_short_and_longer_caches(hd, P, tile, monkeypatch):
-    """Blocks of 16 prompt tokens and 8 query heads are 128 rows: tiles of 64 keys in caches of up to 80 tokens, of 128 in longer ones."""
-    b, k, B = need_gpu(), 2, 3
+@pytest.mark.parametrize("hd,B,P,tile,split", [(128, 3, 49, 64, False)] + [(hd, 3, P, 64 if P < 68 else 128, False) for hd in (64, 128) for P in (64, 65, 67, 84, 100, 128, 130, 260)]
+                         + [(hd, 1, P, 64, True) for hd in (64, 128) for P in (150, 190, 193)])
+def test_prompts_in_tiles_of_64_and_128_keys(hd, B, P, tile, split, monkeypatch):
+    """Blocks of 16 prompt tokens and 8 query heads are 128 rows: tiles of 64 keys where one or two of them hold all keys, and in several ranges."""
+    b, k = need_gpu(), 2
     base = configs.shrunk(configs.get(2), n_layers=2, vocab=4096, n_docs=500, d_ff=1024)
     cfg = replace(base, model=replace(base.model, d_model=16 * hd, n_q_heads=16, n_kv_heads=2, head_dim=hd), prompt_len=P)
     plans, prefill = [], b.tasc_prefill
@@ -53,6 +54,6 @@ def test_prompts_in_short_and_longer_caches(hd, P, tile, monkeypatch):
 
     monkeypatch.setattr(b, "tasc_prefill", watched)
     s = make_setup(cfg)
-    rep = lockstep(s, corpus.make_prompts(cfg, B, prompt_len=P), 2, k, oracle_rows=[0, B - 1], lengths=[P, P // 2, P - 5], spare=-16, **BF16_TOL)
+    rep = lockstep(s, corpus.make_prompts(cfg, B, prompt_len=P), 2, k, oracle_rows=sorted({0, B - 1}), lengths=[P, P // 2, P - 5][:B], spare=-16, **BF16_TOL)
     check(rep, f"tcgen05 attention, prompts of {P}, heads of {hd}")
-    assert [(p["tcgen05"], p["tile"]) for p in plans] == [(True, tile)]
+    assert [(p["tcgen05"], p["tile"], p["splits"] > 1) for p in plans] == [(True, tile, split)]
