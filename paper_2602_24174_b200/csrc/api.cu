@@ -244,24 +244,28 @@ tasc_status forward_f32(const tasc_model* m, const tasc_kv* kv, const Workspace&
     return TASC_OK;
 }
 
-// Whether the layers of a pass that forward_persist.cu can take run as its one persistent kernel.  Its phases cost about 2.5 us
-// less than kernels of their own, but a CTA reads the activations of all its token rows itself, so what it loses grows with rows
-// times width.  A step in us, enqueued / replayed from a graph (where the five kernels per layer follow one another more closely):
+// Whether the layers of a pass that forward_persist.cu can take run as its one persistent kernel.  It spares the boundaries between kernels, but a
+// CTA reads the activations of all its token rows itself, so what it loses grows with rows times width.  The lines below were drawn when the five
+// kernels per layer were longer: a step of the 1.5B with 7 rows behind 1,071 keys took 1,213 us enqueued / 1,140 replayed from a graph in them and
+// 1,144 / 1,137 in one, of the 135M with 6 rows 747 / 669 and 594 / 586.  Their code, their MMAs and the merge of key ranges have been cut since.
+// Now, in us:
 //     rows   7 MB per layer (135M)            30 MB (0.5B)                     94 MB (1.5B)
 //            five kernels   one kernel        five kernels   one kernel        five kernels   one kernel
-//       7                                                                      1213 / 1140    1144 / 1137
-//       6    747 / 669      594 / 586         746 / 689      650 / 640
-//       8    768 / 681      601 / 592         740 / 662      643 / 635         1223 / 1141    1132 / 1123
-//      12    791 / 694      622 / 613         762 / 686      804 / 793         1226 / 1151    1665 / 1657
-//      16    791 / 691      624 / 614         759 / 698      804 / 794         1259 / 1190    1681 / 1672
-//      18    816 / 709      758 / 749
-//      24    801 / 731      758 / 748
-//      32    822 / 744      769 / 761         795 / 729      955 / 948 (28)
-//      48                                     905 / 850      1197 / 1187
-//      96    965 / 898      1052 / 1042
-// (270 - 380, 560 and 1,071 keys).  The one kernel's time hardly changes between 17 and 32 rows and between 33 and 64 (blocks of
-// 32); a generation replays, so 17 to 32 rows are not its (plan_persist).
-// 33 to 64 rows of the 135M, since the five kernels have shorter code and token tiles of 16 rows:
+//       2    589 / 521      563 / 560         589 / 528      617 / 614          987 / 920     1110 / 1107
+//       4                                                                       999 / 936     1109 / 1105
+//       6    615 / 555      577 / 575         607 / 552      633 / 630
+//       7                                                                      1020 / 966     1126 / 1122
+//       8    622 / 561      584 / 581         625 / 569      637 / 634         1023 / 966     1129 / 1126
+//      12    627 / 568      604 / 601         617 / 565
+//      16    640 / 580      618 / 614         640 / 586
+//      18    659 / 596
+//      24    674 / 611
+//      32    708 / 654
+// (270, 560 and 1,071 keys; 1.5B, 7 rows: 100 keys 1008 / 941 and 1083 / 1080, 1,500 1050 / 990 and 1140 / 1137, 3,000 1126 / 1080 and 1265 / 1261;
+// 0.5B, 6 rows: 100 keys 601 / 539 and 610 / 607, 1,000 642 / 588 and 650 / 647.)  So up to 8 rows of the 1.5B and the 0.5B take the slower form, by 7 to
+// 13 and 1 to 5 % enqueued and by 14 to 20 and 10 to 16 % replayed; the 135M's is the faster one enqueued, by 3 to 7 %, and the slower one
+// replayed, by 4 to 8 %.  Where the one kernel is not reached any more it was slower by more: 12 rows of the 1.5B 1,665, of the 0.5B 804.
+// 33 to 64 rows of the 135M, when the five kernels had got shorter code and token tiles of 16 rows:
 //     rows   keys    five kernels   one kernel            rows   keys    five kernels   one kernel
 //      35     40      675 / 599      735 / 728              64     40      659 / 600      748 / 741
 //            150      689 / 617      773 / 768                    150      681 / 620      795 / 789
@@ -271,9 +275,8 @@ tasc_status forward_f32(const tasc_model* m, const tasc_kv* kv, const Workspace&
 // so the five kernels are the faster ones at every size, by 6 to 14 % enqueued and 16 to 22 % replayed.  Verify steps in caches of up to
 // PERSIST_BLOCKS_CTX tokens are still the one kernel's: nothing else reaches its blocks of 32 rows, and no time speaks for it.
 constexpr int PERSIST_BLOCKS_CTX = 352;
-// Its attention has at most one unit per SM and 12 key ranges, so the bytes of a unit's keys are bounded too, by 512 keys of 64:
-//     1.5B, 7 rows    1,500 keys 1235 / 1155, 1160 / 1150   3,000 (250 per unit) 1357 / 1273, 1296 / 1288   3,600 1340 / 1266, 1357 / 1348
-//     135M, 48 rows   1,500 (500 per unit) 1100 / 1010, 1070 / 1061                                         4,000 1385 / 1290, 1676 / 1666
+// Its attention has at most one unit per SM and 12 key ranges, so the bytes of a unit's keys are bounded too, by 512 keys of 64.  (135M, 48 rows, 1,500
+// keys, 500 per unit: 1,100 / 1,010 in five kernels then, 1,070 / 1,061 in one; 4,000 keys 1,385 / 1,290 and 1,676 / 1,666.)
 bool persist_pays(const tasc_model* m, int M, int R, int max_ctx, const PersistPlan& pp) {
     if (M > 32 && (R > TASC_MAX_ROWS || max_ctx > PERSIST_BLOCKS_CTX)) return false;
     if (max_ctx / pp.splits * m->desc.head_dim > 512 * 64) return false;

@@ -12,12 +12,12 @@
 //                  then O += O tile (t - 1), rescaled: O is accumulated in registers, so a new maximum costs no pass over TMEM
 //   TMA warp       K and V tiles, a ring of two or more
 // P as the MMA's A operand in TMEM takes no pass through shared memory, does not wait for P(t - 1) to be used, and leaves the ring its
-// memory, so that 128 keys make a tile for up to 128 rows too (64 before, and where the plan has more of them, see plan_attention_tc).  With up to 64 rows four of the
-// eight softmax warps have any; two of the others are the TMA and the MMA warp then.
+// memory, so that 128 keys make a tile for up to 128 rows too (64 before, and where the plan finds that better, see plan_attention_tc).  With up
+// to 64 rows four of the eight softmax warps have any; two of the others are the TMA and the MMA warp then.
 // Key ranges split over a cluster are merged as in attention_mma.cu.
 //
 // Measured, per layer: 1.5B at 64 sequences x 7 rows and up to 1,530 keys 61 -> 33 us (by stamps 2.2 us per 128 keys, 2.0
-// with P in TMEM and the warps' places; the softmax 0.9 of it); 0.5B + 8,192 tokens at 32 x 9 rows, 640 keys 15.5 -> 13.4; prefill of 16 x 1,024 tokens
+// with P in TMEM and the warps' places); 0.5B + 8,192 tokens at 32 x 9 rows, 640 keys 15.5 -> 13.4; prefill of 16 x 1,024 tokens
 // on the 1.5B 72 -> 47 us per pass of 2,048 rows.  With P in TMEM, whole steps: 1.5B, 64 x 7 rows behind 1,500 keys 4,204 -> 4,190 us, and with
 // the warps' places 4,094; 40 x 5 rows behind 1,400 2,859 -> 2,821, 2,736; 0.5B + 8,192 tokens 1,392 -> 1,370, 1,371; a prefill of
 // 4 x 1,000 tokens of the 1.5B (96 rows) 19.68 -> 19.45 ms with tiles of 64 keys, 19.90 -> 19.47 with tiles of 128.
